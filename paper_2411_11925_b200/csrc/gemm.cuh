@@ -350,6 +350,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
               for (int j = 0; j < kChunk; ++j) a0[j] = silu_t<true>(a0[j] + bias_s[c * kChunk + j]);
             } else
               modulate_chunk(a0, a1, bias_s + c * kChunk, bias_s + TN + c * kChunk, hv, rs);
+            // One thread per chunk: the row's second chunk lands where another warp reads the first chunk's h from, so every
+            // thread must have read its h before any writes.  (With two chunks per thread the order is the thread's own.)
+            if (EPI == EPI_MOD && CPT == 1) asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
             // 64 bytes of row rloc in box c / 2 (TMA's 128-byte swizzle); the modulate epilogue writes over the h it read
             uint8_t* row = (EPI == EPI_MOD ? h_s + 2 * (c >> 1) * (kTileM * 128) : out_s + (c >> 1) * (kTileM * 128)) + rloc * 128;
             __align__(16) ACT o[kChunk];
@@ -368,7 +371,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
         }
         if (EPI == EPI_GATE_RES || Cfg::kStagedOut) fence_proxy_async_smem();
         tc_fence_before_sync();   // orders the TMEM reads before the barrier that releases the buffer
-      }
+      } else if (EPI == EPI_MOD && CPT == 1) asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");   // the barrier above
       if (EPI == EPI_GATE_RES) {
         // one (mean, M2) partial per row and 64-column group
         if (CPT == 2) {            // TN = 128: this thread's two chunks are one group
