@@ -62,6 +62,7 @@ struct csd_ctx {
   cudaStream_t side[2] = {nullptr, nullptr};
   cudaEvent_t ev_fork = nullptr, ev_done[2] = {nullptr, nullptr};
   int* d_err = nullptr;
+  unsigned long long* tally() const { return reinterpret_cast<unsigned long long*>(d_err + 2); }   // tally_cap_hits
   int64_t launches = 0;
   int chain_mode = CSD_CHAIN_LAYERS;   // csd_set_chain_mode
   EncodeTiledFn encode = nullptr;
@@ -899,25 +900,41 @@ Chain make_lv_chain(csd_ctx* ctx, int slot, cudaStream_t st, const csd_head* hd,
   return c;
 }
 
+// Launches of the short kernels: the next one's blocks are set up while the preceding kernel still runs (each waits for it
+// before it touches memory), which takes about a microsecond off every kernel boundary.
+template <typename... KArgs, typename... Args>
+int launch_short(csd_ctx* ctx, cudaStream_t st, void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, const Args&... args) {
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3(grid); lc.blockDim = dim3(block); lc.dynamicSmemBytes = smem; lc.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at; lc.numAttrs = 1;
+  CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, kern, static_cast<KArgs>(args)...));
+  ctx->launches++;
+  return CSD_OK;
+}
+
 int accept_scan_lv(csd_ctx* ctx, cudaStream_t st, int B, int gamma, int C, const float* x0, const float* mu_q,
                    const float* lv_q, const float* hld_q, const float* mu_p, const float* lv_p, const float* hld_p,
                    const float* u, float* logratio, float* log_sigma_rows, int32_t* n_accept, uint32_t* mask) {
-  accept_scan_lv_kernel<<<(B + 3) / 4, 128, 0, st>>>(B, gamma, C, x0, mu_q, lv_q, hld_q, mu_p, lv_p, hld_p, u, logratio,
-                                                     log_sigma_rows, n_accept, mask);
-  ctx->launches++;
-  CSD_CUDA(ctx, cudaGetLastError());
-  return CSD_OK;
+  return launch_short(ctx, st, accept_scan_lv_kernel, (B + 3) / 4, 128, 0, B, gamma, C, x0, mu_q, lv_q, hld_q, mu_p, lv_p, hld_p,
+                      u, logratio, log_sigma_rows, n_accept, mask);
+}
+
+template <bool LV>
+int launch_resample(csd_ctx* ctx, cudaStream_t st, const ResampleParams& p) {
+  return launch_short(ctx, st, resample_kernel<LV>, (p.B + 3) / 4, 128, 0, p);
 }
 
 int resample_lv(csd_ctx* ctx, cudaStream_t st, int B, int gamma, int C, int cap, const float* log_sigma_rows,
                 const int32_t* n_accept, const float* mu_p, const float* lv_p, const float* mu_q, const float* lv_q,
                 const float* xi, const float* v, float* x_new, int32_t* n_prop, uint32_t* flags, int32_t* cap_hits) {
-  CSD_CUDA(ctx, cudaMemsetAsync(cap_hits, 0, sizeof(int32_t), st));
-  resample_lv_kernel<<<(B + 3) / 4, 128, 0, st>>>(B, gamma, C, cap, log_sigma_rows, n_accept, mu_p, lv_p, mu_q, lv_q, xi, v,
-                                                  x_new, n_prop, flags, cap_hits);
-  ctx->launches++;
-  CSD_CUDA(ctx, cudaGetLastError());
-  return CSD_OK;
+  ResampleParams p{};
+  p.B = B; p.gamma = gamma; p.C = C; p.cap = cap; p.log_sigma_rows = log_sigma_rows; p.lv_p = lv_p; p.lv_q = lv_q;
+  p.n_accept = n_accept; p.mu_p = mu_p; p.mu_q = mu_q; p.xi = xi; p.v = v; p.x_new = x_new; p.n_prop = n_prop; p.flags = flags;
+  p.cap_hits = cap_hits; p.tally = ctx->tally();
+  return launch_resample<true>(ctx, st, p);
 }
 
 double log_sigma_term(const csd_schedule* q, const csd_schedule* p, int C) {
@@ -932,24 +949,19 @@ int accept_scan(csd_ctx* ctx, cudaStream_t st, int B, int gamma, int C, double l
   const double lc = log_sigma + C * (std::log(static_cast<double>(sq1)) - std::log(static_cast<double>(sp1)));
   const float inv2vp = static_cast<float>(0.5 / (static_cast<double>(sp1) * sp1));
   const float inv2vq = static_cast<float>(0.5 / (static_cast<double>(sq1) * sq1));
-  accept_scan_kernel<<<(B + 3) / 4, 128, 0, st>>>(B, gamma, C, static_cast<float>(lc), inv2vp, inv2vq, x0, mu_q, mu_p, u,
-                                                  logratio, n_accept, mask, offset);
-  ctx->launches++;
-  CSD_CUDA(ctx, cudaGetLastError());
-  return CSD_OK;
+  return launch_short(ctx, st, accept_scan_kernel, (B + 3) / 4, 128, 0, B, gamma, C, static_cast<float>(lc), inv2vp, inv2vq, x0,
+                      mu_q, mu_p, u, logratio, n_accept, mask, offset);
 }
 
 int resample(csd_ctx* ctx, cudaStream_t st, int B, int gamma, int C, int cap, double log_sigma, float sp1, float sq1,
              const int32_t* n_accept, const float* mu_p, const float* mu_q, const float* xi, const float* v,
              float* x_new, int32_t* n_prop, uint32_t* flags, int32_t* cap_hits) {
-  CSD_CUDA(ctx, cudaMemsetAsync(cap_hits, 0, sizeof(int32_t), st));
-  resample_kernel<<<(B + 3) / 4, 128, 0, st>>>(B, gamma, C, cap, static_cast<float>(log_sigma), sp1, sq1,
-                                               static_cast<float>(std::log(static_cast<double>(sp1))),
-                                               static_cast<float>(std::log(static_cast<double>(sq1))), n_accept, mu_p,
-                                               mu_q, xi, v, x_new, n_prop, flags, cap_hits);
-  ctx->launches++;
-  CSD_CUDA(ctx, cudaGetLastError());
-  return CSD_OK;
+  ResampleParams p{};
+  p.B = B; p.gamma = gamma; p.C = C; p.cap = cap; p.log_sigma = static_cast<float>(log_sigma); p.sp1 = sp1; p.sq1 = sq1;
+  p.log_sp1 = static_cast<float>(std::log(static_cast<double>(sp1))); p.log_sq1 = static_cast<float>(std::log(static_cast<double>(sq1)));
+  p.n_accept = n_accept; p.mu_p = mu_p; p.mu_q = mu_q; p.xi = xi; p.v = v; p.x_new = x_new; p.n_prop = n_prop; p.flags = flags;
+  p.cap_hits = cap_hits; p.tally = ctx->tally();
+  return launch_resample<false>(ctx, st, p);
 }
 
 // Target chain over the R = B gamma verified positions with the B rows of position gamma + 1 appended (Alg. 1
@@ -1042,8 +1054,8 @@ int csd_create(csd_ctx** out, int device, void* cuda_stream) {
     ok = ok && cudaEventCreateWithFlags(&c->ev_done[i], cudaEventDisableTiming) == cudaSuccess;
   }
   ok = ok && cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess;
-  ok = ok && cudaMalloc(&c->d_err, 2 * sizeof(int)) == cudaSuccess;   // [0] first failed wait, [1] non-finite value seen
-  ok = ok && cudaMemset(c->d_err, 0, 2 * sizeof(int)) == cudaSuccess;
+  ok = ok && cudaMalloc(&c->d_err, 4 * sizeof(int)) == cudaSuccess;   // [0] first failed wait, [1] non-finite value seen, [2..3] tally_cap_hits
+  ok = ok && cudaMemset(c->d_err, 0, 4 * sizeof(int)) == cudaSuccess;
   void* fn = nullptr;
   cudaDriverEntryPointQueryResult qres;
   ok = ok && cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess &&
@@ -1984,10 +1996,7 @@ int csd_gmm_draft_sample(csd_ctx* ctx, int R, int C, const csd_gmm* q, const flo
   if (C < 1 || C > 32) return fail(ctx, CSD_ERR_UNSUPPORTED, "token dim C = %d must be in [1, 32]", C);
   if (!u_comp || !noise || !x) return fail(ctx, CSD_ERR_INVALID_ARG, "null array argument");
   CSD_DEVICE(ctx);
-  gmm_sample_kernel<<<(R + 3) / 4, 128, 0, ctx->stream>>>(R, C, gmm_view(q), u_comp, noise, x, comp);
-  ctx->launches++;
-  CSD_CUDA(ctx, cudaGetLastError());
-  return CSD_OK;
+  return launch_short(ctx, ctx->stream, gmm_sample_kernel, (R + 3) / 4, 128, 0, R, C, gmm_view(q), u_comp, noise, x, comp);
 }
 
 int csd_gmm_verify(csd_ctx* ctx, int B, int gamma, int C, const csd_gmm* q, const csd_gmm* p, const float* x,
@@ -2000,10 +2009,9 @@ int csd_gmm_verify(csd_ctx* ctx, int B, int gamma, int C, const csd_gmm* q, cons
   if (C < 1 || C > 32) return fail(ctx, CSD_ERR_UNSUPPORTED, "token dim C = %d must be in [1, 32]", C);
   if (!x || !u || !logratio || !n_accept) return fail(ctx, CSD_ERR_INVALID_ARG, "null array argument");
   CSD_DEVICE(ctx);
-  gmm_verify_kernel<<<B, 32 * gamma, 0, ctx->stream>>>(B, gamma, C, gmm_view(q), gmm_view(p), x, u, logratio, n_accept, accept_mask);
-  ctx->launches++;
-  CSD_CUDA(ctx, cudaGetLastError());
-  return CSD_OK;
+  auto kern = C <= 16 ? gmm_verify_kernel<16> : gmm_verify_kernel<32>;
+  return launch_short(ctx, ctx->stream, kern, B, 32 * gamma, 0, B, gamma, C, gmm_view(q), gmm_view(p), x, u, logratio, n_accept,
+                      accept_mask);
 }
 
 int csd_gmm_resample(csd_ctx* ctx, int B, int gamma, int C, int cap, const csd_gmm* q, const csd_gmm* p,
@@ -2017,12 +2025,12 @@ int csd_gmm_resample(csd_ctx* ctx, int B, int gamma, int C, int cap, const csd_g
   if (cap < 1) return fail(ctx, CSD_ERR_INVALID_ARG, "cap = %d must be >= 1", cap);
   if (!n_accept || !w || !xi || !v || !x_new || !n_prop || !flags || !cap_hits) return fail(ctx, CSD_ERR_INVALID_ARG, "null array argument");
   CSD_DEVICE(ctx);
-  CSD_CUDA(ctx, cudaMemsetAsync(cap_hits, 0, sizeof(int32_t), ctx->stream));
-  gmm_resample_kernel<<<(B + 3) / 4, 128, 0, ctx->stream>>>(B, gamma, C, cap, gmm_view(q), gmm_view(p), n_accept, w, xi, v, x_new,
-                                                            n_prop, flags, cap_hits);
-  ctx->launches++;
-  CSD_CUDA(ctx, cudaGetLastError());
-  return CSD_OK;
+  GmmResampleParams r{B, gamma, C, cap, gmm_view(q), gmm_view(p), n_accept, w, xi, v, x_new, n_prop, flags, cap_hits, ctx->tally()};
+  const size_t smem = gmm_resample_smem_floats(q->K, p->K, C) * 4;
+  const bool fits = smem <= 48 * 1024;
+  auto kern = C <= 16 ? (fits ? gmm_resample_kernel<16, true> : gmm_resample_kernel<16, false>)
+                      : (fits ? gmm_resample_kernel<32, true> : gmm_resample_kernel<32, false>);
+  return launch_short(ctx, ctx->stream, kern, B, 128, fits ? smem : 0, r);
 }
 
 int csd_round_host(csd_ctx* ctx, const csd_head* head_q, const csd_head* head_p, const csd_schedule* sched_q,

@@ -111,6 +111,8 @@ __device__ __forceinline__ void ch_fail(int* err, int role, int site, int count)
 // launch_dependents: lets the next kernel's CTAs start their prologue on free SMs.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Both, for a short kernel: nothing is read before the preceding kernel's writes are visible.
+__device__ __forceinline__ void griddep_enter() { griddep_wait(); if (threadIdx.x == 0) griddep_launch_dependents(); }
 
 // --------------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* m) {

@@ -416,6 +416,20 @@ single_path_accept_kernel(int B, int gamma, int T, const float* __restrict__ ter
   }
 }
 
+// The C coordinates of one row or proposal, zero beyond C; 16-byte loads where the row allows them.
+__device__ __forceinline__ void load_coords(const float* __restrict__ src, int C, float* z) {
+  if (C == kCPad && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+#pragma unroll
+    for (int c4 = 0; c4 < kCPad / 4; ++c4) {
+      const float4 q = __ldg(reinterpret_cast<const float4*>(src) + c4);
+      z[4 * c4] = q.x; z[4 * c4 + 1] = q.y; z[4 * c4 + 2] = q.z; z[4 * c4 + 3] = q.w;
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < kCPad; ++c) z[c] = c < C ? __ldg(src + c) : 0.0f;
+  }
+}
+
 // ---------------------------------------------------------------------------------------------
 // Verification: one warp per sequence, lane i = draft position i (gamma <= 32).
 //   logratio = log_sigma + C (log sq1 - log sp1) - |x0 - mu_p|^2 / (2 sp1^2) + |x0 - mu_q|^2 / (2 sq1^2)
@@ -426,6 +440,7 @@ accept_scan_kernel(int B, int gamma, int C, float log_const, float inv2vp, float
                    const float* __restrict__ mu_p, const float* __restrict__ u,
                    float* __restrict__ logratio, int32_t* __restrict__ n_accept,
                    uint32_t* __restrict__ accept_mask, const float* __restrict__ offset = nullptr) {
+  griddep_enter();
   const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (b >= B) return;
@@ -433,10 +448,11 @@ accept_scan_kernel(int B, int gamma, int C, float log_const, float inv2vp, float
   if (lane < gamma) {
     const size_t row = static_cast<size_t>(b) * gamma + lane;
     float dp = 0.0f, dq = 0.0f;
-    for (int c = 0; c < C; ++c) {
-      const float x = x0[row * C + c];
-      const float ep = x - mu_p[row * C + c];
-      const float eq = x - mu_q[row * C + c];
+    float xv[kCPad], pv[kCPad], qv[kCPad];       // every load of the row in flight at once
+    load_coords(x0 + row * C, C, xv); load_coords(mu_p + row * C, C, pv); load_coords(mu_q + row * C, C, qv);
+#pragma unroll
+    for (int c = 0; c < kCPad; ++c) {            // (coordinates beyond C add exact zeros)
+      const float ep = xv[c] - pv[c], eq = xv[c] - qv[c];
       dp = fmaf(ep, ep, dp);
       dq = fmaf(eq, eq, dq);
     }
@@ -508,6 +524,7 @@ accept_scan_lv_kernel(int B, int gamma, int C, const float* __restrict__ x0, con
                       const float* __restrict__ lv_p, const float* __restrict__ hld_p, const float* __restrict__ u,
                       float* __restrict__ logratio, float* __restrict__ log_sigma_rows, int32_t* __restrict__ n_accept,
                       uint32_t* __restrict__ accept_mask) {
+  griddep_enter();
   const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (b >= B) return;
@@ -532,54 +549,113 @@ accept_scan_lv_kernel(int B, int gamma, int C, const float* __restrict__ x0, con
   }
 }
 
-// Corollary 1 with diagonal final-step covariances: x' = mu_p + exp(lv_p / 2) xi, alpha_s = max(0, 1 - q(x') / (Sigma p(x')))
-// with the rejected token's own Sigma; one warp per sequence, lane c < C = coordinate.
-__global__ void __launch_bounds__(128)
-resample_lv_kernel(int B, int gamma, int C, int cap, const float* __restrict__ log_sigma_rows,
-                   const int32_t* __restrict__ n_accept, const float* __restrict__ mu_p, const float* __restrict__ lv_p,
-                   const float* __restrict__ mu_q, const float* __restrict__ lv_q, const float* __restrict__ xi,
-                   const float* __restrict__ v, float* __restrict__ x_new, int32_t* __restrict__ n_prop,
-                   uint32_t* __restrict__ flags, int32_t* __restrict__ cap_hits) {
-  const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (b >= B) return;
-  const int n = n_accept[b];
-  if (n >= gamma) {
-    if (lane == 0) { n_prop[b] = 0; flags[b] = 0u; }
-    return;
+// Sum over the 16 (padded) coordinates in the order of a butterfly reduction over 32 lanes whose upper half holds zeros.
+__device__ __forceinline__ float coord_tree_sum(float* v) {
+#pragma unroll
+  for (int o = kCPad / 2; o > 0; o >>= 1)
+#pragma unroll
+    for (int c = 0; c < o; ++c) v[c] = __fadd_rn(v[c], v[c + o]);
+  return v[0];
+}
+
+// The number of sequences whose cap was reached, summed over the blocks without a memset before the launch: every block
+// adds (its hits, 1) to one 64-bit word, the last one to arrive has the sum and leaves the word at zero for the context's
+// next call.  hits: this block's count, valid in thread 0.
+__device__ __forceinline__ void tally_cap_hits(int hits, unsigned long long* tally, int32_t* cap_hits) {
+  if (threadIdx.x != 0) return;
+  unsigned long long before = 0;
+  if (gridDim.x > 1) {
+    before = atomicAdd(tally, (static_cast<unsigned long long>(hits) << 32) | 1ull);
+    if (static_cast<unsigned>(before) != gridDim.x - 1) return;
+    *tally = 0ull;
   }
-  const size_t row = static_cast<size_t>(b) * gamma + n;
-  const bool on = lane < C;
-  const float mp = on ? mu_p[row * C + lane] : 0.0f, mq = on ? mu_q[row * C + lane] : 0.0f;
-  const float lp_d = on ? lv_p[row * C + lane] : 0.0f, lq_d = on ? lv_q[row * C + lane] : 0.0f;
-  const float sp = expf(0.5f * lp_d), ivp = 0.5f * expf(-lp_d), ivq = 0.5f * expf(-lq_d);
-  const float ls = log_sigma_rows[row];
-  float hl = on ? 0.5f * (lq_d - lp_d) : 0.0f;      // (1/2) sum_d (lv_q - lv_p): the normalisers' part of lq - lp ... negated below
+  *cap_hits = static_cast<int32_t>(before >> 32) + hits;
+}
+
+// Resampling (Cor. 1), one warp per sequence, 32 proposals at a time: lane j evaluates proposal k0 + j over all
+// coordinates, the first accepted one in order is taken.  (A warp per proposal, lane = coordinate, walks the proposals
+// one by one, each a trip to memory for xi and v and ten dependent shuffles; the sums keep that form's order.)
+// LV: diagonal final-step covariances, x' = mu_p + exp(lv_p / 2) xi with the rejected token's own Sigma.
+struct ResampleParams {
+  int B, gamma, C, cap;
+  float log_sigma, sp1, sq1, log_sp1, log_sq1;   // fixed variances
+  const float *log_sigma_rows, *lv_p, *lv_q;     // LV
+  const int32_t* n_accept;
+  const float *mu_p, *mu_q, *xi, *v;
+  float* x_new;
+  int32_t* n_prop;
+  uint32_t* flags;
+  int32_t* cap_hits;
+  unsigned long long* tally;
+};
+
+template <bool LV>
+__global__ void __launch_bounds__(128) resample_kernel(const ResampleParams p) {
+  __shared__ int hit_s[4];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int b = blockIdx.x * (blockDim.x >> 5) + warp;
+  int hit = 0;
+  griddep_enter();
+  const int n = b < p.B ? p.n_accept[b] : p.gamma;
+  // the first 32 proposals do not depend on the row: their loads travel with n_accept's
+  float z[kCPad], vk = 0.0f;
+  auto fetch = [&](int k0) {
+    const size_t pr = static_cast<size_t>(b) * p.cap + (k0 + lane < p.cap ? k0 + lane : p.cap - 1);
+    load_coords(p.xi + pr * p.C, p.C, z);
+    vk = __ldg(p.v + pr);
+  };
+  if (b < p.B) fetch(0);
+  if (n >= p.gamma) {
+    if (b < p.B && lane == 0) { p.n_prop[b] = 0; p.flags[b] = 0u; }
+  } else {
+    const size_t row = static_cast<size_t>(b) * p.gamma + n;
+    const bool on = lane < p.C;
+    const size_t o = row * p.C + lane;
+    const float mp = on ? p.mu_p[o] : 0.0f, mq = on ? p.mu_q[o] : 0.0f;
+    float sp = p.sp1, ivp = 0.5f / (p.sp1 * p.sp1), ivq = 0.5f / (p.sq1 * p.sq1), ls = p.log_sigma, hl = 0.0f;
+    if (LV) {
+      const float lp_d = on ? p.lv_p[o] : 0.0f, lq_d = on ? p.lv_q[o] : 0.0f;
+      sp = expf(0.5f * lp_d); ivp = 0.5f * expf(-lp_d); ivq = 0.5f * expf(-lq_d);
+      ls = p.log_sigma_rows[row];
+      hl = on ? 0.5f * (lq_d - lp_d) : 0.0f;       // (1/2) sum_d (lv_q - lv_p): the normalisers' part of lp - lq
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) hl += __shfl_xor_sync(0xffffffffu, hl, o);
-  float xp = 0.0f;
-  int k = 0;
-  bool done = false;
-  for (; k < cap && !done; ++k) {
-    const float z = on ? xi[(static_cast<size_t>(b) * cap + k) * C + lane] : 0.0f;
-    xp = mp + sp * z;
-    float ep = on ? (xp - mp) : 0.0f, eq = on ? (xp - mq) : 0.0f;
-    ep = ep * ep * ivp; eq = eq * eq * ivq;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      ep += __shfl_xor_sync(0xffffffffu, ep, o);
-      eq += __shfl_xor_sync(0xffffffffu, eq, o);
+      for (int s = 16; s > 0; s >>= 1) hl += __shfl_xor_sync(0xffffffffu, hl, s);
     }
-    // lq - lp = -(1/2) sum lv_q - eq + (1/2) sum lv_p + ep = -hl - eq + ep
-    const float alpha = fmaxf(0.0f, -expm1f(fminf(0.0f, (ep - eq) - hl - ls)));
-    done = v[static_cast<size_t>(b) * cap + k] <= alpha;
+    int k = p.cap;
+    bool done = false;
+    for (int k0 = 0; k0 < p.cap && !done; k0 += 32) {
+      if (k0 > 0) fetch(k0);
+      float ep[kCPad], eq[kCPad];
+#pragma unroll
+      for (int c = 0; c < kCPad; ++c) {
+        const float mpc = __shfl_sync(0xffffffffu, mp, c), mqc = __shfl_sync(0xffffffffu, mq, c);
+        const float spc = LV ? __shfl_sync(0xffffffffu, sp, c) : sp;
+        const float x = fmaf(spc, z[c], mpc);
+        const float dp = x - mpc, dq = x - mqc;
+        ep[c] = __fmul_rn(dp, dp); eq[c] = __fmul_rn(dq, dq);
+        if (LV) { ep[c] = __fmul_rn(ep[c], __shfl_sync(0xffffffffu, ivp, c)); eq[c] = __fmul_rn(eq[c], __shfl_sync(0xffffffffu, ivq, c)); }
+        if (c >= p.C) { ep[c] = 0.0f; eq[c] = 0.0f; }
+      }
+      const float se = coord_tree_sum(ep), sq = coord_tree_sum(eq);
+      float d;                                       // log q(x') - log Sigma - log p(x')
+      if (LV) d = (se - sq) - hl - ls;               // lq - lp = -(1/2) sum lv_q - sq + (1/2) sum lv_p + se
+      else {
+        const float lp = -p.C * p.log_sp1 - se * ivp;
+        const float lq = -p.C * p.log_sq1 - sq * ivq;
+        d = lq - ls - lp;
+      }
+      const float alpha = fmaxf(0.0f, -expm1f(fminf(0.0f, d)));
+      const uint32_t ok = __ballot_sync(0xffffffffu, k0 + lane < p.cap && vk <= alpha);
+      if (ok) { k = k0 + __ffs(ok); done = true; }
+    }
+    // the proposal taken (the last one when the cap was reached)
+    if (on) p.x_new[static_cast<size_t>(b) * p.C + lane] = fmaf(sp, p.xi[(static_cast<size_t>(b) * p.cap + k - 1) * p.C + lane], mp);
+    if (lane == 0) { p.n_prop[b] = k; p.flags[b] = 1u | (done ? 0u : 2u); }
+    hit = done ? 0 : 1;
   }
-  if (on) x_new[static_cast<size_t>(b) * C + lane] = xp;
-  if (lane == 0) {
-    n_prop[b] = k;
-    flags[b] = 1u | (done ? 0u : 2u);
-    if (!done) atomicAdd(cap_hits, 1);
-  }
+  if (lane == 0) hit_s[warp] = hit;
+  __syncthreads();
+  tally_cap_hits(hit_s[0] + hit_s[1] + hit_s[2] + hit_s[3], p.tally, p.cap_hits);
 }
 
 // Self-test of the bounded waits: one thread waits on a barrier on which nobody ever arrives, so the wait runs
@@ -590,53 +666,6 @@ __global__ void wait_timeout_selftest_kernel(int* err) {
   if (threadIdx.x == 0) { mbar_init(&bar, 1); fence_mbar_init(); }
   __syncthreads();
   if (threadIdx.x == 0 && !ch_wait<false>(&bar, 0, err)) ch_fail(err, 4, 1, 0);
-}
-
-// Resampling: one warp per sequence, lane c < C = coordinate.  Proposals are consumed in order.
-__global__ void __launch_bounds__(128)
-resample_kernel(int B, int gamma, int C, int cap, float log_sigma, float sp1, float sq1,
-                float log_sp1, float log_sq1, const int32_t* __restrict__ n_accept,
-                const float* __restrict__ mu_p, const float* __restrict__ mu_q,
-                const float* __restrict__ xi, const float* __restrict__ v,
-                float* __restrict__ x_new, int32_t* __restrict__ n_prop,
-                uint32_t* __restrict__ flags, int32_t* __restrict__ cap_hits) {
-  const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (b >= B) return;
-  const int n = n_accept[b];
-  if (n >= gamma) {
-    if (lane == 0) { n_prop[b] = 0; flags[b] = 0u; }
-    return;
-  }
-  const size_t row = static_cast<size_t>(b) * gamma + n;
-  const float mp = (lane < C) ? mu_p[row * C + lane] : 0.0f;
-  const float mq = (lane < C) ? mu_q[row * C + lane] : 0.0f;
-  const float inv2vp = 0.5f / (sp1 * sp1), inv2vq = 0.5f / (sq1 * sq1);
-  float xp = 0.0f;
-  int k = 0;
-  bool done = false;
-  for (; k < cap && !done; ++k) {
-    const float z = (lane < C) ? xi[(static_cast<size_t>(b) * cap + k) * C + lane] : 0.0f;
-    xp = mp + sp1 * z;
-    float ep = (lane < C) ? (xp - mp) : 0.0f;
-    float eq = (lane < C) ? (xp - mq) : 0.0f;
-    ep *= ep; eq *= eq;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      ep += __shfl_xor_sync(0xffffffffu, ep, o);
-      eq += __shfl_xor_sync(0xffffffffu, eq, o);
-    }
-    const float lp = -C * log_sp1 - ep * inv2vp;
-    const float lq = -C * log_sq1 - eq * inv2vq;
-    const float alpha = fmaxf(0.0f, -expm1f(fminf(0.0f, lq - log_sigma - lp)));
-    done = v[static_cast<size_t>(b) * cap + k] <= alpha;
-  }
-  if (lane < C) x_new[static_cast<size_t>(b) * C + lane] = xp;
-  if (lane == 0) {
-    n_prop[b] = k;
-    flags[b] = 1u | (done ? 0u : 2u);
-    if (!done) atomicAdd(cap_hits, 1);
-  }
 }
 
 }  // namespace csd
