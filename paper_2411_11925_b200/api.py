@@ -1,7 +1,8 @@
 """ctypes binding of libcsd.so: argument marshalling only.
 
 Every step of the hot path runs inside the CUDA library; this module passes
-pointers and sizes.  torch is used for device memory and streams.  There is no
+pointers and sizes (the calls that are a single short kernel go through the native
+_marshal module, the rest through ctypes).  torch is used for device memory and streams.  There is no
 CPU path: importing this module raises if the library is missing.
 """
 from __future__ import annotations
@@ -54,10 +55,6 @@ class _Schedule(C.Structure):
                 ("tfeat", C.c_void_p)]
 
 
-class _Gmm(C.Structure):
-    _fields_ = [("K", C.c_int), ("logw", C.c_void_p), ("mu", C.c_void_p), ("log_sigma", C.c_void_p)]
-
-
 class _ScheduleLV(C.Structure):
     _fields_ = [("T", C.c_int), ("a", _c_float_p), ("b", _c_float_p), ("lv_min", _c_float_p), ("lv_max", _c_float_p),
                 ("tfeat", C.c_void_p)]
@@ -85,13 +82,8 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
     lib.csd_schedule_lv_ddpm.argtypes = [i32, f64p, f64] + [_c_float_p] * 4
     lib.csd_draft_denoise_lv.argtypes = [vp, vp, C.POINTER(_ScheduleLV), i32, i32, f32] + [vp] * 8
     lib.csd_verify_lv.argtypes = [vp, vp, C.POINTER(_ScheduleLV), i32, i32, i32, f32] + [vp] * 15
-    lib.csd_resample_lv.argtypes = [vp, i32, i32, i32, i32] + [vp] * 12
     lib.csd_round_lv.argtypes = ([vp, vp, vp, C.POINTER(_ScheduleLV), C.POINTER(_ScheduleLV), i32, i32, i32, f32, i32]
                                  + [vp] * 22)
-    gp = C.POINTER(_Gmm)
-    lib.csd_gmm_draft_sample.argtypes = [vp, i32, i32, gp] + [vp] * 4
-    lib.csd_gmm_verify.argtypes = [vp, i32, i32, i32, gp, gp] + [vp] * 5
-    lib.csd_gmm_resample.argtypes = [vp, i32, i32, i32, i32, gp, gp] + [vp] * 8
     lib.csd_profile.argtypes = [vp, i32]
     lib.csd_profile_read.argtypes = [vp, i32, C.POINTER(C.c_int64), C.POINTER(f64), C.POINTER(f64)]
     lib.csd_head_create.argtypes = [vp, C.POINTER(_HeadDesc), C.POINTER(_HeadWeights), C.POINTER(vp)]
@@ -108,8 +100,6 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
     lib.csd_verify_bonus.argtypes = [vp, vp, C.POINTER(_Schedule), C.POINTER(_Schedule), i32, i32, i32, f32] + [vp] * 15
     lib.csd_round_bonus.argtypes = ([vp, vp, vp, C.POINTER(_Schedule), C.POINTER(_Schedule), i32, i32, i32, f32, i32]
                                     + [vp] * 22)
-    lib.csd_accept_scan.argtypes = [vp, i32, i32, i32, f64, f32, f32] + [vp] * 7
-    lib.csd_resample.argtypes = [vp, i32, i32, i32, i32, f64, f32, f32] + [vp] * 9
     round_args = [vp, vp, vp, C.POINTER(_Schedule), C.POINTER(_Schedule), i32, i32, i32, f32, i32] + [vp] * 17
     lib.csd_round.argtypes = round_args
     lib.csd_round_host.argtypes = round_args
@@ -120,6 +110,7 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
 
 
 _LIB = load_library()
+from . import _marshal as _fast  # noqa: E402  (linked against the library loaded above)
 
 
 def _schedule_out(n: int):
@@ -174,6 +165,9 @@ def _ptr(t) -> Optional[int]:
     raise TypeError(type(t))
 
 
+_fast.set_ptr_of(_ptr)
+
+
 class Schedule:
     """Keeps the host coefficient arrays and the device feature table alive."""
 
@@ -218,6 +212,7 @@ class Context:
         rc = _LIB.csd_create(C.byref(self._h), device, sp)
         if rc != 0:
             raise CsdError(rc, "csd_create failed")
+        self._addr = self._h.value
         self._heads = []
 
     def _check(self, rc: int):
@@ -264,6 +259,7 @@ class Context:
         if self._h:
             _LIB.csd_destroy(self._h)
             self._h = C.c_void_p()
+            self._addr = 0
 
     def __del__(self):
         try:
@@ -331,15 +327,17 @@ class Context:
 
     def csd_accept_scan(self, B, gamma, Cdim, log_sigma, sigma1_p, sigma1_q, x0_q, mu1_q, mu1_p, u, logratio,
                         n_accept, accept_mask=None):
-        self._check(_LIB.csd_accept_scan(self._h, B, gamma, Cdim, log_sigma, sigma1_p, sigma1_q, _ptr(x0_q),
-                                         _ptr(mu1_q), _ptr(mu1_p), _ptr(u), _ptr(logratio), _ptr(n_accept),
-                                         _ptr(accept_mask)))
+        rc = _fast.accept_scan(self._addr, B, gamma, Cdim, log_sigma, sigma1_p, sigma1_q, x0_q, mu1_q, mu1_p, u, logratio,
+                               n_accept, accept_mask)
+        if rc:
+            self._check(rc)
 
     def csd_resample(self, B, gamma, Cdim, cap, log_sigma, sigma1_p, sigma1_q, n_accept, mu1_p, mu1_q, xi, v,
                      x_new, n_prop, flags, cap_hits):
-        self._check(_LIB.csd_resample(self._h, B, gamma, Cdim, cap, log_sigma, sigma1_p, sigma1_q, _ptr(n_accept),
-                                      _ptr(mu1_p), _ptr(mu1_q), _ptr(xi), _ptr(v), _ptr(x_new), _ptr(n_prop),
-                                      _ptr(flags), _ptr(cap_hits)))
+        rc = _fast.resample(self._addr, B, gamma, Cdim, cap, log_sigma, sigma1_p, sigma1_q, n_accept, mu1_p, mu1_q, xi, v,
+                            x_new, n_prop, flags, cap_hits)
+        if rc:
+            self._check(rc)
 
     def csd_draft_denoise_lv(self, head: "Head", sched: ScheduleLV, R, cfg, cfg_scale, z, x_T, eps, x0, mu1, lv1,
                              half_logdet, x1=None):
@@ -356,9 +354,10 @@ class Context:
 
     def csd_resample_lv(self, B, gamma, Cdim, cap, log_sigma_rows, n_accept, mu1_p, lv1_p, mu1_q, lv1_q, xi, v, x_new,
                         n_prop, flags, cap_hits):
-        self._check(_LIB.csd_resample_lv(self._h, B, gamma, Cdim, cap,
-                                         *[_ptr(t) for t in (log_sigma_rows, n_accept, mu1_p, lv1_p, mu1_q, lv1_q, xi, v,
-                                                             x_new, n_prop, flags, cap_hits)]))
+        rc = _fast.resample_lv(self._addr, B, gamma, Cdim, cap, log_sigma_rows, n_accept, mu1_p, lv1_p, mu1_q, lv1_q, xi, v,
+                               x_new, n_prop, flags, cap_hits)
+        if rc:
+            self._check(rc)
 
     def csd_round_lv(self, head_q, head_p, sched_q: ScheduleLV, sched_p: ScheduleLV, B, gamma, cfg, cfg_scale, cap,
                      z_q, z_p, x_T, eps, u, xi, v, x0, mu1_q, lv1_q, half_logdet_q, mu1_p, lv1_p, half_logdet_p,
@@ -369,25 +368,21 @@ class Context:
                                                           mu1_p, lv1_p, half_logdet_p, log_sigma_rows, logratio, n_accept,
                                                           accept_mask, x_new, n_prop, flags, cap_hits)]))
 
-    @staticmethod
-    def _gmm(m):
-        """m: (logw [rows,K], mu [rows,K,C], log_sigma [rows,K,C]) device tensors."""
-        logw, mu, ls = m
-        return _Gmm(int(logw.shape[1]), _ptr(logw), _ptr(mu), _ptr(ls))
-
+    # mixtures q, p: (logw [rows,K], mu [rows,K,C], log_sigma [rows,K,C]) device tensors
     def csd_gmm_draft_sample(self, R, Cdim, q, u_comp, noise, x, comp=None):
-        g = self._gmm(q)
-        self._check(_LIB.csd_gmm_draft_sample(self._h, R, Cdim, C.byref(g), _ptr(u_comp), _ptr(noise), _ptr(x), _ptr(comp)))
+        rc = _fast.gmm_draft_sample(self._addr, R, Cdim, q, u_comp, noise, x, comp)
+        if rc:
+            self._check(rc)
 
     def csd_gmm_verify(self, B, gamma, Cdim, q, p, x, u, logratio, n_accept, accept_mask=None):
-        gq, gp_ = self._gmm(q), self._gmm(p)
-        self._check(_LIB.csd_gmm_verify(self._h, B, gamma, Cdim, C.byref(gq), C.byref(gp_), _ptr(x), _ptr(u), _ptr(logratio),
-                                        _ptr(n_accept), _ptr(accept_mask)))
+        rc = _fast.gmm_verify(self._addr, B, gamma, Cdim, q, p, x, u, logratio, n_accept, accept_mask)
+        if rc:
+            self._check(rc)
 
     def csd_gmm_resample(self, B, gamma, Cdim, cap, q, p, n_accept, w, xi, v, x_new, n_prop, flags, cap_hits):
-        gq, gp_ = self._gmm(q), self._gmm(p)
-        self._check(_LIB.csd_gmm_resample(self._h, B, gamma, Cdim, cap, C.byref(gq), C.byref(gp_), _ptr(n_accept), _ptr(w),
-                                          _ptr(xi), _ptr(v), _ptr(x_new), _ptr(n_prop), _ptr(flags), _ptr(cap_hits)))
+        rc = _fast.gmm_resample(self._addr, B, gamma, Cdim, cap, q, p, n_accept, w, xi, v, x_new, n_prop, flags, cap_hits)
+        if rc:
+            self._check(rc)
 
     def _round(self, fn, head_q, head_p, sched_q, sched_p, B, gamma, cfg, cfg_scale, cap, z_q, z_p, x_T, eps, u,
                xi, v, x0, mu1_q, mu1_p, logratio, n_accept, accept_mask, x_new, n_prop, flags, cap_hits):
