@@ -22,6 +22,7 @@
 #include "rowops.cuh"
 #include "smallbatch.cuh"
 #include "pchain.cuh"
+#include "f32chain.cuh"
 
 using namespace csd;
 
@@ -335,6 +336,21 @@ int launch_simt(csd_ctx* ctx, cudaStream_t st, const float* A0, int lda0, const 
   return CSD_OK;
 }
 
+// Launches of the short kernels: the next one's blocks are set up while the preceding kernel still runs (each waits for it
+// before it touches memory), which takes about a microsecond off every kernel boundary.
+template <typename... KArgs, typename... Args>
+int launch_short(csd_ctx* ctx, cudaStream_t st, void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, const Args&... args) {
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3(grid); lc.blockDim = dim3(block); lc.dynamicSmemBytes = smem; lc.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at; lc.numAttrs = 1;
+  CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, kern, static_cast<KArgs>(args)...));
+  ctx->launches++;
+  return CSD_OK;
+}
+
 int check_sched(csd_ctx* ctx, const csd_schedule* s, bool full) {
   if (!s) return fail(ctx, CSD_ERR_INVALID_ARG, "schedule is null");
   if (s->T < 1) return fail(ctx, CSD_ERR_INVALID_ARG, "schedule T = %d must be >= 1", s->T);
@@ -356,6 +372,31 @@ constexpr bool kPersistentChains = CSD_PERSISTENT_CHAINS != 0;
 #define CSD_FOLD_PAIRS 1
 #endif
 constexpr bool kFoldPairs = CSD_FOLD_PAIRS != 0;
+
+// fp32 heads: the persistent chain kernel for groups of G rows (f32chain.cuh).  False where its shared memory does not fit.
+template <int G>
+bool fc_ready(const csd_ctx* ctx, const csd_head_desc& d) {
+  static int known[kMaxDevices] = {};
+  int& k = known[ctx->device];
+  if (k == 0) {
+    k = cudaFuncSetAttribute(f32_chain_kernel<G, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess &&
+        cudaFuncSetAttribute(f32_chain_kernel<G, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess ? 1 : -1;
+    cudaGetLastError();
+  }
+  return k == 1 && fc_layout(G, d.W, d.var_out ? kCPad2 : kCPad).total * 4 <= 227 * 1024;
+}
+
+// Rows per group: the fewest that keep all groups of the chains side by side resident at once (a cluster of 8 SMs each,
+// about one cluster per GPC stays unused), where a step costs the least time; with more groups than that, the most rows
+// that fit, because every group reads all the weights.  0: none fits (W beyond about 4000).  The choice changes no bit.
+int fc_rows(const csd_ctx* ctx, const csd_head_desc& d, int R, int cfg, int chains) {
+  const int clusters = ctx->num_sms / kFcCluster - 2;
+  auto few = [&](int g) { const int per = g / (cfg ? 2 : 1); return (R + per - 1) / per * chains <= clusters; };
+  const bool ok4 = fc_ready<4>(ctx, d), ok8 = fc_ready<8>(ctx, d), ok16 = fc_ready<16>(ctx, d);
+  if (ok4 && few(4)) return 4;
+  if (ok8 && few(8)) return 8;
+  return ok16 ? 16 : ok8 ? 8 : ok4 ? 4 : 0;
+}
 
 // Shared-memory opt-in of the folded block kernels, once per device and operand type.
 bool fold_kernels_ready(const csd_ctx* ctx, const csd_head_desc& d) {
@@ -431,6 +472,7 @@ struct Chain {
   int Rh = 0, W = 0, L = 0, T = 0, tn = kTileN;
   bool sbk = false;       // the whole chain runs in the small-batch kernel (smallbatch.cuh)
   bool pck = false;       // the whole chain runs in the persistent chain kernel (pchain.cuh)
+  int fcg = 0;            // fp32 head: the whole chain runs in the fp32 chain kernel with groups of this many rows (f32chain.cuh)
   bool fold = false;      // blocks 1.. run as two kernels (fold.cuh) instead of three
   CUtensorMap tm_ap{};
   bool mod64 = false;     // modulate kernels in 64-wide tiles although the others use 128
@@ -560,10 +602,13 @@ struct Chain {
             !batch_Rin && !lv_min && !ctx->prof_on && d.C <= kCPad && pchain_kernel_ready(ctx, d.dtype);
       if (pck) { fold = false; pair = false; }
     }
+    // fp32 heads: one persistent kernel per chain, except where a row's bits have to be those of a batched pass
+    fcg = !tc && ctx->chain_mode != CSD_CHAIN_LAYERS_PLAIN && !batch_Rin && !ctx->prof_on ? fc_rows(ctx, d, R, cfg, chains) : 0;
     ChainWs& ws = ctx->ws[slot];
     int rc = batch_Rin ? ensure_ws(ctx, ws, d, ws_steps * batch_Rin * (cfg ? 2 : 1), ws_steps * batch_Rin, Ts)
                        : ensure_ws(ctx, ws, d, Rh, R, Ts);
     if (rc) return rc;
+    if (fcg) return launch_f32_chain();
     if (!batch_reuse) {
       const dim3 grid((W + 31) / 32, (Ts + 31) / 32);
       small_gemm_nt_kernel<true><<<grid, 256, 0, st>>>(sc->tfeat, hd->Wt1, hd->bt1, ws.hid, Ts, W, d.F);
@@ -707,6 +752,57 @@ struct Chain {
     return CSD_OK;
   }
 
+  static RowsGemm rows_gemm(const float* A, const float* B, const float* bias, float* C, int M, int N, int K, bool silu) {
+    return RowsGemm{A, B, bias, C, M, N, K, silu ? 1 : 0, (N + kRgCols - 1) / kRgCols};
+  }
+  int launch_rows_gemm(const RowsGemm& a, const RowsGemm* b) {
+    auto blocks = [](const RowsGemm& g) { return g.blocks_n * ((g.M + kRgRows - 1) / kRgRows); };
+    RowsGemmPair pr{{a, b ? *b : a}, blocks(a)};
+    return launch_short(ctx, st, rows_gemm_kernel, blocks(a) + (b ? blocks(*b) : 0), 256, 0, pr);
+  }
+
+  // fp32 heads: hidden layer of the timestep embedding and condition projection, the embedding, then the chain.
+  int launch_f32_chain() {
+    const csd_head_desc& d = hd->d;
+    ChainWs& ws = ctx->ws[slot];
+    const RowsGemm hid = rows_gemm(sc->tfeat, hd->Wt1, hd->bt1, ws.hid, Ts, W, d.F, true), te = rows_gemm(ws.hid, hd->Wt2, hd->bt2, ws.te, Ts, W, W, false),
+                   cz = rows_gemm(z, static_cast<const float*>(hd->Wz), hd->bz, ws.cz, Rh, W, d.Dz, false);
+    int rc;
+    if ((rc = launch_rows_gemm(hid, &cz)) || (rc = launch_rows_gemm(te, nullptr))) return rc;
+    FcParams p{};
+    p.R = R; p.cfg = cfg; p.C = d.C; p.W = W; p.L = L; p.T = Ts; p.per = fcg / (cfg ? 2 : 1); p.sample_last = sample_last; p.lv = lv_min ? 1 : 0;
+    p.cfg_scale = cfg_scale;
+    p.w = static_cast<const float*>(hd->Wss[0]); p.bias = hd->bsh[0];   // csd_head_create lays both out block after block
+    p.win = hd->win; p.bin = hd->bin; p.wout_t = hd->wout_t; p.bout = hd->bout;
+    p.cz = ws.cz; p.te = ws.te; p.x_T = x_T; p.eps = eps; p.x = ws.x; p.x0 = x0; p.mu1 = mu1; p.x1 = x1;
+    p.traj_x = traj_x; p.traj_mu = traj_mu; p.lv1 = lv1; p.half_logdet = half_logdet; p.status = ctx->d_err + 1;
+    const int groups = (R + p.per - 1) / p.per;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3(static_cast<unsigned>(groups) * kFcCluster); lc.blockDim = dim3(fcg == 16 ? FcThreads<16>::value : FcThreads<8>::value); lc.stream = st;
+    lc.dynamicSmemBytes = static_cast<size_t>(fc_layout(fcg, W, lv_min ? kCPad2 : kCPad).total) * 4;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kFcCluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at; lc.numAttrs = 2;
+    const bool narrow = W / kFcCluster <= 32;
+    auto kern = narrow ? (fcg == 16 ? f32_chain_kernel<16, 2> : fcg == 8 ? f32_chain_kernel<8, 2> : f32_chain_kernel<4, 2>)
+                       : (fcg == 16 ? f32_chain_kernel<16, 4> : fcg == 8 ? f32_chain_kernel<8, 4> : f32_chain_kernel<4, 4>);
+    for (p.t_hi = Ts; p.t_hi >= 1; p.t_hi = p.t_lo - 1) {
+      p.t_lo = p.t_hi > kFcMaxSteps ? p.t_hi - kFcMaxSteps + 1 : 1;
+      for (int t = p.t_lo; t <= p.t_hi; ++t) {
+        const int i = t - p.t_lo;
+        p.a[i] = sc->a[t - 1]; p.b[i] = sc->b[t - 1];
+        p.s0[i] = lv_min ? lv_min[t - 1] : sc->sigma[t - 1];
+        p.s1[i] = lv_min ? lv_max[t - 1] : 0.0f;
+      }
+      CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, kern, p));
+      ctx->launches++;
+    }
+    return CSD_OK;
+  }
+
   // The persistent small-batch kernel: s of every step, zeroed counters, the schedule on the device, one launch.
   int launch_small_batch() {
     const csd_head_desc& d = hd->d;
@@ -759,7 +855,7 @@ struct Chain {
   }
 
   int step(int t) {
-    if (sbk || pck) return CSD_OK;   // already enqueued by begin()
+    if (sbk || pck || fcg) return CSD_OK;   // already enqueued by begin()
     const csd_head_desc& d = hd->d;
     ChainWs& ws = ctx->ws[slot];
     cur_t = t;
@@ -898,21 +994,6 @@ Chain make_lv_chain(csd_ctx* ctx, int slot, cudaStream_t st, const csd_head* hd,
   Chain c{ctx, slot, st, hd, view, R, cfg, cfg_scale, z, x_T, eps, sample_last, x0, mu1, x1};
   c.lv_min = sc->lv_min; c.lv_max = sc->lv_max; c.lv1 = lv1; c.half_logdet = half_logdet;
   return c;
-}
-
-// Launches of the short kernels: the next one's blocks are set up while the preceding kernel still runs (each waits for it
-// before it touches memory), which takes about a microsecond off every kernel boundary.
-template <typename... KArgs, typename... Args>
-int launch_short(csd_ctx* ctx, cudaStream_t st, void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, const Args&... args) {
-  cudaLaunchConfig_t lc{};
-  lc.gridDim = dim3(grid); lc.blockDim = dim3(block); lc.dynamicSmemBytes = smem; lc.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  lc.attrs = at; lc.numAttrs = 1;
-  CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, kern, static_cast<KArgs>(args)...));
-  ctx->launches++;
-  return CSD_OK;
 }
 
 int accept_scan_lv(csd_ctx* ctx, cudaStream_t st, int B, int gamma, int C, const float* x0, const float* mu_q,
@@ -1303,6 +1384,7 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
   for (size_t c = 0; c < C; ++c) { bout_pad[c] = w->bout[c]; if (d.var_out) bout_pad[kCPad + c] = w->bout[C + c]; }
   const size_t f_win = put(win_pad.data(), win_pad.size()), f_wout = put(wout_t.data(), wout_t.size()),
                f_bout = put(bout_pad.data(), epw);
+  // (block after block, then the final pair: f32_chain_kernel walks them with one stride, as it does the matrices above)
   std::vector<size_t> f_bsh(L), f_bsc(L), f_bg(L), f_b1(L), f_b2(L);
   for (size_t k = 0; k < L; ++k) {
     f_bsh[k] = put(w->bada + k * 3 * W, W); f_bsc[k] = put(w->bada + k * 3 * W + W, W);
