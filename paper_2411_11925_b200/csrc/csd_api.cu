@@ -201,19 +201,6 @@ int make_tmap(csd_ctx* ctx, CUtensorMap* m, int dtype, const void* ptr, uint64_t
   return CSD_OK;
 }
 
-// fp32 [rows, cols] matrix read in boxes of 32 floats (128 bytes, swizzled) x 128 rows.
-int make_tmap_f32(csd_ctx* ctx, CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols) {
-  const cuuint64_t gdim[2] = {cols, rows};
-  const cuuint64_t gstride[1] = {cols * 4};
-  const cuuint32_t box[2] = {static_cast<cuuint32_t>(kChunk), static_cast<cuuint32_t>(kTileM)};
-  const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = ctx->encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(ptr), gdim, gstride, box, estr,
-                                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) return fail(ctx, CSD_ERR_CUDA, "cuTensorMapEncodeTiled (fp32) failed with code %d", (int)r);
-  return CSD_OK;
-}
-
 // Byte offsets of a chain's intermediates inside its workspace (each piece rounded up to 1 KiB) and their total.
 // The one place that knows the layout: the growable workspaces and the fixed static scratch both use it.
 struct WsLayout {
@@ -266,7 +253,7 @@ int ensure_ws(csd_ctx* ctx, ChainWs& ws, const csd_head_desc& d, int Rh, int R, 
 
 template <int EPI, int NSEG, int NMUL, int TN, typename ACT, bool PAIR>
 int launch_tc_t(csd_ctx* ctx, cudaStream_t st, const CUtensorMap& a0, const CUtensorMap& b0, const CUtensorMap& a1,
-                const CUtensorMap& b1, const CUtensorMap& th, int K0, int K1, int dep_k, int N, const EpiParams& ep,
+                const CUtensorMap& b1, int K0, int K1, int dep_k, int N, const EpiParams& ep,
                 const CUtensorMap* tout = nullptr) {
   constexpr int MMA_N = NMUL * TN;
   auto kern = gemm_tc_kernel<EPI, ACT, NSEG, MMA_N, TN, std::is_same<ACT, __half>::value ? 0 : 1, PAIR>;
@@ -299,7 +286,7 @@ int launch_tc_t(csd_ctx* ctx, cudaStream_t st, const CUtensorMap& a0, const CUte
   cfg.attrs = at; cfg.numAttrs = na;
   EpiParams e = ep;
   e.nt = N / kStatCols;   // eps partials are per 64-column group for both tile widths
-  CSD_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, a0, b0, a1, b1, th, tout ? *tout : th, K0 / kBlockK, K1 / kBlockK, dep_k / kBlockK, tiles_n, units, e,
+  CSD_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, a0, b0, a1, b1, tout ? *tout : a0, K0 / kBlockK, K1 / kBlockK, dep_k / kBlockK, tiles_n, units, e,
                                    ctx->d_err));
   ctx->launches++;
   return CSD_OK;
@@ -311,16 +298,16 @@ int launch_tc_t(csd_ctx* ctx, cudaStream_t st, const CUtensorMap& a0, const CUte
 // written by the preceding kernel.
 template <int EPI, int NSEG, int NMUL>
 int launch_tc(csd_ctx* ctx, int dtype, int tn, bool pair, cudaStream_t st, const CUtensorMap& a0, const CUtensorMap& b0,
-              const CUtensorMap& a1, const CUtensorMap& b1, const CUtensorMap& th, int K0, int K1, int dep_k,
+              const CUtensorMap& a1, const CUtensorMap& b1, int K0, int K1, int dep_k,
               int N, const EpiParams& ep, const CUtensorMap* tout = nullptr) {
   if (dtype == CSD_F16) {
-    if (tn == 64) return launch_tc_t<EPI, NSEG, NMUL, 64, __half, false>(ctx, st, a0, b0, a1, b1, th, K0, K1, dep_k, N, ep, tout);
-    if (pair) return launch_tc_t<EPI, NSEG, NMUL, 128, __half, true>(ctx, st, a0, b0, a1, b1, th, K0, K1, dep_k, N, ep, tout);
-    return launch_tc_t<EPI, NSEG, NMUL, 128, __half, false>(ctx, st, a0, b0, a1, b1, th, K0, K1, dep_k, N, ep, tout);
+    if (tn == 64) return launch_tc_t<EPI, NSEG, NMUL, 64, __half, false>(ctx, st, a0, b0, a1, b1, K0, K1, dep_k, N, ep, tout);
+    if (pair) return launch_tc_t<EPI, NSEG, NMUL, 128, __half, true>(ctx, st, a0, b0, a1, b1, K0, K1, dep_k, N, ep, tout);
+    return launch_tc_t<EPI, NSEG, NMUL, 128, __half, false>(ctx, st, a0, b0, a1, b1, K0, K1, dep_k, N, ep, tout);
   }
-  if (tn == 64) return launch_tc_t<EPI, NSEG, NMUL, 64, __nv_bfloat16, false>(ctx, st, a0, b0, a1, b1, th, K0, K1, dep_k, N, ep, tout);
-  if (pair) return launch_tc_t<EPI, NSEG, NMUL, 128, __nv_bfloat16, true>(ctx, st, a0, b0, a1, b1, th, K0, K1, dep_k, N, ep, tout);
-  return launch_tc_t<EPI, NSEG, NMUL, 128, __nv_bfloat16, false>(ctx, st, a0, b0, a1, b1, th, K0, K1, dep_k, N, ep, tout);
+  if (tn == 64) return launch_tc_t<EPI, NSEG, NMUL, 64, __nv_bfloat16, false>(ctx, st, a0, b0, a1, b1, K0, K1, dep_k, N, ep, tout);
+  if (pair) return launch_tc_t<EPI, NSEG, NMUL, 128, __nv_bfloat16, true>(ctx, st, a0, b0, a1, b1, K0, K1, dep_k, N, ep, tout);
+  return launch_tc_t<EPI, NSEG, NMUL, 128, __nv_bfloat16, false>(ctx, st, a0, b0, a1, b1, K0, K1, dep_k, N, ep, tout);
 }
 
 template <int EPI, int NSEG, int MMA_N>
@@ -480,7 +467,7 @@ struct Chain {
   bool tc = false, pair = false;
   // s is double-buffered by step parity (index t & 1): the boundary kernel that ends step t writes s of step t - 2,
   // so no product of s ever waits for the kernel right before it
-  CUtensorMap tm_z{}, tm_sb[2]{}, tm_u{}, tm_v{}, tm_h{};
+  CUtensorMap tm_z{}, tm_sb[2]{}, tm_u{}, tm_v{}, tm_u_out{}, tm_v_out{};   // _out: boxes of 32 rows, what an epilogue warp stores
   void* sbuf[2] = {nullptr, nullptr};
   int cur_t = 0;
   EpiParams ep{};
@@ -632,7 +619,8 @@ struct Chain {
       if ((rc = make_tmap(ctx, &tm_sb[0], d.dtype, ws.s2, Rh, W, W, kTileM))) return rc;
       if ((rc = make_tmap(ctx, &tm_u, d.dtype, ws.u, Rh, W, W, kTileM))) return rc;
       if ((rc = make_tmap(ctx, &tm_v, d.dtype, ws.v, Rh, W, W, kTileM))) return rc;
-      if ((rc = make_tmap_f32(ctx, &tm_h, ws.h, Rh, W))) return rc;
+      if ((rc = make_tmap(ctx, &tm_u_out, d.dtype, ws.u, Rh, W, W, 32))) return rc;
+      if ((rc = make_tmap(ctx, &tm_v_out, d.dtype, ws.v, Rh, W, W, 32))) return rc;
       if ((rc = make_tmap(ctx, &tm_ap, d.dtype, ws.ap, Rh, W, W, kTileM))) return rc;
     }
     // cz = z Wz^T + bz
@@ -641,7 +629,7 @@ struct Chain {
     e.M = Rz;
     e.bias0 = hd->bz; e.out_f32 = ws.cz;
     if (batch_reuse) rc = CSD_OK;
-    else if (tc) rc = launch_tc<EPI_BIAS_F32, 1, 1>(ctx, d.dtype, tn, pair, st, tm_z, tmw.Wz, tm_z, tmw.Wz, tm_h, d.Dz, 0, 0, W, e);
+    else if (tc) rc = launch_tc<EPI_BIAS_F32, 1, 1>(ctx, d.dtype, tn, pair, st, tm_z, tmw.Wz, tm_z, tmw.Wz, d.Dz, 0, 0, W, e);
     else rc = launch_simt<EPI_BIAS_F32, 1, 128>(ctx, st, z, d.Dz, static_cast<const float*>(hd->Wz), d.Dz, nullptr, 0,
                                                 nullptr, 0, W, e);
     if (rc) return rc;
@@ -690,7 +678,7 @@ struct Chain {
     if (!ctx->prof_on) { at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[na].val.programmaticStreamSerializationAllowed = 1; ++na; }
     lc.attrs = at; lc.numAttrs = na;
     const CUtensorMap& ts = tm_sb[cur_t & 1];
-#define CSD_FOLD_LAUNCH(ACT, FMT, KIND, PAIR) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, fold_kernel<ACT, FMT, KIND, PAIR>, ts, *tp, *ta, *tw, *tout, tm_h, tiles_n, p))
+#define CSD_FOLD_LAUNCH(ACT, FMT, KIND, PAIR) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, fold_kernel<ACT, FMT, KIND, PAIR>, ts, *tp, *ta, *tw, *tout, tiles_n, p))
     if (d.dtype == CSD_F16) {
       if (kind == FOLD_W1) { if (fp) CSD_FOLD_LAUNCH(__half, 0, FOLD_W1, true); else CSD_FOLD_LAUNCH(__half, 0, FOLD_W1, false); }
       else { if (fp) CSD_FOLD_LAUNCH(__half, 0, FOLD_GATE, true); else CSD_FOLD_LAUNCH(__half, 0, FOLD_GATE, false); }
@@ -881,8 +869,8 @@ struct Chain {
       // s of the first step is written by the kernel right before the first modulate kernel; every later s is older
       const int dep_mod = (k == 0 && t == T) ? 0 : W;
       if (folded_in) rc = CSD_OK;
-      else if (tc && mod64) rc = launch_tc<EPI_MOD, 1, 2>(ctx, d.dtype, 64, false, st, tm_s, hd->tm[0].Wss[k], tm_s, hd->tm[0].Wss[k], tm_h, W, 0, dep_mod, W, e, &tm_u);
-      else if (tc) rc = launch_tc<EPI_MOD, 1, 2>(ctx, d.dtype, tn, pair, st, tm_s, tmw.Wss[k], tm_s, tmw.Wss[k], tm_h, W, 0, dep_mod, W, e, &tm_u);
+      else if (tc && mod64) rc = launch_tc<EPI_MOD, 1, 2>(ctx, d.dtype, 64, false, st, tm_s, hd->tm[0].Wss[k], tm_s, hd->tm[0].Wss[k], W, 0, dep_mod, W, e, &tm_u_out);
+      else if (tc) rc = launch_tc<EPI_MOD, 1, 2>(ctx, d.dtype, tn, pair, st, tm_s, tmw.Wss[k], tm_s, tmw.Wss[k], W, 0, dep_mod, W, e, &tm_u_out);
       else rc = launch_simt<EPI_MOD, 1, 256>(ctx, st, sf, W, static_cast<const float*>(hd->Wss[k]), W, nullptr, 0,
                                              nullptr, 0, W, e);
       if (rc) return rc;
@@ -893,15 +881,15 @@ struct Chain {
         // CTA pairs over 256 x 256 tiles: per MMA byte the pair loads half as many operand bytes as with 256 x 128
         // tiles, and the first layer (one accumulator, K = W) is the kernel bound by that feed
         const CUtensorMap& w1 = hd->tm[1].W1[k];   // 128-row boxes: each CTA of the pair loads half of the 256 rows
-        rc = d.dtype == CSD_F16 ? launch_tc_t<EPI_SILU_ACT, 1, 1, 256, __half, true>(ctx, st, tm_u, w1, tm_u, w1, tm_h, W, 0, 0, W, e, &tm_v)
-                                : launch_tc_t<EPI_SILU_ACT, 1, 1, 256, __nv_bfloat16, true>(ctx, st, tm_u, w1, tm_u, w1, tm_h, W, 0, 0, W, e, &tm_v);
+        rc = d.dtype == CSD_F16 ? launch_tc_t<EPI_SILU_ACT, 1, 1, 256, __half, true>(ctx, st, tm_u, w1, tm_u, w1, W, 0, 0, W, e, &tm_v_out)
+                                : launch_tc_t<EPI_SILU_ACT, 1, 1, 256, __nv_bfloat16, true>(ctx, st, tm_u, w1, tm_u, w1, W, 0, 0, W, e, &tm_v_out);
       }
       else if (tc && w1_wide) {
         const CUtensorMap& w1 = hd->W1_wide[k];
-        rc = d.dtype == CSD_F16 ? launch_tc_t<EPI_SILU_ACT, 1, 1, 256, __half, false>(ctx, st, tm_u, w1, tm_u, w1, tm_h, W, 0, 0, W, e, &tm_v)
-                                : launch_tc_t<EPI_SILU_ACT, 1, 1, 256, __nv_bfloat16, false>(ctx, st, tm_u, w1, tm_u, w1, tm_h, W, 0, 0, W, e, &tm_v);
+        rc = d.dtype == CSD_F16 ? launch_tc_t<EPI_SILU_ACT, 1, 1, 256, __half, false>(ctx, st, tm_u, w1, tm_u, w1, W, 0, 0, W, e, &tm_v_out)
+                                : launch_tc_t<EPI_SILU_ACT, 1, 1, 256, __nv_bfloat16, false>(ctx, st, tm_u, w1, tm_u, w1, W, 0, 0, W, e, &tm_v_out);
       }
-      else if (tc) rc = launch_tc<EPI_SILU_ACT, 1, 1>(ctx, d.dtype, tn, pair, st, tm_u, tmw.W1[k], tm_u, tmw.W1[k], tm_h, W, 0, 0, W, e, &tm_v);
+      else if (tc) rc = launch_tc<EPI_SILU_ACT, 1, 1>(ctx, d.dtype, tn, pair, st, tm_u, tmw.W1[k], tm_u, tmw.W1[k], W, 0, 0, W, e, &tm_v_out);
       else rc = launch_simt<EPI_SILU_ACT, 1, 128>(ctx, st, uf, W, static_cast<const float*>(hd->W1[k]), W, nullptr, 0,
                                                   nullptr, 0, W, e);
       if (rc) return rc;
@@ -912,7 +900,7 @@ struct Chain {
       else if (tc) {
         EpiParams g = e;
         g.bias0 = hd->bg[k]; g.bias1 = hd->b2[k];
-        rc = launch_tc<EPI_GATE_RES, 2, 1>(ctx, d.dtype, tn, pair, st, tm_s, tmw.Wg[k], tm_v, tmw.W2[k], tm_h, W, W, W, W, g);
+        rc = launch_tc<EPI_GATE_RES, 2, 1>(ctx, d.dtype, tn, pair, st, tm_s, tmw.Wg[k], tm_v, tmw.W2[k], W, W, W, W, g);
       }
       else rc = launch_simt<EPI_GATE_RES, 2, 128>(ctx, st, vf, W, static_cast<const float*>(hd->W2[k]), W, sf, W,
                                                   static_cast<const float*>(hd->Wg[k]), W, W, e);
@@ -921,13 +909,13 @@ struct Chain {
     EpiParams e = ep;
     e.h = ws.h; e.stats = ws.stats; e.bias0 = hd->bfsh; e.bias1 = hd->bfsc; e.wout_t = hd->wout_t; e.epart = ws.epart;
     if (d.var_out) {   // 32 output columns: eps_hat | variance parameter
-      if (tc && mod64) rc = launch_tc<EPI_MODF2, 1, 2>(ctx, d.dtype, 64, false, st, tm_s, hd->tm[0].Wfss, tm_s, hd->tm[0].Wfss, tm_h, W, 0, W, W, e);
-      else if (tc) rc = launch_tc<EPI_MODF2, 1, 2>(ctx, d.dtype, tn, pair, st, tm_s, tmw.Wfss, tm_s, tmw.Wfss, tm_h, W, 0, W, W, e);
+      if (tc && mod64) rc = launch_tc<EPI_MODF2, 1, 2>(ctx, d.dtype, 64, false, st, tm_s, hd->tm[0].Wfss, tm_s, hd->tm[0].Wfss, W, 0, W, W, e);
+      else if (tc) rc = launch_tc<EPI_MODF2, 1, 2>(ctx, d.dtype, tn, pair, st, tm_s, tmw.Wfss, tm_s, tmw.Wfss, W, 0, W, W, e);
       else rc = launch_simt<EPI_MODF2, 1, 256>(ctx, st, sf, W, static_cast<const float*>(hd->Wfss), W, nullptr, 0, nullptr,
                                                0, W, e);
     }
-    else if (tc && mod64) rc = launch_tc<EPI_MODF, 1, 2>(ctx, d.dtype, 64, false, st, tm_s, hd->tm[0].Wfss, tm_s, hd->tm[0].Wfss, tm_h, W, 0, W, W, e);
-    else if (tc) rc = launch_tc<EPI_MODF, 1, 2>(ctx, d.dtype, tn, pair, st, tm_s, tmw.Wfss, tm_s, tmw.Wfss, tm_h, W, 0, W, W, e);
+    else if (tc && mod64) rc = launch_tc<EPI_MODF, 1, 2>(ctx, d.dtype, 64, false, st, tm_s, hd->tm[0].Wfss, tm_s, hd->tm[0].Wfss, W, 0, W, W, e);
+    else if (tc) rc = launch_tc<EPI_MODF, 1, 2>(ctx, d.dtype, tn, pair, st, tm_s, tmw.Wfss, tm_s, tmw.Wfss, W, 0, W, W, e);
     else rc = launch_simt<EPI_MODF, 1, 256>(ctx, st, sf, W, static_cast<const float*>(hd->Wfss), W, nullptr, 0, nullptr,
                                             0, W, e);
     if (rc) return rc;

@@ -36,12 +36,24 @@ struct EpiParams {
   const float* bias1;    // [N]
   float* out_f32;        // EPI_BIAS_F32
   void* out_act;         // EPI_SILU_ACT, EPI_MOD
-  float* h;              // EPI_MOD / EPI_MODF (read), EPI_GATE_RES (read-modify-write)
+  float* h;              // EPI_MOD / EPI_MODF (read), EPI_GATE_RES (read-modify-write); tensor-core kernels: tiled_off
   int nt;                // eps partials per row: N/64 (tensor-core kernel), N/128 (FMA kernel)
-  float* stats;          // [M, ldo/64, 2] (mean, M2) per 64-column group of h
+  float* stats;          // [M, ldo/64, 2] (mean, M2) per 64-column group of h; tensor-core kernels: tiled_off
   const float* wout_t;   // [N, 16 or 32] fp32, Wout transposed and zero padded (EPI_MODF, EPI_MODF2)
   float* epart;          // [M, nt, 16 or 32] (EPI_MODF, EPI_MODF2)
 };
+
+// Layout of the residual stream h [M, W] and of the LayerNorm partials [M, 2 W/64] on the tensor-core path: tiles of 32 rows,
+// inside a tile quads of four columns, inside a quad the tile's rows (the last tile has as many as are left).  An epilogue
+// thread owns a row and a warp 32 of them, so a warp's 16-byte access covers 512 contiguous bytes and its 32 columns are one
+// contiguous 4 KB block; row-major an access would touch 32 lines, and such bursts held up the mainloop's operand loads.
+__host__ __device__ __forceinline__ int tiled_rows(int m, int M) { const int left = M - (m & ~31); return left < 32 ? left : 32; }
+// Offset in floats of column quad c4 of row m.
+__host__ __device__ __forceinline__ size_t tiled_off(int m, int c4, int M, int cols) {
+  return static_cast<size_t>(m & ~31) * cols + (static_cast<size_t>(c4) * tiled_rows(m, M) + (m & 31)) * 4;
+}
+// Offset in float2 of the (mean, M2) partial of 64-column group g of row m (G groups a row).
+__host__ __device__ __forceinline__ size_t tiled_stat_off(int m, int g, int M, int G) { return tiled_off(m, g >> 1, M, 2 * G) / 2 + (g & 1); }
 
 __device__ __forceinline__ float silu_f(float x) { return x / (1.0f + expf(-x)); }
 // Fast variant for the tensor-core path (its result is rounded to a 16-bit operand anyway).
@@ -126,16 +138,16 @@ __device__ __forceinline__ void chan_merge_equal(float& ma, float& m2a, float mb
 // no chain of dependent divisions.  Sums run in group order, so the result does not depend on which
 // CTA computes it.  Up to 24 groups (W <= 1536) are loaded once, as one batch of 16-byte loads.
 // CG: read past the L1 cache (the partials were written by other CTAs of the same kernel).
-// p: the row's G (mean, M2) pairs, 16-byte aligned.
+// p: the row's G (mean, M2) pairs, 16-byte aligned; two pairs per float4, stride apart.
 template <bool CG = false>
-__device__ __forceinline__ void row_stats_at(const float4* p, int W, float& mean, float& rstd) {
+__device__ __forceinline__ void row_stats_at(const float4* p, int W, float& mean, float& rstd, int stride = 1) {
   const int G = W / kStatCols;   // even: W is a multiple of 128
   constexpr int kB = 12;         // 16-byte loads (two groups each) per batch
   float sum = 0.0f, m2 = 0.0f, q = 0.0f;
   if (G <= 2 * kB) {
     float4 b[kB];
 #pragma unroll
-    for (int j = 0; j < kB; ++j) b[j] = (2 * j < G) ? (CG ? __ldcg(p + j) : p[j]) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int j = 0; j < kB; ++j) b[j] = (2 * j < G) ? (CG ? __ldcg(p + j * stride) : p[j * stride]) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
     for (int j = 0; j < kB; ++j)
       if (2 * j < G) { sum += b[j].x; sum += b[j].z; m2 += b[j].y; m2 += b[j].w; }
@@ -144,10 +156,10 @@ __device__ __forceinline__ void row_stats_at(const float4* p, int W, float& mean
     for (int j = 0; j < kB; ++j)
       if (2 * j < G) { const float d0 = b[j].x - mean, d1 = b[j].z - mean; q = fmaf(d0, d0, q); q = fmaf(d1, d1, q); }
   } else {
-    for (int j = 0; j < G / 2; ++j) { const float4 b = CG ? __ldcg(p + j) : p[j]; sum += b.x; sum += b.z; m2 += b.y; m2 += b.w; }
+    for (int j = 0; j < G / 2; ++j) { const float4 b = CG ? __ldcg(p + j * stride) : p[j * stride]; sum += b.x; sum += b.z; m2 += b.y; m2 += b.w; }
     mean = sum / static_cast<float>(G);
     for (int j = 0; j < G / 2; ++j) {
-      const float4 b = CG ? __ldcg(p + j) : p[j];
+      const float4 b = CG ? __ldcg(p + j * stride) : p[j * stride];
       const float d0 = b.x - mean, d1 = b.z - mean;
       q = fmaf(d0, d0, q); q = fmaf(d1, d1, q);
     }
@@ -161,9 +173,35 @@ __device__ __forceinline__ void row_stats(const float* stats, int m, int W, floa
   row_stats_at<CG>(reinterpret_cast<const float4*>(stats) + static_cast<size_t>(m) * (W / kStatCols / 2), W, mean, rstd);
 }
 
-template <int EPI>
+// The same from partials in the tiled layout (M rows).
+__device__ __forceinline__ void row_stats_tiled(const float* stats, int m, int M, int W, float& mean, float& rstd) {
+  row_stats_at<true>(reinterpret_cast<const float4*>(stats + tiled_off(m, 0, M, W / kStatCols * 2)), W, mean, rstd, tiled_rows(m, M));
+}
+
+// 32 consecutive columns (from n0) of row m of h in the tiled layout.
+__device__ __forceinline__ void load_h_tiled(const float* h, int m, int n0, int M, int W, float* v) {
+  const int rt = tiled_rows(m, M);
+  const float4* s = reinterpret_cast<const float4*>(h + tiled_off(m, n0 >> 2, M, W));
+#pragma unroll
+  for (int j = 0; j < kChunk / 4; ++j) {
+    const float4 x = __ldcg(s + j * rt);
+    v[4 * j] = x.x; v[4 * j + 1] = x.y; v[4 * j + 2] = x.z; v[4 * j + 3] = x.w;
+  }
+}
+__device__ __forceinline__ void store_h_tiled(float* h, int m, int n0, int M, int W, const float* v) {
+  const int rt = tiled_rows(m, M);
+  float4* d = reinterpret_cast<float4*>(h + tiled_off(m, n0 >> 2, M, W));
+#pragma unroll
+  for (int j = 0; j < kChunk / 4; ++j) d[j * rt] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+}
+
+// TILED: the tensor-core path's layout of the partials.
+template <int EPI, bool TILED>
 __device__ __forceinline__ void epi_row_begin(const EpiParams& ep, int m, RowState& rs) {
-  if constexpr (EPI == EPI_MOD || epi_is_modf<EPI>()) row_stats<false>(ep.stats, m, ep.ldo, rs.mean, rs.rstd);
+  if constexpr (EPI == EPI_MOD || epi_is_modf<EPI>()) {
+    if constexpr (TILED) row_stats_tiled(ep.stats, m, ep.M, ep.ldo, rs.mean, rs.rstd);
+    else row_stats<false>(ep.stats, m, ep.ldo, rs.mean, rs.rstd);
+  }
   if constexpr (epi_is_modf<EPI>()) {
 #pragma unroll
     for (int c = 0; c < epi_out_width<EPI>(); ++c) rs.eacc[c] = 0.0f;
@@ -254,8 +292,10 @@ __device__ __forceinline__ void epi_chunk(const EpiParams& ep, int m, int n0, fl
 }
 
 // Writes the (mean, M2) partial of one row over 64-column group g.
+template <bool TILED>
 __device__ __forceinline__ void store_group_stats(const EpiParams& ep, int m, int g, float mean, float m2) {
-  reinterpret_cast<float2*>(ep.stats)[static_cast<size_t>(m) * (ep.ldo / kStatCols) + g] = make_float2(mean, m2);
+  const int G = ep.ldo / kStatCols;
+  reinterpret_cast<float2*>(ep.stats)[TILED ? tiled_stat_off(m, g, ep.M, G) : static_cast<size_t>(m) * G + g] = make_float2(mean, m2);
 }
 
 template <int EPI>

@@ -55,7 +55,7 @@ template <typename ACT, int AB_FMT, int KIND, bool PAIR>
 __global__ void __launch_bounds__(kFoldThreads, 1)
 fold_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ CUtensorMap tmWp,
             const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
-            const __grid_constant__ CUtensorMap tmOut, const __grid_constant__ CUtensorMap tmHst, int tiles_n,
+            const __grid_constant__ CUtensorMap tmOut, int tiles_n,
             const FoldParams p) {
   using Cfg = FoldCfg<KIND>;
   // Ring stages.  Alone: three of 64 KB; early product [A 16 KB | packed 256-row weight tile 32 KB], dependent product two
@@ -86,7 +86,6 @@ fold_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ CUt
   if (threadIdx.x == 0) {
     tma_prefetch_desc(&tmS); tma_prefetch_desc(&tmWp); tma_prefetch_desc(&tmA); tma_prefetch_desc(&tmW);
     tma_prefetch_desc(&tmOut);
-    if (KIND == FOLD_GATE) tma_prefetch_desc(&tmHst);
     for (int s = 0; s < SP; ++s) { mbar_init(&full_bar[s], 3); mbar_init(&empty_bar[s], 1); }
     mbar_init(&acc_full[0], 1); mbar_init(&acc_full[1], 1);
     fence_mbar_init();
@@ -225,20 +224,15 @@ fold_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ CUt
     if (et == 0) griddep_launch_dependents();   // (letting the next kernel start before this wait was measured slower)
     float hv2[2][kChunk];
     if (KIND == FOLD_GATE) {
-      // h of this thread's 64 columns, read past L1 (its writer may have overlapped this kernel's start)
+      // h of this thread's 64 columns, requested before the accumulators are awaited
 #pragma unroll
       for (int ci = 0; ci < 2; ++ci) {
-        const float4* src = reinterpret_cast<const float4*>(p.h + static_cast<size_t>(valid ? m : 0) * W + n_base + (2 * half + ci) * kChunk);
-#pragma unroll
-        for (int i = 0; i < kChunk / 4; ++i) {
-          const float4 v4 = __ldcg(src + i);
-          hv2[ci][4 * i] = v4.x; hv2[ci][4 * i + 1] = v4.y; hv2[ci][4 * i + 2] = v4.z; hv2[ci][4 * i + 3] = v4.w;
-        }
+        if (valid) load_h_tiled(p.h, m, n_base + (2 * half + ci) * kChunk, p.M, W, hv2[ci]);
       }
     }
-    // The outputs leave through shared memory and TMA stores: a thread owns a row, so direct stores would touch 32
+    // The 16-bit output leaves through shared memory and TMA stores: a thread owns a row, so direct stores would touch 32
     // rows per instruction, 16 bytes each (measured: they, not the arithmetic, set the epilogue's length).  The ring
-    // is free once the last MMA has completed: 16-bit tile in two boxes of 64 columns at its start, fp32 h behind.
+    // is free once the last MMA has completed: two boxes of 64 columns at its start.  (h has a layout of its own: tiled_off.)
     auto stage_act = [&](int c, const float* v) {
       uint8_t* row = ring + (c >> 1) * (kTileM * 128) + rloc * 128;
       ACT o[kChunk];
@@ -250,7 +244,7 @@ fold_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ CUt
     };
     RowState rs;
     rs.mean = 0.0f; rs.rstd = 0.0f; rs.pm = 0.0f; rs.pm2 = 0.0f; rs.pn = 0.0f;
-    if (KIND == FOLD_W1 && valid) row_stats<true>(p.stats_in, m, W, rs.mean, rs.rstd);
+    if (KIND == FOLD_W1 && valid) row_stats_tiled(p.stats_in, m, p.M, W, rs.mean, rs.rstd);
     asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");   // constants are in place
     bar_wait(&acc_full[0], 3);
     bar_wait(&acc_full[1], 4);
@@ -277,7 +271,7 @@ fold_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ CUt
         } else {
           float* hv = hv2[ci];
           gate_res_chunk(a0, am, bias_s + c * kChunk, bias_s + 128 + c * kChunk, hv, rs);
-          store_swizzled_row32(ring + 32768 + c * (kTileM * 128), rloc, hv);   // new h, one fp32 box per chunk
+          if (valid) store_h_tiled(p.h, m, n_base + c * kChunk, p.M, W, hv);
           const float* ks = bias_s + 256 + c * kChunk;
 #pragma unroll
           for (int j = 0; j < kChunk; ++j) hv[j] = __fmul_rn(hv[j], __fadd_rn(1.0f, __fadd_rn(a1[j], ks[j])));
@@ -285,17 +279,13 @@ fold_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ CUt
         }
       }
       if (KIND == FOLD_GATE && valid)
-        reinterpret_cast<float2*>(p.stats_out)[static_cast<size_t>(m) * (W / kStatCols) + tile_n * 2 + half] = make_float2(rs.pm, rs.pm2);
+        reinterpret_cast<float2*>(p.stats_out)[tiled_stat_off(m, tile_n * 2 + half, p.M, W / kStatCols)] = make_float2(rs.pm, rs.pm2);
     }
     fence_proxy_async_smem();
     asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
     if (et == 0 && ok) {
       tma_store_2d(&tmOut, ring, n_base, row0);
       tma_store_2d(&tmOut, ring + kTileM * 128, n_base + 64, row0);
-      if (KIND == FOLD_GATE) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) tma_store_2d(&tmHst, ring + 32768 + c * (kTileM * 128), n_base + c * kChunk, row0);
-      }
       tma_store_commit();
       tma_store_wait_all();
     }

@@ -18,10 +18,10 @@ namespace csd {
 
 constexpr int kBlockK = 64;  // bf16 elements per TMA box row = 128 bytes = one swizzle row
 // Warp roles: warp 0 TMA (A), warp 1 MMA, then the epilogue warps, last warp TMA (B).  A tile has
-// TN/32 column chunks x 4 TMEM lane quarters; the cheap epilogues of 128-wide tiles run 16 warps
-// (one chunk per thread), everything else 8 warps (two chunks per thread, or one when TN = 64).
+// TN/32 column chunks x 4 TMEM lane quarters; 256-wide tiles run 16 warps, everything else 8 (two chunks per
+// thread, or one when TN = 64), the condition projection 16 with one chunk per thread.
 template <int EPI, int TN> struct TcWarps {
-  static constexpr int kEpi = (TN >= 128 && (EPI == EPI_SILU_ACT || EPI == EPI_BIAS_F32)) ? 16 : 8;
+  static constexpr int kEpi = (TN == 256 || (TN == 128 && EPI == EPI_BIAS_F32)) ? 16 : 8;
   static constexpr int kThreads = (kEpi + 3) * 32;
   static constexpr int kChunksPerThread = (TN / kChunk) * 4 / kEpi;
 };
@@ -31,7 +31,6 @@ enum DevErr : int { DEV_OK = 0, DEV_ERR_TMA_WAIT = 1, DEV_ERR_MMA_WAIT = 2, DEV_
 // PAIR: two CTAs of a cluster share one MMA (cta_group::2, M = 256): each holds its own 128 rows of A
 // and half of the B rows, which cuts the shared-memory traffic per CTA and k-block.
 template <int EPI, int MMA_N, int TN, bool PAIR> struct TcCfg {
-  static constexpr bool kStageH = EPI == EPI_MOD || epi_is_modf<EPI>() || EPI == EPI_GATE_RES;
   // A stage holds kKps k-blocks of 64 elements (one TMA box per operand and k-block).  The kernels whose
   // MMAs are 128 wide use two: fewer barrier round trips per byte.
   static constexpr int kKps = ((EPI == EPI_SILU_ACT || EPI == EPI_GATE_RES) && MMA_N <= 128) ? 2 : 1;
@@ -41,40 +40,28 @@ template <int EPI, int MMA_N, int TN, bool PAIR> struct TcCfg {
   static constexpr int kABytes = kKps * kABoxBytes;
   static constexpr int kBBytes = kKps * kBBoxBytes;
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kHTileBytes = kTileM * TN * 4;        // fp32 h tile staged in shared memory
-  static constexpr int kHBytes = kStageH ? kHTileBytes : 0;
   // 16-bit output tiles (SiLU and modulate epilogues) leave through shared memory and TMA stores: a thread owns a row,
   // so direct stores touch 32 lines per instruction, and such bursts hold up the TMA loads of the next tile's
-  // mainloop.  The modulate epilogue reuses the h tile it has just read; the SiLU epilogue gets a buffer of its own.
+  // mainloop.  Each warp stores its own 32 rows x 64 columns (4 KB) as soon as it has them: a whole tile in one go kept the
+  // TMA unit from the mainloop's loads for 1.5 to 2 k cycles.
   static constexpr bool kStagedOut = EPI == EPI_SILU_ACT || EPI == EPI_MOD;
-  static constexpr int kOutBytes = EPI == EPI_SILU_ACT ? kTileM * TN * 2 : 0;
   static constexpr int kWoutBytes = epi_is_modf<EPI>() ? kTileM * epi_out_width<EPI>() * 4 : 0;   // Wout^T tile [TN][16 or 32], reused for [128 rows][..] partials
-  static constexpr int kXchBytes = (EPI == EPI_GATE_RES || epi_is_modf<EPI>()) ? kTileM * 16 : 0;   // per-row exchange between column halves
-  static constexpr int kMiscBytes = 2 * TN * 4 + kXchBytes;     // two bias slices + exchange
+  // h comes in through shared memory, a warp's 32 x 32 block at a time (4 KB, contiguous), requested a tile ahead: loads into
+  // registers at the start of a tile took 4 k cycles behind the operand traffic and stood in front of every epilogue.  The
+  // ring's depth is what covers the operands' latency, so the gated kernel stages one of a warp's two blocks and loads the
+  // other late, and the modulate kernel's outgoing piece takes the place of the block it has read.
+  static constexpr int kHChunks = !epi_reads_h<EPI>() ? 0 : EPI == EPI_GATE_RES ? 1 : TcWarps<EPI, TN>::kChunksPerThread;
+  static constexpr bool kOutOverH = EPI == EPI_MOD && TN == 128;
+  static constexpr int kHBytes = 8 * kHChunks * 4096;
+  static constexpr int kOutBytes = kStagedOut && !kOutOverH ? kTileM * TN * 2 : 0;
+  static constexpr int kXchBytes = EPI == EPI_GATE_RES && TN == 64 ? kTileM * 16 : 0;   // per-row exchange between column halves
+  static constexpr int kBiasSlices = EPI == EPI_SILU_ACT || EPI == EPI_BIAS_F32 ? 1 : 2;
+  static constexpr int kMiscBytes = kBiasSlices * TN * 4 + kXchBytes;     // bias slices + exchange
   static constexpr int kFixedBytes = 1024 + kHBytes + kOutBytes + kWoutBytes + kMiscBytes + 256;
   static constexpr int kStagesMax = (227 * 1024 - kFixedBytes) / kStageBytes;
   static constexpr int kStages = kStagesMax > 8 ? 8 : kStagesMax;
   static constexpr int kSmemBytes = kFixedBytes + kStages * kStageBytes;
 };
-
-// Reads 32 consecutive floats of row r from a [128 rows][128 bytes] tile that TMA wrote with the
-// 128-byte swizzle (16-byte unit j of row r lives at unit j ^ (r & 7)).
-__device__ __forceinline__ void load_swizzled_row32(const uint8_t* tile, int r, float* v) {
-  const uint8_t* row = tile + r * 128;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const float4 q = *reinterpret_cast<const float4*>(row + ((j ^ (r & 7)) << 4));
-    v[4 * j] = q.x; v[4 * j + 1] = q.y; v[4 * j + 2] = q.z; v[4 * j + 3] = q.w;
-  }
-}
-
-// The inverse: writes 32 floats of row r in the layout a TMA store with the 128-byte swizzle expects.
-__device__ __forceinline__ void store_swizzled_row32(uint8_t* tile, int r, const float* v) {
-  uint8_t* row = tile + r * 128;
-#pragma unroll
-  for (int j = 0; j < 8; ++j)
-    *reinterpret_cast<float4*>(row + ((j ^ (r & 7)) << 4)) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-}
 
 // Persistent over tiles: CTA b handles output tiles b, b + gridDim.x, ... (column tile fastest).  The
 // shared-memory ring runs on across tiles; the accumulators are double-buffered in TMEM, so the
@@ -83,13 +70,12 @@ template <int EPI, typename ACT, int NSEG, int MMA_N, int TN, int AB_FMT, bool P
 __global__ void __launch_bounds__(TcWarps<EPI, TN>::kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
                const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
-               const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmOut, int nkb0, int nkb1, int dep_kb,
+               const __grid_constant__ CUtensorMap tmOut, int nkb0, int nkb1, int dep_kb,
                int tiles_n, int tiles_total,
                EpiParams ep, int* err) {
   using Cfg = TcCfg<EPI, MMA_N, TN, PAIR>;
   constexpr int S = Cfg::kStages;
   constexpr int EW = TcWarps<EPI, TN>::kEpi, CPT = TcWarps<EPI, TN>::kChunksPerThread, kEpiThreads = EW * 32;
-  constexpr int NC = TN / kChunk;               // column chunks per tile
   constexpr bool kPacked = (NSEG == 1) && (MMA_N == 2 * TN);
   constexpr int EPW = epi_out_width<EPI>();   // output-projection columns (EPI_MODF, EPI_MODF2)
   constexpr bool kTwoAcc = kPacked || NSEG == 2;
@@ -99,17 +85,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* stage_base = smem;
-  uint8_t* h_s = smem + S * Cfg::kStageBytes;                    // NC chunks of [128 rows][128 B], swizzled
-  uint8_t* out_s = h_s + Cfg::kHBytes;                           // SiLU epilogue: outgoing 16-bit tile, boxes of 64 columns
+  uint8_t* h_s = smem + S * Cfg::kStageBytes;                    // per epilogue warp kHChunks blocks of [8 quads][32 rows][16 B]
+  uint8_t* out_s = h_s + Cfg::kHBytes;                           // outgoing 16-bit tile, pieces of [32 rows][128 B], swizzled
   float* wout_s = reinterpret_cast<float*>(out_s + Cfg::kOutBytes);
-  float* bias_s = reinterpret_cast<float*>(out_s + Cfg::kOutBytes + Cfg::kWoutBytes);
-  float* xch_s = bias_s + 2 * TN;                            // [128 rows][4] exchange between column halves
+  float* bias_s = reinterpret_cast<float*>(out_s + Cfg::kOutBytes + Cfg::kWoutBytes);   // [slices][TN]
+  float* xch_s = bias_s + Cfg::kBiasSlices * TN;       // [128 rows][4] exchange between column halves
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(out_s + Cfg::kOutBytes + Cfg::kWoutBytes + Cfg::kMiscBytes);
   uint64_t* empty_bar = full_bar + S;
   uint64_t* tmem_full_bar = empty_bar + S;      // [2]
   uint64_t* tmem_empty_bar = tmem_full_bar + 2; // [2]
-  uint64_t* h_bar = tmem_empty_bar + 2;
-  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(h_bar + 1);
+  uint64_t* h_bar = tmem_empty_bar + 2;         // [8], one per epilogue warp
+  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(h_bar + 8);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int KPS = Cfg::kKps;
@@ -146,12 +132,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
     tma_prefetch_desc(&tmA0);
     tma_prefetch_desc(&tmB0);
     if (NSEG == 2) { tma_prefetch_desc(&tmA1); tma_prefetch_desc(&tmB1); }
-    if (Cfg::kStageH) tma_prefetch_desc(&tmH);
     if (Cfg::kStagedOut) tma_prefetch_desc(&tmOut);
     for (int s = 0; s < S; ++s) { mbar_init(&full_bar[s], 2); mbar_init(&empty_bar[s], 1); }
-    // a pair's accumulator buffer is released by the epilogues of both CTAs (to the leader's barrier)
-    for (int i = 0; i < 2; ++i) { mbar_init(&tmem_full_bar[i], 1); mbar_init(&tmem_empty_bar[i], PAIR ? 2 : 1); }
-    mbar_init(h_bar, 1);
+    // an accumulator buffer is released by every epilogue warp (of a pair, of both CTAs, to the leader's barrier)
+    for (int i = 0; i < 2; ++i) { mbar_init(&tmem_full_bar[i], 1); mbar_init(&tmem_empty_bar[i], PAIR ? 2 * EW : EW); }
+    if (Cfg::kHChunks) for (int i = 0; i < 8; ++i) mbar_init(&h_bar[i], 1);
     fence_mbar_init();
   }
   if (warp == 1) {
@@ -214,7 +199,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
       for (int i = 0; i < my_tiles && ok; ++i) {
         const int ab = i & 1;
         // the epilogue must have drained this accumulator buffer (tile i - 2)
-        if (i >= 2 && !mbar_wait(&tmem_empty_bar[ab], ((i >> 1) - 1) & 1)) { if (leader) atomicExch(err, DEV_ERR_MMA_WAIT); ok = false; break; }
+        if (i >= 2 && !ch_wait<PAIR>(&tmem_empty_bar[ab], ((i >> 1) - 1) & 1, err)) { if (leader) atomicExch(err, DEV_ERR_MMA_WAIT); ok = false; break; }
         tc_fence_after_sync();
         for (int kb = 0; kb < total_kb; ++kb, ++it) {
           const int s = it % S;
@@ -257,21 +242,54 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
     // (at most one kernel runs ahead).
     // per-tile constants (biases, the Wout^T tile): not written by any kernel, so those of the first tile
     // are staged before the wait
-    auto stage_consts = [&](int tile_n) {
+    auto epi_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); };
+    // (two steps: the loads are requested with the tile's other loads, what they bring is put away after them)
+    float cb0 = 0.0f, cb1 = 0.0f;
+    float4 cw[epi_is_modf<EPI>() ? TN * EPW / 4 / kEpiThreads : 1];
+    auto fetch_consts = [&](int tile_n) {
       if (et < TN) {
-        bias_s[et] = ep.bias0[tile_n * TN + et];
-        bias_s[TN + et] = ep.bias1 ? ep.bias1[tile_n * TN + et] : 0.0f;
+        cb0 = __ldg(ep.bias0 + tile_n * TN + et);
+        if (Cfg::kBiasSlices == 2) cb1 = __ldg(ep.bias1 + tile_n * TN + et);
       }
       if (epi_is_modf<EPI>()) {
         const float4* src = reinterpret_cast<const float4*>(ep.wout_t + static_cast<size_t>(tile_n) * TN * EPW);
-        float4* dst = reinterpret_cast<float4*>(wout_s);
 #pragma unroll
-        for (int j = 0; j < TN * EPW / 4 / kEpiThreads; ++j) dst[et + j * kEpiThreads] = src[et + j * kEpiThreads];
+        for (int j = 0; j < TN * EPW / 4 / kEpiThreads; ++j) cw[j] = __ldg(src + et + j * kEpiThreads);
       }
     };
-    stage_consts(unit % tiles_n);
+    auto put_consts = [&]() {
+      if (et < TN) {
+        bias_s[et] = cb0;
+        if (Cfg::kBiasSlices == 2) bias_s[TN + et] = cb1;
+      }
+      if (epi_is_modf<EPI>()) {
+#pragma unroll
+        for (int j = 0; j < TN * EPW / 4 / kEpiThreads; ++j) reinterpret_cast<float4*>(wout_s)[et + j * kEpiThreads] = cw[j];
+      }
+    };
+    fetch_consts(unit % tiles_n);
     griddep_wait();
     if (et == 0) griddep_launch_dependents();
+    // this warp's piece of the output tile: 32 rows x 64 columns; with 64-wide tiles two warps fill one piece
+    uint8_t* const piece = Cfg::kOutOverH ? h_s + (warp - 2) * Cfg::kHChunks * 4096 : out_s + (CPT == 2 ? half * 4 + q : q) * 4096;
+    const bool stores = lane == 0 && (CPT == 2 || half == 0);
+    auto piece_sync = [&]() {
+      if (CPT == 2) __syncwarp(); else asm volatile("bar.sync %0, 64;" ::"r"(2 + q) : "memory");
+    };
+    // this warp's blocks of h of its tile i
+    uint8_t* const h_piece = h_s + (warp - 2) * Cfg::kHChunks * 4096;
+    uint32_t h_loads = 0;                        // tiles whose h has been awaited
+    auto h_request = [&](int i) {
+      const int t = unit + i * nunits;
+      const int n = (t % tiles_n) * TN + CPT * half * kChunk, row = (PAIR ? 2 * (t / tiles_n) + rank : t / tiles_n) * kTileM + q * 32;
+      if (Cfg::kHChunks && lane == 0 && row < ep.M) {
+        const uint32_t bytes = tiled_rows(row, ep.M) * 128;
+        mbar_arrive_expect_tx(&h_bar[warp - 2], Cfg::kHChunks * bytes);
+#pragma unroll
+        for (int ci = 0; ci < Cfg::kHChunks; ++ci) bulk_load(h_piece + ci * 4096, ep.h + tiled_off(row, (n + ci * kChunk) >> 2, ep.M, ep.ldo), bytes, &h_bar[warp - 2]);
+      }
+    };
+    h_request(0);
     bool ok = true;
     for (int i = 0; i < my_tiles; ++i) {
       const int t = unit + i * nunits;
@@ -279,51 +297,28 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
       const int ab = i & 1;
       const int m = tile_m * kTileM + rloc;
       const bool valid = m < ep.M;
-      // every epilogue thread is done with the previous tile: its accumulator buffer, the h tile and
-      // the per-tile constants may be replaced
-      asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
-      if (et == 0) {
-        if (i >= 1) {
-          if (PAIR) mbar_arrive_cluster(mapa_shared(smem_u32(&tmem_empty_bar[ab ^ 1]), 0));
-          else mbar_arrive(&tmem_empty_bar[ab ^ 1]);
-        }
-        if (Cfg::kStagedOut && i >= 1) {
-          // the previous tile's 16-bit output sits in shared memory (the modulate epilogue wrote it over the h tile)
-          const int tp = unit + (i - 1) * nunits;
-          const int pn = tp % tiles_n, pm = PAIR ? 2 * (tp / tiles_n) + rank : tp / tiles_n;
-#pragma unroll
-          for (int b = 0; b < TN / 64; ++b)
-            tma_store_2d(&tmOut, (EPI == EPI_MOD ? h_s + 2 * b * (kTileM * 128) : out_s + b * (kTileM * 128)), pn * TN + b * 64, pm * kTileM);
-          tma_store_commit();
-          tma_store_wait_read();   // before this tile's h lands on it / the epilogue writes the next tile
-        }
-        if (EPI == EPI_GATE_RES && i >= 1) {
-          // the previous tile's new h sits in the h tile (the threads that own its rows wrote it in place): TMA
-          // stores instead of row-per-thread stores, which touch 32 rows per instruction
-          const int tp = unit + (i - 1) * nunits;
-          const int pn = tp % tiles_n, pm = PAIR ? 2 * (tp / tiles_n) + rank : tp / tiles_n;
-#pragma unroll
-          for (int c = 0; c < NC; ++c) tma_store_2d(&tmH, h_s + c * (kTileM * 128), pn * TN + c * kChunk, pm * kTileM);
-          tma_store_commit();
-          tma_store_wait_read();   // before the next h tile lands on it
-        }
-        if (Cfg::kStageH) {
-          // requested before this thread block's further pipeline traffic queues up behind it: ordinary
-          // loads issued while the pipeline saturates the SM's shared-memory port take thousands of cycles
-          mbar_arrive_expect_tx(h_bar, Cfg::kHTileBytes);
-#pragma unroll
-          for (int c = 0; c < NC; ++c)
-            tma_load_2d(h_s + c * (kTileM * 128), &tmH, h_bar, tile_n * TN + c * kChunk, tile_m * kTileM);
-        }
-      }
-      if (i > 0) stage_consts(tile_n);
+      // everything the epilogue takes from memory is requested before the accumulators are awaited
       RowState rs;
-      if (valid) epi_row_begin<EPI>(ep, m, rs);
-      asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");   // biases and the Wout^T tile are in place
+      rs.pm = 0.0f; rs.pm2 = 0.0f; rs.pn = 0.0f; rs.mean = 0.0f; rs.rstd = 0.0f;
+      if (i > 0) fetch_consts(tile_n);
+      if (valid) epi_row_begin<EPI, true>(ep, m, rs);
+      float hlate[kChunk];                       // the block of h that is not staged
+      if (epi_reads_h<EPI>() && Cfg::kHChunks < CPT && valid) load_h_tiled(ep.h, m, tile_n * TN + (CPT * half + 1) * kChunk, ep.M, ep.ldo, hlate);
+      if (i > 0) epi_sync();                     // every thread is done with the previous tile's constants
+      put_consts();
+      epi_sync();                                // the constants are in place
       if (ok) ok = mbar_wait(&tmem_full_bar[ab], (i >> 1) & 1);
-      if (ok && Cfg::kStageH) ok = mbar_wait(h_bar, i & 1);
+      const bool h_here = Cfg::kHChunks && tile_m * kTileM + q * 32 < ep.M;
+      if (h_here) {
+        if (ok) ok = mbar_wait(&h_bar[warp - 2], h_loads & 1);
+        ++h_loads;
+      }
       if (!ok) atomicExch(err, DEV_ERR_EPI_WAIT);
       ok = __all_sync(0xffffffffu, ok);
+      if (Cfg::kStagedOut && !Cfg::kOutOverH && i > 0) {   // the previous tile's piece has left
+        if (stores) tma_store_wait_read();
+        piece_sync();
+      }
       if (ok) {
         tc_fence_after_sync();
         const uint32_t trow = tmem_base + ab * kAccCols + (static_cast<uint32_t>(q * 32) << 16);
@@ -334,54 +329,82 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
           const int col0 = kPacked ? (c >> 1) * 128 + (c & 1) * kChunk : c * kChunk;   // first accumulator
           tmem_ld32(trow + col0, a0);
           if (kTwoAcc) tmem_ld32(trow + col0 + (kPacked ? kStatCols : TN), a1);
-          if (Cfg::kStageH) load_swizzled_row32(h_s + c * (kTileM * 128), rloc, hv);
+          if (epi_reads_h<EPI>()) {
+            if (ci < Cfg::kHChunks) {
+              const float4* hp = reinterpret_cast<const float4*>(h_piece + ci * 4096) + lane;
+              const int rt = tiled_rows(tile_m * kTileM + q * 32, ep.M);
+              if (valid) {
+#pragma unroll
+                for (int j = 0; j < kChunk / 4; ++j) { const float4 x = hp[j * rt]; hv[4 * j] = x.x; hv[4 * j + 1] = x.y; hv[4 * j + 2] = x.z; hv[4 * j + 3] = x.w; }
+              }
+            } else {
+#pragma unroll
+              for (int j = 0; j < kChunk; ++j) hv[j] = hlate[j];
+            }
+          }
           tmem_ld_wait();
+          if (Cfg::kHChunks && !Cfg::kOutOverH && ci == Cfg::kHChunks - 1 && i + 1 < my_tiles) { __syncwarp(); h_request(i + 1); }
+          if (Cfg::kOutOverH && ci == 0) __syncwarp();   // every lane has read the block: the piece may take its place
+          if (ci == CPT - 1) {                   // this warp's last read of the buffer: the MMAs of tile i + 2 may have it
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) {
+              if (PAIR) mbar_arrive_cluster_tmem(mapa_shared(smem_u32(&tmem_empty_bar[ab]), 0));
+              else mbar_arrive(&tmem_empty_bar[ab]);
+            }
+          }
+          const float *b0 = bias_s + c * kChunk, *b1 = bias_s + (Cfg::kBiasSlices - 1) * TN + c * kChunk;
           float efirst[EPW];
           if (epi_is_modf<EPI>() && ci == 1) {
 #pragma unroll
             for (int e = 0; e < EPW; ++e) { efirst[e] = rs.eacc[e]; rs.eacc[e] = 0.0f; }
           }
           if (EPI == EPI_GATE_RES) {
-            gate_res_chunk(a0, a1, bias_s + c * kChunk, bias_s + TN + c * kChunk, hv, rs);
-            store_swizzled_row32(h_s + c * (kTileM * 128), rloc, hv);   // in place; leaves by TMA store
+            gate_res_chunk(a0, a1, b0, b1, hv, rs);
+            if (valid) store_h_tiled(ep.h, m, tile_n * TN + c * kChunk, ep.M, ep.ldo, hv);
           } else if (Cfg::kStagedOut) {
             if (EPI == EPI_SILU_ACT) {
 #pragma unroll
-              for (int j = 0; j < kChunk; ++j) a0[j] = silu_t<true>(a0[j] + bias_s[c * kChunk + j]);
-            } else
-              modulate_chunk(a0, a1, bias_s + c * kChunk, bias_s + TN + c * kChunk, hv, rs);
-            // One thread per chunk: the row's second chunk lands where another warp reads the first chunk's h from, so every
-            // thread must have read its h before any writes.  (With two chunks per thread the order is the thread's own.)
-            if (EPI == EPI_MOD && CPT == 1) asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
-            // 64 bytes of row rloc in box c / 2 (TMA's 128-byte swizzle); the modulate epilogue writes over the h it read
-            uint8_t* row = (EPI == EPI_MOD ? h_s + 2 * (c >> 1) * (kTileM * 128) : out_s + (c >> 1) * (kTileM * 128)) + rloc * 128;
+              for (int j = 0; j < kChunk; ++j) a0[j] = silu_t<true>(a0[j] + b0[j]);
+            } else modulate_chunk(a0, a1, b0, b1, hv, rs);
+            uint8_t* row = piece + lane * 128;   // TMA's 128-byte swizzle
             __align__(16) ACT o[kChunk];
 #pragma unroll
             for (int j = 0; j < kChunk; ++j) o[j] = to_act<ACT>(a0[j]);
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-              *reinterpret_cast<uint4*>(row + ((((c & 1) * 4 + u) ^ (rloc & 7)) << 4)) = reinterpret_cast<const uint4*>(o)[u];
+              *reinterpret_cast<uint4*>(row + ((((c & 1) * 4 + u) ^ (lane & 7)) << 4)) = reinterpret_cast<const uint4*>(o)[u];
           } else if (valid)
-            epi_chunk<EPI, ACT, true>(ep, m, tile_n * TN + c * kChunk, a0, a1, bias_s + c * kChunk,
-                                      bias_s + TN + c * kChunk, hv, rs, wout_s + c * kChunk * EPW);
+            epi_chunk<EPI, ACT, true>(ep, m, tile_n * TN + c * kChunk, a0, a1, b0, b1, hv, rs, wout_s + c * kChunk * EPW);
           if (epi_is_modf<EPI>() && ci == 1) {
 #pragma unroll
             for (int e = 0; e < EPW; ++e) rs.eacc[e] = efirst[e] + rs.eacc[e];
           }
         }
-        if (EPI == EPI_GATE_RES || Cfg::kStagedOut) fence_proxy_async_smem();
-        tc_fence_before_sync();   // orders the TMEM reads before the barrier that releases the buffer
-      } else if (EPI == EPI_MOD && CPT == 1) asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");   // the barrier above
+      }
+      if (Cfg::kStagedOut) {
+        fence_proxy_async_smem();
+        piece_sync();
+        if (stores && ok && tile_m * kTileM + q * 32 < ep.M) {
+          tma_store_2d(&tmOut, piece, tile_n * TN + (CPT == 2 ? half * 64 : 0), tile_m * kTileM + q * 32);
+          tma_store_commit();
+        }
+      }
+      if (Cfg::kOutOverH && i + 1 < my_tiles) {  // the next tile's h once the piece has left
+        if (stores) tma_store_wait_read();
+        __syncwarp();
+        h_request(i + 1);
+      }
       if (EPI == EPI_GATE_RES) {
         // one (mean, M2) partial per row and 64-column group
-        if (CPT == 2) {            // TN = 128: this thread's two chunks are one group
-          if (ok && valid) store_group_stats(ep, m, tile_n * 2 + half, rs.pm, rs.pm2);
+        if (CPT == 2) {            // this thread's two chunks are one group
+          if (ok && valid) store_group_stats<true>(ep, m, tile_n * (TN / kStatCols) + half, rs.pm, rs.pm2);
         } else {                   // TN = 64: chunk 1 (warps 6..9) is merged into chunk 0 (warps 2..5)
           if (half == 1) { xch_s[rloc * 4] = rs.pm; xch_s[rloc * 4 + 1] = rs.pm2; }
-          asm volatile("bar.sync 1, 256;" ::: "memory");
+          epi_sync();
           if (half == 0 && ok && valid) {
             chan_merge_equal(rs.pm, rs.pm2, xch_s[rloc * 4], xch_s[rloc * 4 + 1], static_cast<float>(kChunk));
-            store_group_stats(ep, m, tile_n, rs.pm, rs.pm2);
+            store_group_stats<true>(ep, m, tile_n, rs.pm, rs.pm2);
           }
         }
       }
@@ -391,13 +414,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
         if (CPT == 2) {            // TN = 128: this thread's two chunks are one group
           if (ok && valid) epi_row_end<EPI>(ep, m, tile_n * 2 + half, rs);
         } else {                   // TN = 64: chunk 1 (warps 6..9) is added to chunk 0 (warps 2..5)
-          asm volatile("bar.sync 1, 256;" ::: "memory");   // every thread is done reading the Wout^T tile
+          epi_sync();                                      // every thread is done reading the Wout^T tile
           float* part = wout_s;                            // [128 rows][EPW]
           if (half == 1 && ok) {
 #pragma unroll
             for (int c = 0; c < EPW; ++c) part[rloc * EPW + c] = rs.eacc[c];
           }
-          asm volatile("bar.sync 1, 256;" ::: "memory");
+          epi_sync();
           if (half == 0 && ok && valid) {
 #pragma unroll
             for (int c = 0; c < EPW; ++c) rs.eacc[c] += part[rloc * EPW + c];
@@ -406,31 +429,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
         }
       }
     }
-    if (Cfg::kStagedOut) {
-      // the last tile's output
-      asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
-      if (et == 0 && ok) {
-        const int tp = unit + (my_tiles - 1) * nunits;
-        const int pn = tp % tiles_n, pm = PAIR ? 2 * (tp / tiles_n) + rank : tp / tiles_n;
-#pragma unroll
-        for (int b = 0; b < TN / 64; ++b)
-          tma_store_2d(&tmOut, (EPI == EPI_MOD ? h_s + 2 * b * (kTileM * 128) : out_s + b * (kTileM * 128)), pn * TN + b * 64, pm * kTileM);
-        tma_store_commit();
-      }
-      if (et == 0) tma_store_wait_all();
-    }
-    if (EPI == EPI_GATE_RES) {
-      // the last tile's new h
-      asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
-      if (et == 0 && ok) {
-        const int tp = unit + (my_tiles - 1) * nunits;
-        const int pn = tp % tiles_n, pm = PAIR ? 2 * (tp / tiles_n) + rank : tp / tiles_n;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) tma_store_2d(&tmH, h_s + c * (kTileM * 128), pn * TN + c * kChunk, pm * kTileM);
-        tma_store_commit();
-      }
-      if (et == 0) tma_store_wait_all();
-    }
+    if (Cfg::kStagedOut && stores) tma_store_wait_all();
   }
   tc_fence_before_sync();
   __syncthreads();
@@ -509,7 +508,7 @@ gemm_simt_kernel(const float* __restrict__ A0, int lda0, const float* __restrict
   if (m < ep.M) {
     const int n0 = tile_n * kTileN + warp * kChunk;
     float hv[kChunk];
-    epi_row_begin<EPI>(ep, m, rs);
+    epi_row_begin<EPI, false>(ep, m, rs);
     if (epi_reads_h<EPI>()) load_chunk_f32(ep.h + static_cast<size_t>(m) * ep.ldo + n0, hv);
     epi_chunk<EPI, float, false>(ep, m, n0, acc0, acc1, ep.bias0 + n0, ep.bias1 ? ep.bias1 + n0 : ep.bias0 + n0, hv, rs,
                                  kStageWout ? wout_s + warp * kChunk * EPW
@@ -523,7 +522,7 @@ gemm_simt_kernel(const float* __restrict__ A0, int lda0, const float* __restrict
     if (m < ep.M && !(warp & 1)) {
       chan_merge_equal(rs.pm, rs.pm2, scr[((warp + 1) * kSimtRows + lane) * 4], scr[((warp + 1) * kSimtRows + lane) * 4 + 1],
                        static_cast<float>(kChunk));
-      store_group_stats(ep, m, tile_n * 2 + (warp >> 1), rs.pm, rs.pm2);
+      store_group_stats<false>(ep, m, tile_n * 2 + (warp >> 1), rs.pm, rs.pm2);
     }
   }
   if constexpr (epi_is_modf<EPI>()) {

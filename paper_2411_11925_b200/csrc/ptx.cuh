@@ -128,6 +128,13 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m
       : "memory");
 }
 
+// Contiguous copy global -> this CTA's shared memory (16-byte aligned, a multiple of 16 bytes), completion counted in bytes.
+__device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(smem_u32(smem_dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+
 // 2-D tiled store shared -> global (rows beyond the tensor's extent are clipped).  x * elem_size must be a
 // multiple of 16 bytes and neither coordinate negative.  Completion is tracked per thread in bulk groups.
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* m, const void* smem_src, int x, int y) {
@@ -218,6 +225,12 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 // arrive on a barrier of another CTA of the cluster (shared::cluster address)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+// The same to say that tensor memory has been read: the reads are complete (tcgen05.wait::ld) and ordered by
+// tcgen05.fence::before_thread_sync, no ordinary memory is handed over.  A releasing arrive would wait for the thread's
+// outstanding stores first: 2 to 3 k cycles per tile in the gated kernel's epilogue.
+__device__ __forceinline__ void mbar_arrive_cluster_tmem(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // Counter in shared memory that CTAs of the cluster bump remotely: relaxed add (the caller fences once
 // before a batch of them), read with acquire.

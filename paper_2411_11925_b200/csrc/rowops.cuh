@@ -2,6 +2,7 @@
 // (eps_hat reduction, classifier-free guidance, DDPM update, input projection, LayerNorm partials,
 // condition vector s), and the verification / resampling kernels.
 #pragma once
+#include <type_traits>
 #include "epilogue.cuh"
 #include "ptx.cuh"
 
@@ -80,6 +81,41 @@ __device__ __forceinline__ void input_proj_group(const float* wa, const float* w
   for (int o = 16; o > 0; o >>= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
 }
 
+// h and the LayerNorm partials of up to RB consecutive token rows (their guidance twins hold the same values) over the
+// 64-column group g, by one warp: lane holds columns 64 g + lane and + 32 in acc.  Tiled layout (tensor-core path): the values
+// pass through tile_s [RB][64] so that the rows' 16-byte quads, which are neighbours in memory, are written together.
+template <bool TILED, int RB>
+__device__ __forceinline__ void write_h_group(float* h, float* stats, const float (&acc)[RB][2], const float (&mean)[RB], const float (&m2)[RB],
+                                              float* tile_s, int g, int r0, int nrow, int nrep, int R, int W, int lane) {
+  const int M = R * nrep, G = W / kStatCols;
+  if (!TILED) {
+#pragma unroll
+    for (int rr = 0; rr < RB; ++rr)
+      for (int rep = 0; rr < nrow && rep < nrep; ++rep) {
+        const size_t row = static_cast<size_t>(r0 + rr) + static_cast<size_t>(rep) * R;
+        if (lane == 0) reinterpret_cast<float2*>(stats)[row * G + g] = make_float2(mean[rr], m2[rr]);
+        h[row * W + g * kStatCols + lane] = acc[rr][0];
+        h[row * W + g * kStatCols + 32 + lane] = acc[rr][1];
+      }
+    return;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int rr = 0; rr < RB; ++rr) { tile_s[rr * kStatCols + lane] = acc[rr][0]; tile_s[rr * kStatCols + 32 + lane] = acc[rr][1]; }
+  __syncwarp();
+  for (int rep = 0; rep < nrep; ++rep) {
+#pragma unroll
+    for (int rr = 0; rr < RB; ++rr)
+      if (rr < nrow && lane == rr) reinterpret_cast<float2*>(stats)[tiled_stat_off(r0 + rr + rep * R, g, M, G)] = make_float2(mean[rr], m2[rr]);
+#pragma unroll
+    for (int k = 0; k < (RB * 16 + 31) / 32; ++k) {
+      const int idx = k * 32 + lane, rr = idx % RB, c4 = idx / RB;
+      if (c4 < 16 && rr < nrow)
+        *reinterpret_cast<float4*>(h + tiled_off(r0 + rr + rep * R, g * 16 + c4, M, W)) = *reinterpret_cast<const float4*>(tile_s + rr * kStatCols + c4 * 4);
+    }
+  }
+}
+
 struct StepParams {
   int R, cfg, C, W, NT;          // token rows, guidance flag, token dim, width, number of column tiles
   float cfg_scale, a, b, sigma;  // coefficients of the step being finished (t)
@@ -94,7 +130,7 @@ struct StepParams {
   const float* bin;
   const float* cz;               // [Rh, W]
   const float* te_next;          // [W] embedding of the step being prepared
-  float* h;                      // [Rh, W]
+  float* h;                      // [Rh, W] (16-bit operands: tiled layout, as stats)
   float* stats;                  // [Rh, W/64, 2]
   void* s;                       // [Rh, W] activations: s of the step te_next belongs to (null: none)
   void* s_b;                     // a second s to prepare (first boundary only), with its embedding te_b
@@ -128,6 +164,8 @@ __global__ void __launch_bounds__(256, RB == 4 ? 3 : 0) step_kernel(StepParams p
   __shared__ float xs[RB][kCPad];
   __shared__ float eh[RB][2][kCPad];
   __shared__ float wv[LV ? RB : 1][kCPad];
+  constexpr bool kTiled = !std::is_same<ACT, float>::value;
+  __shared__ __align__(16) float tile_s[kTiled ? 8 : 1][RB * kStatCols];
   const int r0 = blockIdx.x * RB, tid = threadIdx.x;
   const int nrep = p.cfg ? 2 : 1;
   const int nrow = min(RB, p.R - r0);
@@ -229,21 +267,20 @@ __global__ void __launch_bounds__(256, RB == 4 ? 3 : 0) step_kernel(StepParams p
           const size_t row = static_cast<size_t>(r0 + rr) + static_cast<size_t>(rep) * p.R;
           czv[rr][rep][j] = (rr < nrow && rep < nrep && (s || s_b)) ? __ldg(p.cz + row * p.W + g * kStatCols + j * 32 + lane) : 0.0f;
         }
+    float acc[RB][2], mean[RB], m2[RB];
+#pragma unroll
+    for (int rr = 0; rr < RB; ++rr) input_proj_group(wa, wb, ba, bb, xs[rr], acc[rr], mean[rr], m2[rr]);   // (rows beyond nrow: x = 0)
+    write_h_group<kTiled, RB>(p.h, p.stats, acc, mean, m2, tile_s[kTiled ? warp : 0], g, r0, nrow, nrep, p.R, p.W, lane);
 #pragma unroll
     for (int rr = 0; rr < RB; ++rr) {
       if (rr >= nrow) break;
-      float acc[2], mean, m2;
-      input_proj_group(wa, wb, ba, bb, xs[rr], acc, mean, m2);
 #pragma unroll
       for (int rep = 0; rep < 2; ++rep) {
         if (rep >= nrep) break;
         const size_t row = static_cast<size_t>(r0 + rr) + static_cast<size_t>(rep) * p.R;
-        if (lane == 0)
-          reinterpret_cast<float2*>(p.stats)[row * (p.W / kStatCols) + g] = make_float2(mean, m2);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           const int n = g * kStatCols + j * 32 + lane;
-          p.h[row * p.W + n] = acc[j];
           if (s) s[row * p.W + n] = to_act<ACT>(silu_f(czv[rr][rep][j] + te[j]));
           if (s_b) s_b[row * p.W + n] = to_act<ACT>(silu_f(czv[rr][rep][j] + teb[j]));
         }
@@ -280,6 +317,8 @@ template <typename ACT>
 __global__ void __launch_bounds__(256) batch_prepare_kernel(BatchParams p) {
   constexpr int RB = 4;
   __shared__ float xs[RB][kCPad];
+  constexpr bool kTiled = !std::is_same<ACT, float>::value;
+  __shared__ __align__(16) float tile_s[kTiled ? 8 : 1][RB * kStatCols];
   const int r0 = blockIdx.x * RB, tid = threadIdx.x;
   const int nrep = p.cfg ? 2 : 1;
   const int nrow = min(RB, p.Rtok - r0);
@@ -320,20 +359,17 @@ __global__ void __launch_bounds__(256) batch_prepare_kernel(BatchParams p) {
         czv[rr][rep][1] = __ldg(p.cz + zrow * p.W + nb);
       }
     }
+    float acc[RB][2], mean[RB], m2[RB];
+#pragma unroll
+    for (int rr = 0; rr < RB; ++rr) input_proj_group(wa, wb, ba, bb, xs[rr], acc[rr], mean[rr], m2[rr]);   // (rows beyond nrow: x = 0)
+    write_h_group<kTiled, RB>(p.h, p.stats, acc, mean, m2, tile_s[kTiled ? warp : 0], g, r0, nrow, nrep, p.Rtok, p.W, lane);
 #pragma unroll
     for (int rr = 0; rr < RB; ++rr) {
       if (rr >= nrow) break;
-      const int rt = r0 + rr;
-      float acc[2], mean, m2;
-      input_proj_group(wa, wb, ba, bb, xs[rr], acc, mean, m2);
 #pragma unroll
       for (int rep = 0; rep < 2; ++rep) {
         if (rep >= nrep) break;
-        const size_t row = static_cast<size_t>(rt) + static_cast<size_t>(rep) * p.Rtok;
-        if (lane == 0)
-          reinterpret_cast<float2*>(p.stats)[row * (p.W / kStatCols) + g] = make_float2(mean, m2);
-        p.h[row * p.W + na] = acc[0];
-        p.h[row * p.W + nb] = acc[1];
+        const size_t row = static_cast<size_t>(r0 + rr) + static_cast<size_t>(rep) * p.Rtok;
         s[row * p.W + na] = to_act<ACT>(silu_f(czv[rr][rep][0] + tev[rr][0]));
         s[row * p.W + nb] = to_act<ACT>(silu_f(czv[rr][rep][1] + tev[rr][1]));
       }
