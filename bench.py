@@ -27,8 +27,6 @@ import numpy as np  # noqa: E402
 # dram__bytes_read + dram__bytes_write per launch of a kernel class, from the ncu capture summarised under
 # profiles/ for (workload, class); absent = no capture of the kernel as it stands (reported as null)
 NCU_DRAM_BYTES_PER_LAUNCH = {
-    # profiles/mar256_sequential_draft_sb_chain_kernel_ncu.md: 99.4 MB read + 51.8 MB written per launch
-    ("mar256", "sb_chain"): 151.2e6,
     # profiles/mar256_persistent_chain_kernel_ncu.md: 6.02 GB read + 43.6 MB written per launch of the target chain
     ("mar256", "pchain_target"): 6.062e9,
 }
@@ -339,27 +337,27 @@ def measure(name, args, peaks, steps, warmup, rounds_per_step, full):
         r1 = DeviceRound(inp1, ctx=ctx, device=local, heads=(rounds[0].head_q, rounds[0].head_p))
         seq_step = lambda i: [r1.draft() for _ in range(wl.gamma)]
         timed(seq_step, 3)
+        ctx.set_chain_mode(api.Context.CHAIN_LAYER_KERNELS)
+        timed(seq_step, 3)
         layers_secs = timed(seq_step, few)
-        # the persistent small-batch kernel (csd_set_chain_mode): chains of at most 128 head rows
-        ctx.set_chain_mode(api.Context.CHAIN_SMALL_BATCH)
+        ctx.set_chain_mode(api.Context.CHAIN_LAYERS)      # the group chain kernel where it applies
         timed(seq_step, 3)
         l1 = ctx.launch_count()
         seq_secs = timed(seq_step, few)
         launches_per_call = int((ctx.launch_count() - l1) // (few * wl.gamma))
-        ctx.set_chain_mode(api.Context.CHAIN_LAYERS)
         d = wl.draft
         wbytes = 2.0 * (d.W * d.Dz + d.L * 5 * d.W * d.W + 2 * d.W * d.W)     # 16-bit GEMM weights of the draft head
         per_call = seq_secs / (few * wl.gamma)
         out["sequential_draft"] = {
             "calls_per_round": wl.gamma, "head_rows_per_call": wl.B * (2 if wl.cfg else 1),
-            "chain_mode": "CSD_CHAIN_SMALL_BATCH" if launches_per_call < 50 else "CSD_CHAIN_LAYERS (small-batch kernel not eligible)",
+            "chain_mode": "group chain kernel" if launches_per_call < 50 else "layer kernels (group chain kernel not eligible)",
             "ms_per_call": 1e3 * per_call, "us_per_denoising_step": 1e6 * per_call / wl.T,
             "layer_kernels_ms_per_call": 1e3 * layers_secs / (few * wl.gamma),
             "launches_per_call": launches_per_call,
             "value": wl.B * wl.gamma * few / seq_secs, "unit": UNIT,
             "bound": "hbm", "weight_bytes_per_step": wbytes, "achieved": wbytes * wl.T / per_call / 1e9,
             "peak": peaks["hbm_gbs"], "roofline_unit": "GB/s", "frac": wbytes * wl.T / per_call / 1e9 / peaks["hbm_gbs"],
-            "traffic": NCU_DRAM_BYTES_PER_LAUNCH.get((wl.name, "sb_chain")) if launches_per_call < 50 else None,
+            "traffic": None,
             "note": "algorithmic bytes = draft weight bytes x T per call; the weights fit L2 (126 MB), so the "
                     "fraction says how far the call is from streaming them from HBM once per step"}
 

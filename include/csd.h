@@ -139,26 +139,23 @@ int64_t csd_launch_count(const csd_ctx *ctx);
  *                       to itself (csd_draft_denoise or csd_verify called alone) is about a tenth faster with
  *                       CSD_CHAIN_LAYER_KERNELS, whose kernels spread over the idle SMs; the default is chosen
  *                       per chain, not per call, so that csd_round and the three separate calls give the same bits.
+ *                     - A chain of few rows on a 16-bit head with W in {512, 1024, 1536} and var_out = 0 (groups of
+ *                       16 tokens, or 8 with guidance: up to 17, 8 and 4 groups) runs as the group chain kernel:
+ *                       everything that depends on the condition vector only is formed ahead, for many steps at a
+ *                       time, and a cluster of W / 128 CTAs carries each group through the steps, activations
+ *                       passing through distributed shared memory.  This is the calling pattern Alg. 1 forces on
+ *                       the draft model (x_i ~ q_i one position at a time).  Every block is folded.
  *                     - Otherwise one kernel per layer, chained with programmatic dependent launch; a layer's
  *                       independent part overlaps its predecessor on otherwise idle SMs.  For 16-bit heads on
  *                       grids of one wave, blocks 2..L run as two kernels instead of three: LayerNorm is folded
  *                       into the first layer's epilogue.
  *                     Folding is algebraically the same function, rounded differently: the layouts agree within
  *                     the parity tolerance, not bit for bit, and which one runs depends on the call's row count.
- *   CSD_CHAIN_LAYER_KERNELS: as CSD_CHAIN_LAYERS without the persistent kernel (layer kernels, folded where
+ *   CSD_CHAIN_LAYER_KERNELS: as CSD_CHAIN_LAYERS without the chain kernels (layer kernels, folded where
  *                     that applies): what csd_draft_denoise_static always runs.
  *   CSD_CHAIN_LAYERS_PLAIN: layer kernels without the folded blocks (three kernels per block everywhere); a
  *                     row's bits then do not depend on how many rows the call has.
- *   CSD_CHAIN_SMALL_BATCH: as CSD_CHAIN_LAYERS, except that a chain of at most 128 head rows (R (1 + cfg) <= 128)
- *                     on a 16-bit head with W in {512, 1024, 1536} and var_out = 0 runs as ONE persistent kernel
- *                     that spreads every layer over the whole GPU (weights as the MMA's M operand, a cluster of 8
- *                     CTAs per group of 16 rows, the products of the condition vector computed a step ahead by the
- *                     remaining SMs).  This is the calling pattern Alg. 1 forces on the draft model (x_i ~ q_i one
- *                     position at a time), where the layer kernels are bound by kernel latency.  Every block is
- *                     folded, so results agree with the other layouts within the parity tolerance.  The kernel
- *                     needs the GPU to itself: csd_round then runs its two chains one after the other, and two
- *                     contexts should not run such chains at the same time (the kernels would wait for each
- *                     other's SMs until the wait limit and report CSD_ERR_TIMEOUT).
+ *   CSD_CHAIN_SMALL_BATCH: the same as CSD_CHAIN_LAYERS, which chooses the kernels for few rows by itself.
  * Takes effect for calls made after it returns. */
 enum { CSD_CHAIN_LAYERS = 0, CSD_CHAIN_SMALL_BATCH = 1, CSD_CHAIN_LAYERS_PLAIN = 2, CSD_CHAIN_LAYER_KERNELS = 3 };
 int csd_set_chain_mode(csd_ctx *ctx, int mode);
@@ -170,7 +167,7 @@ int csd_set_chain_mode(csd_ctx *ctx, int mode);
  * kernel class, the launches recorded since: their count, device time (ms) and algorithmic FLOPs
  * (2*M*N*K per GEMM).  Classes: 0 condition projection, 1 block MLP first layer (+SiLU),
  * 2 AdaLN modulate (shift|scale), 3 block MLP second layer + gate + residual, 4 final modulate +
- * output projection, 5 per-step boundary kernel, 6 small-batch chain kernel. */
+ * output projection, 5 per-step boundary kernel, 6 a whole chain (not recorded: with profiling on, chains run as layer kernels). */
 int csd_profile(csd_ctx *ctx, int enable);
 int csd_profile_read(csd_ctx *ctx, int kernel_class, int64_t *launches, double *total_ms,
                      double *total_flops);
@@ -216,8 +213,8 @@ int csd_draft_denoise(csd_ctx *ctx, const csd_head *head, const csd_schedule *sc
 /* csd_draft_denoise without any allocation (the paper has no counterpart: this is a deployment
  * variant of the call above with the same arguments; it runs the layer kernels, so its results are
  * bit-identical to csd_draft_denoise in the modes CSD_CHAIN_LAYER_KERNELS and CSD_CHAIN_LAYERS_PLAIN, and
- * in the default mode whenever that call does not take the persistent chain kernel, whose buffers
- * grow with T and cannot live in a fixed array; otherwise the two agree within the parity tolerance).
+ * in the default mode whenever that call takes neither the persistent nor the group chain kernel,
+ * whose buffers grow with T and cannot live in a fixed array; otherwise the two agree within the parity tolerance).
  * Who needs it: code that must not, or cannot, reach the CUDA allocator when the call is made -
  * a serving process whose framework has handed all free device memory to its own pool so that
  * cudaMalloc fails, a latency-critical loop where cudaMalloc's implicit device synchronisation is

@@ -228,10 +228,9 @@ class Context:
     CHAIN_LAYERS, CHAIN_SMALL_BATCH, CHAIN_LAYERS_PLAIN, CHAIN_LAYER_KERNELS = 0, 1, 2, 3
 
     def set_chain_mode(self, mode: int):
-        """csd_set_chain_mode: CHAIN_LAYERS (default: the persistent chain kernel where it applies, else one kernel per
-        layer with folded blocks where they apply), CHAIN_LAYER_KERNELS (never the persistent chain kernel),
-        CHAIN_LAYERS_PLAIN (three kernels per block everywhere) or CHAIN_SMALL_BATCH (chains of at most 128 head rows
-        run as one persistent kernel over the whole GPU)."""
+        """csd_set_chain_mode: CHAIN_LAYERS (default: the group or the persistent chain kernel where one applies, else one
+        kernel per layer with folded blocks where they apply), CHAIN_LAYER_KERNELS (neither chain kernel),
+        CHAIN_LAYERS_PLAIN (three kernels per block everywhere) or CHAIN_SMALL_BATCH (as the default)."""
         self._check(_LIB.csd_set_chain_mode(self._h, int(mode)))
 
     def set_wait_limit(self, cycles: int):

@@ -20,7 +20,7 @@
 #include "gemm.cuh"
 #include "gmm.cuh"
 #include "rowops.cuh"
-#include "smallbatch.cuh"
+#include "groupchain.cuh"
 #include "pchain.cuh"
 #include "f32chain.cuh"
 
@@ -73,7 +73,10 @@ struct csd_ctx {
   HostIo bn;       // csd_bonus_token: samples of every sequence before the selection
   HostIo sp;       // csd_verify_single_path: schedule constants, mu^p of one pass, running log-ratio
   HostIo pc[3];    // persistent chain kernel (per chain slot): s of all steps, a', v, partials, counters, schedule
-  HostIo sb[2];    // small-batch chain kernel (per chain slot): s of all steps, early products, a', v, counters, schedule
+  HostIo gc[2];    // group chain kernel (per chain slot): s of all steps, schedule
+  HostIo gm[2];    // its condition products: two chunks of steps
+  cudaStream_t aux[2] = {nullptr, nullptr};        // (per chain slot) where they are formed
+  cudaEvent_t ev_prep[2] = {}, ev_mods[2][2] = {}, ev_read[2][2] = {};   // preparation done; a chunk is written / has been read
   char err[512] = {0};
   // optional per-launch timing (csd_profile)
   bool prof_on = false;
@@ -107,17 +110,16 @@ struct csd_head {
   std::vector<CUtensorMap> Wgs, Wf;
   std::vector<CUtensorMap> Wgs_half, Wf_half;   // the same matrices in 128-row boxes: what one CTA of a pair loads
   std::vector<float*> c1, c2;   // first MLP layer with 256-row boxes (W a multiple of 256)
-  // small-batch chain kernel (smallbatch.cuh): usable for this head; device tables (tensor maps of W1_k, W2_k, then of
-  // the matrices multiplied by s: per block Wf_k, Wg_k, Wss_k, then Wfss, all in 128-row boxes; early tiles; biases)
-  bool sb_ready = false;
+  // group chain kernel (groupchain.cuh): the dependent layers' maps W1_k, W2_k (device table, boxes of 128 rows) and the matrix
+  // multiplied by s: scale_0 | per block W1_k Wscale_k, W1_k Wshift_k, gate_k, scale_{k+1} | final shift, scale
+  bool gc_ready = false;
+  CUtensorMap* d_gc_maps = nullptr;
+  void* mblob = nullptr;
+  CUtensorMap Wm{};
   // persistent chain kernel (pchain.cuh): per phase the early and the dependent weight maps; per phase three bias rows
   bool pc_ready = false;
   CUtensorMap* d_pc_maps = nullptr;
   const float** d_pc_bias = nullptr;
-  int sb_ntasks = 0;
-  CUtensorMap* d_sb_maps = nullptr;
-  SbTask* d_sb_tasks = nullptr;
-  const float** d_sb_bias = nullptr;
 };
 
 namespace {
@@ -424,30 +426,34 @@ bool pchain_kernel_ready(const csd_ctx* ctx, int dtype) {
   return k == 1;
 }
 
-// Whether the small-batch chain kernel can run on this device: its clusters of 8 CTAs (one per SM, ~213 KB of
-// shared memory each) must all be resident at once.  Returns the number of clusters the GPU holds (0: unusable).
+// Clusters of the group chain kernel for width W that the device holds at a time (0: it cannot run), and its opt-ins, once
+// per device and operand type.
 template <typename ACT, int FMT>
-int sb_clusters_of(csd_ctx* ctx) {
-  static int known[kMaxDevices] = {};   // 0 unknown, > 0 clusters, -1 unusable
-  int& k = known[ctx->device];
+int gchain_clusters_of(const csd_ctx* ctx, int W) {
+  static int known[kMaxDevices][kGcMaxCl + 1] = {};
+  int& k = known[ctx->device][W / 128];
   if (k == 0) {
-    k = -1;
-    auto kern = sb_chain_kernel<ACT, FMT>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSbSmemBytes) == cudaSuccess &&
-        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 0) == cudaSuccess) {
-      cudaLaunchConfig_t lc{};
-      lc.gridDim = dim3(kSbCluster); lc.blockDim = dim3(kSbThreads); lc.dynamicSmemBytes = kSbSmemBytes;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = kSbCluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-      lc.attrs = at; lc.numAttrs = 1;
-      int ncl = 0;
-      if (cudaOccupancyMaxActiveClusters(&ncl, kern, &lc) == cudaSuccess && ncl >= 1) k = ncl;
-    }
+    auto kern = group_chain_kernel<ACT, FMT>;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = static_cast<unsigned>(W / 128); at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3(static_cast<unsigned>(W / 128)); lc.blockDim = dim3(kGcThreads); lc.dynamicSmemBytes = gc_layout(W).total + 1024;
+    lc.attrs = at; lc.numAttrs = 1;
+    int n = 0;
+    const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess &&
+                    cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                    cudaFuncSetAttribute(mods_gemm_kernel<FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMgSmemBytes) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&n, kern, &lc) == cudaSuccess;
     cudaGetLastError();
+    k = ok && n > 0 ? n : -1;
   }
-  return k > 0 ? k : 0;
+  return k < 0 ? 0 : k;
 }
+int gchain_clusters(const csd_ctx* ctx, int dtype, int W) {
+  return dtype == CSD_F16 ? gchain_clusters_of<__half, 0>(ctx, W) : gchain_clusters_of<__nv_bfloat16, 1>(ctx, W);
+}
+constexpr size_t kGcChunkBytes = size_t(512) << 20;   // condition products of one chunk of steps
 
 // One head's denoising chain for R token rows on stream `st` with workspace slot `slot`:
 // begin() enqueues the per-call work (timestep embedding, condition projection, first boundary
@@ -457,7 +463,7 @@ struct Chain {
   int R, cfg; float cfg_scale; const float *z, *x_T, *eps; int sample_last; float *x0, *mu1, *x1;
   int chains = 1;   // chains that run concurrently with this one (itself included)
   int Rh = 0, W = 0, L = 0, T = 0, tn = kTileN;
-  bool sbk = false;       // the whole chain runs in the small-batch kernel (smallbatch.cuh)
+  bool gck = false;       // the whole chain runs in the group chain kernel (groupchain.cuh)
   bool pck = false;       // the whole chain runs in the persistent chain kernel (pchain.cuh)
   int fcg = 0;            // fp32 head: the whole chain runs in the fp32 chain kernel with groups of this many rows (f32chain.cuh)
   bool fold = false;      // blocks 1.. run as two kernels (fold.cuh) instead of three
@@ -573,18 +579,21 @@ struct Chain {
       fold = tc && (ctx->chain_mode == CSD_CHAIN_LAYERS || ctx->chain_mode == CSD_CHAIN_LAYER_KERNELS) && !pair && L >= 2 && !hd->Wf.empty() &&
              8 * t128 > ctx->num_sms && 2 * t128 <= ctx->num_sms && fold_kernels_ready(ctx, d);
     }
-    // Few rows: one persistent kernel for the whole chain (opt-in per context).  It needs the GPU to itself, so a
-    // round that uses it runs its two chains one after the other (chains == 1 here).
-    sbk = tc && ctx->chain_mode == CSD_CHAIN_SMALL_BATCH && Rh <= kSbRows && hd->sb_ready && chains == 1 && slot != 2 &&
-          !traj_x && !batch_Rin && !lv_min && !ctx->prof_on &&
-          (d.dtype == CSD_F16 ? sb_clusters_of<__half, 0>(ctx) : sb_clusters_of<__nv_bfloat16, 1>(ctx)) > kSbRows / kSbGroup;
-    if (sbk) { fold = false; pair = false; }
+    // Few rows: condition products ahead, one kernel for the rest (groupchain.cuh).
+    // Few rows: condition products ahead, one kernel for the rest (groupchain.cuh).  A step takes it as long for one group as
+    // for all that are resident (W = 1024: 15 clusters), so it wins up to there; the two chains of a round run together, and a
+    // call of one chain takes the same kernels as the round does, so each gets half.  Beyond: 1536-wide, 8 groups where 7
+    // clusters fit, 42 ms a round against the layer kernels' 27.
+    gck = tc && (ctx->chain_mode == CSD_CHAIN_LAYERS || ctx->chain_mode == CSD_CHAIN_SMALL_BATCH) && hd->gc_ready &&
+          slot != 2 && !batch_Rin && !lv_min && !ctx->prof_on &&
+          (R + (cfg ? 7 : 15)) / (cfg ? 8 : 16) <= (gchain_clusters(ctx, d.dtype, W) + 1) / 2;
+    if (gck) { fold = false; pair = false; }
     // One wave of 128 x 128 tiles per layer and W = 1024: one persistent kernel per chain (pchain.cuh).  Row blocks are
     // paired: an odd number is rounded up with a block of rows that belong to no token.
     {
       const int row_tiles = (Rh + kTileM - 1) / kTileM, nb = cfg ? (R + 63) / 64 : (R + 127) / 128;
       const int t128 = (W / kTileN) * row_tiles;
-      pck = kPersistentChains && tc && ctx->chain_mode == CSD_CHAIN_LAYERS && !pair && !sbk && slot != 2 && hd->pc_ready &&
+      pck = kPersistentChains && tc && ctx->chain_mode == CSD_CHAIN_LAYERS && !pair && !gck && slot != 2 && hd->pc_ready &&
             8 * t128 > ctx->num_sms && 2 * t128 <= ctx->num_sms && W / kTileN == kPcColTiles && row_tiles == nb &&
             !batch_Rin && !lv_min && !ctx->prof_on && d.C <= kCPad && pchain_kernel_ready(ctx, d.dtype);
       if (pck) { fold = false; pair = false; }
@@ -597,10 +606,8 @@ struct Chain {
     if (rc) return rc;
     if (fcg) return launch_f32_chain();
     if (!batch_reuse) {
-      const dim3 grid((W + 31) / 32, (Ts + 31) / 32);
-      small_gemm_nt_kernel<true><<<grid, 256, 0, st>>>(sc->tfeat, hd->Wt1, hd->bt1, ws.hid, Ts, W, d.F);
-      small_gemm_nt_kernel<false><<<grid, 256, 0, st>>>(ws.hid, hd->Wt2, hd->bt2, ws.te, Ts, W, W);
-      ctx->launches += 2;
+      if ((rc = launch_rows_gemm(rows_gemm(sc->tfeat, hd->Wt1, hd->bt1, ws.hid, Ts, W, d.F, true), nullptr)) ||
+          (rc = launch_rows_gemm(rows_gemm(ws.hid, hd->Wt2, hd->bt2, ws.te, Ts, W, W, false), nullptr))) return rc;
     }
     CSD_CUDA(ctx, cudaGetLastError());
     ep.M = Rh; ep.ldo = W;
@@ -634,7 +641,7 @@ struct Chain {
                                                 nullptr, 0, W, e);
     if (rc) return rc;
     sbuf[0] = ws.s2; sbuf[1] = ws.s;
-    if (sbk) return launch_small_batch();
+    if (gck) return launch_group_chain();
     if (pck) return launch_pchain();
     if (batch_Rin) return launch_batch(0);   // a pass has one step (t = 1): its s is sbuf[1]
     sp.traj_x = traj_x; sp.traj_mu = nullptr; sp.status = ctx->d_err + 1;
@@ -716,9 +723,9 @@ struct Chain {
     CSD_CUDA(ctx, cudaMemcpyAsync(d_sched, sc->a, Ts * sizeof(float), cudaMemcpyHostToDevice, st));
     CSD_CUDA(ctx, cudaMemcpyAsync(d_sched + Ts, sc->b, Ts * sizeof(float), cudaMemcpyHostToDevice, st));
     CSD_CUDA(ctx, cudaMemcpyAsync(d_sched + 2 * Ts, sc->sigma, Ts * sizeof(float), cudaMemcpyHostToDevice, st));
-    const dim3 sgrid(static_cast<unsigned>(rows), static_cast<unsigned>(Ts));
-    if (d.dtype == CSD_F16) pc_cond_all_kernel<__half><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__half*>(b + o_s), R, cfg, W, static_cast<int>(rows));
-    else pc_cond_all_kernel<__nv_bfloat16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__nv_bfloat16*>(b + o_s), R, cfg, W, static_cast<int>(rows));
+    const dim3 sgrid(static_cast<unsigned>(rows), static_cast<unsigned>((Ts + kCondSteps - 1) / kCondSteps));
+    if (d.dtype == CSD_F16) cond_all_kernel<__half, 128><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__half*>(b + o_s), R, cfg, W, static_cast<int>(rows), Ts);
+    else cond_all_kernel<__nv_bfloat16, 128><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__nv_bfloat16*>(b + o_s), R, cfg, W, static_cast<int>(rows), Ts);
     ctx->launches++;
     CSD_CUDA(ctx, cudaGetLastError());
     PcParams p{};
@@ -791,59 +798,84 @@ struct Chain {
     return CSD_OK;
   }
 
-  // The persistent small-batch kernel: s of every step, zeroed counters, the schedule on the device, one launch.
-  int launch_small_batch() {
+  // The group chain kernel: s of every step in its row order, then chunk by chunk the condition products (on the slot's
+  // own stream, ahead of the chain) and the chain.
+  int launch_group_chain() {
     const csd_head_desc& d = hd->d;
     ChainWs& ws = ctx->ws[slot];
-    const size_t asz = 2, nm = static_cast<size_t>(5 * L + 2) * W;
+    const int per = cfg ? 8 : 16, groups = (R + per - 1) / per, rows = groups * kGcRows, cl = W / 128;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 1024); return o; };
-    const size_t o_s = take(static_cast<size_t>(Ts) * kSbRows * W * asz), o_mods = take(2 * kSbRows * nm * 4),
-                 o_ap = take(static_cast<size_t>(kSbRows) * W * asz), o_v = take(static_cast<size_t>(kSbRows) * W * asz),
-                 o_sync = take(static_cast<size_t>(Ts + 2) * 4), o_sched = take(static_cast<size_t>(3) * Ts * 4),
-                 o_h = take(static_cast<size_t>(kSbRows) * W * 4), o_st = take(static_cast<size_t>(kSbRows) * (W / kStatCols) * 8);
-    int rc = ensure_side(ctx, ctx->sb[slot], off, "the small-batch chain buffers");
+    const size_t o_s = take(static_cast<size_t>(Ts) * rows * W * 2), o_sched = take(static_cast<size_t>(3) * Ts * 4);
+    int rc = ensure_side(ctx, ctx->gc[slot], off, "the group chain buffers");
     if (rc) return rc;
-    char* b = static_cast<char*>(ctx->sb[slot].base);
-    CUtensorMap tm_a{}, tm_vv{}, tm_sa{};
-    if ((rc = make_tmap(ctx, &tm_a, d.dtype, b + o_ap, kSbRows, W, W, kSbGroup))) return rc;     // boxes of one row group
-    if ((rc = make_tmap(ctx, &tm_vv, d.dtype, b + o_v, kSbRows, W, W, kSbGroup))) return rc;
-    if ((rc = make_tmap(ctx, &tm_sa, d.dtype, b + o_s, static_cast<uint64_t>(Ts) * kSbRows, W, W, kTileM))) return rc;
-    CSD_CUDA(ctx, cudaMemsetAsync(b + o_sync, 0, static_cast<size_t>(Ts + 2) * 4, st));
-    // small pageable sources: staged by the runtime before the calls return
+    // Steps per chunk: a first chunk of a tile's width of rows, because nothing overlaps its products; then twice as many
+    // each time, as far as the buffers go.
+    const size_t wrows = static_cast<size_t>(4 * L + 2) * W;
+    auto chunk_bytes = [&](int steps) { return wrows * ((static_cast<size_t>(steps) * rows + 255) / 256) * 256 * 4; };
+    int most = Ts;
+    while (most > 1 && chunk_bytes(most) > kGcChunkBytes) most = (most + 1) / 2;
+    if ((rc = ensure_side(ctx, ctx->gm[slot], 2 * chunk_bytes(most), "the condition products"))) return rc;
+    char* b = static_cast<char*>(ctx->gc[slot].base);
+    CUtensorMap tm_s{};
+    if ((rc = make_tmap(ctx, &tm_s, d.dtype, b + o_s, static_cast<uint64_t>(Ts) * rows, W, W, kTileM))) return rc;
     float* d_sched = reinterpret_cast<float*>(b + o_sched);
-    CSD_CUDA(ctx, cudaMemcpyAsync(d_sched, sc->a, Ts * sizeof(float), cudaMemcpyHostToDevice, st));
-    CSD_CUDA(ctx, cudaMemcpyAsync(d_sched + Ts, sc->b, Ts * sizeof(float), cudaMemcpyHostToDevice, st));
-    CSD_CUDA(ctx, cudaMemcpyAsync(d_sched + 2 * Ts, sc->sigma, Ts * sizeof(float), cudaMemcpyHostToDevice, st));
-    const dim3 sgrid(static_cast<unsigned>(kSbRows), static_cast<unsigned>(Ts));
-    if (d.dtype == CSD_F16) sb_cond_all_kernel<__half><<<sgrid, 256, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__half*>(b + o_s), R, cfg, W, Ts);
-    else sb_cond_all_kernel<__nv_bfloat16><<<sgrid, 256, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__nv_bfloat16*>(b + o_s), R, cfg, W, Ts);
+    // pageable source: staged by the runtime before the call returns
+    std::vector<float> hs(static_cast<size_t>(3) * Ts);
+    for (int t = 0; t < Ts; ++t) { hs[t] = sc->a[t]; hs[Ts + t] = sc->b[t]; hs[2 * Ts + t] = sc->sigma[t]; }
+    CSD_CUDA(ctx, cudaMemcpyAsync(d_sched, hs.data(), hs.size() * 4, cudaMemcpyHostToDevice, st));
+    const dim3 sgrid(static_cast<unsigned>(rows), static_cast<unsigned>((Ts + kCondSteps - 1) / kCondSteps));
+    if (d.dtype == CSD_F16) cond_all_kernel<__half, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__half*>(b + o_s), R, cfg, W, rows, Ts);
+    else cond_all_kernel<__nv_bfloat16, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__nv_bfloat16*>(b + o_s), R, cfg, W, rows, Ts);
     ctx->launches++;
     CSD_CUDA(ctx, cudaGetLastError());
-    const int ncl = d.dtype == CSD_F16 ? sb_clusters_of<__half, 0>(ctx) : sb_clusters_of<__nv_bfloat16, 1>(ctx);
-    SbParams p{};
-    p.R = R; p.Rh = Rh; p.cfg = cfg; p.W = W; p.L = L; p.T = Ts; p.C = d.C; p.sample_last = sample_last; p.cfg_scale = cfg_scale;
-    const int per = cfg ? 8 : 16;                 // tokens per row group
-    p.nd = (R + per - 1) / per; p.ne = ncl - p.nd; p.ntasks = hd->sb_ntasks; p.nm = static_cast<int>(nm);
-    p.maps = hd->d_sb_maps; p.tasks = hd->d_sb_tasks; p.sched = d_sched; p.bias = hd->d_sb_bias;
-    p.mods = reinterpret_cast<float*>(b + o_mods); p.h = reinterpret_cast<float*>(b + o_h); p.stats = reinterpret_cast<float*>(b + o_st);
-    p.ap = b + o_ap; p.v = b + o_v; p.x = ws.x;
-    p.win = hd->win; p.bin = hd->bin; p.wout_t = hd->wout_t; p.bout = hd->bout; p.x_T = x_T; p.eps = eps;
-    p.x0 = x0; p.mu1 = mu1; p.x1 = x1; p.sync = reinterpret_cast<int*>(b + o_sync); p.err = ctx->d_err; p.status = ctx->d_err + 1;
-    cudaLaunchConfig_t lc{};
-    lc.gridDim = dim3((p.nd + p.ne) * kSbCluster); lc.blockDim = dim3(kSbThreads); lc.dynamicSmemBytes = kSbSmemBytes; lc.stream = st;
+    cudaStream_t gst = ctx->aux[slot];
+    CSD_CUDA(ctx, cudaEventRecord(ctx->ev_prep[slot], st));
+    CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_prep[slot], 0));
+    GcParams p{};
+    p.R = R; p.cfg = cfg; p.W = W; p.L = L; p.C = d.C; p.T = Ts; p.rows = rows; p.sample_last = sample_last; p.cfg_scale = cfg_scale;
+    p.maps = hd->d_gc_maps; p.c1 = hd->c1[0]; p.bg = hd->bg[0]; p.b2 = hd->b2[0]; p.bsc = hd->bsc[0]; p.bfsh = hd->bfsh; p.bfsc = hd->bfsc;
+    p.sched = d_sched; p.win = hd->win; p.bin = hd->bin; p.wout_t = hd->wout_t; p.bout = hd->bout; p.x_T = x_T; p.eps = eps;
+    p.x = ws.x; p.x0 = x0; p.mu1 = mu1; p.x1 = x1; p.traj_x = traj_x; p.traj_mu = traj_mu; p.err = ctx->d_err; p.status = ctx->d_err + 1;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kSbCluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t lc{};
     lc.attrs = at; lc.numAttrs = 1;
-    if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, sb_chain_kernel<__half, 0>, tm_a, tm_vv, tm_sa, p));
-    else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, sb_chain_kernel<__nv_bfloat16, 1>, tm_a, tm_vv, tm_sa, p));
-    ctx->launches++;
+    int n = (256 + rows - 1) / rows;
+    for (int t_hi = Ts, c = 0; t_hi >= 1; ++c, n *= 2) {
+      if (n > most) n = most;
+      if (n > t_hi) n = t_hi;
+      const int t_lo = t_hi - n + 1, buf = c & 1;
+      float4* mods = reinterpret_cast<float4*>(static_cast<char*>(ctx->gm[slot].base) + buf * chunk_bytes(most));
+      MgParams m{};
+      m.nkb = W / kBlockK; m.tiles_n = (n * rows + 255) / 256; m.units = m.tiles_n * static_cast<int>(wrows / 256);
+      m.s_row0 = (t_lo - 1) * rows; m.out = mods; m.err = ctx->d_err;
+      if (c >= 2) CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_read[slot][buf], 0));
+      // beside a running chain the products take the SMs it leaves
+      int pairs = (c == 0 ? ctx->num_sms : ctx->num_sms - chains * groups * cl) / 2;
+      if (pairs < 8) pairs = 8;
+      if (pairs > m.units) pairs = m.units;
+      lc.gridDim = dim3(static_cast<unsigned>(2 * pairs)); lc.blockDim = dim3(kMgThreads); lc.dynamicSmemBytes = kMgSmemBytes; lc.stream = gst;
+      at[0].val.clusterDim.x = 2;
+      if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<0>, hd->Wm, tm_s, m));
+      else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<1>, hd->Wm, tm_s, m));
+      CSD_CUDA(ctx, cudaEventRecord(ctx->ev_mods[slot][buf], gst));
+      CSD_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_mods[slot][buf], 0));
+      p.t_hi = t_hi; p.t_lo = t_lo; p.mods = mods; p.nq = m.tiles_n * 64;
+      lc.gridDim = dim3(static_cast<unsigned>(groups * cl)); lc.blockDim = dim3(kGcThreads); lc.dynamicSmemBytes = gc_layout(W).total + 1024; lc.stream = st;
+      at[0].val.clusterDim.x = static_cast<unsigned>(cl);
+      if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, group_chain_kernel<__half, 0>, p));
+      else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, group_chain_kernel<__nv_bfloat16, 1>, p));
+      CSD_CUDA(ctx, cudaEventRecord(ctx->ev_read[slot][buf], st));
+      ctx->launches += 2;
+      t_hi = t_lo - 1;
+    }
     return CSD_OK;
   }
 
   int step(int t) {
-    if (sbk || pck || fcg) return CSD_OK;   // already enqueued by begin()
+    if (gck || pck || fcg) return CSD_OK;   // already enqueued by begin()
     const csd_head_desc& d = hd->d;
     ChainWs& ws = ctx->ws[slot];
     cur_t = t;
@@ -1049,7 +1081,7 @@ size_t bonus_buf_bytes(const csd_head_desc& d, int Rt, int cfg, int T) {
 int ensure_side(csd_ctx* ctx, HostIo& io, size_t need, const char* what) {
   if (need <= io.cap) return CSD_OK;
   CSD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  for (int i = 0; i < 2; ++i) CSD_CUDA(ctx, cudaStreamSynchronize(ctx->side[i]));
+  for (int i = 0; i < 2; ++i) { CSD_CUDA(ctx, cudaStreamSynchronize(ctx->side[i])); CSD_CUDA(ctx, cudaStreamSynchronize(ctx->aux[i])); }
   if (io.base) CSD_CUDA(ctx, cudaFree(io.base));
   io.base = nullptr; io.cap = 0;
   if (cudaMalloc(&io.base, need) != cudaSuccess) {
@@ -1121,6 +1153,11 @@ int csd_create(csd_ctx** out, int device, void* cuda_stream) {
   for (int i = 0; i < 2; ++i) {
     ok = ok && cudaStreamCreateWithPriority(&c->side[i], cudaStreamNonBlocking, i == 1 ? prio_hi : prio_lo) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->ev_done[i], cudaEventDisableTiming) == cudaSuccess;
+    ok = ok && cudaStreamCreateWithPriority(&c->aux[i], cudaStreamNonBlocking, prio_lo) == cudaSuccess;
+    ok = ok && cudaEventCreateWithFlags(&c->ev_prep[i], cudaEventDisableTiming) == cudaSuccess;
+    for (int j = 0; j < 2; ++j)
+      ok = ok && cudaEventCreateWithFlags(&c->ev_mods[i][j], cudaEventDisableTiming) == cudaSuccess &&
+           cudaEventCreateWithFlags(&c->ev_read[i][j], cudaEventDisableTiming) == cudaSuccess;
   }
   ok = ok && cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess;
   ok = ok && cudaMalloc(&c->d_err, 4 * sizeof(int)) == cudaSuccess;   // [0] first failed wait, [1] non-finite value seen, [2..3] tally_cap_hits
@@ -1145,6 +1182,12 @@ int csd_destroy(csd_ctx* c) {
   cudaStreamSynchronize(c->stream);
   for (int i = 0; i < 2; ++i) {
     if (c->side[i]) { cudaStreamSynchronize(c->side[i]); cudaStreamDestroy(c->side[i]); }
+    if (c->aux[i]) { cudaStreamSynchronize(c->aux[i]); cudaStreamDestroy(c->aux[i]); }
+    if (c->ev_prep[i]) cudaEventDestroy(c->ev_prep[i]);
+    for (int j = 0; j < 2; ++j) {
+      if (c->ev_mods[i][j]) cudaEventDestroy(c->ev_mods[i][j]);
+      if (c->ev_read[i][j]) cudaEventDestroy(c->ev_read[i][j]);
+    }
     if (c->ev_done[i]) cudaEventDestroy(c->ev_done[i]);
   }
   for (ChainWs& w : c->ws)
@@ -1155,7 +1198,8 @@ int csd_destroy(csd_ctx* c) {
   if (c->sp.base) cudaFree(c->sp.base);
   if (c->un.base) cudaFree(c->un.base);
   if (c->bn.base) cudaFree(c->bn.base);
-  for (HostIo& b : c->sb) if (b.base) cudaFree(b.base);
+  for (HostIo& b : c->gc) if (b.base) cudaFree(b.base);
+  for (HostIo& b : c->gm) if (b.base) cudaFree(b.base);
   for (HostIo& b : c->pc) if (b.base) cudaFree(b.base);
   if (c->d_err) cudaFree(c->d_err);
   cudaGetLastError();
@@ -1382,11 +1426,11 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
   const size_t f_bfsh = put(w->bfada, W), f_bfsc = put(w->bfada + W, W);
   // folded blocks: c1_k = W1_k (1 + bscale_k), c2_k = W1_k bshift_k + b1_k  (double accumulation, rounded once)
   const bool folded = d.dtype != CSD_F32 && L >= 2;
-  // the small-batch chain kernel folds every block, the first included
-  const bool sbk = d.dtype != CSD_F32 && W % 512 == 0 && W <= static_cast<size_t>(kSbMaxW) && !d.var_out;
-  const size_t kfold0 = sbk ? 0 : 1;      // first block that has folded weights
+  // the group chain kernel and the persistent chain kernel fold every block, the first included
+  const bool gck = d.dtype != CSD_F32 && W % 512 == 0 && W <= static_cast<size_t>(kGcMaxW) && !d.var_out;
+  const size_t kfold0 = gck ? 0 : 1;      // first block that has folded weights
   std::vector<size_t> f_c1(L, 0), f_c2(L, 0);
-  if (folded || sbk) {
+  if (folded || gck) {
     std::vector<float> v1(W), v2(W);
     for (size_t k = kfold0; k < L; ++k) {
       const float* W1k = w->W1 + k * W * W;
@@ -1407,7 +1451,7 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
   h->win = fb + f_win; h->bin = fb + f_bin; h->wout_t = fb + f_wout; h->bout = fb + f_bout;
   h->bfsh = fb + f_bfsh; h->bfsc = fb + f_bfsc;
   h->c1.assign(L, nullptr); h->c2.assign(L, nullptr);
-  if (folded || sbk) for (size_t k = kfold0; k < L; ++k) { h->c1[k] = fb + f_c1[k]; h->c2[k] = fb + f_c2[k]; }
+  if (folded || gck) for (size_t k = kfold0; k < L; ++k) { h->c1[k] = fb + f_c1[k]; h->c2[k] = fb + f_c2[k]; }
   h->bsh.resize(L); h->bsc.resize(L); h->bg.resize(L); h->b1.resize(L); h->b2.resize(L);
   for (size_t k = 0; k < L; ++k) { h->bsh[k] = fb + f_bsh[k]; h->bsc[k] = fb + f_bsc[k]; h->bg[k] = fb + f_bg[k]; h->b1[k] = fb + f_b1[k]; h->b2[k] = fb + f_b2[k]; }
 
@@ -1426,15 +1470,25 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
       }
       if (!rc) rc = make_tmap(ctx, &tm.Wfss, d.dtype, h->Wfss, 2 * W, W, W, 2 * tn);
     }
-    std::vector<CUtensorMap> wf128(L);
-    if (!rc && (folded || sbk)) {
-      // xblob: Wgs_0 .. Wgs_{L-2} | Wf_1 .. Wf_{L-1} | Wf_0 (small-batch kernel only), each [2 W, W] in operand format
-      const size_t per = 2 * W * W, nx = (2 * (L - 1) + (sbk ? 1 : 0)) * per;
+    std::vector<float> ms;    // the matrix multiplied by s for the group chain kernel
+    if (!rc && (folded || gck)) {
+      // xblob: Wgs_0 .. Wgs_{L-2} | Wf_1 .. Wf_{L-1} | Wf_0 (where block 0 is folded too), each [2 W, W] in operand format
+      const size_t per = 2 * W * W, nx = (2 * (L - 1) + (gck ? 1 : 0)) * per;
       auto wf_slot = [&](size_t k) { return k == 0 ? 2 * (L - 1) : L - 1 + k - 1; };
       std::vector<float> xs;
       try { xs.resize(nx); } catch (...) { return bail(CSD_ERR_WORKSPACE, "out of host memory"); }
       float *dA = nullptr, *dB = nullptr, *dC = nullptr;
       std::vector<float> f1(W * W), f2(W * W);
+      auto mput = [&](const float* src, size_t sec) { memcpy(&ms[sec * W * W], src, W * W * 4); };
+      if (gck) {
+        try { ms.resize((4 * L + 2) * W * W); } catch (...) { return bail(CSD_ERR_WORKSPACE, "out of host memory"); }
+        mput(w->Wada + W * W, 0);
+        for (size_t k = 0; k < L; ++k) {
+          mput(w->Wada + k * 3 * W * W + 2 * W * W, 3 + 4 * k);
+          if (k + 1 < L) mput(w->Wada + (k + 1) * 3 * W * W + W * W, 4 + 4 * k);
+        }
+        mput(w->Wfada, 4 * L); mput(w->Wfada + W * W, 4 * L + 1);
+      }
       bool okx = cudaMalloc(&dA, W * W * 4) == cudaSuccess && cudaMalloc(&dB, W * W * 4) == cudaSuccess && cudaMalloc(&dC, W * W * 4) == cudaSuccess;
       for (size_t k = 0; k + 1 < L && okx; ++k)     // gate of block k | scale of block k + 1
         interleave(w->Wada + k * 3 * W * W + 2 * W * W, w->Wada + (k + 1) * 3 * W * W + W * W, &xs[k * per]);
@@ -1449,6 +1503,7 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
         if (okx) square_matmul_kernel<<<grid, 256>>>(dA, dB, dC, static_cast<int>(W));
         okx = okx && cudaMemcpy(f2.data(), dC, W * W * 4, cudaMemcpyDeviceToHost) == cudaSuccess;
         if (okx) interleave(f1.data(), f2.data(), &xs[wf_slot(k) * per]);
+        if (okx && gck) { mput(f1.data(), 1 + 4 * k); mput(f2.data(), 2 + 4 * k); }
       }
       if (dA) cudaFree(dA);
       if (dB) cudaFree(dB);
@@ -1466,42 +1521,28 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
       for (size_t k = 1; k < L && !rc; ++k) rc = make_tmap(ctx, &h->Wf[k], d.dtype, xbase + wf_slot(k) * per * 2, 2 * W, W, W, 256);
       for (size_t k = 0; k + 1 < L && !rc; ++k) rc = make_tmap(ctx, &h->Wgs_half[k], d.dtype, xbase + k * per * 2, 2 * W, W, W, 128);
       for (size_t k = kfold0; k < L && !rc; ++k) rc = make_tmap(ctx, &h->Wf_half[k], d.dtype, xbase + wf_slot(k) * per * 2, 2 * W, W, W, 128);
-      for (size_t k = kfold0; k < L && !rc && sbk; ++k) rc = make_tmap(ctx, &wf128[k], d.dtype, xbase + wf_slot(k) * per * 2, 2 * W, W, W, 128);
     }
     if (!rc && W % 256 == 0) {
       h->W1_wide.resize(L);
       for (size_t k = 0; k < L && !rc; ++k) rc = make_tmap(ctx, &h->W1_wide[k], d.dtype, h->W1[k], W, W, W, 256);
     }
     if (rc) { csd_head_destroy(h); return rc; }
-    if (sbk) {
-      // tables of the small-batch chain kernel
+    if (gck) {
+      // tables of the group chain kernel
       std::vector<CUtensorMap> maps;
       for (size_t k = 0; k < L; ++k) { maps.push_back(h->tm[1].W1[k]); maps.push_back(h->tm[1].W2[k]); }
-      std::vector<SbTask> tasks;
-      auto add = [&](const CUtensorMap& m, size_t rows, size_t col0) {
-        const int mi = static_cast<int>(maps.size());
-        maps.push_back(m);
-        for (size_t r = 0; r < rows; r += 128) tasks.push_back(SbTask{mi, static_cast<int>(r), static_cast<int>(col0 + r), 0});
-      };
-      for (size_t k = 0; k < L; ++k) {           // mods columns of block k: [P1 | P2 : 2 W][gate : W][shift | scale : 2 W]
-        add(wf128[k], 2 * W, 5 * k * W);
-        add(h->tm[1].Wg[k], W, 5 * k * W + 2 * W);
-        add(h->tm[0].Wss[k], 2 * W, 5 * k * W + 3 * W);
-      }
-      add(h->tm[0].Wfss, 2 * W, 5 * L * W);
-      std::vector<const float*> bt;
-      for (size_t k = 0; k < L; ++k) { bt.push_back(h->c1[k]); bt.push_back(h->c2[k]); bt.push_back(h->bg[k]); bt.push_back(h->b2[k]); bt.push_back(h->bsc[k]); }
-      bt.push_back(h->bfsh); bt.push_back(h->bfsc);
-      if (cudaMalloc(&h->d_sb_maps, maps.size() * sizeof(CUtensorMap)) != cudaSuccess ||
-          cudaMalloc(&h->d_sb_tasks, tasks.size() * sizeof(SbTask)) != cudaSuccess ||
-          cudaMalloc(&h->d_sb_bias, bt.size() * sizeof(float*)) != cudaSuccess) { cudaGetLastError(); return bail(CSD_ERR_WORKSPACE, "cannot allocate device memory for the small-batch tables"); }
-      if (cudaMemcpy(h->d_sb_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess ||
-          cudaMemcpy(h->d_sb_tasks, tasks.data(), tasks.size() * sizeof(SbTask), cudaMemcpyHostToDevice) != cudaSuccess ||
-          cudaMemcpy(h->d_sb_bias, bt.data(), bt.size() * sizeof(float*), cudaMemcpyHostToDevice) != cudaSuccess) return bail(CSD_ERR_CUDA, "small-batch table upload failed");
-      h->sb_ntasks = static_cast<int>(tasks.size());
-      h->sb_ready = true;
+      std::vector<uint16_t> mb;
+      try { mb.resize(ms.size()); } catch (...) { return bail(CSD_ERR_WORKSPACE, "out of host memory"); }
+      if (d.dtype == CSD_BF16) { for (size_t i = 0; i < ms.size(); ++i) mb[i] = f32_to_bf16_bits(ms[i]); }
+      else { for (size_t i = 0; i < ms.size(); ++i) { const __half hv = __float2half_rn(ms[i]); memcpy(&mb[i], &hv, 2); } }
+      if (cudaMalloc(&h->mblob, mb.size() * 2) != cudaSuccess ||
+          cudaMalloc(&h->d_gc_maps, maps.size() * sizeof(CUtensorMap)) != cudaSuccess) { cudaGetLastError(); return bail(CSD_ERR_WORKSPACE, "cannot allocate device memory for the group-chain tables"); }
+      if (cudaMemcpy(h->mblob, mb.data(), mb.size() * 2, cudaMemcpyHostToDevice) != cudaSuccess ||
+          cudaMemcpy(h->d_gc_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess) return bail(CSD_ERR_CUDA, "group-chain table upload failed");
+      if ((rc = make_tmap(ctx, &h->Wm, d.dtype, h->mblob, (4 * L + 2) * W, W, W, kTileM))) { csd_head_destroy(h); return rc; }
+      h->gc_ready = true;
     }
-    if (sbk && W / kTileN == static_cast<size_t>(kPcColTiles)) {
+    if (gck && W / kTileN == static_cast<size_t>(kPcColTiles)) {
       // tables of the persistent chain kernel: phases B, (W1_k, GATE_k) for every block, F
       const size_t NP = 2 * L + 2;
       std::vector<CUtensorMap> maps(2 * NP);
@@ -1538,9 +1579,8 @@ int csd_head_destroy(csd_head* h) {
   if (h->xblob) cudaFree(h->xblob);
   if (h->d_pc_maps) cudaFree(h->d_pc_maps);
   if (h->d_pc_bias) cudaFree(h->d_pc_bias);
-  if (h->d_sb_maps) cudaFree(h->d_sb_maps);
-  if (h->d_sb_tasks) cudaFree(h->d_sb_tasks);
-  if (h->d_sb_bias) cudaFree(h->d_sb_bias);
+  if (h->d_gc_maps) cudaFree(h->d_gc_maps);
+  if (h->mblob) cudaFree(h->mblob);
   cudaGetLastError();
   delete h;
   return CSD_OK;
@@ -1859,24 +1899,19 @@ static int round_impl(csd_ctx* ctx, const csd_head* head_q, const csd_head* head
   if ((rc = ensure_ws(ctx, ctx->ws[0], head_q->d, R * (cfg ? 2 : 1), R, sched_q->T))) return rc;
   if ((rc = ensure_ws(ctx, ctx->ws[1], head_p->d, Rp * (cfg ? 2 : 1), Rp, sched_p->T))) return rc;
   if (bonus && (rc = ensure_side(ctx, ctx->bn, bonus_buf_bytes(head_p->d, Rp, cfg, T), "the bonus rows"))) return rc;
-  // Few rows in small-batch mode: each chain is one persistent kernel that wants the whole GPU, so the two run one
-  // after the other on the context's stream (the same kernels, hence the same bits, as the separate calls).
-  const bool seq = ctx->chain_mode == CSD_CHAIN_SMALL_BATCH && Rp * (cfg ? 2 : 1) <= kSbRows && head_q->sb_ready && head_p->sb_ready;
-  if (!seq) {
-    CSD_CUDA(ctx, cudaEventRecord(ctx->ev_fork, ctx->stream));
-    for (int i = 0; i < 2; ++i) CSD_CUDA(ctx, cudaStreamWaitEvent(ctx->side[i], ctx->ev_fork, 0));
-  }
+  CSD_CUDA(ctx, cudaEventRecord(ctx->ev_fork, ctx->stream));
+  for (int i = 0; i < 2; ++i) CSD_CUDA(ctx, cudaStreamWaitEvent(ctx->side[i], ctx->ev_fork, 0));
   // the two chains' launches are interleaved step by step so that neither stream starves
   // the chain with more work per row goes to the higher-priority stream
   const double wq = static_cast<double>(head_q->d.L) * head_q->d.W * head_q->d.W, wp = static_cast<double>(head_p->d.L) * head_p->d.W * head_p->d.W;
   const int sq = wq > wp ? 1 : 0;
-  cudaStream_t st_q = seq ? ctx->stream : ctx->side[sq], st_p = seq ? ctx->stream : ctx->side[1 - sq];
+  cudaStream_t st_q = ctx->side[sq], st_p = ctx->side[1 - sq];
   BonusBuf bb{};
   if (bonus && (rc = gather_bonus_inputs(ctx, st_p, head_p->d, R, B, cfg, T, z_p, x_T, eps, z_next, x_T_next, eps_next, bb))) return rc;
   Chain cq{ctx, 0, st_q, head_q, sched_q, R, cfg, cfg_scale, z_q, x_T, eps, 1, x0, mu1_q, nullptr};
   Chain cp = bonus ? Chain{ctx, 1, st_p, head_p, sched_p, Rp, cfg, cfg_scale, bb.z, bb.x_T, bb.eps, 1, bb.x0, bb.mu1, nullptr}
                    : Chain{ctx, 1, st_p, head_p, sched_p, R, cfg, cfg_scale, z_p, x_T, eps, 0, nullptr, mu1_p, nullptr};
-  cq.chains = cp.chains = seq ? 1 : 2;
+  cq.chains = cp.chains = 2;
   rc = cp.begin();
   int rc2 = cq.begin();
   for (int t = sched_p->T; t >= 1 && !rc && !rc2; --t) {
@@ -1884,7 +1919,7 @@ static int round_impl(csd_ctx* ctx, const csd_head* head_q, const csd_head* head
     if (!rc) rc2 = cq.step(t);
   }
   if (bonus && !rc) CSD_CUDA(ctx, cudaMemcpyAsync(mu1_p, bb.mu1, static_cast<size_t>(R) * C * 4, cudaMemcpyDeviceToDevice, st_p));
-  for (int i = 0; i < 2 && !seq; ++i) {
+  for (int i = 0; i < 2; ++i) {
     CSD_CUDA(ctx, cudaEventRecord(ctx->ev_done[i], ctx->side[i]));
     CSD_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_done[i], 0));
   }

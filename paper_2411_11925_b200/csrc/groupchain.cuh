@@ -1,0 +1,580 @@
+// A denoising chain of few rows (W in {512, 1024, 1536}, 16-bit operands) in two parts:
+//
+// 1. mods_gemm_kernel: everything a head takes from the condition vector - gates, scales, the folded first-layer terms
+//    P1 | P2 of fold.cuh, the final shift and scale: two thirds of its multiply-adds - does not depend on x_t.  It is
+//    formed for many steps at once, as one dense product over the rows of a chunk of steps, in fp32.
+// 2. group_chain_kernel: what depends on x_t.  Token rows never exchange data, so the rows are cut into groups of 16 (with
+//    guidance 8 tokens' conditional rows and their unconditional twins) and a cluster of W / 128 CTAs owns a group for all
+//    steps of the chunk; CTA r owns output columns [128 r, 128 r + 128) of every layer.  Groups never wait for each other and
+//    nothing waits for a kernel that runs beside it, so any number of chains may run at a time.
+//
+// Few rows are bound by latency: per layer a CTA multiplies its 128 weight rows (the MMA's M operand, streamed ahead through
+// a ring) with the group's 16 rows (its N), 64 instructions or 2.6 k cycles at W = 1024, and the results have to reach the
+// other CTAs of the cluster.  They do so by bulk copies from shared memory to shared memory (4 KB to each, 0.7 to 2 k cycles;
+// each CTA's MMAs start on whichever tile its own turn order reaches first, its own tile first), counted in by mbarriers: no
+// trip through L2, no proxy fence, no cluster barrier.  The two activation buffers (a', v) need no hand-back: a CTA sends its
+// part of one only after its product on the other, which took every peer's part of that.  LayerNorm partials travel as
+// 8-byte remote stores, the residual stream h stays in registers (a thread owns a column of 16 rows), and every CTA of the
+// cluster updates the group's token states x_t for itself from the exchanged output-projection partials.
+//
+// The kernel this replaces (products of s by other CTAs of the same kernel, activations through L2, a cluster barrier per
+// layer) took 38.6 us a step on a 3 x 1024 head of 128 rows and needed the GPU to itself.
+#pragma once
+#include "fold.cuh"
+
+namespace csd {
+
+// ------------------------------------------------------------------------------------------ products of s_t
+constexpr int kMgStages = 6, kMgStageBytes = 32768;   // per stage: 128 weight rows | 128 rows of s, one k-block of 64
+constexpr int kMgEpiWarps = 8;
+constexpr int kMgThreads = (kMgEpiWarps + 3) * 32;
+constexpr int kMgSmemBytes = 1024 + kMgStages * kMgStageBytes + 256;
+
+// After a wait that ran out, copies may be in flight that nobody waits for: they land within microseconds.
+__device__ __forceinline__ void gc_settle(const int* err) {
+  if (*reinterpret_cast<const volatile int*>(err) != 0)
+    for (int i = 0; i < 64; ++i) __nanosleep(1000);
+}
+
+struct MgParams {
+  int nkb, tiles_n, units;     // k-blocks; tiles of 256 rows of s; tiles in all (s fastest: the weights stream past once)
+  int s_row0;                  // first row of s
+  float4* out;                 // [weight row / 128][row of s / 4][128 weight rows][4 rows of s]
+  int* err;
+};
+
+// out = weights s^T in 256 x 256 tiles per CTA pair, written from registers: a lane holds one weight row, so a warp's 16-byte
+// stores cover 512 contiguous bytes, and a group's 16 rows of one column tile are one contiguous 8 KB block.
+template <int AB_FMT>
+__global__ void __launch_bounds__(kMgThreads, 1)
+mods_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmS, const MgParams p) {
+  constexpr int S = kMgStages;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + S * kMgStageBytes);
+  uint64_t* empty_bar = full_bar + S;
+  uint64_t* acc_full = empty_bar + S;     // [2]
+  uint64_t* acc_empty = acc_full + 2;     // [2], every epilogue warp of both CTAs
+  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(acc_empty + 2);     // and whether the context is free of errors
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = static_cast<int>(cluster_ctarank());
+  const int unit0 = static_cast<int>(blockIdx.x >> 1), nunits = static_cast<int>(gridDim.x >> 1);
+  const int my_tiles = (p.units - unit0 + nunits - 1) / nunits;
+  if (threadIdx.x == 0) {
+    tma_prefetch_desc(&tmW); tma_prefetch_desc(&tmS);
+    for (int s = 0; s < S; ++s) { mbar_init(&full_bar[s], 2); mbar_init(&empty_bar[s], 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 2 * kMgEpiWarps); }
+    tmem_base_s[1] = *reinterpret_cast<const volatile int*>(p.err) == 0;    // one reading for all warps
+    fence_mbar_init();
+  }
+  if (warp == 1) { tmem_alloc_pair(tmem_base_s, 512); tmem_relinquish_pair(); }
+  tc_fence_before_sync();
+  __syncthreads();
+  cluster_arrive(); cluster_wait();       // the peer's barriers exist before anything signals them
+  tc_fence_after_sync();
+  const uint32_t tmem_base = *tmem_base_s;
+  const bool run = tmem_base_s[1] != 0;
+
+  if (run && (warp == 0 || warp == kMgEpiWarps + 2)) {
+    const bool is_w = warp == 0;
+    if (lane == 0) {
+      bool ok = true;
+      int it = 0;
+      for (int i = 0; i < my_tiles && ok; ++i) {
+        const int u = unit0 + i * nunits;
+        const int row = (is_w ? (u / p.tiles_n) * 256 : p.s_row0 + (u % p.tiles_n) * 256) + rank * 128;
+        for (int kb = 0; kb < p.nkb; ++kb, ++it) {
+          const int s = it % S;
+          if (it >= S && !ch_wait<false>(&empty_bar[s], ((it / S) & 1) ^ 1, p.err)) { ch_fail(p.err, DEV_ERR_TMA_WAIT, 1, it); ok = false; break; }
+          if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], 32768);     // both CTAs' bytes of this operand
+          tma_load_2d_pair(smem + s * kMgStageBytes + (is_w ? 0 : 16384), is_w ? &tmW : &tmS, mapa_shared(smem_u32(&full_bar[s]), 0), kb * kBlockK, row);
+        }
+      }
+    }
+    __syncwarp();
+  } else if (run && warp == 1 && rank == 0) {
+    const bool leader = elect_one();
+    constexpr uint32_t idesc = umma_idesc_f16(256, AB_FMT, 256);
+    bool ok = true;
+    int it = 0;
+    for (int i = 0; i < my_tiles && ok; ++i) {
+      const int ab = i & 1;
+      if (i >= 2 && !ch_wait<true>(&acc_empty[ab], ((i >> 1) - 1) & 1, p.err)) { if (leader) ch_fail(p.err, DEV_ERR_MMA_WAIT, 1, i); ok = false; break; }
+      tc_fence_after_sync();
+      for (int kb = 0; kb < p.nkb; ++kb, ++it) {
+        const int s = it % S;
+        if (!ch_wait<false>(&full_bar[s], (it / S) & 1, p.err)) { if (leader) ch_fail(p.err, DEV_ERR_MMA_WAIT, 2, it); ok = false; break; }
+        tc_fence_after_sync();
+        if (leader) {
+          const uint32_t sa = smem_u32(smem + s * kMgStageBytes);
+          const uint64_t da = umma_smem_desc_sw128(sa), db = umma_smem_desc_sw128(sa + 16384);
+#pragma unroll
+          for (int k = 0; k < kBlockK / 16; ++k) umma_f16_pair(tmem_base + ab * 256, da + 2 * k, db + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+          umma_commit_pair(&empty_bar[s]);
+        }
+        __syncwarp();
+      }
+      if (ok && leader) umma_commit_pair(&acc_full[ab]);
+      __syncwarp();
+    }
+  } else if (run && warp >= 2 && warp < kMgEpiWarps + 2) {
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    bool ok = true;
+    for (int i = 0; i < my_tiles && ok; ++i) {
+      const int u = unit0 + i * nunits, ab = i & 1;
+      ok = ch_wait<false>(&acc_full[ab], (i >> 1) & 1, p.err);
+      if (!ok) ch_fail(p.err, DEV_ERR_EPI_WAIT, 1, i);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after_sync();
+      const uint32_t trow = tmem_base + ab * 256 + half * 128 + (static_cast<uint32_t>(q * 32) << 16);
+      float4* o = p.out + ((static_cast<size_t>(u / p.tiles_n) * 2 + rank) * (p.tiles_n * 64) + (u % p.tiles_n) * 64 + half * 32) * 128 + q * 32 + lane;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        float a[kChunk];
+        tmem_ld32(trow + c * kChunk, a);
+        tmem_ld_wait();
+        if (c == 3) {            // this warp's last read of the buffer
+          tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster_tmem(mapa_shared(smem_u32(&acc_empty[ab]), 0));
+        }
+#pragma unroll
+        for (int j = 0; j < kChunk / 4; ++j) o[(c * 8 + j) * 128] = make_float4(a[4 * j], a[4 * j + 1], a[4 * j + 2], a[4 * j + 3]);
+      }
+    }
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  gc_settle(p.err);
+  cluster_arrive(); cluster_wait();   // neither CTA leaves while the pair's MMAs or signals may touch it
+  if (warp == 1) tmem_dealloc_pair(tmem_base, 512);
+}
+
+// ------------------------------------------------------------------------------------------ the chain
+constexpr int kGcRows = 16;               // rows of a group = MMA N
+constexpr int kGcThreads = 256;           // warps: weights 0, MMA 1, condition products 2, (3), epilogue 4..7
+constexpr int kGcMaxW = 1536;
+constexpr int kGcMaxCl = kGcMaxW / 128;
+constexpr int kGcWinLd = kCPad + 1;       // a row of Win and its bias in shared memory (odd: lanes walk rows)
+constexpr int kGcTile = kGcRows * 256;    // bytes of one CTA's part of an activation buffer: two k-blocks of [16 rows][128 B]
+
+struct GcLayout { int act, ring, stages, mods, stage, win, wout, stats, misc, total; };
+__host__ __device__ inline GcLayout gc_layout(int W) {
+  GcLayout l{};
+  int o = 0;
+  auto take = [&](int n) { const int r = o; o += n; return r; };
+  l.stages = W > 1024 ? 2 : 3;
+  l.act = take(2 * kGcRows * W * 2);      // a' | v
+  l.ring = take(l.stages * 32768);        // stages of two k-blocks of [128 weight rows][128 B]
+  l.mods = take(2 * 16384);               // two items' condition products, each [product][row quad][128 columns][4]
+  l.stage = take(2 * kGcTile + 1024);     // outgoing tiles, by turns, and the outgoing partial: a peer's tile of one phase says that it
+                                          // has received this CTA's of the phase before, so two buffers never overrun a copy
+  l.win = take(128 * kGcWinLd * 4);
+  l.wout = take(128 * kCPad * 4);
+  l.stats = take(W / 32 * kGcRows * 8);   // [32-column group][row] (mean, M2)
+  l.misc = take(1024 + 512 + 512);        // x [16 tokens][16], (mean, rstd) per warp [4][16], barriers
+  l.total = o;
+  return l;
+}
+
+struct GcParams {
+  int R, cfg, W, L, C, T, t_hi, t_lo, rows, sample_last;   // rows: kernel rows (groups x 16)
+  float cfg_scale;
+  const CUtensorMap* maps;     // [2 L]: W1_k, W2_k in boxes of 128 rows
+  const float4* mods; int nq;  // products of the chunk, nq row quads per weight row
+  const float *c1, *bg, *b2, *bsc, *bfsh, *bfsc;   // block 0; c1_k | c2_k are 2 W floats a block, the others 5 W apart
+  const float* sched;          // a[T], b[T], sigma[T]
+  const float *win, *bin, *wout_t, *bout;
+  const float *x_T, *eps;
+  float *x, *x0, *mu1, *x1, *traj_x, *traj_mu;
+  int* err;
+  int* status;
+};
+
+// Shared memory of this CTA -> the same or another CTA of the cluster, completion counted in bytes on a barrier there.
+__device__ __forceinline__ void gc_copy(uint32_t dst_cluster, const void* src, uint32_t bytes, uint32_t bar_cluster) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst_cluster), "r"(smem_u32(src)), "r"(bytes), "r"(bar_cluster) : "memory");
+}
+__device__ __forceinline__ void gc_st_async(uint32_t dst_cluster, float a, float b, uint32_t bar_cluster) {
+  const unsigned long long v = (static_cast<unsigned long long>(__float_as_uint(b)) << 32) | __float_as_uint(a);
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(dst_cluster), "l"(v), "r"(bar_cluster) : "memory");
+}
+// Sums 16 values over the warp, transposing: lane l ends with value l / 2.
+__device__ __forceinline__ float gc_reduce16(const float (&in)[kGcRows], int lane) {
+  float v[kGcRows];
+#pragma unroll
+  for (int i = 0; i < kGcRows; ++i) v[i] = in[i];
+#pragma unroll
+  for (int n = 8; n >= 1; n >>= 1) {
+    const int o = 2 * n;
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i < n) {
+        const float send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+template <typename ACT, int AB_FMT>
+__global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid_constant__ GcParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int W = p.W, L = p.L, T = p.T, CL = W / 128, NI = 2 * L + 2;   // items with condition products per step
+  const GcLayout lo = gc_layout(W);
+  const int act_bytes = kGcRows * W * 2;
+  uint8_t* act = smem + lo.act;
+  uint8_t* stage = smem + lo.stage;
+  float4* part_out = reinterpret_cast<float4*>(stage + 2 * kGcTile);
+  float* win_s = reinterpret_cast<float*>(smem + lo.win);
+  float* wout_s = reinterpret_cast<float*>(smem + lo.wout);
+  float2* stats_s = reinterpret_cast<float2*>(smem + lo.stats);
+  float* xs = reinterpret_cast<float*>(smem + lo.misc);
+  float2* norm_all = reinterpret_cast<float2*>(smem + lo.misc + 1024);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + lo.misc + 1536);
+  uint64_t *w_full = bars, *w_empty = bars + 3, *act_full = bars + 6, *acc_full = act_full + 2 * kGcMaxCl, *mods_full = acc_full + 1,
+           *mods_free = mods_full + 2, *stats_full = mods_free + 2, *part_full = stats_full + 1;
+  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(part_full + 1);     // and whether the context is free of errors
+  // free at the end of a step, when every product that reads them is complete here: the columns' modulated h (read by this
+  // CTA only), the peers' output-projection partials
+  float* uf_s = reinterpret_cast<float*>(act);                       // [16][kUfLd]
+  float* part_s = reinterpret_cast<float*>(act + act_bytes);         // [CL][16][16]
+  constexpr int kUfLd = 132;
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = static_cast<int>(cluster_ctarank()), grp = static_cast<int>(blockIdx.x) / CL;
+  const int n_base = rank * 128;
+  if (tid == 0) {
+    for (int s = 0; s < 3; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); }
+    for (int i = 0; i < 2 * kGcMaxCl; ++i) mbar_init(&act_full[i], 1);
+    mbar_init(acc_full, 1);
+    for (int i = 0; i < 2; ++i) { mbar_init(&mods_full[i], 1); mbar_init(&mods_free[i], 4); }
+    mbar_init(stats_full, 1); mbar_init(part_full, 1);
+    tmem_base_s[1] = *reinterpret_cast<const volatile int*>(p.err) == 0;    // one reading for all warps
+    fence_mbar_init();
+  }
+  if (warp == 1) { tmem_alloc(tmem_base_s, 32); tmem_relinquish(); }
+  for (int i = tid; i < 128 * kCPad; i += kGcThreads) {
+    win_s[(i / kCPad) * kGcWinLd + i % kCPad] = p.win[static_cast<size_t>(n_base) * kCPad + i];
+    wout_s[i] = p.wout_t[static_cast<size_t>(n_base) * kCPad + i];
+  }
+  if (tid < 128) win_s[tid * kGcWinLd + kCPad] = p.bin[n_base + tid];
+  tc_fence_before_sync();
+  __syncthreads();
+  cluster_arrive(); cluster_wait();       // the peers' barriers exist before anything signals them
+  tc_fence_after_sync();
+  const uint32_t tmem_base = *tmem_base_s;
+  const bool run = tmem_base_s[1] != 0;
+
+  // (a CTA that gives up on a wait goes on through its barriers without waiting: its peers' waits end by the context's
+  // error word)
+  if (run && warp == 0) {
+    // ---------------------------------------------------------------- weights, k-blocks in this CTA's turn order
+    if (lane == 0) {
+      uint32_t it = 0, s = 0, par = 1;
+      bool ok = true;
+      for (int t = p.t_hi; t >= p.t_lo && ok; --t)
+        for (int ph = 0; ph < 2 * L && ok; ++ph)
+          for (int j = 0; j < CL; ++j, ++it) {
+            const int src = rank + j < CL ? rank + j : rank + j - CL;
+            if (it >= static_cast<uint32_t>(lo.stages) && !ch_wait<false>(&w_empty[s], par, p.err)) { ch_fail(p.err, DEV_ERR_TMA_WAIT, 1, static_cast<int>(it)); ok = false; break; }
+            mbar_arrive_expect_tx(&w_full[s], 32768);
+            uint8_t* dst = smem + lo.ring + s * 32768;
+            tma_load_2d(dst, p.maps + ph, &w_full[s], src * 128, n_base);
+            tma_load_2d(dst + 16384, p.maps + ph, &w_full[s], src * 128 + kBlockK, n_base);
+            if (++s == static_cast<uint32_t>(lo.stages)) { s = 0; par ^= 1; }
+          }
+    }
+    __syncwarp();
+  } else if (run && warp == 1) {
+    // ---------------------------------------------------------------- MMA issue
+    const bool leader = elect_one();
+    constexpr uint32_t idesc = umma_idesc_f16(kGcRows, AB_FMT);
+    bool ok = true;
+    uint32_t s = 0, par = 0, use = 0;
+    for (int t = p.t_hi; t >= p.t_lo && ok; --t)
+      for (int ph = 0; ph < 2 * L && ok; ++ph) {
+        const int buf = ph & 1;
+        if (lane < CL) mbar_arrive_expect_tx(&act_full[buf * kGcMaxCl + lane], kGcTile);
+        __syncwarp();
+        for (int j = 0; j < CL; ++j) {
+          const int src = rank + j < CL ? rank + j : rank + j - CL;
+          ok = ch_wait<false>(&act_full[buf * kGcMaxCl + src], use & 1, p.err) && ch_wait<false>(&w_full[s], par, p.err);
+          if (!ok) { if (leader) ch_fail(p.err, DEV_ERR_MMA_WAIT, 2, ph); break; }
+          tc_fence_after_sync();
+          if (leader) {
+            const uint32_t sa = smem_u32(smem + lo.ring + s * 32768), sb = smem_u32(act + buf * act_bytes + src * kGcTile);
+#pragma unroll
+            for (int jj = 0; jj < 2; ++jj) {
+              const uint64_t da = umma_smem_desc_sw128(sa + jj * 16384), db = umma_smem_desc_sw128(sb + jj * (kGcRows * 128));
+#pragma unroll
+              for (int k = 0; k < kBlockK / 16; ++k) umma_f16(tmem_base, da + 2 * k, db + 2 * k, idesc, (j > 0 || jj > 0 || k > 0) ? 1u : 0u);
+            }
+            umma_commit(&w_empty[s]);
+          }
+          __syncwarp();
+          if (++s == static_cast<uint32_t>(lo.stages)) { s = 0; par ^= 1; }
+        }
+        if (ok && leader) umma_commit(acc_full);
+        __syncwarp();
+        if (buf == 1) ++use;
+      }
+  } else if (run && warp == 2) {
+    // ---------------------------------------------------------------- condition products, an item ahead
+    if (lane == 0) {
+      uint32_t n = 0;
+      bool ok = true;
+      for (int t = p.t_hi; t >= p.t_lo && ok; --t)
+        for (int item = 0; item < NI; ++item, ++n) {
+          const int b = n & 1;
+          if (n >= 2 && !ch_wait<false>(&mods_free[b], ((n >> 1) - 1) & 1, p.err)) { ch_fail(p.err, DEV_ERR_TMA_WAIT, 3, item); ok = false; break; }
+          const int sec = item == 0 ? 0 : item == NI - 1 ? 4 * L : 2 * item - 1, ns = item == 0 || item == 2 * L ? 1 : 2;
+          mbar_arrive_expect_tx(&mods_full[b], ns * 8192);
+          const size_t q0 = (static_cast<size_t>(t - p.t_lo) * p.rows + grp * kGcRows) / 4;
+          for (int u = 0; u < ns; ++u)
+            bulk_load(smem + lo.mods + b * 16384 + u * 8192, p.mods + (static_cast<size_t>((sec + u) * CL + rank) * p.nq + q0) * 128, 8192, &mods_full[b]);
+        }
+    }
+    __syncwarp();
+  } else if (run && warp >= 4) {
+    // ---------------------------------------------------------------- epilogue: thread = one column of the group's 16 rows
+    const int ew = warp - 4, et = tid - 128, c = ew * 32 + lane, col = n_base + c;
+    const int per = p.cfg ? 8 : 16, tok0 = grp * per;        // tokens of the group; row i is token i % per
+    float2* norm_s = norm_all + ew * kGcRows;                // this warp's copy of the rows' (mean, rstd)
+    bool ok = true;
+    uint32_t n_item = 0, n_acc = 0, n_stat = 0, n_part = 0, n_tile = 0;
+    auto epi_sync = [&]() { asm volatile("bar.sync 1, 128;" ::: "memory"); };
+    auto wait = [&](uint64_t* bar, uint32_t parity, int site) {
+      if (ok && !ch_wait<true>(bar, parity, p.err)) { ch_fail(p.err, DEV_ERR_EPI_WAIT, site, static_cast<int>(n_item)); ok = false; }
+    };
+    // this item's condition products of the column
+    auto take = [&](float* m0, float* m1) {
+      const int b = n_item & 1;
+      wait(&mods_full[b], (n_item >> 1) & 1, 4);
+      const float4* src = reinterpret_cast<const float4*>(smem + lo.mods + b * 16384) + c;
+#pragma unroll
+      for (int q = 0; q < kGcRows / 4; ++q) {
+        const float4 v = src[q * 128];
+        m0[4 * q] = v.x; m0[4 * q + 1] = v.y; m0[4 * q + 2] = v.z; m0[4 * q + 3] = v.w;
+        if (m1) { const float4 w = src[512 + q * 128]; m1[4 * q] = w.x; m1[4 * q + 1] = w.y; m1[4 * q + 2] = w.z; m1[4 * q + 3] = w.w; }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&mods_free[b]);
+      ++n_item;
+    };
+    // 16-bit tile of this CTA's columns, to every CTA's activation buffer `buf`
+    auto send_tile = [&](const float (&v)[kGcRows], int buf) {
+      uint8_t* const out = stage + (n_tile++ & 1) * kGcTile;
+      uint8_t* kb = out + (c >> 6) * (kGcRows * 128);
+      const int u = (c & 63) >> 3, b = (c & 7) * 2;
+#pragma unroll
+      for (int i = 0; i < kGcRows; ++i) *reinterpret_cast<ACT*>(kb + i * 128 + ((u ^ (i & 7)) << 4) + b) = to_act<ACT>(v[i]);
+      fence_proxy_async_smem();
+      epi_sync();
+      if (ok && ew == 0 && lane < CL) {
+        const int peer = rank + lane < CL ? rank + lane : rank + lane - CL;
+        gc_copy(mapa_shared(smem_u32(act + buf * act_bytes + rank * kGcTile), peer), out, kGcTile, mapa_shared(smem_u32(&act_full[buf * kGcMaxCl + rank]), peer));
+      }
+      __syncwarp();
+    };
+    // (mean, M2) of each row over this warp's 32 columns, to every CTA
+    auto send_stats = [&](const float (&v)[kGcRows]) {
+      const float mean = gc_reduce16(v, lane) * (1.0f / 32.0f);     // of row lane / 2
+      float d[kGcRows];
+#pragma unroll
+      for (int i = 0; i < kGcRows; ++i) { const float e = v[i] - __shfl_sync(0xffffffffu, mean, 2 * i); d[i] = e * e; }
+      const float m2 = gc_reduce16(d, lane);
+      const uint32_t at = smem_u32(stats_s + (rank * 4 + ew) * kGcRows + (lane >> 1)), bar = smem_u32(stats_full);
+      for (int r = lane & 1; ok && r < CL; r += 2) gc_st_async(mapa_shared(at, r), mean, m2, mapa_shared(bar, r));
+    };
+    const uint32_t stats_bytes = static_cast<uint32_t>(CL) * 4 * kGcRows * 8, part_bytes = static_cast<uint32_t>(CL) * kGcRows * kCPad * 4;
+    // the rows' (mean, rstd) from all partials, into norm_s (32-column groups merged as equal-count partials)
+    auto norms = [&]() {
+      wait(stats_full, n_stat & 1, 5);
+      if (et == 0) mbar_arrive_expect_tx(stats_full, stats_bytes);   // the next phase's
+      ++n_stat;
+      const int row = lane & 15, h = lane >> 4, G = CL * 2;          // two lanes per row, half of the W / 32 partials each
+      const float2* src = stats_s + h * G * kGcRows + row;
+      float sm = 0.0f, m2 = 0.0f, q = 0.0f;
+      for (int g = 0; g < G; ++g) { const float2 v = src[g * kGcRows]; sm += v.x; m2 += v.y; }
+      sm += __shfl_xor_sync(0xffffffffu, sm, 16);
+      const float mean = sm / static_cast<float>(2 * G);
+      for (int g = 0; g < G; ++g) { const float d = src[g * kGcRows].x - mean; q = fmaf(d, d, q); }
+      m2 = fmaf(32.0f, q, m2);
+      m2 += __shfl_xor_sync(0xffffffffu, m2, 16);
+      if (lane < kGcRows) norm_s[row] = make_float2(mean, 1.0f / sqrtf(m2 / static_cast<float>(W) + 1e-6f));
+      __syncwarp();
+    };
+    auto acc_load = [&](float (&a)[kGcRows]) {
+      wait(acc_full, n_acc & 1, 6);
+      ++n_acc;
+      tc_fence_after_sync();
+      tmem_ld16(tmem_base + (static_cast<uint32_t>(ew * 32) << 16), a);
+      tmem_ld_wait();
+      tc_fence_before_sync();
+    };
+
+    if (et == 0) { mbar_arrive_expect_tx(stats_full, stats_bytes); mbar_arrive_expect_tx(part_full, part_bytes); }
+    // state of the group's tokens
+    const bool first = p.t_hi == T;
+    for (int i = et; i < per * kCPad; i += 128) {
+      const int tok = tok0 + (i >> 4), e = i & 15;
+      float v = 0.0f;
+      if (tok < p.R && e < p.C) {
+        const size_t o = static_cast<size_t>(tok) * p.C + e;
+        v = first ? p.x_T[o] : p.x[o];
+        if (first && rank == 0 && p.traj_x) p.traj_x[o] = v;
+      }
+      xs[i] = v;
+    }
+    epi_sync();
+    for (int t = p.t_hi; t >= p.t_lo; --t) {
+      float h[kGcRows], m0[kGcRows], m1[kGcRows], a[kGcRows];
+      // ---- h = Win x + bin for the column, a' = h (1 + scale_0)
+      {
+        float w[kCPad];
+#pragma unroll
+        for (int e = 0; e < kCPad; ++e) w[e] = win_s[c * kGcWinLd + e];
+        const float bi = win_s[c * kGcWinLd + kCPad], bs = __ldg(p.bsc + col);
+#pragma unroll
+        for (int i = 0; i < kGcRows; ++i) {
+          if (i >= 8 && p.cfg) { h[i] = h[i - 8]; continue; }
+          const float4* xq = reinterpret_cast<const float4*>(xs + i * kCPad);
+          float v = bi;
+#pragma unroll
+          for (int q = 0; q < kCPad / 4; ++q) {
+            const float4 x = xq[q];
+            v = fmaf(w[4 * q], x.x, v); v = fmaf(w[4 * q + 1], x.y, v); v = fmaf(w[4 * q + 2], x.z, v); v = fmaf(w[4 * q + 3], x.w, v);
+          }
+          h[i] = v;
+        }
+        take(m0, nullptr);
+#pragma unroll
+        for (int i = 0; i < kGcRows; ++i) a[i] = __fmul_rn(h[i], __fadd_rn(1.0f, __fadd_rn(m0[i], bs)));
+        send_tile(a, 0);
+        send_stats(h);
+      }
+#pragma unroll 1
+      for (int k = 0; k < L; ++k) {
+        // ---- v = SiLU(rstd (a' W1^T - mean (P1 + c1)) + P2 + c2)
+        {
+          const float k0 = __ldg(p.c1 + static_cast<size_t>(2 * k) * W + col), k1 = __ldg(p.c1 + static_cast<size_t>(2 * k + 1) * W + col);
+          take(m0, m1);
+          norms();
+          acc_load(a);
+#pragma unroll
+          for (int i = 0; i < kGcRows; ++i) {
+            const float2 nr = norm_s[i];
+            const float t1 = __fsub_rn(a[i], __fmul_rn(nr.x, __fadd_rn(m0[i], k0)));
+            a[i] = silu_t<true>(fmaf(nr.y, t1, __fadd_rn(m1[i], k1)));
+          }
+          send_tile(a, 1);
+        }
+        // ---- h += gate (v W2^T + b2); a' = h (1 + scale_{k+1})
+        {
+          const bool last = k + 1 == L;
+          const float kg = __ldg(p.bg + static_cast<size_t>(5 * k) * W + col), kb = __ldg(p.b2 + static_cast<size_t>(5 * k) * W + col),
+                      ks = last ? 0.0f : __ldg(p.bsc + static_cast<size_t>(5 * (k + 1)) * W + col);
+          if (last) take(m0, nullptr); else take(m0, m1);
+          acc_load(a);
+#pragma unroll
+          for (int i = 0; i < kGcRows; ++i) h[i] = fmaf(__fadd_rn(m0[i], kg), __fadd_rn(a[i], kb), h[i]);
+          if (!last) {
+#pragma unroll
+            for (int i = 0; i < kGcRows; ++i) a[i] = __fmul_rn(h[i], __fadd_rn(1.0f, __fadd_rn(m1[i], ks)));
+            send_tile(a, 0);
+          }
+          send_stats(h);
+        }
+      }
+      // ---- output projection of (LN(h)(1 + scale_f) + shift_f): this CTA's columns' part, to every CTA
+      const float sa = p.sched[t - 1], sb = p.sched[T + t - 1], sg = p.sched[2 * T + t - 1];
+      float noise[2] = {0.0f, 0.0f};
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int i = et + u * 128, tok = tok0 + (i >> 4), e = i & 15;
+        if (i < per * kCPad && tok < p.R && e < p.C) noise[u] = p.eps[(static_cast<size_t>(t - 1) * p.R + tok) * p.C + e];
+      }
+      {
+        const float k0 = __ldg(p.bfsh + col), k1 = __ldg(p.bfsc + col);
+        take(m0, m1);
+        norms();
+#pragma unroll
+        for (int i = 0; i < kGcRows; ++i) {
+          const float2 nr = norm_s[i];
+          uf_s[i * kUfLd + c] = fmaf(__fmul_rn(__fsub_rn(h[i], nr.x), nr.y), __fadd_rn(1.0f, m1[i] + k1), m0[i] + k0);
+        }
+        epi_sync();
+        // four outputs of one row over half of the columns per thread, the halves a quarter apart (bank conflicts)
+        const int quad = lane & 3, row = ew * 4 + ((lane >> 2) & 3), hf = lane >> 4;
+        float4 o = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 8
+        for (int j = 0; j < 64; ++j) {
+          const int cc = hf * 64 + ((j + hf * 16) & 63);
+          const float u = uf_s[row * kUfLd + cc];
+          const float4 w = *reinterpret_cast<const float4*>(wout_s + cc * kCPad + quad * 4);
+          o.x = fmaf(u, w.x, o.x); o.y = fmaf(u, w.y, o.y); o.z = fmaf(u, w.z, o.z); o.w = fmaf(u, w.w, o.w);
+        }
+        o.x += __shfl_xor_sync(0xffffffffu, o.x, 16); o.y += __shfl_xor_sync(0xffffffffu, o.y, 16);
+        o.z += __shfl_xor_sync(0xffffffffu, o.z, 16); o.w += __shfl_xor_sync(0xffffffffu, o.w, 16);
+        if (hf == 0) part_out[row * 4 + quad] = o;
+        fence_proxy_async_smem();
+        epi_sync();
+        if (ok && ew == 0 && lane < CL)
+          gc_copy(mapa_shared(smem_u32(part_s + rank * kGcRows * kCPad), lane), part_out, kGcRows * kCPad * 4, mapa_shared(smem_u32(part_full), lane));
+        __syncwarp();
+      }
+      // ---- guidance and Eq. 3, by every CTA alike (CTA 0 writes what leaves the chip)
+      wait(part_full, n_part & 1, 7);
+      if (et == 0) mbar_arrive_expect_tx(part_full, part_bytes);
+      ++n_part;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int i = et + u * 128, q = i >> 4, e = i & 15, tok = tok0 + q;
+        if (i >= per * kCPad) continue;
+        auto out = [&](int row) {
+          float s = 0.0f;
+          for (int r = 0; r < CL; ++r) s += part_s[(r * kGcRows + row) * kCPad + e];
+          return s + p.bout[e];
+        };
+        float xn = 0.0f;
+        if (tok < p.R && e < p.C) {
+          const size_t o = static_cast<size_t>(tok) * p.C + e;
+          float ee = out(q);
+          if (p.cfg) ee = cfg_combine(ee, out(8 + q), p.cfg_scale);
+          const float xo = xs[i], mu = ddpm_mean(sa, xo, sb, ee);
+          xn = ddpm_sample(mu, sg, noise[u]);
+          if (rank == 0) {
+            if (!(fabsf(xn) <= 3.0e38f)) *p.status = 1;
+            if (t == 1) {
+              p.mu1[o] = mu;
+              if (p.x1) p.x1[o] = xo;
+              if (p.sample_last && p.x0) p.x0[o] = xn;
+            } else {
+              if (t == p.t_lo) p.x[o] = xn;                    // the next launch starts from it
+              if (p.traj_x) {
+                const size_t slot = static_cast<size_t>(p.R) * p.C;
+                p.traj_x[static_cast<size_t>(T - t + 1) * slot + o] = xn;
+                p.traj_mu[static_cast<size_t>(T - t) * slot + o] = mu;
+              }
+            }
+          }
+        }
+        xs[i] = xn;
+      }
+      epi_sync();
+    }
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  gc_settle(p.err);
+  cluster_arrive(); cluster_wait();       // no CTA leaves while a peer may still write to it
+  if (warp == 1) tmem_dealloc(tmem_base, 32);
+}
+
+}  // namespace csd

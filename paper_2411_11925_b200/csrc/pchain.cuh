@@ -21,7 +21,7 @@
 //           a' = h (1 + scale_{k+1})
 //   F     : early [shift_f | scale_f];  eps partial = (LN(h)(1 + scale_f) + shift_f) Wout^T tile
 //   U     : (token-parallel, between steps) eps reduction, guidance, Eq. 3 update of x.
-// s_t of every step is precomputed (pc_cond_all_kernel) in the kernel's row order: a row block holds 64 tokens'
+// s_t of every step is precomputed (cond_all_kernel) in the kernel's row order: a row block holds 64 tokens'
 // conditional rows followed by their unconditional twins (128 tokens without guidance).
 #pragma once
 #include "fold.cuh"
@@ -125,14 +125,6 @@ __device__ __forceinline__ bool pc_wait_flag(const uint32_t* smem_word, uint32_t
       else if (now - t0 > *reinterpret_cast<volatile long long*>(&g_wait_limit_cycles)) return false;
     }
   }
-}
-
-// Token and guidance row (0 conditional, 1 unconditional) of kernel row rho.
-__host__ __device__ __forceinline__ int pc_row_token(int rho, int cfg, int* rep) {
-  const int blk = rho >> 7, r = rho & 127;
-  if (!cfg) { *rep = 0; return blk * 128 + r; }
-  *rep = r >> 6;
-  return blk * 64 + (r & 63);
 }
 
 template <typename ACT, int AB_FMT>
@@ -635,32 +627,6 @@ pchain_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ C
   __syncthreads();
   cluster_arrive(); cluster_wait();   // neither CTA leaves while the pair's MMAs or signals may touch it
   if (warp == 1) tmem_dealloc_pair(tmem_base, 512);
-}
-
-// s_t = SiLU(cz + te_t) of every step, in the kernel's row order and operand format: s_all[(t - 1) rows + rho][col];
-// rows of tokens beyond R are zero.
-template <typename ACT>
-__global__ void __launch_bounds__(128) pc_cond_all_kernel(const float* __restrict__ cz, const float* __restrict__ te,
-                                                          ACT* __restrict__ s_all, int R, int cfg, int W, int rows) {
-  const int t = blockIdx.y, rho = blockIdx.x;
-  int rep;
-  const int i = pc_row_token(rho, cfg, &rep);
-  uint4* dst = reinterpret_cast<uint4*>(s_all + (static_cast<size_t>(t) * rows + rho) * W);     // 8 values per store
-  if (i >= R) {
-    for (int j = threadIdx.x; j < W / 8; j += blockDim.x) dst[j] = make_uint4(0u, 0u, 0u, 0u);
-    return;
-  }
-  const float4* c4 = reinterpret_cast<const float4*>(cz + (static_cast<size_t>(rep) * R + i) * W);
-  const float4* t4 = reinterpret_cast<const float4*>(te + static_cast<size_t>(t) * W);
-  for (int j = threadIdx.x; j < W / 8; j += blockDim.x) {
-    const float4 a = c4[2 * j], b = c4[2 * j + 1], ta = __ldg(t4 + 2 * j), tb = __ldg(t4 + 2 * j + 1);
-    __align__(16) ACT o[8];
-    o[0] = to_act<ACT>(silu_f(a.x + ta.x)); o[1] = to_act<ACT>(silu_f(a.y + ta.y));
-    o[2] = to_act<ACT>(silu_f(a.z + ta.z)); o[3] = to_act<ACT>(silu_f(a.w + ta.w));
-    o[4] = to_act<ACT>(silu_f(b.x + tb.x)); o[5] = to_act<ACT>(silu_f(b.y + tb.y));
-    o[6] = to_act<ACT>(silu_f(b.z + tb.z)); o[7] = to_act<ACT>(silu_f(b.w + tb.w));
-    dst[j] = *reinterpret_cast<const uint4*>(o);
-  }
 }
 
 }  // namespace csd

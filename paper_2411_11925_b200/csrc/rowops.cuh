@@ -8,47 +8,53 @@
 
 namespace csd {
 
-// Timestep embedding te[t, :] = Wt2 SiLU(Wt1 tfeat_t + bt1) + bt2 for all T steps: two small fp32 products
-// C[m, n] = act(sum_k A[m, k] B[n, k] + bias[n]) in 32 x 32 tiles (each weight row is read once per 32 steps,
-// not once per step).
-template <bool SILU>
-__global__ void __launch_bounds__(256)
-small_gemm_nt_kernel(const float* __restrict__ A, const float* __restrict__ B, const float* __restrict__ bias,
-                     float* __restrict__ C, int M, int N, int K) {
-  __shared__ float As[32][33], Bs[32][33];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;      // 32 x 8 threads, 4 rows of the tile each
-  const int m0 = blockIdx.y * 32, n0 = blockIdx.x * 32;
-  float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  for (int k0 = 0; k0 < K; k0 += 32) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int row = ty * 4 + r, k = k0 + tx;
-      As[row][tx] = (m0 + row < M && k < K) ? A[static_cast<size_t>(m0 + row) * K + k] : 0.0f;
-      Bs[row][tx] = (n0 + row < N && k < K) ? B[static_cast<size_t>(n0 + row) * K + k] : 0.0f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 32; ++k) {
-      const float b = Bs[tx][k];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) acc[r] = fmaf(As[ty * 4 + r][k], b, acc[r]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int m = m0 + ty * 4 + r, n = n0 + tx;
-    if (m < M && n < N) {
-      const float v = acc[r] + bias[n];
-      C[static_cast<size_t>(m) * N + n] = SILU ? silu_f(v) : v;
-    }
-  }
-}
-
 template <typename ACT>
 __global__ void convert_act_kernel(const float* __restrict__ src, ACT* __restrict__ dst, size_t n) {
   const size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i < n) dst[i] = to_act<ACT>(src[i]);
+}
+
+// Token and guidance row of row rho of a chain whose rows come in groups of G: with guidance G / 2 tokens' conditional rows,
+// then their unconditional twins.
+template <int G>
+__device__ __forceinline__ int group_row_token(int rho, int cfg, int* rep) {
+  const int blk = rho / G, r = rho % G;
+  if (!cfg) { *rep = 0; return rho; }
+  *rep = r / (G / 2);
+  return blk * (G / 2) + r % (G / 2);
+}
+
+// s_t = SiLU(cz + te_t) of every step, in that row order and operand format: s_all[(t - 1) rows + rho][col]; rows of tokens
+// beyond R are zero.  A block keeps its row of cz in registers over kCondSteps steps: one step per block was bound by the
+// trip to memory (115 us for 1024 rows of 1024 and 100 steps, 210 MB written).
+constexpr int kCondSteps = 10;
+template <typename ACT, int G>
+__global__ void __launch_bounds__(128) cond_all_kernel(const float* __restrict__ cz, const float* __restrict__ te, ACT* __restrict__ s_all,
+                                                       int R, int cfg, int W, int rows, int T) {
+  const int rho = blockIdx.x, t0 = blockIdx.y * kCondSteps, t1 = min(T, t0 + kCondSteps);
+  int rep;
+  const int i = group_row_token<G>(rho, cfg, &rep);
+  for (int j = threadIdx.x; j < W / 8; j += blockDim.x) {
+    uint4* dst = reinterpret_cast<uint4*>(s_all + static_cast<size_t>(rho) * W) + j;     // 8 values per store
+    const size_t step = static_cast<size_t>(rows) * W / 8;
+    if (i >= R) {
+      for (int t = t0; t < t1; ++t) dst[t * step] = make_uint4(0u, 0u, 0u, 0u);
+      continue;
+    }
+    const float4* c4 = reinterpret_cast<const float4*>(cz + (static_cast<size_t>(rep) * R + i) * W) + 2 * j;
+    const float4 a = c4[0], b = c4[1];
+#pragma unroll 2
+    for (int t = t0; t < t1; ++t) {
+      const float4* t4 = reinterpret_cast<const float4*>(te + static_cast<size_t>(t) * W) + 2 * j;
+      const float4 ta = __ldg(t4), tb = __ldg(t4 + 1);
+      __align__(16) ACT o[8];
+      o[0] = to_act<ACT>(silu_f(a.x + ta.x)); o[1] = to_act<ACT>(silu_f(a.y + ta.y));
+      o[2] = to_act<ACT>(silu_f(a.z + ta.z)); o[3] = to_act<ACT>(silu_f(a.w + ta.w));
+      o[4] = to_act<ACT>(silu_f(b.x + tb.x)); o[5] = to_act<ACT>(silu_f(b.y + tb.y));
+      o[6] = to_act<ACT>(silu_f(b.z + tb.z)); o[7] = to_act<ACT>(silu_f(b.w + tb.w));
+      dst[t * step] = *reinterpret_cast<const uint4*>(o);
+    }
+  }
 }
 
 enum StepMode : int { STEP_INIT = 0, STEP_MID = 1, STEP_LAST = 2 };

@@ -1,0 +1,57 @@
+"""The group chain kernel (few rows, 16-bit heads) at its edges: one row, ragged groups, every width, the largest number of
+groups it takes and one more, schedules that end in, at and beyond a chunk of steps, two contexts at a time."""
+import numpy as np
+import pytest
+
+from paper_2411_11925_b200 import inputs as gen
+from _parity import TOL_X
+from test_gpu_parity import _check, _wl
+
+pytestmark = pytest.mark.gpu
+
+H = gen.HeadSpec
+CASES = [
+    dict(B=1, gamma=1, T=3, draft=H(1, 1024, 128), target=H(2, 512, 128)),                                          # one row
+    dict(B=17, gamma=1, T=5, operand="bf16", draft=H(2, 512, 128), target=H(1, 1536, 128)),                         # one row in the last group
+    dict(B=3, gamma=3, T=4, cfg=True, cfg_scale=2.0, draft=H(1, 1536, 64), target=H(3, 1024, 64)),                  # guided, one token in the last group
+    dict(B=16, gamma=8, T=3, draft=H(1, 1024, 64), target=H(1, 1024, 64)),                                          # 8 groups: the most at W = 1024
+    dict(B=43, gamma=3, T=3, draft=H(1, 1024, 64), target=H(1, 1536, 64)),                                          # 9 groups: layer kernels
+]
+
+
+@pytest.mark.parametrize("kw", CASES)
+def test_group_chain_matches_checker_and_fused_round_matches_the_calls(kw):
+    from paper_2411_11925_b200.runner import DeviceRound
+    kw = {"bf16": True, **kw}
+    inp = gen.make_round_inputs(_wl(**kw))
+    _, a, _ = _check(inp, f"group chain {kw}")
+    dr = DeviceRound(inp)
+    dr.fused_round()
+    b = dr.results()
+    for k in ("x0", "mu1_q", "mu1_p", "logratio"):
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+    dr.ctx.close()
+
+
+@pytest.mark.parametrize("B,T", [(1, 16), (1, 17), (1, 49), (40, 5), (40, 6), (40, 17)])      # chunks of 16, 32, .. and of 5, 10, .. steps
+def test_trajectory_across_chunks_of_steps(B, T):
+    from paper_2411_11925_b200 import api
+    from paper_2411_11925_b200.runner import DeviceRound
+    inp = gen.make_round_inputs(_wl(bf16=True, B=B, gamma=1, T=T, draft=H(1, 512, 64), target=H(1, 512, 64)))
+    drs = [DeviceRound(inp), DeviceRound(inp)]
+    for dr in drs:                                     # two contexts, nothing between their launches
+        dr.draft_traj()
+    for dr in drs:
+        dr.ctx.sync()
+    x, mu = drs[0].traj_x.clone(), drs[0].traj_mu.clone()
+    assert bool((x == drs[1].traj_x).all()) and bool((mu == drs[1].traj_mu).all())
+    drs[0].draft()
+    drs[0].ctx.sync()
+    assert bool((x[-1] == drs[0].x0).all())
+    drs[0].ctx.set_chain_mode(api.Context.CHAIN_LAYERS_PLAIN)
+    drs[0].draft_traj()
+    drs[0].ctx.sync()
+    # both carry their own rounding
+    assert float((x - drs[0].traj_x).abs().max()) <= TOL_X["f16"] / 4 and float((mu - drs[0].traj_mu).abs().max()) <= TOL_X["f16"] / 4
+    for dr in drs:
+        dr.ctx.close()
