@@ -154,27 +154,35 @@ mods_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 
 // ------------------------------------------------------------------------------------------ the chain
 constexpr int kGcRows = 16;               // rows of a group = MMA N
-constexpr int kGcThreads = 256;           // warps: weights 0, MMA 1, condition products 2, (3), epilogue 4..7
+constexpr int kGcHalf = kGcRows / 2;      // rows of an epilogue thread
+constexpr int kGcEpi = 256;               // warps 0..7: epilogue
+// Three pairs of a loading warp (11..13) and an MMA-issuing warp (8..10), each with its own part of the weight ring and its own
+// accumulator, take k-blocks in turn.  One pair spends 370 cycles on loading and 530 on issuing a k-block (waits, the
+// instructions' own latency, the commit), which the tensor pipe finishes in 160.  The ring is divided because waits on a
+// barrier's parity are only sound for one warp that follows its phases in order.
+constexpr int kGcMma = 3;
+constexpr int kGcThreads = kGcEpi + 2 * kGcMma * 32;
 constexpr int kGcMaxW = 1536;
 constexpr int kGcMaxCl = kGcMaxW / 128;
-constexpr int kGcWinLd = kCPad + 1;       // a row of Win and its bias in shared memory (odd: lanes walk rows)
 constexpr int kGcTile = kGcRows * 256;    // bytes of one CTA's part of an activation buffer: two k-blocks of [16 rows][128 B]
+constexpr int kGcMaxStages = 12;          // of one k-block of [128 weight rows][128 B]; a multiple of the pairs
 
-struct GcLayout { int act, ring, stages, mods, stage, win, wout, stats, misc, total; };
+struct GcLayout { int act, ring, stages, part, wout, stats, misc, total; };
 __host__ __device__ inline GcLayout gc_layout(int W) {
   GcLayout l{};
   int o = 0;
   auto take = [&](int n) { const int r = o; o += n; return r; };
-  l.stages = W > 1024 ? 2 : 3;
   l.act = take(2 * kGcRows * W * 2);      // a' | v
-  l.ring = take(l.stages * 32768);        // stages of two k-blocks of [128 weight rows][128 B]
-  l.mods = take(2 * 16384);               // two items' condition products, each [product][row quad][128 columns][4]
-  l.stage = take(2 * kGcTile + 1024);     // outgoing tiles, by turns, and the outgoing partial: a peer's tile of one phase says that it
-                                          // has received this CTA's of the phase before, so two buffers never overrun a copy
-  l.win = take(128 * kGcWinLd * 4);
   l.wout = take(128 * kCPad * 4);
   l.stats = take(W / 32 * kGcRows * 8);   // [32-column group][row] (mean, M2)
-  l.misc = take(1024 + 512 + 512);        // x [16 tokens][16], (mean, rstd) per warp [4][16], barriers
+  l.part = take(kGcRows * kCPad * 4);     // the outgoing output-projection partial
+  l.misc = take(1024 + 512 + 512);        // x [16 tokens][16], (mean, rstd) per epilogue warp [8][8], barriers
+  l.stages = (226 * 1024 - o) / 16384;    // all that is left streams weights: 12, 9, 6 stages
+  l.stages = (l.stages > kGcMaxStages ? kGcMaxStages : l.stages) / kGcMma * kGcMma;
+  l.ring = take(0);
+  o = (o + 1023) / 1024 * 1024;
+  l.ring = o;
+  o += l.stages * 16384;
   l.total = o;
   return l;
 }
@@ -202,46 +210,52 @@ __device__ __forceinline__ void gc_st_async(uint32_t dst_cluster, float a, float
   const unsigned long long v = (static_cast<unsigned long long>(__float_as_uint(b)) << 32) | __float_as_uint(a);
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(dst_cluster), "l"(v), "r"(bar_cluster) : "memory");
 }
-// Sums 16 values over the warp, transposing: lane l ends with value l / 2.
-__device__ __forceinline__ float gc_reduce16(const float (&in)[kGcRows], int lane) {
-  float v[kGcRows];
+// Sums 8 values over the warp, transposing: lane l ends with value l / 4.
+__device__ __forceinline__ float gc_reduce8(const float (&in)[kGcHalf], int lane) {
+  float v[kGcHalf];
 #pragma unroll
-  for (int i = 0; i < kGcRows; ++i) v[i] = in[i];
+  for (int i = 0; i < kGcHalf; ++i) v[i] = in[i];
 #pragma unroll
-  for (int n = 8; n >= 1; n >>= 1) {
-    const int o = 2 * n;
+  for (int n = 4; n >= 1; n >>= 1) {
+    const int o = 4 * n;
     const bool up = (lane & o) != 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < 4; ++i)
       if (i < n) {
         const float send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
         v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
       }
   }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
   return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+// Issued where it stands: the products of a phase are on their way while its MMAs run.
+__device__ __forceinline__ float4 gc_ld(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
 }
 
 template <typename ACT, int AB_FMT>
 __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid_constant__ GcParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int W = p.W, L = p.L, T = p.T, CL = W / 128, NI = 2 * L + 2;   // items with condition products per step
+  const int W = p.W, L = p.L, T = p.T, CL = W / 128;
   const GcLayout lo = gc_layout(W);
   const int act_bytes = kGcRows * W * 2;
+  const int SR = lo.stages / kGcMma;       // stages of a pair
   uint8_t* act = smem + lo.act;
-  uint8_t* stage = smem + lo.stage;
-  float4* part_out = reinterpret_cast<float4*>(stage + 2 * kGcTile);
-  float* win_s = reinterpret_cast<float*>(smem + lo.win);
+  float4* part_out = reinterpret_cast<float4*>(smem + lo.part);
   float* wout_s = reinterpret_cast<float*>(smem + lo.wout);
   float2* stats_s = reinterpret_cast<float2*>(smem + lo.stats);
   float* xs = reinterpret_cast<float*>(smem + lo.misc);
   float2* norm_all = reinterpret_cast<float2*>(smem + lo.misc + 1024);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + lo.misc + 1536);
-  uint64_t *w_full = bars, *w_empty = bars + 3, *act_full = bars + 6, *acc_full = act_full + 2 * kGcMaxCl, *mods_full = acc_full + 1,
-           *mods_free = mods_full + 2, *stats_full = mods_free + 2, *part_full = stats_full + 1;
+  uint64_t *w_full = bars, *w_empty = w_full + kGcMaxStages, *act_full = w_empty + kGcMaxStages, *acc_full = act_full + 2 * kGcMaxCl,
+           *stats_full = acc_full + 1, *part_full = stats_full + 1;
   uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(part_full + 1);     // and whether the context is free of errors
-  // free at the end of a step, when every product that reads them is complete here: the columns' modulated h (read by this
-  // CTA only), the peers' output-projection partials
+  // free at the end of a step, when every product that reads them is complete here and every peer has its copy: the columns'
+  // modulated h (read by this CTA only), the peers' output-projection partials
   float* uf_s = reinterpret_cast<float*>(act);                       // [16][kUfLd]
   float* part_s = reinterpret_cast<float*>(act + act_bytes);         // [CL][16][16]
   constexpr int kUfLd = 132;
@@ -250,20 +264,14 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
   const int rank = static_cast<int>(cluster_ctarank()), grp = static_cast<int>(blockIdx.x) / CL;
   const int n_base = rank * 128;
   if (tid == 0) {
-    for (int s = 0; s < 3; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); }
+    for (int s = 0; s < kGcMaxStages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); }
     for (int i = 0; i < 2 * kGcMaxCl; ++i) mbar_init(&act_full[i], 1);
-    mbar_init(acc_full, 1);
-    for (int i = 0; i < 2; ++i) { mbar_init(&mods_full[i], 1); mbar_init(&mods_free[i], 4); }
-    mbar_init(stats_full, 1); mbar_init(part_full, 1);
+    mbar_init(acc_full, kGcMma); mbar_init(stats_full, 1); mbar_init(part_full, 1);
     tmem_base_s[1] = *reinterpret_cast<const volatile int*>(p.err) == 0;    // one reading for all warps
     fence_mbar_init();
   }
-  if (warp == 1) { tmem_alloc(tmem_base_s, 32); tmem_relinquish(); }
-  for (int i = tid; i < 128 * kCPad; i += kGcThreads) {
-    win_s[(i / kCPad) * kGcWinLd + i % kCPad] = p.win[static_cast<size_t>(n_base) * kCPad + i];
-    wout_s[i] = p.wout_t[static_cast<size_t>(n_base) * kCPad + i];
-  }
-  if (tid < 128) win_s[tid * kGcWinLd + kCPad] = p.bin[n_base + tid];
+  if (warp == 8) { tmem_alloc(tmem_base_s, 64); tmem_relinquish(); }
+  for (int i = tid; i < 128 * kCPad; i += kGcThreads) wout_s[i] = p.wout_t[static_cast<size_t>(n_base) * kCPad + i];
   tc_fence_before_sync();
   __syncthreads();
   cluster_arrive(); cluster_wait();       // the peers' barriers exist before anything signals them
@@ -273,124 +281,105 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
 
   // (a CTA that gives up on a wait goes on through its barriers without waiting: its peers' waits end by the context's
   // error word)
-  if (run && warp == 0) {
+  if (run && warp >= 8 + kGcMma) {
     // ---------------------------------------------------------------- weights, k-blocks in this CTA's turn order
     if (lane == 0) {
-      uint32_t it = 0, s = 0, par = 1;
+      const int m = warp - 8 - kGcMma;
+      int j = m, s = 0;
+      uint32_t par = 1;
       bool ok = true;
       for (int t = p.t_hi; t >= p.t_lo && ok; --t)
-        for (int ph = 0; ph < 2 * L && ok; ++ph)
-          for (int j = 0; j < CL; ++j, ++it) {
-            const int src = rank + j < CL ? rank + j : rank + j - CL;
-            if (it >= static_cast<uint32_t>(lo.stages) && !ch_wait<false>(&w_empty[s], par, p.err)) { ch_fail(p.err, DEV_ERR_TMA_WAIT, 1, static_cast<int>(it)); ok = false; break; }
-            mbar_arrive_expect_tx(&w_full[s], 32768);
-            uint8_t* dst = smem + lo.ring + s * 32768;
-            tma_load_2d(dst, p.maps + ph, &w_full[s], src * 128, n_base);
-            tma_load_2d(dst + 16384, p.maps + ph, &w_full[s], src * 128 + kBlockK, n_base);
-            if (++s == static_cast<uint32_t>(lo.stages)) { s = 0; par ^= 1; }
+        for (int ph = 0; ph < 2 * L && ok; ++ph, j -= 2 * CL)
+          for (; j < 2 * CL; j += kGcMma) {
+            const int kb = 2 * rank + j < 2 * CL ? 2 * rank + j : 2 * rank + j - 2 * CL, st = m * SR + s;
+            if (!ch_wait<false>(&w_empty[st], par, p.err)) { ch_fail(p.err, DEV_ERR_TMA_WAIT, 1, ph); ok = false; break; }   // (fresh: passes)
+            mbar_arrive_expect_tx(&w_full[st], 16384);
+            tma_load_2d(smem + lo.ring + st * 16384, p.maps + ph, &w_full[st], kb * kBlockK, n_base);
+            if (++s == SR) { s = 0; par ^= 1; }
           }
     }
     __syncwarp();
-  } else if (run && warp == 1) {
-    // ---------------------------------------------------------------- MMA issue
+  } else if (run && warp >= 8) {
+    // ---------------------------------------------------------------- MMA issue, into 16 columns per pair (the epilogue adds
+    // the pairs' up)
     const bool leader = elect_one();
     constexpr uint32_t idesc = umma_idesc_f16(kGcRows, AB_FMT);
+    const int m = warp - 8;
+    const uint32_t acc = tmem_base + m * kGcRows;
     bool ok = true;
-    uint32_t s = 0, par = 0, use = 0;
+    int j = m, s = 0;
+    uint32_t par = 0, use = 0;
     for (int t = p.t_hi; t >= p.t_lo && ok; --t)
-      for (int ph = 0; ph < 2 * L && ok; ++ph) {
+      for (int ph = 0; ph < 2 * L && ok; ++ph, j -= 2 * CL) {
         const int buf = ph & 1;
-        if (lane < CL) mbar_arrive_expect_tx(&act_full[buf * kGcMaxCl + lane], kGcTile);
+        uint64_t* const tile = act_full + buf * kGcMaxCl;
+        if (m == 0 && lane < CL && lane != rank) mbar_arrive_expect_tx(&tile[lane], kGcTile);   // (its own: the epilogue arrives)
         __syncwarp();
-        for (int j = 0; j < CL; ++j) {
-          const int src = rank + j < CL ? rank + j : rank + j - CL;
-          ok = ch_wait<false>(&act_full[buf * kGcMaxCl + src], use & 1, p.err) && ch_wait<false>(&w_full[s], par, p.err);
+        ok = ch_wait<false>(&tile[rank], use & 1, p.err);      // this CTA's tile is also the word that the accumulators are free
+        uint32_t more = 0;
+        for (; j < 2 * CL; j += kGcMma) {
+          const int src = rank + (j >> 1) < CL ? rank + (j >> 1) : rank + (j >> 1) - CL, st = m * SR + s;
+          ok = ok && ch_wait<false>(&tile[src], use & 1, p.err) && ch_wait<false>(&w_full[st], par, p.err);
           if (!ok) { if (leader) ch_fail(p.err, DEV_ERR_MMA_WAIT, 2, ph); break; }
           tc_fence_after_sync();
           if (leader) {
-            const uint32_t sa = smem_u32(smem + lo.ring + s * 32768), sb = smem_u32(act + buf * act_bytes + src * kGcTile);
+            const uint64_t da = umma_smem_desc_sw128(smem_u32(smem + lo.ring + st * 16384)),
+                           db = umma_smem_desc_sw128(smem_u32(act + buf * act_bytes + src * kGcTile + (j & 1) * (kGcRows * 128)));
 #pragma unroll
-            for (int jj = 0; jj < 2; ++jj) {
-              const uint64_t da = umma_smem_desc_sw128(sa + jj * 16384), db = umma_smem_desc_sw128(sb + jj * (kGcRows * 128));
-#pragma unroll
-              for (int k = 0; k < kBlockK / 16; ++k) umma_f16(tmem_base, da + 2 * k, db + 2 * k, idesc, (j > 0 || jj > 0 || k > 0) ? 1u : 0u);
-            }
-            umma_commit(&w_empty[s]);
+            for (int k = 0; k < kBlockK / 16; ++k) umma_f16(acc, da + 2 * k, db + 2 * k, idesc, k > 0 ? 1u : more);
+            umma_commit(&w_empty[st]);
           }
+          more = 1;
           __syncwarp();
-          if (++s == static_cast<uint32_t>(lo.stages)) { s = 0; par ^= 1; }
+          if (++s == SR) { s = 0; par ^= 1; }
         }
         if (ok && leader) umma_commit(acc_full);
         __syncwarp();
         if (buf == 1) ++use;
       }
-  } else if (run && warp == 2) {
-    // ---------------------------------------------------------------- condition products, an item ahead
-    if (lane == 0) {
-      uint32_t n = 0;
-      bool ok = true;
-      for (int t = p.t_hi; t >= p.t_lo && ok; --t)
-        for (int item = 0; item < NI; ++item, ++n) {
-          const int b = n & 1;
-          if (n >= 2 && !ch_wait<false>(&mods_free[b], ((n >> 1) - 1) & 1, p.err)) { ch_fail(p.err, DEV_ERR_TMA_WAIT, 3, item); ok = false; break; }
-          const int sec = item == 0 ? 0 : item == NI - 1 ? 4 * L : 2 * item - 1, ns = item == 0 || item == 2 * L ? 1 : 2;
-          mbar_arrive_expect_tx(&mods_full[b], ns * 8192);
-          const size_t q0 = (static_cast<size_t>(t - p.t_lo) * p.rows + grp * kGcRows) / 4;
-          for (int u = 0; u < ns; ++u)
-            bulk_load(smem + lo.mods + b * 16384 + u * 8192, p.mods + (static_cast<size_t>((sec + u) * CL + rank) * p.nq + q0) * 128, 8192, &mods_full[b]);
-        }
-    }
-    __syncwarp();
-  } else if (run && warp >= 4) {
-    // ---------------------------------------------------------------- epilogue: thread = one column of the group's 16 rows
-    const int ew = warp - 4, et = tid - 128, c = ew * 32 + lane, col = n_base + c;
+  } else if (run && warp < 8) {
+    // ---------------------------------------------------------------- epilogue: thread = 8 rows of the group in one column
+    const int ew = warp, et = tid, q4 = ew & 3, half = ew >> 2, c = q4 * 32 + lane, col = n_base + c, r0 = half * kGcHalf;
     const int per = p.cfg ? 8 : 16, tok0 = grp * per;        // tokens of the group; row i is token i % per
-    float2* norm_s = norm_all + ew * kGcRows;                // this warp's copy of the rows' (mean, rstd)
+    float2* norm_s = norm_all + ew * kGcHalf;                // this warp's copy of its rows' (mean, rstd)
     bool ok = true;
-    uint32_t n_item = 0, n_acc = 0, n_stat = 0, n_part = 0, n_tile = 0;
-    auto epi_sync = [&]() { asm volatile("bar.sync 1, 128;" ::: "memory"); };
+    uint32_t n_acc = 0, n_stat = 0, n_part = 0;
+    auto epi_sync = [&]() { asm volatile("bar.sync 1, 256;" ::: "memory"); };
     auto wait = [&](uint64_t* bar, uint32_t parity, int site) {
-      if (ok && !ch_wait<true>(bar, parity, p.err)) { ch_fail(p.err, DEV_ERR_EPI_WAIT, site, static_cast<int>(n_item)); ok = false; }
+      if (ok && !ch_wait<true>(bar, parity, p.err)) { ch_fail(p.err, DEV_ERR_EPI_WAIT, site, static_cast<int>(n_acc)); ok = false; }
     };
-    // this item's condition products of the column
-    auto take = [&](float* m0, float* m1) {
-      const int b = n_item & 1;
-      wait(&mods_full[b], (n_item >> 1) & 1, 4);
-      const float4* src = reinterpret_cast<const float4*>(smem + lo.mods + b * 16384) + c;
-#pragma unroll
-      for (int q = 0; q < kGcRows / 4; ++q) {
-        const float4 v = src[q * 128];
-        m0[4 * q] = v.x; m0[4 * q + 1] = v.y; m0[4 * q + 2] = v.z; m0[4 * q + 3] = v.w;
-        if (m1) { const float4 w = src[512 + q * 128]; m1[4 * q] = w.x; m1[4 * q + 1] = w.y; m1[4 * q + 2] = w.z; m1[4 * q + 3] = w.w; }
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&mods_free[b]);
-      ++n_item;
+    // product `sec` of step t, this thread's column and rows
+    auto take = [&](float (&m)[kGcHalf], int t, int sec) {
+      const float4* src = p.mods + (static_cast<size_t>(sec * CL + rank) * p.nq + (static_cast<size_t>(t - p.t_lo) * p.rows + grp * kGcRows + r0) / 4) * 128 + c;
+      const float4 a = gc_ld(src), b = gc_ld(src + 128);
+      m[0] = a.x; m[1] = a.y; m[2] = a.z; m[3] = a.w; m[4] = b.x; m[5] = b.y; m[6] = b.z; m[7] = b.w;
     };
-    // 16-bit tile of this CTA's columns, to every CTA's activation buffer `buf`
-    auto send_tile = [&](const float (&v)[kGcRows], int buf) {
-      uint8_t* const out = stage + (n_tile++ & 1) * kGcTile;
-      uint8_t* kb = out + (c >> 6) * (kGcRows * 128);
+    // 16-bit tile of this CTA's columns: into its own activation buffer `buf`, and from there into every peer's
+    auto send_tile = [&](const float (&v)[kGcHalf], int buf) {
+      uint8_t* const out = act + buf * act_bytes + rank * kGcTile;
+      uint8_t* kb = out + (c >> 6) * (kGcRows * 128) + r0 * 128;
       const int u = (c & 63) >> 3, b = (c & 7) * 2;
 #pragma unroll
-      for (int i = 0; i < kGcRows; ++i) *reinterpret_cast<ACT*>(kb + i * 128 + ((u ^ (i & 7)) << 4) + b) = to_act<ACT>(v[i]);
+      for (int i = 0; i < kGcHalf; ++i) *reinterpret_cast<ACT*>(kb + i * 128 + ((u ^ i) << 4) + b) = to_act<ACT>(v[i]);
       fence_proxy_async_smem();
       epi_sync();
       if (ok && ew == 0 && lane < CL) {
+        const uint32_t bar = smem_u32(&act_full[buf * kGcMaxCl + rank]);
         const int peer = rank + lane < CL ? rank + lane : rank + lane - CL;
-        gc_copy(mapa_shared(smem_u32(act + buf * act_bytes + rank * kGcTile), peer), out, kGcTile, mapa_shared(smem_u32(&act_full[buf * kGcMaxCl + rank]), peer));
+        if (lane == 0) mbar_arrive(&act_full[buf * kGcMaxCl + rank]);
+        else gc_copy(mapa_shared(smem_u32(out), peer), out, kGcTile, mapa_shared(bar, peer));
       }
       __syncwarp();
     };
     // (mean, M2) of each row over this warp's 32 columns, to every CTA
-    auto send_stats = [&](const float (&v)[kGcRows]) {
-      const float mean = gc_reduce16(v, lane) * (1.0f / 32.0f);     // of row lane / 2
-      float d[kGcRows];
+    auto send_stats = [&](const float (&v)[kGcHalf]) {
+      const float mean = gc_reduce8(v, lane) * (1.0f / 32.0f);      // of row lane / 4
+      float d[kGcHalf];
 #pragma unroll
-      for (int i = 0; i < kGcRows; ++i) { const float e = v[i] - __shfl_sync(0xffffffffu, mean, 2 * i); d[i] = e * e; }
-      const float m2 = gc_reduce16(d, lane);
-      const uint32_t at = smem_u32(stats_s + (rank * 4 + ew) * kGcRows + (lane >> 1)), bar = smem_u32(stats_full);
-      for (int r = lane & 1; ok && r < CL; r += 2) gc_st_async(mapa_shared(at, r), mean, m2, mapa_shared(bar, r));
+      for (int i = 0; i < kGcHalf; ++i) { const float e = v[i] - __shfl_sync(0xffffffffu, mean, 4 * i); d[i] = e * e; }
+      const float m2 = gc_reduce8(d, lane);
+      const uint32_t at = smem_u32(stats_s + (rank * 4 + q4) * kGcRows + r0 + (lane >> 2)), bar = smem_u32(stats_full);
+      for (int r = lane & 3; ok && r < CL; r += 4) gc_st_async(mapa_shared(at, r), mean, m2, mapa_shared(bar, r));
     };
     const uint32_t stats_bytes = static_cast<uint32_t>(CL) * 4 * kGcRows * 8, part_bytes = static_cast<uint32_t>(CL) * kGcRows * kCPad * 4;
     // the rows' (mean, rstd) from all partials, into norm_s (32-column groups merged as equal-count partials)
@@ -398,65 +387,70 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
       wait(stats_full, n_stat & 1, 5);
       if (et == 0) mbar_arrive_expect_tx(stats_full, stats_bytes);   // the next phase's
       ++n_stat;
-      const int row = lane & 15, h = lane >> 4, G = CL * 2;          // two lanes per row, half of the W / 32 partials each
-      const float2* src = stats_s + h * G * kGcRows + row;
+      const int row = lane & 7, h = lane >> 3;                       // four lanes per row, a quarter of the W / 32 partials each
+      const float2* src = stats_s + h * CL * kGcRows + r0 + row;
       float sm = 0.0f, m2 = 0.0f, q = 0.0f;
-      for (int g = 0; g < G; ++g) { const float2 v = src[g * kGcRows]; sm += v.x; m2 += v.y; }
+      for (int g = 0; g < CL; ++g) { const float2 v = src[g * kGcRows]; sm += v.x; m2 += v.y; }
+      sm += __shfl_xor_sync(0xffffffffu, sm, 8);
       sm += __shfl_xor_sync(0xffffffffu, sm, 16);
-      const float mean = sm / static_cast<float>(2 * G);
-      for (int g = 0; g < G; ++g) { const float d = src[g * kGcRows].x - mean; q = fmaf(d, d, q); }
+      const float mean = sm / static_cast<float>(4 * CL);
+      for (int g = 0; g < CL; ++g) { const float d = src[g * kGcRows].x - mean; q = fmaf(d, d, q); }
       m2 = fmaf(32.0f, q, m2);
+      m2 += __shfl_xor_sync(0xffffffffu, m2, 8);
       m2 += __shfl_xor_sync(0xffffffffu, m2, 16);
-      if (lane < kGcRows) norm_s[row] = make_float2(mean, 1.0f / sqrtf(m2 / static_cast<float>(W) + 1e-6f));
+      if (lane < kGcHalf) norm_s[row] = make_float2(mean, 1.0f / sqrtf(m2 / static_cast<float>(W) + 1e-6f));
       __syncwarp();
     };
-    auto acc_load = [&](float (&a)[kGcRows]) {
+    auto acc_load = [&](float (&a)[kGcHalf]) {
       wait(acc_full, n_acc & 1, 6);
       ++n_acc;
       tc_fence_after_sync();
-      tmem_ld16(tmem_base + (static_cast<uint32_t>(ew * 32) << 16), a);
+      float b[kGcMma][kGcHalf];
+#pragma unroll
+      for (int m = 0; m < kGcMma; ++m) tmem_ld8(tmem_base + (static_cast<uint32_t>(q4 * 32) << 16) + m * kGcRows + r0, b[m]);
       tmem_ld_wait();
+#pragma unroll
+      for (int i = 0; i < kGcHalf; ++i) a[i] = (b[0][i] + b[1][i]) + b[2][i];
       tc_fence_before_sync();
     };
 
     if (et == 0) { mbar_arrive_expect_tx(stats_full, stats_bytes); mbar_arrive_expect_tx(part_full, part_bytes); }
     // state of the group's tokens
     const bool first = p.t_hi == T;
-    for (int i = et; i < per * kCPad; i += 128) {
-      const int tok = tok0 + (i >> 4), e = i & 15;
+    if (et < per * kCPad) {
+      const int tok = tok0 + (et >> 4), e = et & 15;
       float v = 0.0f;
       if (tok < p.R && e < p.C) {
         const size_t o = static_cast<size_t>(tok) * p.C + e;
         v = first ? p.x_T[o] : p.x[o];
         if (first && rank == 0 && p.traj_x) p.traj_x[o] = v;
       }
-      xs[i] = v;
+      xs[et] = v;
     }
+    float h[kGcHalf], m0[kGcHalf], m1[kGcHalf], a[kGcHalf];
+    take(m0, p.t_hi, 0);
     epi_sync();
     for (int t = p.t_hi; t >= p.t_lo; --t) {
-      float h[kGcRows], m0[kGcRows], m1[kGcRows], a[kGcRows];
       // ---- h = Win x + bin for the column, a' = h (1 + scale_0)
       {
-        float w[kCPad];
+        const float4* wq = reinterpret_cast<const float4*>(p.win + static_cast<size_t>(col) * kCPad);
+        const float4 w0 = __ldg(wq), w1 = __ldg(wq + 1), w2 = __ldg(wq + 2), w3 = __ldg(wq + 3);
+        const float bi = __ldg(p.bin + col), bs = __ldg(p.bsc + col);
 #pragma unroll
-        for (int e = 0; e < kCPad; ++e) w[e] = win_s[c * kGcWinLd + e];
-        const float bi = win_s[c * kGcWinLd + kCPad], bs = __ldg(p.bsc + col);
-#pragma unroll
-        for (int i = 0; i < kGcRows; ++i) {
-          if (i >= 8 && p.cfg) { h[i] = h[i - 8]; continue; }
-          const float4* xq = reinterpret_cast<const float4*>(xs + i * kCPad);
+        for (int i = 0; i < kGcHalf; ++i) {
+          const float4* xq = reinterpret_cast<const float4*>(xs + ((p.cfg ? 0 : r0) + i) * kCPad);
+          const float4 x0 = xq[0], x1 = xq[1], x2 = xq[2], x3 = xq[3];
           float v = bi;
-#pragma unroll
-          for (int q = 0; q < kCPad / 4; ++q) {
-            const float4 x = xq[q];
-            v = fmaf(w[4 * q], x.x, v); v = fmaf(w[4 * q + 1], x.y, v); v = fmaf(w[4 * q + 2], x.z, v); v = fmaf(w[4 * q + 3], x.w, v);
-          }
+          v = fmaf(w0.x, x0.x, v); v = fmaf(w0.y, x0.y, v); v = fmaf(w0.z, x0.z, v); v = fmaf(w0.w, x0.w, v);
+          v = fmaf(w1.x, x1.x, v); v = fmaf(w1.y, x1.y, v); v = fmaf(w1.z, x1.z, v); v = fmaf(w1.w, x1.w, v);
+          v = fmaf(w2.x, x2.x, v); v = fmaf(w2.y, x2.y, v); v = fmaf(w2.z, x2.z, v); v = fmaf(w2.w, x2.w, v);
+          v = fmaf(w3.x, x3.x, v); v = fmaf(w3.y, x3.y, v); v = fmaf(w3.z, x3.z, v); v = fmaf(w3.w, x3.w, v);
           h[i] = v;
         }
-        take(m0, nullptr);
 #pragma unroll
-        for (int i = 0; i < kGcRows; ++i) a[i] = __fmul_rn(h[i], __fadd_rn(1.0f, __fadd_rn(m0[i], bs)));
+        for (int i = 0; i < kGcHalf; ++i) a[i] = __fmul_rn(h[i], __fadd_rn(1.0f, __fadd_rn(m0[i], bs)));
         send_tile(a, 0);
+        take(m0, t, 1); take(m1, t, 2);
         send_stats(h);
       }
 #pragma unroll 1
@@ -464,11 +458,10 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
         // ---- v = SiLU(rstd (a' W1^T - mean (P1 + c1)) + P2 + c2)
         {
           const float k0 = __ldg(p.c1 + static_cast<size_t>(2 * k) * W + col), k1 = __ldg(p.c1 + static_cast<size_t>(2 * k + 1) * W + col);
-          take(m0, m1);
           norms();
           acc_load(a);
 #pragma unroll
-          for (int i = 0; i < kGcRows; ++i) {
+          for (int i = 0; i < kGcHalf; ++i) {
             const float2 nr = norm_s[i];
             const float t1 = __fsub_rn(a[i], __fmul_rn(nr.x, __fadd_rn(m0[i], k0)));
             a[i] = silu_t<true>(fmaf(nr.y, t1, __fadd_rn(m1[i], k1)));
@@ -478,51 +471,55 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
         // ---- h += gate (v W2^T + b2); a' = h (1 + scale_{k+1})
         {
           const bool last = k + 1 == L;
+          take(m0, t, 4 * k + 3);
+          if (!last) take(m1, t, 4 * k + 4);
           const float kg = __ldg(p.bg + static_cast<size_t>(5 * k) * W + col), kb = __ldg(p.b2 + static_cast<size_t>(5 * k) * W + col),
                       ks = last ? 0.0f : __ldg(p.bsc + static_cast<size_t>(5 * (k + 1)) * W + col);
-          if (last) take(m0, nullptr); else take(m0, m1);
           acc_load(a);
 #pragma unroll
-          for (int i = 0; i < kGcRows; ++i) h[i] = fmaf(__fadd_rn(m0[i], kg), __fadd_rn(a[i], kb), h[i]);
+          for (int i = 0; i < kGcHalf; ++i) h[i] = fmaf(__fadd_rn(m0[i], kg), __fadd_rn(a[i], kb), h[i]);
           if (!last) {
 #pragma unroll
-            for (int i = 0; i < kGcRows; ++i) a[i] = __fmul_rn(h[i], __fadd_rn(1.0f, __fadd_rn(m1[i], ks)));
+            for (int i = 0; i < kGcHalf; ++i) a[i] = __fmul_rn(h[i], __fadd_rn(1.0f, __fadd_rn(m1[i], ks)));
             send_tile(a, 0);
           }
+          const int sec = last ? 4 * L : 4 * k + 5;           // the final shift and scale, or the next block's P1, P2
+          take(m0, t, sec); take(m1, t, sec + 1);
           send_stats(h);
         }
       }
       // ---- output projection of (LN(h)(1 + scale_f) + shift_f): this CTA's columns' part, to every CTA
       const float sa = p.sched[t - 1], sb = p.sched[T + t - 1], sg = p.sched[2 * T + t - 1];
-      float noise[2] = {0.0f, 0.0f};
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int i = et + u * 128, tok = tok0 + (i >> 4), e = i & 15;
-        if (i < per * kCPad && tok < p.R && e < p.C) noise[u] = p.eps[(static_cast<size_t>(t - 1) * p.R + tok) * p.C + e];
-      }
+      float noise = 0.0f;
+      const int q = et >> 4, e = et & 15, tok = tok0 + q;                 // this thread's entry of the state
+      const bool mine = et < per * kCPad && tok < p.R && e < p.C;
+      if (mine) noise = p.eps[(static_cast<size_t>(t - 1) * p.R + tok) * p.C + e];
       {
         const float k0 = __ldg(p.bfsh + col), k1 = __ldg(p.bfsc + col);
-        take(m0, m1);
         norms();
 #pragma unroll
-        for (int i = 0; i < kGcRows; ++i) {
+        for (int i = 0; i < kGcHalf; ++i) {
           const float2 nr = norm_s[i];
-          uf_s[i * kUfLd + c] = fmaf(__fmul_rn(__fsub_rn(h[i], nr.x), nr.y), __fadd_rn(1.0f, m1[i] + k1), m0[i] + k0);
+          uf_s[(r0 + i) * kUfLd + c] = fmaf(__fmul_rn(__fsub_rn(h[i], nr.x), nr.y), __fadd_rn(1.0f, m1[i] + k1), m0[i] + k0);
         }
+        if (t > p.t_lo) take(m0, t - 1, 0);
         epi_sync();
-        // four outputs of one row over half of the columns per thread, the halves a quarter apart (bank conflicts)
-        const int quad = lane & 3, row = ew * 4 + ((lane >> 2) & 3), hf = lane >> 4;
+        // four outputs of one row over a quarter of the columns per thread, the quarters apart (bank conflicts)
+        const int quad = lane & 3, row = ew * 2 + ((lane >> 2) & 1), qt = lane >> 3;
         float4 o = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll 8
-        for (int j = 0; j < 64; ++j) {
-          const int cc = hf * 64 + ((j + hf * 16) & 63);
+        for (int j = 0; j < 32; ++j) {
+          const int cc = qt * 32 + ((j + qt * 8) & 31);
           const float u = uf_s[row * kUfLd + cc];
           const float4 w = *reinterpret_cast<const float4*>(wout_s + cc * kCPad + quad * 4);
           o.x = fmaf(u, w.x, o.x); o.y = fmaf(u, w.y, o.y); o.z = fmaf(u, w.z, o.z); o.w = fmaf(u, w.w, o.w);
         }
-        o.x += __shfl_xor_sync(0xffffffffu, o.x, 16); o.y += __shfl_xor_sync(0xffffffffu, o.y, 16);
-        o.z += __shfl_xor_sync(0xffffffffu, o.z, 16); o.w += __shfl_xor_sync(0xffffffffu, o.w, 16);
-        if (hf == 0) part_out[row * 4 + quad] = o;
+#pragma unroll
+        for (int d = 8; d <= 16; d <<= 1) {
+          o.x += __shfl_xor_sync(0xffffffffu, o.x, d); o.y += __shfl_xor_sync(0xffffffffu, o.y, d);
+          o.z += __shfl_xor_sync(0xffffffffu, o.z, d); o.w += __shfl_xor_sync(0xffffffffu, o.w, d);
+        }
+        if (qt == 0) part_out[row * 4 + quad] = o;
         fence_proxy_async_smem();
         epi_sync();
         if (ok && ew == 0 && lane < CL)
@@ -530,25 +527,23 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
         __syncwarp();
       }
       // ---- guidance and Eq. 3, by every CTA alike (CTA 0 writes what leaves the chip)
+      const float bo = mine ? p.bout[e] : 0.0f;
       wait(part_full, n_part & 1, 7);
       if (et == 0) mbar_arrive_expect_tx(part_full, part_bytes);
       ++n_part;
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int i = et + u * 128, q = i >> 4, e = i & 15, tok = tok0 + q;
-        if (i >= per * kCPad) continue;
+      if (et < per * kCPad) {
         auto out = [&](int row) {
           float s = 0.0f;
           for (int r = 0; r < CL; ++r) s += part_s[(r * kGcRows + row) * kCPad + e];
-          return s + p.bout[e];
+          return s + bo;
         };
         float xn = 0.0f;
-        if (tok < p.R && e < p.C) {
+        if (mine) {
           const size_t o = static_cast<size_t>(tok) * p.C + e;
           float ee = out(q);
           if (p.cfg) ee = cfg_combine(ee, out(8 + q), p.cfg_scale);
-          const float xo = xs[i], mu = ddpm_mean(sa, xo, sb, ee);
-          xn = ddpm_sample(mu, sg, noise[u]);
+          const float xo = xs[et], mu = ddpm_mean(sa, xo, sb, ee);
+          xn = ddpm_sample(mu, sg, noise);
           if (rank == 0) {
             if (!(fabsf(xn) <= 3.0e38f)) *p.status = 1;
             if (t == 1) {
@@ -565,7 +560,7 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
             }
           }
         }
-        xs[i] = xn;
+        xs[et] = xn;
       }
       epi_sync();
     }
@@ -574,7 +569,7 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
   __syncthreads();
   gc_settle(p.err);
   cluster_arrive(); cluster_wait();       // no CTA leaves while a peer may still write to it
-  if (warp == 1) tmem_dealloc(tmem_base, 32);
+  if (warp == 8) tmem_dealloc(tmem_base, 64);
 }
 
 }  // namespace csd
