@@ -390,10 +390,12 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
       const int row = lane & 7, h = lane >> 3;                       // four lanes per row, a quarter of the W / 32 partials each
       const float2* src = stats_s + h * CL * kGcRows + r0 + row;
       float sm = 0.0f, m2 = 0.0f, q = 0.0f;
+#pragma unroll 4
       for (int g = 0; g < CL; ++g) { const float2 v = src[g * kGcRows]; sm += v.x; m2 += v.y; }
       sm += __shfl_xor_sync(0xffffffffu, sm, 8);
       sm += __shfl_xor_sync(0xffffffffu, sm, 16);
       const float mean = sm / static_cast<float>(4 * CL);
+#pragma unroll 4
       for (int g = 0; g < CL; ++g) { const float d = src[g * kGcRows].x - mean; q = fmaf(d, d, q); }
       m2 = fmaf(32.0f, q, m2);
       m2 += __shfl_xor_sync(0xffffffffu, m2, 8);
@@ -428,14 +430,16 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
       xs[et] = v;
     }
     float h[kGcHalf], m0[kGcHalf], m1[kGcHalf], a[kGcHalf];
+    float4 w0, w1, w2, w3;                                   // the column's input weights, on their way while the partials meet
+    const float4* const win4 = reinterpret_cast<const float4*>(p.win + static_cast<size_t>(col) * kCPad);
+    const float bi = __ldg(p.bin + col), bs = __ldg(p.bsc + col);
+    auto take_win = [&]() { w0 = gc_ld(win4); w1 = gc_ld(win4 + 1); w2 = gc_ld(win4 + 2); w3 = gc_ld(win4 + 3); };
     take(m0, p.t_hi, 0);
+    take_win();
     epi_sync();
     for (int t = p.t_hi; t >= p.t_lo; --t) {
       // ---- h = Win x + bin for the column, a' = h (1 + scale_0)
       {
-        const float4* wq = reinterpret_cast<const float4*>(p.win + static_cast<size_t>(col) * kCPad);
-        const float4 w0 = __ldg(wq), w1 = __ldg(wq + 1), w2 = __ldg(wq + 2), w3 = __ldg(wq + 3);
-        const float bi = __ldg(p.bin + col), bs = __ldg(p.bsc + col);
 #pragma unroll
         for (int i = 0; i < kGcHalf; ++i) {
           const float4* xq = reinterpret_cast<const float4*>(xs + ((p.cfg ? 0 : r0) + i) * kCPad);
@@ -504,27 +508,38 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
         }
         if (t > p.t_lo) take(m0, t - 1, 0);
         epi_sync();
-        // four outputs of one row over a quarter of the columns per thread, the quarters apart (bank conflicts)
-        const int quad = lane & 3, row = ew * 2 + ((lane >> 2) & 1), qt = lane >> 3;
-        float4 o = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll 8
-        for (int j = 0; j < 32; ++j) {
-          const int cc = qt * 32 + ((j + qt * 8) & 31);
-          const float u = uf_s[row * kUfLd + cc];
-          const float4 w = *reinterpret_cast<const float4*>(wout_s + cc * kCPad + quad * 4);
-          o.x = fmaf(u, w.x, o.x); o.y = fmaf(u, w.y, o.y); o.z = fmaf(u, w.z, o.z); o.w = fmaf(u, w.w, o.w);
-        }
+        // four outputs of two rows over 16 columns per thread, the rows 2 ew, 2 ew + 1 in a warp; columns cg, cg + 8, ..
+        const int quad = lane & 3, cg = lane >> 2;
+        const float* u0 = uf_s + 2 * ew * kUfLd + cg;
+        const float4* wq = reinterpret_cast<const float4*>(wout_s) + cg * 4 + quad;
+        float o[8];
 #pragma unroll
-        for (int d = 8; d <= 16; d <<= 1) {
-          o.x += __shfl_xor_sync(0xffffffffu, o.x, d); o.y += __shfl_xor_sync(0xffffffffu, o.y, d);
-          o.z += __shfl_xor_sync(0xffffffffu, o.z, d); o.w += __shfl_xor_sync(0xffffffffu, o.w, d);
+        for (int i = 0; i < 8; ++i) o[i] = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const float4 w = wq[j * 32];
+          const float a0 = u0[j * 8], a1 = u0[kUfLd + j * 8];
+          o[0] = fmaf(a0, w.x, o[0]); o[1] = fmaf(a0, w.y, o[1]); o[2] = fmaf(a0, w.z, o[2]); o[3] = fmaf(a0, w.w, o[3]);
+          o[4] = fmaf(a1, w.x, o[4]); o[5] = fmaf(a1, w.y, o[5]); o[6] = fmaf(a1, w.z, o[6]); o[7] = fmaf(a1, w.w, o[7]);
         }
-        if (qt == 0) part_out[row * 4 + quad] = o;
+        // sum over cg, transposing: lane (cg, quad) ends with value cg = 4 row + output
+#pragma unroll
+        for (int n = 4; n >= 1; n >>= 1) {
+          const bool up = (cg & n) != 0;
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (i < n) {
+              const float send = up ? o[i] : o[i + n], keep = up ? o[i + n] : o[i];
+              o[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * n);
+            }
+        }
+        reinterpret_cast<float*>(part_out)[(2 * ew + (cg >> 2)) * kCPad + quad * 4 + (cg & 3)] = o[0];
         fence_proxy_async_smem();
         epi_sync();
         if (ok && ew == 0 && lane < CL)
           gc_copy(mapa_shared(smem_u32(part_s + rank * kGcRows * kCPad), lane), part_out, kGcRows * kCPad * 4, mapa_shared(smem_u32(part_full), lane));
         __syncwarp();
+        take_win();
       }
       // ---- guidance and Eq. 3, by every CTA alike (CTA 0 writes what leaves the chip)
       const float bo = mine ? p.bout[e] : 0.0f;
