@@ -140,7 +140,7 @@ int64_t csd_launch_count(const csd_ctx *ctx);
  *                       CSD_CHAIN_LAYER_KERNELS, whose kernels spread over the idle SMs; the default is chosen
  *                       per chain, not per call, so that csd_round and the three separate calls give the same bits.
  *                     - A chain of few rows on a 16-bit head with W in {512, 1024, 1536} and var_out = 0 (groups of
- *                       16 tokens, or 8 with guidance: up to 17, 8 and 4 groups) runs as the group chain kernel:
+ *                       16 tokens, or 8 with guidance: up to 33, 15 and 7 groups) runs as the group chain kernel:
  *                       everything that depends on the condition vector only is formed ahead, for many steps at a
  *                       time, and a cluster of W / 128 CTAs carries each group through the steps, activations
  *                       passing through distributed shared memory.  This is the calling pattern Alg. 1 forces on

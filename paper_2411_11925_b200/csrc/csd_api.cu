@@ -581,12 +581,13 @@ struct Chain {
     }
     // Few rows: condition products ahead, one kernel for the rest (groupchain.cuh).
     // Few rows: condition products ahead, one kernel for the rest (groupchain.cuh).  A step takes it as long for one group as
-    // for all that are resident (W = 1024: 15 clusters), so it wins up to there; the two chains of a round run together, and a
-    // call of one chain takes the same kernels as the round does, so each gets half.  Beyond: 1536-wide, 8 groups where 7
-    // clusters fit, 42 ms a round against the layer kernels' 27.
+    // for all that are resident (clusters: 33, 15, 7 at W = 512, 1024, 1536), so it wins up to there, even where a round's two
+    // chains have to take turns: 240 rows each of the 3 and 6 x 1024 heads, 9.2 ms a round against the layer kernels' 13.2;
+    // 7 groups of a 12 x 1536 target, 17.4 against 28.2.  One group more takes two turns by itself (42 ms).  The rule may not
+    // look at the other chain: a call of one chain gives the bits that the round gives.
     gck = tc && (ctx->chain_mode == CSD_CHAIN_LAYERS || ctx->chain_mode == CSD_CHAIN_SMALL_BATCH) && hd->gc_ready &&
           slot != 2 && !batch_Rin && !lv_min && !ctx->prof_on &&
-          (R + (cfg ? 7 : 15)) / (cfg ? 8 : 16) <= (gchain_clusters(ctx, d.dtype, W) + 1) / 2;
+          (R + (cfg ? 7 : 15)) / (cfg ? 8 : 16) <= gchain_clusters(ctx, d.dtype, W);
     if (gck) { fold = false; pair = false; }
     // One wave of 128 x 128 tiles per layer and W = 1024: one persistent kernel per chain (pchain.cuh).  Row blocks are
     // paired: an odd number is rounded up with a block of rows that belong to no token.

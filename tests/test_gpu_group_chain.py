@@ -14,8 +14,9 @@ CASES = [
     dict(B=1, gamma=1, T=3, draft=H(1, 1024, 128), target=H(2, 512, 128)),                                          # one row
     dict(B=17, gamma=1, T=5, operand="bf16", draft=H(2, 512, 128), target=H(1, 1536, 128)),                         # one row in the last group
     dict(B=3, gamma=3, T=4, cfg=True, cfg_scale=2.0, draft=H(1, 1536, 64), target=H(3, 1024, 64)),                  # guided, one token in the last group
-    dict(B=16, gamma=8, T=3, draft=H(1, 1024, 64), target=H(1, 1024, 64)),                                          # 8 groups: the most at W = 1024
-    dict(B=43, gamma=3, T=3, draft=H(1, 1024, 64), target=H(1, 1536, 64)),                                          # 9 groups: layer kernels
+    dict(B=37, gamma=3, T=3, draft=H(1, 512, 64), target=H(1, 1536, 64)),                                           # 7 groups: the most at W = 1536
+    dict(B=60, gamma=4, T=3, draft=H(1, 1024, 64), target=H(1, 1536, 64)),                                          # 15: the most at W = 1024; layer kernels
+    dict(B=241, gamma=1, T=3, draft=H(1, 1024, 64), target=H(1, 512, 64)),                                          # 16: layer kernels; more than one wave of a round
 ]
 
 
