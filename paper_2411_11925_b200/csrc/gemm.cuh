@@ -343,7 +343,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
             }
           }
           tmem_ld_wait();
-          if (Cfg::kHChunks && !Cfg::kOutOverH && ci == Cfg::kHChunks - 1 && i + 1 < my_tiles) { __syncwarp(); h_request(i + 1); }
           if (Cfg::kOutOverH && ci == 0) __syncwarp();   // every lane has read the block: the piece may take its place
           if (ci == CPT - 1) {                   // this warp's last read of the buffer: the MMAs of tile i + 2 may have it
             tc_fence_before_sync();
@@ -376,6 +375,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
               *reinterpret_cast<uint4*>(row + ((((c & 1) * 4 + u) ^ (lane & 7)) << 4)) = reinterpret_cast<const uint4*>(o)[u];
           } else if (valid)
             epi_chunk<EPI, ACT, true>(ep, m, tile_n * TN + c * kChunk, a0, a1, b0, b1, hv, rs, wout_s + c * kChunk * EPW);
+          // the next tile's h, once every lane has made use of what it read: a shared-memory load that is only issued may still
+          // be queued when the copy writes over its source
+          if (Cfg::kHChunks && !Cfg::kOutOverH && ci == Cfg::kHChunks - 1 && i + 1 < my_tiles) { __syncwarp(); h_request(i + 1); }
           if (epi_is_modf<EPI>() && ci == 1) {
 #pragma unroll
             for (int e = 0; e < EPW; ++e) rs.eacc[e] = efirst[e] + rs.eacc[e];
