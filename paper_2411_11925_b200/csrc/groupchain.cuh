@@ -11,14 +11,14 @@
 // Few rows are bound by latency: per layer a CTA multiplies its 128 weight rows (the MMA's M operand, streamed ahead through
 // a ring) with the group's 16 rows (its N), 64 instructions or 2.6 k cycles at W = 1024, and the results have to reach the
 // other CTAs of the cluster.  They do so by bulk copies from shared memory to shared memory (4 KB to each, 0.7 to 2 k cycles;
-// each CTA's MMAs start on whichever tile its own turn order reaches first, its own tile first), counted in by mbarriers: no
-// trip through L2, no proxy fence, no cluster barrier.  The two activation buffers (a', v) need no hand-back: a CTA sends its
+// a CTA's turn order starts with its own tile), counted in by mbarriers: no
+// trip through L2, no cluster barrier.  The two activation buffers (a', v) need no hand-back: a CTA sends its
 // part of one only after its product on the other, which took every peer's part of that.  LayerNorm partials travel as
-// 8-byte remote stores, the residual stream h stays in registers (a thread owns a column of 16 rows), and every CTA of the
+// 8-byte remote stores, the residual stream h stays in registers (a thread owns 8 rows of a column), and every CTA of the
 // cluster updates the group's token states x_t for itself from the exchanged output-projection partials.
 //
 // The kernel this replaces (products of s by other CTAs of the same kernel, activations through L2, a cluster barrier per
-// layer) took 38.6 us a step on a 3 x 1024 head of 128 rows and needed the GPU to itself.
+// layer) took 38.6 us a step on a 3 x 1024 head of 128 rows and needed the GPU to itself; this one 26.8.
 #pragma once
 #include "fold.cuh"
 
