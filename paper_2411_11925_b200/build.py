@@ -38,7 +38,7 @@ def _run(cmd) -> subprocess.CompletedProcess:
 def build_library(force: bool = False, verbose: bool = False) -> str:
     if force or needs_build():
         res = _run([_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
-                    "-shared", "-Xcompiler", "-fPIC", "-cudart", "static", "--split-compile=0", "-Xptxas", "-v" if verbose else "-O3",
+                    "-shared", "-Xcompiler", "-fPIC", "-cudart", "static", "-Xptxas", "-v" if verbose else "-O3",
                     "-Xlinker", "-soname=libcsd.so", "-o", LIB_PATH] + [os.path.join(CSRC, s) for s in SOURCES])
         if verbose:
             print(res.stderr)
