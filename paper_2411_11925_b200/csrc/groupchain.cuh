@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
         uint32_t more = 0;
         for (; j < 2 * CL; j += kGcMma) {
           const int src = rank + (j >> 1) < CL ? rank + (j >> 1) : rank + (j >> 1) - CL, st = m * SR + s;
-          // half of the lanes wait for the weights, half for the tile (one after the other: 2.91 instead of 2.68 ms a call of
+          // half of the lanes wait for the weights, half for the tile (one after the other: 2.79 instead of 2.73 ms a call of
           // 128 rows, 3 x 1024, 100 steps)
           ok = ok && ch_wait<false>(lane & 1 ? &w_full[st] : &tile[src], lane & 1 ? par : use & 1, p.err);
           ok = __all_sync(0xffffffffu, ok);

@@ -350,11 +350,12 @@ pchain_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ C
       if (et == 0) pc_arrive(ctr);   // release: cumulative over the writes the barrier ordered before it
     };
     // The accumulators may be overwritten once every epilogue warp of the pair has read its part: each warp says so
-    // right after its last read, before the arithmetic on what it read.
+    // right after its last read, before the arithmetic on what it read.  Relaxed: nothing in ordinary memory is handed over,
+    // and a releasing arrive waits for the warp's outstanding stores (target chain of 1024 rows 15.9 -> 15.1 ms).
     auto release_acc = [&]() {
       tc_fence_before_sync();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(mapa_shared(smem_u32(acc_empty), 0));
+      if (lane == 0) mbar_arrive_cluster_tmem(mapa_shared(smem_u32(acc_empty), 0));
     };
     auto stage_act = [&](int c, const float* v) {
       uint8_t* row = stage_out + (c >> 1) * (kTileM * 128) + rloc * 128;
