@@ -328,9 +328,9 @@ int launch_simt(csd_ctx* ctx, cudaStream_t st, const float* A0, int lda0, const 
 // Launches of the short kernels: the next one's blocks are set up while the preceding kernel still runs (each waits for it
 // before it touches memory), which takes about a microsecond off every kernel boundary.
 template <typename... KArgs, typename... Args>
-int launch_short(csd_ctx* ctx, cudaStream_t st, void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, const Args&... args) {
+int launch_short(csd_ctx* ctx, cudaStream_t st, void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem, const Args&... args) {
   cudaLaunchConfig_t lc{};
-  lc.gridDim = dim3(grid); lc.blockDim = dim3(block); lc.dynamicSmemBytes = smem; lc.stream = st;
+  lc.gridDim = grid; lc.blockDim = dim3(block); lc.dynamicSmemBytes = smem; lc.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -607,8 +607,7 @@ struct Chain {
     if (rc) return rc;
     if (fcg) return launch_f32_chain();
     if (!batch_reuse) {
-      if ((rc = launch_rows_gemm(rows_gemm(sc->tfeat, hd->Wt1, hd->bt1, ws.hid, Ts, W, d.F, true), nullptr)) ||
-          (rc = launch_rows_gemm(rows_gemm(ws.hid, hd->Wt2, hd->bt2, ws.te, Ts, W, W, false), nullptr))) return rc;
+      if ((rc = launch_embed<true>(sc->tfeat, hd->Wt1, hd->bt1, ws.hid, d.F)) || (rc = launch_embed<false>(ws.hid, hd->Wt2, hd->bt2, ws.te, W))) return rc;
     }
     CSD_CUDA(ctx, cudaGetLastError());
     ep.M = Rh; ep.ldo = W;
@@ -748,6 +747,13 @@ struct Chain {
     return CSD_OK;
   }
 
+  // One layer of the timestep embedding of all steps: [Ts, W] from [Ts, K].
+  template <bool SILU>
+  int launch_embed(const float* A, const float* B, const float* bias, float* C, int K) {
+    const bool wide = Ts >= 64;
+    const int rows = wide ? 32 : 8;
+    return launch_short(ctx, st, wide ? embed_kernel<4, SILU> : embed_kernel<1, SILU>, dim3((W + 31) / 32, (Ts + rows - 1) / rows), 64, 0, A, B, bias, C, Ts, W, K);
+  }
   static RowsGemm rows_gemm(const float* A, const float* B, const float* bias, float* C, int M, int N, int K, bool silu) {
     return RowsGemm{A, B, bias, C, M, N, K, silu ? 1 : 0, (N + kRgCols - 1) / kRgCols};
   }

@@ -8,6 +8,85 @@
 
 namespace csd {
 
+// C[m, n] = act(sum_k A[m, k] B[n, k] + bias[n]), fp32, k in ascending order: the timestep embeddings of all steps wherever the
+// layer kernels or a chain of tensor-core products read them.  The order is part of the result: one fp32 ulp of te flips
+// 16-bit roundings of s that T steps carry on (summed lane-wise and through a butterfly, as rows_gemm_kernel sums, the rounds
+// of 4096 rows moved by 1e-4 to 4e-4 of their norm), so a sum is one chain of K FMAs and a thread runs 4 MR of them side by
+// side.  Bound by shared-memory loads and that chain.  Tile 8 MR x 32, 64 threads; operands arrive by cp.async, four pieces of
+// 32 k ahead.  MR = 4 for the schedules of ~100 steps (one CTA per SM at W = 1024), MR = 1 where few rows leave more SMs idle
+// than the wider tile saves loads.
+constexpr int kEmbK = 32, kEmbStages = 4, kEmbLd = kEmbK + 4;   // (row stride of nine 16-byte units: conflict-free)
+
+// Element-sized or 16-byte asynchronous copy to shared memory; nothing is read where n is 0 (the destination is zeroed).
+template <int BYTES> __device__ __forceinline__ void cp_async(float* dst, const float* src, int n) {
+  if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n) : "memory");
+}
+
+template <int MR, bool SILU>
+__global__ void __launch_bounds__(64) embed_kernel(const float* __restrict__ A, const float* __restrict__ B, const float* __restrict__ bias,
+                                                   float* __restrict__ C, int M, int N, int K) {
+  __shared__ __align__(16) float sm[kEmbStages][(8 * MR + 32) * kEmbLd];
+  const int tid = threadIdx.x, mi = tid >> 3, ni = tid & 7, m0 = blockIdx.y * 8 * MR, n0 = blockIdx.x * 32;
+  const bool vec = K % 4 == 0 && ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0;
+  const int pieces = (K + kEmbK - 1) / kEmbK;
+  griddep_enter();
+  auto fetch = [&](int p) {       // rows 0 .. 8 MR - 1: A, the other 32: B; zero beyond M, N, K
+    if (p < pieces) {
+      float* s = sm[p % kEmbStages];
+      const int w = vec ? 4 : 1;
+      for (int i = tid; i < (8 * MR + 32) * (kEmbK / w); i += 64) {
+        const int r = i / (kEmbK / w), k = i % (kEmbK / w) * w, row = r < 8 * MR ? m0 + r : n0 + r - 8 * MR;
+        const bool in = p * kEmbK + k < K && row < (r < 8 * MR ? M : N);
+        const float* src = r < 8 * MR ? A : B;
+        if (in) src += static_cast<size_t>(row) * K + p * kEmbK + k;
+        if (vec) cp_async<16>(s + r * kEmbLd + k, src, in ? 16 : 0);
+        else cp_async<4>(s + r * kEmbLd + k, src, in ? 4 : 0);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float acc[MR][4];
+#pragma unroll
+  for (int i = 0; i < MR; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
+  for (int p = 0; p < kEmbStages - 1; ++p) fetch(p);
+  for (int p = 0; p < pieces; ++p) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kEmbStages - 2) : "memory");
+    __syncthreads();              // piece p is there, and everybody is done with the one whose place is taken next
+    fetch(p + kEmbStages - 1);
+    const float* a = sm[p % kEmbStages] + mi * kEmbLd;
+    const float* b = sm[p % kEmbStages] + (8 * MR + ni) * kEmbLd;
+#pragma unroll
+    for (int k = 0; k < kEmbK; k += 4) {
+      float4 av[MR], bv[4];
+#pragma unroll
+      for (int i = 0; i < MR; ++i) av[i] = *reinterpret_cast<const float4*>(a + 8 * i * kEmbLd + k);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) bv[j] = *reinterpret_cast<const float4*>(b + 8 * j * kEmbLd + k);
+#pragma unroll
+      for (int i = 0; i < MR; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float s = acc[i][j];
+          s = fmaf(av[i].x, bv[j].x, s); s = fmaf(av[i].y, bv[j].y, s); s = fmaf(av[i].z, bv[j].z, s); s = fmaf(av[i].w, bv[j].w, s);
+          acc[i][j] = s;
+        }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < MR; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int m = m0 + mi + 8 * i, n = n0 + ni + 8 * j;
+      if (m < M && n < N) {
+        const float v = acc[i][j] + bias[n];
+        C[static_cast<size_t>(m) * N + n] = SILU ? silu_f(v) : v;
+      }
+    }
+}
+
 template <typename ACT>
 __global__ void convert_act_kernel(const float* __restrict__ src, ACT* __restrict__ dst, size_t n) {
   const size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
