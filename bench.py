@@ -340,11 +340,12 @@ def measure(name, args, peaks, steps, warmup, rounds_per_step, full):
         ctx.set_chain_mode(api.Context.CHAIN_LAYER_KERNELS)
         timed(seq_step, 3)
         layers_secs = timed(seq_step, few)
-        ctx.set_chain_mode(api.Context.CHAIN_LAYERS)      # the group chain kernel where it applies
+        ctx.set_chain_mode(api.Context.CHAIN_SMALL_BATCH)      # the group chain kernel where it applies
         timed(seq_step, 3)
         l1 = ctx.launch_count()
         seq_secs = timed(seq_step, few)
         launches_per_call = int((ctx.launch_count() - l1) // (few * wl.gamma))
+        ctx.set_chain_mode(api.Context.CHAIN_LAYERS)
         d = wl.draft
         wbytes = 2.0 * (d.W * d.Dz + d.L * 5 * d.W * d.W + 2 * d.W * d.W)     # 16-bit GEMM weights of the draft head
         per_call = seq_secs / (few * wl.gamma)

@@ -230,7 +230,8 @@ class Context:
     def set_chain_mode(self, mode: int):
         """csd_set_chain_mode: CHAIN_LAYERS (default: the group or the persistent chain kernel where one applies, else one
         kernel per layer with folded blocks where they apply), CHAIN_LAYER_KERNELS (neither chain kernel),
-        CHAIN_LAYERS_PLAIN (three kernels per block everywhere) or CHAIN_SMALL_BATCH (as the default)."""
+        CHAIN_LAYERS_PLAIN (three kernels per block everywhere) or CHAIN_SMALL_BATCH (as CHAIN_LAYERS_PLAIN, with the group chain
+        kernel for few rows, folded up to 128 head rows: faster, rounded more often)."""
         self._check(_LIB.csd_set_chain_mode(self._h, int(mode)))
 
     def set_wait_limit(self, cycles: int):

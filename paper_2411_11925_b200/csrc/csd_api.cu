@@ -111,11 +111,12 @@ struct csd_head {
   std::vector<CUtensorMap> Wgs_half, Wf_half;   // the same matrices in 128-row boxes: what one CTA of a pair loads
   std::vector<float*> c1, c2;   // first MLP layer with 256-row boxes (W a multiple of 256)
   // group chain kernel (groupchain.cuh): the dependent layers' maps W1_k, W2_k (device table, boxes of 128 rows) and the matrix
-  // multiplied by s: scale_0 | per block W1_k Wscale_k, W1_k Wshift_k, gate_k, scale_{k+1} | final shift, scale
-  bool gc_ready = false;
+  // multiplied by s: all blocks' rows where they lie (Wss_0 to Wfss), or its own one for the folded form: scale_0 | per block
+  // W1_k Wscale_k, W1_k Wshift_k, gate_k, scale_{k+1} | final shift, scale
+  bool gc_ready = false, gf_ready = false;
   CUtensorMap* d_gc_maps = nullptr;
   void* mblob = nullptr;
-  CUtensorMap Wm{};
+  CUtensorMap Wrows{}, Wm{};
   // persistent chain kernel (pchain.cuh): per phase the early and the dependent weight maps; per phase three bias rows
   bool pc_ready = false;
   CUtensorMap* d_pc_maps = nullptr;
@@ -433,7 +434,11 @@ int gchain_clusters_of(const csd_ctx* ctx, int W) {
   static int known[kMaxDevices][kGcMaxCl + 1] = {};
   int& k = known[ctx->device][W / 128];
   if (k == 0) {
-    auto kern = group_chain_kernel<ACT, FMT>;
+    auto kern = group_chain_kernel<ACT, FMT, false>, folded = group_chain_kernel<ACT, FMT, true>;
+    auto opt_in = [](auto k) {
+      return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess &&
+             cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    };
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = static_cast<unsigned>(W / 128); at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
@@ -441,8 +446,7 @@ int gchain_clusters_of(const csd_ctx* ctx, int W) {
     lc.gridDim = dim3(static_cast<unsigned>(W / 128)); lc.blockDim = dim3(kGcThreads); lc.dynamicSmemBytes = gc_layout(W).total + 1024;
     lc.attrs = at; lc.numAttrs = 1;
     int n = 0;
-    const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess &&
-                    cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+    const bool ok = opt_in(kern) && opt_in(folded) &&
                     cudaFuncSetAttribute(mods_gemm_kernel<FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMgSmemBytes) == cudaSuccess &&
                     cudaOccupancyMaxActiveClusters(&n, kern, &lc) == cudaSuccess;
     cudaGetLastError();
@@ -463,7 +467,7 @@ struct Chain {
   int R, cfg; float cfg_scale; const float *z, *x_T, *eps; int sample_last; float *x0, *mu1, *x1;
   int chains = 1;   // chains that run concurrently with this one (itself included)
   int Rh = 0, W = 0, L = 0, T = 0, tn = kTileN;
-  bool gck = false;       // the whole chain runs in the group chain kernel (groupchain.cuh)
+  bool gck = false, gfold = false;   // the whole chain runs in the group chain kernel (groupchain.cuh), in its folded form
   bool pck = false;       // the whole chain runs in the persistent chain kernel (pchain.cuh)
   int fcg = 0;            // fp32 head: the whole chain runs in the fp32 chain kernel with groups of this many rows (f32chain.cuh)
   bool fold = false;      // blocks 1.. run as two kernels (fold.cuh) instead of three
@@ -579,7 +583,6 @@ struct Chain {
       fold = tc && (ctx->chain_mode == CSD_CHAIN_LAYERS || ctx->chain_mode == CSD_CHAIN_LAYER_KERNELS) && !pair && L >= 2 && !hd->Wf.empty() &&
              8 * t128 > ctx->num_sms && 2 * t128 <= ctx->num_sms && fold_kernels_ready(ctx, d);
     }
-    // Few rows: condition products ahead, one kernel for the rest (groupchain.cuh).
     // Few rows: condition products ahead, one kernel for the rest (groupchain.cuh).  A step takes it as long for one group as
     // for all that are resident (clusters: 33, 15, 7 at W = 512, 1024, 1536), so it wins up to there, even where a round's two
     // chains have to take turns: 240 rows each of the 3 and 6 x 1024 heads, 9.2 ms a round against the layer kernels' 13.2;
@@ -589,6 +592,8 @@ struct Chain {
           slot != 2 && !batch_Rin && !lv_min && !ctx->prof_on &&
           (R + (cfg ? 7 : 15)) / (cfg ? 8 : 16) <= gchain_clusters(ctx, d.dtype, W);
     if (gck) { fold = false; pair = false; }
+    // Its folded form is a quarter faster a layer and less precise: only in the mode that says so, up to the rows that it names
+    gfold = gck && ctx->chain_mode == CSD_CHAIN_SMALL_BATCH && Rh <= 128 && hd->gf_ready;
     // One wave of 128 x 128 tiles per layer and W = 1024: one persistent kernel per chain (pchain.cuh).  Row blocks are
     // paired: an odd number is rounded up with a block of rows that belong to no token.
     {
@@ -818,7 +823,7 @@ struct Chain {
     if (rc) return rc;
     // Steps per chunk: a first chunk of a tile's width of rows, because nothing overlaps its products; then twice as many
     // each time, as far as the buffers go.
-    const size_t wrows = static_cast<size_t>(4 * L + 2) * W;
+    const size_t wrows = static_cast<size_t>((gfold ? 4 : 3) * L + 2) * W;
     auto chunk_bytes = [&](int steps) { return wrows * ((static_cast<size_t>(steps) * rows + 255) / 256) * 256 * 4; };
     int most = Ts;
     while (most > 1 && chunk_bytes(most) > kGcChunkBytes) most = (most + 1) / 2;
@@ -841,7 +846,8 @@ struct Chain {
     CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_prep[slot], 0));
     GcParams p{};
     p.R = R; p.cfg = cfg; p.W = W; p.L = L; p.C = d.C; p.T = Ts; p.rows = rows; p.sample_last = sample_last; p.cfg_scale = cfg_scale;
-    p.maps = hd->d_gc_maps; p.c1 = hd->c1[0]; p.bg = hd->bg[0]; p.b2 = hd->b2[0]; p.bsc = hd->bsc[0]; p.bfsh = hd->bfsh; p.bfsc = hd->bfsc;
+    p.maps = hd->d_gc_maps; p.c1 = hd->c1[0]; p.bsh = hd->bsh[0]; p.bsc = hd->bsc[0]; p.bg = hd->bg[0]; p.b1 = hd->b1[0]; p.b2 = hd->b2[0];
+    p.bfsh = hd->bfsh; p.bfsc = hd->bfsc;
     p.sched = d_sched; p.win = hd->win; p.bin = hd->bin; p.wout_t = hd->wout_t; p.bout = hd->bout; p.x_T = x_T; p.eps = eps;
     p.x = ws.x; p.x0 = x0; p.mu1 = mu1; p.x1 = x1; p.traj_x = traj_x; p.traj_mu = traj_mu; p.err = ctx->d_err; p.status = ctx->d_err + 1;
     cudaLaunchAttribute at[1];
@@ -857,6 +863,7 @@ struct Chain {
       float4* mods = reinterpret_cast<float4*>(static_cast<char*>(ctx->gm[slot].base) + buf * chunk_bytes(most));
       MgParams m{};
       m.nkb = W / kBlockK; m.tiles_n = (n * rows + 255) / 256; m.units = m.tiles_n * static_cast<int>(wrows / 256);
+      m.run = gfold ? static_cast<int>(wrows / 256) : 3 * W / 256; m.stride = 5 * W;   // plain: a block's layers lie between
       m.s_row0 = (t_lo - 1) * rows; m.out = mods; m.err = ctx->d_err;
       if (c >= 2) CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_read[slot][buf], 0));
       // beside a running chain the products take the SMs it leaves
@@ -865,15 +872,15 @@ struct Chain {
       if (pairs > m.units) pairs = m.units;
       lc.gridDim = dim3(static_cast<unsigned>(2 * pairs)); lc.blockDim = dim3(kMgThreads); lc.dynamicSmemBytes = kMgSmemBytes; lc.stream = gst;
       at[0].val.clusterDim.x = 2;
-      if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<0>, hd->Wm, tm_s, m));
-      else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<1>, hd->Wm, tm_s, m));
+      if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<0>, gfold ? hd->Wm : hd->Wrows, tm_s, m));
+      else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<1>, gfold ? hd->Wm : hd->Wrows, tm_s, m));
       CSD_CUDA(ctx, cudaEventRecord(ctx->ev_mods[slot][buf], gst));
       CSD_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_mods[slot][buf], 0));
       p.t_hi = t_hi; p.t_lo = t_lo; p.mods = mods; p.nq = m.tiles_n * 64;
       lc.gridDim = dim3(static_cast<unsigned>(groups * cl)); lc.blockDim = dim3(kGcThreads); lc.dynamicSmemBytes = gc_layout(W).total + 1024; lc.stream = st;
       at[0].val.clusterDim.x = static_cast<unsigned>(cl);
-      if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, group_chain_kernel<__half, 0>, p));
-      else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, group_chain_kernel<__nv_bfloat16, 1>, p));
+      if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, gfold ? group_chain_kernel<__half, 0, true> : group_chain_kernel<__half, 0, false>, p));
+      else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, gfold ? group_chain_kernel<__nv_bfloat16, 1, true> : group_chain_kernel<__nv_bfloat16, 1, false>, p));
       CSD_CUDA(ctx, cudaEventRecord(ctx->ev_read[slot][buf], st));
       ctx->launches += 2;
       t_hi = t_lo - 1;
@@ -1546,8 +1553,9 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
           cudaMalloc(&h->d_gc_maps, maps.size() * sizeof(CUtensorMap)) != cudaSuccess) { cudaGetLastError(); return bail(CSD_ERR_WORKSPACE, "cannot allocate device memory for the group-chain tables"); }
       if (cudaMemcpy(h->mblob, mb.data(), mb.size() * 2, cudaMemcpyHostToDevice) != cudaSuccess ||
           cudaMemcpy(h->d_gc_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess) return bail(CSD_ERR_CUDA, "group-chain table upload failed");
-      if ((rc = make_tmap(ctx, &h->Wm, d.dtype, h->mblob, (4 * L + 2) * W, W, W, kTileM))) { csd_head_destroy(h); return rc; }
-      h->gc_ready = true;
+      if ((rc = make_tmap(ctx, &h->Wm, d.dtype, h->mblob, (4 * L + 2) * W, W, W, kTileM)) ||
+          (rc = make_tmap(ctx, &h->Wrows, d.dtype, h->Wss[0], (5 * L + 2) * W, W, W, kTileM))) { csd_head_destroy(h); return rc; }
+      h->gc_ready = h->gf_ready = true;
     }
     if (gck && W / kTileN == static_cast<size_t>(kPcColTiles)) {
       // tables of the persistent chain kernel: phases B, (W1_k, GATE_k) for every block, F

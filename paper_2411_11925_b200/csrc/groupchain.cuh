@@ -1,8 +1,8 @@
 // A denoising chain of few rows (W in {512, 1024, 1536}, 16-bit operands) in two parts:
 //
-// 1. mods_gemm_kernel: everything a head takes from the condition vector - gates, scales, the folded first-layer terms
-//    P1 | P2 of fold.cuh, the final shift and scale: two thirds of its multiply-adds - does not depend on x_t.  It is
-//    formed for many steps at once, as one dense product over the rows of a chunk of steps, in fp32.
+// 1. mods_gemm_kernel: everything a head takes from the condition vector - shifts, scales, gates: three fifths of its
+//    multiply-adds - does not depend on x_t.  It is formed for many steps at once, as one dense product over the rows of a chunk
+//    of steps, in fp32.
 // 2. group_chain_kernel: what depends on x_t.  Token rows never exchange data, so the rows are cut into groups of 16 (with
 //    guidance 8 tokens' conditional rows and their unconditional twins) and a cluster of W / 128 CTAs owns a group for all
 //    steps of the chunk; CTA r owns output columns [128 r, 128 r + 128) of every layer.  Groups never wait for each other and
@@ -17,8 +17,13 @@
 // 8-byte remote stores, the residual stream h stays in registers (a thread owns 8 rows of a column), and every CTA of the
 // cluster updates the group's token states x_t for itself from the exchanged output-projection partials.
 //
-// The kernel this replaces (products of s by other CTAs of the same kernel, activations through L2, a cluster barrier per
-// layer) took 38.6 us a step on a 3 x 1024 head of 128 rows and needed the GPU to itself; this one 25 to 27.
+// Two forms.  Plain (the default mode): the operand of a block's first layer is u = LN(h)(1 + scale) + shift, rounded once, as in
+// the layer kernels, and the LayerNorm partials are awaited before it can leave.  FOLD (CSD_CHAIN_SMALL_BATCH up to 128 head rows):
+// the folded blocks of fold.cuh, first-layer terms P1 | P2 among the products of s; what leaves is a' = h (1 + scale), which waits
+// for nothing.  Folding rounds the fused weights as well, and the mean goes only after the product: against float64 its error
+// is 1.02 to 1.20 times that of the layer kernels (geometric means over 12 draws of 9 to 91 tokens each; 2 x 512 to 12 x 1536, both
+// formats), the plain form's 0.90 to 1.03 times.  The wait costs 1 to 9 %: 3 x 1024, T = 40, 12 tokens with guidance 1.03 -> 1.07 ms,
+// 12 x 1536 5.8 -> 6.3 ms (layer kernels 2.2 and 9.6).
 #pragma once
 #include "fold.cuh"
 
@@ -38,6 +43,7 @@ __device__ __forceinline__ void gc_settle(const int* err) {
 
 struct MgParams {
   int nkb, tiles_n, units;     // k-blocks; tiles of 256 rows of s; tiles in all (s fastest: the weights stream past once)
+  int run, stride;             // tiles of 256 weight rows come in runs of this many, whose first rows lie this far apart
   int s_row0;                  // first row of s
   float4* out;                 // [weight row / 128][row of s / 4][128 weight rows][4 rows of s]
   int* err;
@@ -84,7 +90,8 @@ mods_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       int it = 0;
       for (int i = 0; i < my_tiles && ok; ++i) {
         const int u = unit0 + i * nunits;
-        const int row = (is_w ? (u / p.tiles_n) * 256 : p.s_row0 + (u % p.tiles_n) * 256) + rank * 128;
+        const int wt = u / p.tiles_n;
+        const int row = (is_w ? wt / p.run * p.stride + wt % p.run * 256 : p.s_row0 + (u - wt * p.tiles_n) * 256) + rank * 128;
         for (int kb = 0; kb < p.nkb; ++kb, ++it) {
           const int s = it % S;
           if (it >= S && !ch_wait<false>(&empty_bar[s], ((it / S) & 1) ^ 1, p.err)) { ch_fail(p.err, DEV_ERR_TMA_WAIT, 1, it); ok = false; break; }
@@ -193,7 +200,7 @@ struct GcParams {
   float cfg_scale;
   const CUtensorMap* maps;     // [2 L]: W1_k, W2_k in boxes of 128 rows
   const float4* mods; int nq;  // products of the chunk, nq row quads per weight row
-  const float *c1, *bg, *b2, *bsc, *bfsh, *bfsc;   // block 0; c1_k | c2_k are 2 W floats a block, the others 5 W apart
+  const float *c1, *bsh, *bsc, *bg, *b1, *b2, *bfsh, *bfsc;   // block 0; c1_k | c2_k (FOLD) are 2 W floats a block, the others 5 W apart
   const float* sched;          // a[T], b[T], sigma[T]
   const float *win, *bin, *wout_t, *bout;
   const float *x_T, *eps;
@@ -237,7 +244,7 @@ __device__ __forceinline__ float4 gc_ld(const float4* p) {
   return v;
 }
 
-template <typename ACT, int AB_FMT>
+template <typename ACT, int AB_FMT, bool FOLD>
 __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid_constant__ GcParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -352,12 +359,20 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
     auto wait = [&](uint64_t* bar, uint32_t parity, int site) {
       if (ok && !ch_wait<true>(bar, parity, p.err)) { ch_fail(p.err, DEV_ERR_EPI_WAIT, site, static_cast<int>(n_acc)); ok = false; }
     };
-    // product `sec` of step t, this thread's column and rows
-    auto take = [&](float (&m)[kGcHalf], int t, int sec) {
-      const float4* src = p.mods + (static_cast<size_t>(sec * CL + rank) * p.nq + (static_cast<size_t>(t - p.t_lo) * p.rows + grp * kGcRows + r0) / 4) * 128 + c;
+    // product of step t with row `row` of tile `tile` of 128 weight rows, for this thread's rows of the group
+    auto take_row = [&](float (&m)[kGcHalf], int t, int tile, int row) {
+      const float4* src = p.mods + (static_cast<size_t>(tile) * p.nq + (static_cast<size_t>(t - p.t_lo) * p.rows + grp * kGcRows + r0) / 4) * 128 + row;
       const float4 a = gc_ld(src), b = gc_ld(src + 128);
       m[0] = a.x; m[1] = a.y; m[2] = a.z; m[3] = a.w; m[4] = b.x; m[5] = b.y; m[6] = b.z; m[7] = b.w;
     };
+    // FOLD: product `sec` (scale_0 | per block P1, P2, gate, next scale | final shift, scale) in this thread's column
+    auto take = [&](float (&m)[kGcHalf], int t, int sec) { take_row(m, t, sec * CL + rank, c); };
+    // Plain: shift and scale of block k (L: the final pair), whose rows are interleaved in groups of 64, and gate
+    auto take_ss = [&](float (&sh)[kGcHalf], float (&sc)[kGcHalf], int t, int k) {
+      const int tile = 3 * CL * k + 2 * rank + (c >> 6);
+      take_row(sh, t, tile, c & 63); take_row(sc, t, tile, 64 + (c & 63));
+    };
+    auto take_gate = [&](float (&m)[kGcHalf], int t, int k) { take_row(m, t, 3 * CL * k + 2 * CL + rank, c); };
     // 16-bit tile of this CTA's columns: into its own activation buffer `buf`, and from there into every peer's
     auto send_tile = [&](const float (&v)[kGcHalf], int buf) {
       uint8_t* const out = act + buf * act_bytes + rank * kGcTile;
@@ -433,16 +448,27 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
       }
       xs[et] = v;
     }
-    float h[kGcHalf], m0[kGcHalf], m1[kGcHalf], a[kGcHalf];
+    float h[kGcHalf], m0[kGcHalf], m1[kGcHalf], m2[FOLD ? 1 : kGcHalf], a[kGcHalf];
+    // Plain: u = LN(h)(1 + scale) + shift of block k to every CTA
+    auto send_u = [&](const float (&sh)[kGcHalf], const float (&sc)[kGcHalf], float bsh, float bsc) {
+      norms();
+#pragma unroll
+      for (int i = 0; i < kGcHalf; ++i) {
+        const float2 nr = norm_s[i];
+        a[i] = fmaf(__fmul_rn(__fsub_rn(h[i], nr.x), nr.y), __fadd_rn(1.0f, sc[i] + bsc), sh[i] + bsh);
+      }
+      send_tile(a, 0);
+    };
     float4 w0, w1, w2, w3;                                   // the column's input weights, on their way while the partials meet
     const float4* const win4 = reinterpret_cast<const float4*>(p.win + static_cast<size_t>(col) * kCPad);
-    const float bi = __ldg(p.bin + col), bs = __ldg(p.bsc + col);
+    const float bi = __ldg(p.bin + col), bs = __ldg(p.bsc + col), bh = FOLD ? 0.0f : __ldg(p.bsh + col);
     auto take_win = [&]() { w0 = gc_ld(win4); w1 = gc_ld(win4 + 1); w2 = gc_ld(win4 + 2); w3 = gc_ld(win4 + 3); };
-    take(m0, p.t_hi, 0);
+    auto take_first = [&](int t) { if constexpr (FOLD) take(m0, t, 0); else take_ss(m0, m1, t, 0); };
+    take_first(p.t_hi);
     take_win();
     epi_sync();
     for (int t = p.t_hi; t >= p.t_lo; --t) {
-      // ---- h = Win x + bin for the column, a' = h (1 + scale_0)
+      // ---- h = Win x + bin for the column; a' = h (1 + scale_0), or u
       {
 #pragma unroll
         for (int i = 0; i < kGcHalf; ++i) {
@@ -455,16 +481,21 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
           v = fmaf(w3.x, x3.x, v); v = fmaf(w3.y, x3.y, v); v = fmaf(w3.z, x3.z, v); v = fmaf(w3.w, x3.w, v);
           h[i] = v;
         }
+        if constexpr (FOLD) {
 #pragma unroll
-        for (int i = 0; i < kGcHalf; ++i) a[i] = __fmul_rn(h[i], __fadd_rn(1.0f, __fadd_rn(m0[i], bs)));
-        send_tile(a, 0);
-        take(m0, t, 1); take(m1, t, 2);
-        send_stats(h);
+          for (int i = 0; i < kGcHalf; ++i) a[i] = __fmul_rn(h[i], __fadd_rn(1.0f, __fadd_rn(m0[i], bs)));
+          send_tile(a, 0);
+          take(m0, t, 1); take(m1, t, 2);
+          send_stats(h);
+        } else {
+          send_stats(h);
+          send_u(m0, m1, bh, bs);
+        }
       }
 #pragma unroll 1
       for (int k = 0; k < L; ++k) {
-        // ---- v = SiLU(rstd (a' W1^T - mean (P1 + c1)) + P2 + c2)
-        {
+        // ---- v = SiLU(rstd (a' W1^T - mean (P1 + c1)) + P2 + c2), or SiLU(u W1^T + b1)
+        if constexpr (FOLD) {
           const float k0 = __ldg(p.c1 + static_cast<size_t>(2 * k) * W + col), k1 = __ldg(p.c1 + static_cast<size_t>(2 * k + 1) * W + col);
           norms();
           acc_load(a);
@@ -475,10 +506,16 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
             a[i] = silu_t<true>(fmaf(nr.y, t1, __fadd_rn(m1[i], k1)));
           }
           send_tile(a, 1);
+        } else {
+          const float k0 = __ldg(p.b1 + static_cast<size_t>(5 * k) * W + col);
+          acc_load(a);
+#pragma unroll
+          for (int i = 0; i < kGcHalf; ++i) a[i] = silu_t<true>(a[i] + k0);
+          send_tile(a, 1);
         }
-        // ---- h += gate (v W2^T + b2); a' = h (1 + scale_{k+1})
-        {
-          const bool last = k + 1 == L;
+        // ---- h += gate (v W2^T + b2); the next block's a' = h (1 + scale_{k+1}), or u
+        const bool last = k + 1 == L;
+        if constexpr (FOLD) {
           take(m0, t, 4 * k + 3);
           if (!last) take(m1, t, 4 * k + 4);
           const float kg = __ldg(p.bg + static_cast<size_t>(5 * k) * W + col), kb = __ldg(p.b2 + static_cast<size_t>(5 * k) * W + col),
@@ -494,6 +531,16 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
           const int sec = last ? 4 * L : 4 * k + 5;           // the final shift and scale, or the next block's P1, P2
           take(m0, t, sec); take(m1, t, sec + 1);
           send_stats(h);
+        } else {
+          take_gate(m0, t, k);
+          take_ss(m2, m1, t, k + 1);
+          const size_t at = static_cast<size_t>(5 * k) * W + col, nx = last ? 0 : at + static_cast<size_t>(5) * W;
+          const float kg = __ldg(p.bg + at), kb = __ldg(p.b2 + at), kh = __ldg(p.bsh + nx), ks = __ldg(p.bsc + nx);
+          acc_load(a);
+#pragma unroll
+          for (int i = 0; i < kGcHalf; ++i) { h[i] = fmaf(m0[i] + kg, a[i] + kb, h[i]); m0[i] = m2[i]; }
+          send_stats(h);
+          if (!last) send_u(m0, m1, kh, ks);
         }
       }
       // ---- output projection of (LN(h)(1 + scale_f) + shift_f): this CTA's columns' part, to every CTA
@@ -510,7 +557,7 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
           const float2 nr = norm_s[i];
           uf_s[(r0 + i) * kUfLd + c] = fmaf(__fmul_rn(__fsub_rn(h[i], nr.x), nr.y), __fadd_rn(1.0f, m1[i] + k1), m0[i] + k0);
         }
-        if (t > p.t_lo) take(m0, t - 1, 0);
+        if (t > p.t_lo) take_first(t - 1);
         epi_sync();
         // four outputs of two rows over 16 columns per thread, the rows 2 ew, 2 ew + 1 in a warp; columns cg, cg + 8, ..
         const int quad = lane & 3, cg = lane >> 2;
