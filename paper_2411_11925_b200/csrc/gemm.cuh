@@ -375,9 +375,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
               *reinterpret_cast<uint4*>(row + ((((c & 1) * 4 + u) ^ (lane & 7)) << 4)) = reinterpret_cast<const uint4*>(o)[u];
           } else if (valid)
             epi_chunk<EPI, ACT, true>(ep, m, tile_n * TN + c * kChunk, a0, a1, b0, b1, hv, rs, wout_s + c * kChunk * EPW);
-          // the next tile's h, once every lane has made use of what it read: a shared-memory load that is only issued may still
-          // be queued when the copy writes over its source
-          if (Cfg::kHChunks && !Cfg::kOutOverH && ci == Cfg::kHChunks - 1 && i + 1 < my_tiles) { __syncwarp(); h_request(i + 1); }
+          // The next tile's h.  The copy writes, through the async proxy, over what the lanes have read with ordinary loads: the
+          // proxy fence completes them.  (__syncwarp() does not: a load that was issued but whose value nothing had used yet read
+          // the next tile's rows, once in 10^6 tiles; and in the final kernel that use is arithmetic on registers, which
+          // nothing keeps in front of the copy.)
+          if (Cfg::kHChunks && !Cfg::kOutOverH && ci == Cfg::kHChunks - 1 && i + 1 < my_tiles) { fence_proxy_async_smem(); __syncwarp(); h_request(i + 1); }
           if (epi_is_modf<EPI>() && ci == 1) {
 #pragma unroll
             for (int e = 0; e < EPW; ++e) rs.eacc[e] = efirst[e] + rs.eacc[e];
