@@ -331,6 +331,7 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
           // 128 rows, 3 x 1024, 100 steps)
           ok = ok && ch_wait<false>(lane & 1 ? &w_full[st] : &tile[src], lane & 1 ? par : use & 1, p.err);
           ok = __all_sync(0xffffffffu, ok);
+          __syncwarp();        // (a vote orders no memory: the leader issues on what the other lanes have waited for)
           if (!ok) { if (leader) ch_fail(p.err, DEV_ERR_MMA_WAIT, 2, ph); break; }
           tc_fence_after_sync();
           if (leader) {
