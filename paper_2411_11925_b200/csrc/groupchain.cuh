@@ -35,11 +35,7 @@ constexpr int kMgEpiWarps = 8;
 constexpr int kMgThreads = (kMgEpiWarps + 3) * 32;
 constexpr int kMgSmemBytes = 1024 + kMgStages * kMgStageBytes + 256;
 
-// After a wait that ran out, copies may be in flight that nobody waits for: they land within microseconds.
-__device__ __forceinline__ void gc_settle(const int* err) {
-  if (*reinterpret_cast<const volatile int*>(err) != 0)
-    for (int i = 0; i < 64; ++i) __nanosleep(1000);
-}
+__device__ __forceinline__ void gc_settle(const int* err) { if (*reinterpret_cast<const volatile int*>(err) != 0) settle(); }
 
 struct MgParams {
   int nkb, tiles_n, units;     // k-blocks; tiles of 256 rows of s; tiles in all (s fastest: the weights stream past once)

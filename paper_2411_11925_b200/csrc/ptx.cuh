@@ -105,6 +105,11 @@ __device__ __forceinline__ void ch_fail(int* err, int role, int site, int count)
   atomicCAS(err, 0, role | (site << 4) | ((count & 0xffff) << 8) | ((static_cast<int>(blockIdx.x) & 0x7f) << 24));
 }
 
+// After a wait that ran out, copies may be in flight that nobody waits for: they land within microseconds.
+__device__ __forceinline__ void settle() {
+  for (int i = 0; i < 64; ++i) __nanosleep(1000);
+}
+
 // ------------------------------------------------ programmatic dependent launch
 // No-ops unless the kernel was launched with the programmatic-stream-serialization attribute.
 // wait: blocks until the preceding kernel of the stream has completed and its writes are visible.
