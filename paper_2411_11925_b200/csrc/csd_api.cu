@@ -73,7 +73,7 @@ struct csd_ctx {
   HostIo bn;       // csd_bonus_token: samples of every sequence before the selection
   HostIo sp;       // csd_verify_single_path: schedule constants, mu^p of one pass, running log-ratio
   HostIo pc[3];    // persistent chain kernel (per chain slot): s of all steps, a', v, partials, counters, schedule
-  HostIo gc[2];    // group chain kernel (per chain slot): s of all steps, schedule
+  HostIo gc[2];    // group chain kernel (per chain slot): s of all steps
   HostIo gm[2];    // its condition products: two chunks of steps
   cudaStream_t aux[2] = {nullptr, nullptr};        // (per chain slot) where they are formed
   cudaEvent_t ev_prep[2] = {}, ev_mods[2][2] = {}, ev_read[2][2] = {};   // preparation done; a chunk is written / has been read
@@ -816,29 +816,21 @@ struct Chain {
     const csd_head_desc& d = hd->d;
     ChainWs& ws = ctx->ws[slot];
     const int per = cfg ? 8 : 16, groups = (R + per - 1) / per, rows = groups * kGcRows, cl = W / 128;
-    size_t off = 0;
-    auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 1024); return o; };
-    const size_t o_s = take(static_cast<size_t>(Ts) * rows * W * 2), o_sched = take(static_cast<size_t>(3) * Ts * 4);
-    int rc = ensure_side(ctx, ctx->gc[slot], off, "the group chain buffers");
+    int rc = ensure_side(ctx, ctx->gc[slot], static_cast<size_t>(Ts) * rows * W * 2, "the condition vectors of all steps");
     if (rc) return rc;
     // Steps per chunk: a first chunk of a tile's width of rows, because nothing overlaps its products; then twice as many
     // each time, as far as the buffers go.
     const size_t wrows = static_cast<size_t>((gfold ? 4 : 3) * L + 2) * W;
     auto chunk_bytes = [&](int steps) { return wrows * ((static_cast<size_t>(steps) * rows + 255) / 256) * 256 * 4; };
-    int most = Ts;
+    int most = Ts < kGcMaxSteps ? Ts : kGcMaxSteps;
     while (most > 1 && chunk_bytes(most) > kGcChunkBytes) most = (most + 1) / 2;
     if ((rc = ensure_side(ctx, ctx->gm[slot], 2 * chunk_bytes(most), "the condition products"))) return rc;
-    char* b = static_cast<char*>(ctx->gc[slot].base);
+    void* const s_all = ctx->gc[slot].base;
     CUtensorMap tm_s{};
-    if ((rc = make_tmap(ctx, &tm_s, d.dtype, b + o_s, static_cast<uint64_t>(Ts) * rows, W, W, kTileM))) return rc;
-    float* d_sched = reinterpret_cast<float*>(b + o_sched);
-    // pageable source: staged by the runtime before the call returns
-    std::vector<float> hs(static_cast<size_t>(3) * Ts);
-    for (int t = 0; t < Ts; ++t) { hs[t] = sc->a[t]; hs[Ts + t] = sc->b[t]; hs[2 * Ts + t] = sc->sigma[t]; }
-    CSD_CUDA(ctx, cudaMemcpyAsync(d_sched, hs.data(), hs.size() * 4, cudaMemcpyHostToDevice, st));
+    if ((rc = make_tmap(ctx, &tm_s, d.dtype, s_all, static_cast<uint64_t>(Ts) * rows, W, W, kTileM))) return rc;
     const dim3 sgrid(static_cast<unsigned>(rows), static_cast<unsigned>((Ts + kCondSteps - 1) / kCondSteps));
-    if (d.dtype == CSD_F16) cond_all_kernel<__half, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__half*>(b + o_s), R, cfg, W, rows, Ts);
-    else cond_all_kernel<__nv_bfloat16, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__nv_bfloat16*>(b + o_s), R, cfg, W, rows, Ts);
+    if (d.dtype == CSD_F16) cond_all_kernel<__half, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, static_cast<__half*>(s_all), R, cfg, W, rows, Ts);
+    else cond_all_kernel<__nv_bfloat16, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, static_cast<__nv_bfloat16*>(s_all), R, cfg, W, rows, Ts);
     ctx->launches++;
     CSD_CUDA(ctx, cudaGetLastError());
     cudaStream_t gst = ctx->aux[slot];
@@ -848,7 +840,7 @@ struct Chain {
     p.R = R; p.cfg = cfg; p.W = W; p.L = L; p.C = d.C; p.T = Ts; p.rows = rows; p.sample_last = sample_last; p.cfg_scale = cfg_scale;
     p.maps = hd->d_gc_maps; p.c1 = hd->c1[0]; p.bsh = hd->bsh[0]; p.bsc = hd->bsc[0]; p.bg = hd->bg[0]; p.b1 = hd->b1[0]; p.b2 = hd->b2[0];
     p.bfsh = hd->bfsh; p.bfsc = hd->bfsc;
-    p.sched = d_sched; p.win = hd->win; p.bin = hd->bin; p.wout_t = hd->wout_t; p.bout = hd->bout; p.x_T = x_T; p.eps = eps;
+    p.win = hd->win; p.bin = hd->bin; p.wout_t = hd->wout_t; p.bout = hd->bout; p.x_T = x_T; p.eps = eps;
     p.x = ws.x; p.x0 = x0; p.mu1 = mu1; p.x1 = x1; p.traj_x = traj_x; p.traj_mu = traj_mu; p.err = ctx->d_err; p.status = ctx->d_err + 1;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -877,6 +869,7 @@ struct Chain {
       CSD_CUDA(ctx, cudaEventRecord(ctx->ev_mods[slot][buf], gst));
       CSD_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_mods[slot][buf], 0));
       p.t_hi = t_hi; p.t_lo = t_lo; p.mods = mods; p.nq = m.tiles_n * 64;
+      for (int i = 0; i < n; ++i) { p.ca[i] = sc->a[t_lo - 1 + i]; p.cb[i] = sc->b[t_lo - 1 + i]; p.sigma[i] = sc->sigma[t_lo - 1 + i]; }
       lc.gridDim = dim3(static_cast<unsigned>(groups * cl)); lc.blockDim = dim3(kGcThreads); lc.dynamicSmemBytes = gc_layout(W).total + 1024; lc.stream = st;
       at[0].val.clusterDim.x = static_cast<unsigned>(cl);
       if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, gfold ? group_chain_kernel<__half, 0, true> : group_chain_kernel<__half, 0, false>, p));

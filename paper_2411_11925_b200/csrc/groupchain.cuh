@@ -191,18 +191,20 @@ __host__ __device__ inline GcLayout gc_layout(int W) {
   return l;
 }
 
+constexpr int kGcMaxSteps = 128;          // steps per launch: their coefficients travel as kernel parameters
+
 struct GcParams {
   int R, cfg, W, L, C, T, t_hi, t_lo, rows, sample_last;   // rows: kernel rows (groups x 16)
   float cfg_scale;
   const CUtensorMap* maps;     // [2 L]: W1_k, W2_k in boxes of 128 rows
   const float4* mods; int nq;  // products of the chunk, nq row quads per weight row
   const float *c1, *bsh, *bsc, *bg, *b1, *b2, *bfsh, *bfsc;   // block 0; c1_k | c2_k (FOLD) are 2 W floats a block, the others 5 W apart
-  const float* sched;          // a[T], b[T], sigma[T]
   const float *win, *bin, *wout_t, *bout;
   const float *x_T, *eps;
   float *x, *x0, *mu1, *x1, *traj_x, *traj_mu;
   int* err;
   int* status;
+  float ca[kGcMaxSteps], cb[kGcMaxSteps], sigma[kGcMaxSteps];   // index t - t_lo
 };
 
 // Shared memory of this CTA -> the same or another CTA of the cluster, completion counted in bytes on a barrier there.
@@ -541,7 +543,7 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
         }
       }
       // ---- output projection of (LN(h)(1 + scale_f) + shift_f): this CTA's columns' part, to every CTA
-      const float sa = p.sched[t - 1], sb = p.sched[T + t - 1], sg = p.sched[2 * T + t - 1];
+      const float sa = p.ca[t - p.t_lo], sb = p.cb[t - p.t_lo], sg = p.sigma[t - p.t_lo];
       float noise = 0.0f;
       const int q = et >> 4, e = et & 15, tok = tok0 + q;                 // this thread's entry of the state
       const bool mine = et < per * kCPad && tok < p.R && e < p.C;
