@@ -1030,8 +1030,20 @@ int accept_scan_lv(csd_ctx* ctx, cudaStream_t st, int B, int gamma, int C, const
                       u, logratio, log_sigma_rows, n_accept, mask);
 }
 
+// The word through which the blocks of a resampling launch count the sequences that reached the cap, or null, with cap_hits
+// zeroed, where launches of this context may run side by side: a capturing stream (the graph's launches run whenever and
+// wherever the caller says), the per-thread stream handle (one stream for every thread).
+int cap_hits_tally(csd_ctx* ctx, cudaStream_t st, int32_t* cap_hits, unsigned long long** tally) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  CSD_CUDA(ctx, cudaStreamIsCapturing(st, &capture));
+  *tally = capture == cudaStreamCaptureStatusNone && st != cudaStreamPerThread ? ctx->tally() : nullptr;
+  if (!*tally) CSD_CUDA(ctx, cudaMemsetAsync(cap_hits, 0, sizeof(int32_t), st));
+  return CSD_OK;
+}
+
 template <bool LV>
-int launch_resample(csd_ctx* ctx, cudaStream_t st, const ResampleParams& p) {
+int launch_resample(csd_ctx* ctx, cudaStream_t st, ResampleParams& p) {
+  if (int rc = cap_hits_tally(ctx, st, p.cap_hits, &p.tally)) return rc;
   return launch_short(ctx, st, resample_kernel<LV>, (p.B + 3) / 4, 128, 0, p);
 }
 
@@ -1041,7 +1053,7 @@ int resample_lv(csd_ctx* ctx, cudaStream_t st, int B, int gamma, int C, int cap,
   ResampleParams p{};
   p.B = B; p.gamma = gamma; p.C = C; p.cap = cap; p.log_sigma_rows = log_sigma_rows; p.lv_p = lv_p; p.lv_q = lv_q;
   p.n_accept = n_accept; p.mu_p = mu_p; p.mu_q = mu_q; p.xi = xi; p.v = v; p.x_new = x_new; p.n_prop = n_prop; p.flags = flags;
-  p.cap_hits = cap_hits; p.tally = ctx->tally();
+  p.cap_hits = cap_hits;
   return launch_resample<true>(ctx, st, p);
 }
 
@@ -1068,7 +1080,7 @@ int resample(csd_ctx* ctx, cudaStream_t st, int B, int gamma, int C, int cap, do
   p.B = B; p.gamma = gamma; p.C = C; p.cap = cap; p.log_sigma = static_cast<float>(log_sigma); p.sp1 = sp1; p.sq1 = sq1;
   p.log_sp1 = static_cast<float>(std::log(static_cast<double>(sp1))); p.log_sq1 = static_cast<float>(std::log(static_cast<double>(sq1)));
   p.n_accept = n_accept; p.mu_p = mu_p; p.mu_q = mu_q; p.xi = xi; p.v = v; p.x_new = x_new; p.n_prop = n_prop; p.flags = flags;
-  p.cap_hits = cap_hits; p.tally = ctx->tally();
+  p.cap_hits = cap_hits;
   return launch_resample<false>(ctx, st, p);
 }
 
@@ -2138,7 +2150,8 @@ int csd_gmm_resample(csd_ctx* ctx, int B, int gamma, int C, int cap, const csd_g
   if (cap < 1) return fail(ctx, CSD_ERR_INVALID_ARG, "cap = %d must be >= 1", cap);
   if (!n_accept || !w || !xi || !v || !x_new || !n_prop || !flags || !cap_hits) return fail(ctx, CSD_ERR_INVALID_ARG, "null array argument");
   CSD_DEVICE(ctx);
-  GmmResampleParams r{B, gamma, C, cap, gmm_view(q), gmm_view(p), n_accept, w, xi, v, x_new, n_prop, flags, cap_hits, ctx->tally()};
+  GmmResampleParams r{B, gamma, C, cap, gmm_view(q), gmm_view(p), n_accept, w, xi, v, x_new, n_prop, flags, cap_hits, nullptr};
+  if ((rc = cap_hits_tally(ctx, ctx->stream, cap_hits, &r.tally))) return rc;
   const size_t smem = gmm_resample_smem_floats(q->K, p->K, C) * 4;
   const bool fits = smem <= 48 * 1024;
   auto kern = C <= 16 ? (fits ? gmm_resample_kernel<16, true> : gmm_resample_kernel<16, false>)
