@@ -145,7 +145,11 @@ int64_t csd_launch_count(const csd_ctx *ctx);
  *                       time, and a cluster of W / 128 CTAs carries each group through the steps, activations
  *                       passing through distributed shared memory.  This is the calling pattern Alg. 1 forces on
  *                       the draft model (x_i ~ q_i one position at a time).  Blocks are not folded: its error is that
- *                       of three kernels per block.
+ *                       of three kernels per block.  Its buffers, kept by the context per chain of a round: the
+ *                       condition vectors of all steps (T x rows x W 16-bit values) and two chunks of condition
+ *                       products, fp32, (3 L + 2) W x rows x steps, at most 512 MB each (64 tokens with guidance, T = 100,
+ *                       3 x 1024: 26 MB and 2 x 288 MB).  Where the device has less free, chunks are shorter (the same
+ *                       bits); where not even one step fits, the layer kernels run.
  *                     - Otherwise one kernel per layer, chained with programmatic dependent launch; a layer's
  *                       independent part overlaps its predecessor on otherwise idle SMs.  For 16-bit heads on
  *                       grids of one wave, blocks 2..L run as two kernels instead of three: LayerNorm is folded

@@ -75,6 +75,7 @@ struct csd_ctx {
   HostIo pc[3];    // persistent chain kernel (per chain slot): s of all steps, a', v, partials, counters, schedule
   HostIo gc[2];    // group chain kernel (per chain slot): s of all steps
   HostIo gm[2];    // its condition products: two chunks of steps
+  size_t gc_refused[2] = {SIZE_MAX, SIZE_MAX}, gm_refused[2] = {SIZE_MAX, SIZE_MAX};   // sizes that could not be had: not asked for again
   cudaStream_t aux[2] = {nullptr, nullptr};        // (per chain slot) where they are formed
   cudaEvent_t ev_prep[2] = {}, ev_mods[2][2] = {}, ev_read[2][2] = {};   // preparation done; a chunk is written / has been read
   char err[512] = {0};
@@ -457,7 +458,7 @@ int gchain_clusters_of(const csd_ctx* ctx, int W) {
 int gchain_clusters(const csd_ctx* ctx, int dtype, int W) {
   return dtype == CSD_F16 ? gchain_clusters_of<__half, 0>(ctx, W) : gchain_clusters_of<__nv_bfloat16, 1>(ctx, W);
 }
-constexpr size_t kGcChunkBytes = size_t(512) << 20;   // condition products of one chunk of steps
+constexpr size_t kGcChunkBytes = size_t(512) << 20;   // most bytes of condition products of one chunk of steps
 
 // One head's denoising chain for R token rows on stream `st` with workspace slot `slot`:
 // begin() enqueues the per-call work (timestep embedding, condition projection, first boundary
@@ -469,6 +470,7 @@ struct Chain {
   int Rh = 0, W = 0, L = 0, T = 0, tn = kTileN;
   bool gck = false, gfold = false;   // the whole chain runs in the group chain kernel (groupchain.cuh), in its folded form
   bool pck = false;       // the whole chain runs in the persistent chain kernel (pchain.cuh)
+  int gc_rows = 0, gc_most = 0;      // its rows (groups x 16) and the most steps of a chunk
   int fcg = 0;            // fp32 head: the whole chain runs in the fp32 chain kernel with groups of this many rows (f32chain.cuh)
   bool fold = false;      // blocks 1.. run as two kernels (fold.cuh) instead of three
   CUtensorMap tm_ap{};
@@ -591,9 +593,11 @@ struct Chain {
     gck = tc && (ctx->chain_mode == CSD_CHAIN_LAYERS || ctx->chain_mode == CSD_CHAIN_SMALL_BATCH) && hd->gc_ready &&
           slot != 2 && !batch_Rin && !lv_min && !ctx->prof_on &&
           (R + (cfg ? 7 : 15)) / (cfg ? 8 : 16) <= gchain_clusters(ctx, d.dtype, W);
-    if (gck) { fold = false; pair = false; }
     // Its folded form is a quarter faster a layer and less precise: only in the mode that says so, up to the rows that it names
     gfold = gck && ctx->chain_mode == CSD_CHAIN_SMALL_BATCH && Rh <= 128 && hd->gf_ready;
+    int rc = CSD_OK;
+    if (gck && (rc = reserve_group_chain())) return rc;
+    if (gck) { fold = false; pair = false; }
     // One wave of 128 x 128 tiles per layer and W = 1024: one persistent kernel per chain (pchain.cuh).  Row blocks are
     // paired: an odd number is rounded up with a block of rows that belong to no token.
     {
@@ -607,7 +611,7 @@ struct Chain {
     // fp32 heads: one persistent kernel per chain, except where a row's bits have to be those of a batched pass
     fcg = !tc && ctx->chain_mode != CSD_CHAIN_LAYERS_PLAIN && !batch_Rin && !ctx->prof_on ? fc_rows(ctx, d, R, cfg, chains) : 0;
     ChainWs& ws = ctx->ws[slot];
-    int rc = batch_Rin ? ensure_ws(ctx, ws, d, ws_steps * batch_Rin * (cfg ? 2 : 1), ws_steps * batch_Rin, Ts)
+    rc = batch_Rin ? ensure_ws(ctx, ws, d, ws_steps * batch_Rin * (cfg ? 2 : 1), ws_steps * batch_Rin, Ts)
                        : ensure_ws(ctx, ws, d, Rh, R, Ts);
     if (rc) return rc;
     if (fcg) return launch_f32_chain();
@@ -810,21 +814,38 @@ struct Chain {
     return CSD_OK;
   }
 
+  // Weight rows of the condition products, and the bytes of a chunk of steps of them.
+  size_t gc_wrows() const { return static_cast<size_t>((gfold ? 4 : 3) * L + 2) * W; }
+  size_t gc_chunk_bytes(int steps) const { return gc_wrows() * ((static_cast<size_t>(steps) * gc_rows + 255) / 256) * 256 * 4; }
+
+  // Buffers of the group chain kernel.  Shorter chunks cost a launch each and change no bit, so a chunk is halved until its two
+  // buffers can be had; where one step does not fit the chain falls back to the layer kernels (gck), which need none of it.
+  int reserve_group_chain() {
+    gc_rows = (R + (cfg ? 7 : 15)) / (cfg ? 8 : 16) * kGcRows;
+    auto have = [&](HostIo& io, size_t& refused, size_t need, const char* what) {
+      if (need <= io.cap) return static_cast<int>(CSD_OK);
+      const int rc = need < refused ? ensure_side(ctx, io, need, what) : static_cast<int>(CSD_ERR_WORKSPACE);
+      if (rc == CSD_ERR_WORKSPACE && need < refused) refused = need;
+      return rc;
+    };
+    int rc = have(ctx->gc[slot], ctx->gc_refused[slot], static_cast<size_t>(Ts) * gc_rows * W * 2, "the condition vectors of all steps");
+    gc_most = Ts < kGcMaxSteps ? Ts : kGcMaxSteps;
+    while (gc_most > 1 && gc_chunk_bytes(gc_most) > kGcChunkBytes) gc_most = (gc_most + 1) / 2;
+    if (!rc)
+      while ((rc = have(ctx->gm[slot], ctx->gm_refused[slot], 2 * gc_chunk_bytes(gc_most), "the condition products")) == CSD_ERR_WORKSPACE && gc_most > 1)
+        gc_most = (gc_most + 1) / 2;
+    if (rc == CSD_ERR_WORKSPACE) { gck = gfold = false; ctx->err[0] = 0; rc = CSD_OK; }
+    return rc;
+  }
+
   // The group chain kernel: s of every step in its row order, then chunk by chunk the condition products (on the slot's
   // own stream, ahead of the chain) and the chain.
   int launch_group_chain() {
     const csd_head_desc& d = hd->d;
     ChainWs& ws = ctx->ws[slot];
-    const int per = cfg ? 8 : 16, groups = (R + per - 1) / per, rows = groups * kGcRows, cl = W / 128;
-    int rc = ensure_side(ctx, ctx->gc[slot], static_cast<size_t>(Ts) * rows * W * 2, "the condition vectors of all steps");
-    if (rc) return rc;
-    // Steps per chunk: a first chunk of a tile's width of rows, because nothing overlaps its products; then twice as many
-    // each time, as far as the buffers go.
-    const size_t wrows = static_cast<size_t>((gfold ? 4 : 3) * L + 2) * W;
-    auto chunk_bytes = [&](int steps) { return wrows * ((static_cast<size_t>(steps) * rows + 255) / 256) * 256 * 4; };
-    int most = Ts < kGcMaxSteps ? Ts : kGcMaxSteps;
-    while (most > 1 && chunk_bytes(most) > kGcChunkBytes) most = (most + 1) / 2;
-    if ((rc = ensure_side(ctx, ctx->gm[slot], 2 * chunk_bytes(most), "the condition products"))) return rc;
+    const int rows = gc_rows, groups = rows / kGcRows, cl = W / 128, most = gc_most;
+    const size_t wrows = gc_wrows();
+    int rc;
     void* const s_all = ctx->gc[slot].base;
     CUtensorMap tm_s{};
     if ((rc = make_tmap(ctx, &tm_s, d.dtype, s_all, static_cast<uint64_t>(Ts) * rows, W, W, kTileM))) return rc;
@@ -847,12 +868,14 @@ struct Chain {
     at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t lc{};
     lc.attrs = at; lc.numAttrs = 1;
+    // Steps per chunk: a first chunk of a tile's width of rows, because nothing overlaps its products; then twice as many
+    // each time, as far as the buffers go.
     int n = (256 + rows - 1) / rows;
     for (int t_hi = Ts, c = 0; t_hi >= 1; ++c, n *= 2) {
       if (n > most) n = most;
       if (n > t_hi) n = t_hi;
       const int t_lo = t_hi - n + 1, buf = c & 1;
-      float4* mods = reinterpret_cast<float4*>(static_cast<char*>(ctx->gm[slot].base) + buf * chunk_bytes(most));
+      float4* mods = reinterpret_cast<float4*>(static_cast<char*>(ctx->gm[slot].base) + buf * gc_chunk_bytes(most));
       MgParams m{};
       m.nkb = W / kBlockK; m.tiles_n = (n * rows + 255) / 256; m.units = m.tiles_n * static_cast<int>(wrows / 256);
       m.run = gfold ? static_cast<int>(wrows / 256) : 3 * W / 256; m.stride = 5 * W;   // plain: a block's layers lie between
