@@ -111,13 +111,12 @@ struct csd_head {
   std::vector<CUtensorMap> Wgs, Wf;
   std::vector<CUtensorMap> Wgs_half, Wf_half;   // the same matrices in 128-row boxes: what one CTA of a pair loads
   std::vector<float*> c1, c2;   // first MLP layer with 256-row boxes (W a multiple of 256)
-  // group chain kernel (groupchain.cuh): the dependent layers' maps W1_k, W2_k (device table, boxes of 128 rows) and the matrix
-  // multiplied by s: all blocks' rows where they lie (Wss_0 to Wfss), or its own one for the folded form: scale_0 | per block
-  // W1_k Wscale_k, W1_k Wshift_k, gate_k, scale_{k+1} | final shift, scale
-  bool gc_ready = false, gf_ready = false;
+  // group chain kernel (groupchain.cuh): the dependent layers' maps W1_k, W2_k (device table, boxes of 128 rows); the matrices
+  // multiplied by s where they lie (all blocks' rows Wss_0 .. Wfss; xblob), and which tiles of 256 of their rows each form takes
+  bool gc_ready = false;
   CUtensorMap* d_gc_maps = nullptr;
-  void* mblob = nullptr;
-  CUtensorMap Wrows{}, Wm{};
+  CUtensorMap Wrows{}, Wx{};
+  int* d_gc_rows = nullptr;     // plain form, then folded form: first rows (~row: of xblob)
   // persistent chain kernel (pchain.cuh): per phase the early and the dependent weight maps; per phase three bias rows
   bool pc_ready = false;
   CUtensorMap* d_pc_maps = nullptr;
@@ -594,7 +593,7 @@ struct Chain {
           slot != 2 && !batch_Rin && !lv_min && !ctx->prof_on &&
           (R + (cfg ? 7 : 15)) / (cfg ? 8 : 16) <= gchain_clusters(ctx, d.dtype, W);
     // Its folded form is a quarter faster a layer and less precise: only in the mode that says so, up to the rows that it names
-    gfold = gck && ctx->chain_mode == CSD_CHAIN_SMALL_BATCH && Rh <= 128 && hd->gf_ready;
+    gfold = gck && ctx->chain_mode == CSD_CHAIN_SMALL_BATCH && Rh <= 128;
     int rc = CSD_OK;
     if (gck && (rc = reserve_group_chain())) return rc;
     if (gck) { fold = false; pair = false; }
@@ -815,7 +814,7 @@ struct Chain {
   }
 
   // Weight rows of the condition products, and the bytes of a chunk of steps of them.
-  size_t gc_wrows() const { return static_cast<size_t>((gfold ? 4 : 3) * L + 2) * W; }
+  size_t gc_wrows() const { return static_cast<size_t>(gfold ? 4 * L + 3 : 3 * L + 2) * W; }
   size_t gc_chunk_bytes(int steps) const { return gc_wrows() * ((static_cast<size_t>(steps) * gc_rows + 255) / 256) * 256 * 4; }
 
   // Buffers of the group chain kernel.  Shorter chunks cost a launch each and change no bit, so a chunk is halved until its two
@@ -878,7 +877,7 @@ struct Chain {
       float4* mods = reinterpret_cast<float4*>(static_cast<char*>(ctx->gm[slot].base) + buf * gc_chunk_bytes(most));
       MgParams m{};
       m.nkb = W / kBlockK; m.tiles_n = (n * rows + 255) / 256; m.units = m.tiles_n * static_cast<int>(wrows / 256);
-      m.run = gfold ? static_cast<int>(wrows / 256) : 3 * W / 256; m.stride = 5 * W;   // plain: a block's layers lie between
+      m.wrow = hd->d_gc_rows + (gfold ? (3 * L + 2) * W / 256 : 0);
       m.s_row0 = (t_lo - 1) * rows; m.out = mods; m.err = ctx->d_err;
       if (c >= 2) CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_read[slot][buf], 0));
       // beside a running chain the products take the SMs it leaves
@@ -887,8 +886,8 @@ struct Chain {
       if (pairs > m.units) pairs = m.units;
       lc.gridDim = dim3(static_cast<unsigned>(2 * pairs)); lc.blockDim = dim3(kMgThreads); lc.dynamicSmemBytes = kMgSmemBytes; lc.stream = gst;
       at[0].val.clusterDim.x = 2;
-      if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<0>, gfold ? hd->Wm : hd->Wrows, tm_s, m));
-      else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<1>, gfold ? hd->Wm : hd->Wrows, tm_s, m));
+      if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<0>, hd->Wrows, hd->Wx, tm_s, m));
+      else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<1>, hd->Wrows, hd->Wx, tm_s, m));
       CSD_CUDA(ctx, cudaEventRecord(ctx->ev_mods[slot][buf], gst));
       CSD_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_mods[slot][buf], 0));
       p.t_hi = t_hi; p.t_lo = t_lo; p.mods = mods; p.nq = m.tiles_n * 64;
@@ -1512,7 +1511,6 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
       }
       if (!rc) rc = make_tmap(ctx, &tm.Wfss, d.dtype, h->Wfss, 2 * W, W, W, 2 * tn);
     }
-    std::vector<float> ms;    // the matrix multiplied by s for the group chain kernel
     if (!rc && (folded || gck)) {
       // xblob: Wgs_0 .. Wgs_{L-2} | Wf_1 .. Wf_{L-1} | Wf_0 (where block 0 is folded too), each [2 W, W] in operand format
       const size_t per = 2 * W * W, nx = (2 * (L - 1) + (gck ? 1 : 0)) * per;
@@ -1521,16 +1519,6 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
       try { xs.resize(nx); } catch (...) { return bail(CSD_ERR_WORKSPACE, "out of host memory"); }
       float *dA = nullptr, *dB = nullptr, *dC = nullptr;
       std::vector<float> f1(W * W), f2(W * W);
-      auto mput = [&](const float* src, size_t sec) { memcpy(&ms[sec * W * W], src, W * W * 4); };
-      if (gck) {
-        try { ms.resize((4 * L + 2) * W * W); } catch (...) { return bail(CSD_ERR_WORKSPACE, "out of host memory"); }
-        mput(w->Wada + W * W, 0);
-        for (size_t k = 0; k < L; ++k) {
-          mput(w->Wada + k * 3 * W * W + 2 * W * W, 3 + 4 * k);
-          if (k + 1 < L) mput(w->Wada + (k + 1) * 3 * W * W + W * W, 4 + 4 * k);
-        }
-        mput(w->Wfada, 4 * L); mput(w->Wfada + W * W, 4 * L + 1);
-      }
       bool okx = cudaMalloc(&dA, W * W * 4) == cudaSuccess && cudaMalloc(&dB, W * W * 4) == cudaSuccess && cudaMalloc(&dC, W * W * 4) == cudaSuccess;
       for (size_t k = 0; k + 1 < L && okx; ++k)     // gate of block k | scale of block k + 1
         interleave(w->Wada + k * 3 * W * W + 2 * W * W, w->Wada + (k + 1) * 3 * W * W + W * W, &xs[k * per]);
@@ -1545,7 +1533,6 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
         if (okx) square_matmul_kernel<<<grid, 256>>>(dA, dB, dC, static_cast<int>(W));
         okx = okx && cudaMemcpy(f2.data(), dC, W * W * 4, cudaMemcpyDeviceToHost) == cudaSuccess;
         if (okx) interleave(f1.data(), f2.data(), &xs[wf_slot(k) * per]);
-        if (okx && gck) { mput(f1.data(), 1 + 4 * k); mput(f2.data(), 2 + 4 * k); }
       }
       if (dA) cudaFree(dA);
       if (dB) cudaFree(dB);
@@ -1573,17 +1560,20 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
       // tables of the group chain kernel
       std::vector<CUtensorMap> maps;
       for (size_t k = 0; k < L; ++k) { maps.push_back(h->tm[1].W1[k]); maps.push_back(h->tm[1].W2[k]); }
-      std::vector<uint16_t> mb;
-      try { mb.resize(ms.size()); } catch (...) { return bail(CSD_ERR_WORKSPACE, "out of host memory"); }
-      if (d.dtype == CSD_BF16) { for (size_t i = 0; i < ms.size(); ++i) mb[i] = f32_to_bf16_bits(ms[i]); }
-      else { for (size_t i = 0; i < ms.size(); ++i) { const __half hv = __float2half_rn(ms[i]); memcpy(&mb[i], &hv, 2); } }
-      if (cudaMalloc(&h->mblob, mb.size() * 2) != cudaSuccess ||
+      std::vector<int> rows;
+      auto tiles = [&](size_t row, size_t n) { for (size_t r = 0; r < n; r += 256) rows.push_back(static_cast<int>(row + r)); };
+      for (size_t k = 0; k < L; ++k) tiles(5 * k * W, 3 * W);
+      tiles(5 * L * W, 2 * W);
+      const size_t nx = (4 * L - 2) * W;                     // rows of xblob
+      for (size_t r = 0; r < nx; r += 256) rows.push_back(~static_cast<int>(r));
+      tiles(0, 2 * W); tiles((5 * (L - 1) + 2) * W, W); tiles(5 * L * W, 2 * W);
+      if (cudaMalloc(&h->d_gc_rows, rows.size() * sizeof(int)) != cudaSuccess ||
           cudaMalloc(&h->d_gc_maps, maps.size() * sizeof(CUtensorMap)) != cudaSuccess) { cudaGetLastError(); return bail(CSD_ERR_WORKSPACE, "cannot allocate device memory for the group-chain tables"); }
-      if (cudaMemcpy(h->mblob, mb.data(), mb.size() * 2, cudaMemcpyHostToDevice) != cudaSuccess ||
+      if (cudaMemcpy(h->d_gc_rows, rows.data(), rows.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
           cudaMemcpy(h->d_gc_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess) return bail(CSD_ERR_CUDA, "group-chain table upload failed");
-      if ((rc = make_tmap(ctx, &h->Wm, d.dtype, h->mblob, (4 * L + 2) * W, W, W, kTileM)) ||
-          (rc = make_tmap(ctx, &h->Wrows, d.dtype, h->Wss[0], (5 * L + 2) * W, W, W, kTileM))) { csd_head_destroy(h); return rc; }
-      h->gc_ready = h->gf_ready = true;
+      if ((rc = make_tmap(ctx, &h->Wrows, d.dtype, h->Wss[0], (5 * L + 2) * W, W, W, kTileM)) ||
+          (rc = make_tmap(ctx, &h->Wx, d.dtype, h->xblob, nx, W, W, kTileM))) { csd_head_destroy(h); return rc; }
+      h->gc_ready = true;
     }
     if (gck && W / kTileN == static_cast<size_t>(kPcColTiles)) {
       // tables of the persistent chain kernel: phases B, (W1_k, GATE_k) for every block, F
@@ -1623,7 +1613,7 @@ int csd_head_destroy(csd_head* h) {
   if (h->d_pc_maps) cudaFree(h->d_pc_maps);
   if (h->d_pc_bias) cudaFree(h->d_pc_bias);
   if (h->d_gc_maps) cudaFree(h->d_gc_maps);
-  if (h->mblob) cudaFree(h->mblob);
+  if (h->d_gc_rows) cudaFree(h->d_gc_rows);
   cudaGetLastError();
   delete h;
   return CSD_OK;
