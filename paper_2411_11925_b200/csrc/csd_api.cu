@@ -376,6 +376,21 @@ bool fc_ready(const csd_ctx* ctx, const csd_head_desc& d) {
   return k == 1 && fc_layout(G, d.W, d.var_out ? kCPad2 : kCPad).total * 4 <= 227 * 1024;
 }
 
+// Whether the chain kernel is the faster one for Rh head rows.  Its clusters take turns, about 15 at a time, and every group reads
+// all the weights for its 16, 8 or 4 rows (W up to 896, 1664, 3072); the layer kernels' 32 x 128 tiles share them among 32 and cost
+// the less per tile the more tiles there are.  ms a step of one block, chain / layer kernels, by head rows (tiles):
+//   W =  512: 2048 (256) 0.61 / 0.63, 4096 (512) 1.20 / 1.26, 8192 (1024) 2.34 / 2.12
+//   W =  768: 1024 (192) 0.62 / 0.91, 2048 (384) 1.11 / 1.07, 4096 (768) 2.20 / 2.17, 8192 (1536) 4.27 / 3.95
+//   W = 1024: 1024 (256) 0.99 / 1.20, 2048 (512) 1.96 / 2.41, 4096 (1024) 3.80 / 3.91, 8192 (2048) 7.51 / 6.57
+//   W = 1280: 1024 (320) 1.50 / 1.86, 2048 (640) 2.99 / 3.33, 4096 (1280) 5.82 / 5.09
+//   W = 1536:  512 (192) 1.31 / 2.06, 1024 (384) 2.33 / 2.30, 2048 (768) 4.64 / 4.19
+//   W = 2048:  256 (128) 1.41 / 2.81,  512 (256) 2.53 / 2.87, 1024 (512) 5.06 / 4.59
+//   W = 3072:  256 (192) 2.99 / 4.20,  512 (384) 5.33 / 4.49
+// The line: 640 tiles, 256 where a group has four rows only.
+bool fc_pays(const csd_ctx* ctx, const csd_head_desc& d, int Rh) {
+  return (Rh + 31) / 32 * (d.W / 128) <= (fc_ready<8>(ctx, d) ? 640 : 256);
+}
+
 // Rows per group: the fewest that keep all groups of the chains side by side resident at once (a cluster of 8 SMs each,
 // about one cluster per GPC stays unused), where a step costs the least time; with more groups than that, the most rows
 // that fit, because every group reads all the weights.  0: none fits (W beyond about 4000).  The choice changes no bit.
@@ -608,7 +623,7 @@ struct Chain {
       if (pck) { fold = false; pair = false; }
     }
     // fp32 heads: one persistent kernel per chain, except where a row's bits have to be those of a batched pass
-    fcg = !tc && ctx->chain_mode != CSD_CHAIN_LAYERS_PLAIN && !batch_Rin && !ctx->prof_on ? fc_rows(ctx, d, R, cfg, chains) : 0;
+    fcg = !tc && ctx->chain_mode != CSD_CHAIN_LAYERS_PLAIN && !batch_Rin && !ctx->prof_on && fc_pays(ctx, d, Rh) ? fc_rows(ctx, d, R, cfg, chains) : 0;
     ChainWs& ws = ctx->ws[slot];
     rc = batch_Rin ? ensure_ws(ctx, ws, d, ws_steps * batch_Rin * (cfg ? 2 : 1), ws_steps * batch_Rin, Ts)
                        : ensure_ws(ctx, ws, d, Rh, R, Ts);
