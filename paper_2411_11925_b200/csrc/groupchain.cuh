@@ -183,7 +183,7 @@ __host__ __device__ inline GcLayout gc_layout(int W) {
   l.stats = take(W / 32 * kGcRows * 8);   // [32-column group][row] (mean, M2)
   l.part = take(kGcRows * kCPad * 4);     // the outgoing output-projection partial
   l.misc = take(1024 + 512 + 512);        // x [16 tokens][16], (mean, rstd) per epilogue warp [8][8], barriers
-  l.stages = (226 * 1024 - o) / 16384;    // all that is left streams weights: 12, 9, 6 stages
+  l.stages = (226 * 1024 - o) / 16384;    // all that is left streams weights: 9, 9, 6 stages at W = 512, 1024, 1536
   l.stages = (l.stages > kGcMaxStages ? kGcMaxStages : l.stages) / kGcMma * kGcMma;
   l.ring = take(0);
   o = (o + 1023) / 1024 * 1024;
