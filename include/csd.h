@@ -145,14 +145,22 @@ int64_t csd_launch_count(const csd_ctx *ctx);
  *                       time, and a cluster of W / 128 CTAs carries each group through the steps, activations
  *                       passing through distributed shared memory.  This is the calling pattern Alg. 1 forces on
  *                       the draft model (x_i ~ q_i one position at a time).  Blocks are not folded: its error is that
- *                       of three kernels per block.
+ *                       of three kernels per block.  Its buffers, kept by the context per chain of a round: the
+ *                       condition vectors of all steps (T x rows x W 16-bit values) and two chunks of condition
+ *                       products, fp32, (3 L + 2) W x rows x steps, at most 512 MB each (64 tokens with guidance, T = 100,
+ *                       3 x 1024: 26 MB and 2 x 288 MB).  Where the device has less free, chunks are shorter (the same
+ *                       bits); where not even one step fits, the layer kernels run.
+ *                     - A chain of an fp32 head with W up to 3072 runs as one persistent kernel: a cluster of 8 CTAs carries 4
+ *                       to 16 head rows through all layers and steps.  Up to 640 tiles of 32 head rows x 128 columns (256
+ *                       from W = 1792 on; some less with var_out = 1); the layer kernels are faster above.  It needs no
+ *                       buffers of its own, and runs in CSD_CHAIN_LAYER_KERNELS and csd_draft_denoise_static as well.
  *                     - Otherwise one kernel per layer, chained with programmatic dependent launch; a layer's
  *                       independent part overlaps its predecessor on otherwise idle SMs.  For 16-bit heads on
  *                       grids of one wave, blocks 2..L run as two kernels instead of three: LayerNorm is folded
  *                       into the first layer's epilogue.
  *                     Folding is algebraically the same function, rounded differently: the layouts agree within
  *                     the parity tolerance, not bit for bit, and which one runs depends on the call's row count.
- *   CSD_CHAIN_LAYER_KERNELS: as CSD_CHAIN_LAYERS without the chain kernels (layer kernels, folded where
+ *   CSD_CHAIN_LAYER_KERNELS: as CSD_CHAIN_LAYERS without the chain kernels of 16-bit heads (layer kernels, folded where
  *                     that applies): what csd_draft_denoise_static always runs.
  *   CSD_CHAIN_LAYERS_PLAIN: layer kernels without the folded blocks (three kernels per block everywhere); a
  *                     row's bits then do not depend on how many rows the call has.
@@ -215,7 +223,7 @@ int csd_draft_denoise(csd_ctx *ctx, const csd_head *head, const csd_schedule *sc
                       float *x0, float *mu1, float *x1);
 
 /* csd_draft_denoise without any allocation (the paper has no counterpart: this is a deployment
- * variant of the call above with the same arguments; it runs the layer kernels, so its results are
+ * variant of the call above with the same arguments; it runs the kernels of CSD_CHAIN_LAYER_KERNELS, so its results are
  * bit-identical to csd_draft_denoise in the modes CSD_CHAIN_LAYER_KERNELS and CSD_CHAIN_LAYERS_PLAIN, and
  * in the default mode whenever that call takes neither the persistent nor the group chain kernel,
  * whose buffers grow with T and cannot live in a fixed array; otherwise the two agree within the parity tolerance).

@@ -73,8 +73,9 @@ struct csd_ctx {
   HostIo bn;       // csd_bonus_token: samples of every sequence before the selection
   HostIo sp;       // csd_verify_single_path: schedule constants, mu^p of one pass, running log-ratio
   HostIo pc[3];    // persistent chain kernel (per chain slot): s of all steps, a', v, partials, counters, schedule
-  HostIo gc[2];    // group chain kernel (per chain slot): s of all steps, schedule
+  HostIo gc[2];    // group chain kernel (per chain slot): s of all steps
   HostIo gm[2];    // its condition products: two chunks of steps
+  size_t gc_refused[2] = {SIZE_MAX, SIZE_MAX}, gm_refused[2] = {SIZE_MAX, SIZE_MAX};   // sizes that could not be had: not asked for again
   cudaStream_t aux[2] = {nullptr, nullptr};        // (per chain slot) where they are formed
   cudaEvent_t ev_prep[2] = {}, ev_mods[2][2] = {}, ev_read[2][2] = {};   // preparation done; a chunk is written / has been read
   char err[512] = {0};
@@ -110,13 +111,12 @@ struct csd_head {
   std::vector<CUtensorMap> Wgs, Wf;
   std::vector<CUtensorMap> Wgs_half, Wf_half;   // the same matrices in 128-row boxes: what one CTA of a pair loads
   std::vector<float*> c1, c2;   // first MLP layer with 256-row boxes (W a multiple of 256)
-  // group chain kernel (groupchain.cuh): the dependent layers' maps W1_k, W2_k (device table, boxes of 128 rows) and the matrix
-  // multiplied by s: all blocks' rows where they lie (Wss_0 to Wfss), or its own one for the folded form: scale_0 | per block
-  // W1_k Wscale_k, W1_k Wshift_k, gate_k, scale_{k+1} | final shift, scale
-  bool gc_ready = false, gf_ready = false;
+  // group chain kernel (groupchain.cuh): the dependent layers' maps W1_k, W2_k (device table, boxes of 128 rows); the matrices
+  // multiplied by s where they lie (all blocks' rows Wss_0 .. Wfss; xblob), and which tiles of 256 of their rows each form takes
+  bool gc_ready = false;
   CUtensorMap* d_gc_maps = nullptr;
-  void* mblob = nullptr;
-  CUtensorMap Wrows{}, Wm{};
+  CUtensorMap Wrows{}, Wx{};
+  int* d_gc_rows = nullptr;     // plain form, then folded form: first rows (~row: of xblob)
   // persistent chain kernel (pchain.cuh): per phase the early and the dependent weight maps; per phase three bias rows
   bool pc_ready = false;
   CUtensorMap* d_pc_maps = nullptr;
@@ -376,6 +376,21 @@ bool fc_ready(const csd_ctx* ctx, const csd_head_desc& d) {
   return k == 1 && fc_layout(G, d.W, d.var_out ? kCPad2 : kCPad).total * 4 <= 227 * 1024;
 }
 
+// Whether the chain kernel is the faster one for Rh head rows.  Its clusters take turns, about 15 at a time, and every group reads
+// all the weights for its 16, 8 or 4 rows (W up to 896, 1664, 3072); the layer kernels' 32 x 128 tiles share them among 32 and cost
+// the less per tile the more tiles there are.  ms a step of one block, chain / layer kernels, by head rows (tiles):
+//   W =  512: 2048 (256) 0.61 / 0.63, 4096 (512) 1.20 / 1.26, 8192 (1024) 2.34 / 2.12
+//   W =  768: 1024 (192) 0.62 / 0.91, 2048 (384) 1.11 / 1.07, 4096 (768) 2.20 / 2.17, 8192 (1536) 4.27 / 3.95
+//   W = 1024: 1024 (256) 0.99 / 1.20, 2048 (512) 1.96 / 2.41, 4096 (1024) 3.80 / 3.91, 8192 (2048) 7.51 / 6.57
+//   W = 1280: 1024 (320) 1.50 / 1.86, 2048 (640) 2.99 / 3.33, 4096 (1280) 5.82 / 5.09
+//   W = 1536:  512 (192) 1.31 / 2.06, 1024 (384) 2.33 / 2.30, 2048 (768) 4.64 / 4.19
+//   W = 2048:  256 (128) 1.41 / 2.81,  512 (256) 2.53 / 2.87, 1024 (512) 5.06 / 4.59
+//   W = 3072:  256 (192) 2.99 / 4.20,  512 (384) 5.33 / 4.49
+// The line: 640 tiles, 256 where a group has four rows only.
+bool fc_pays(const csd_ctx* ctx, const csd_head_desc& d, int Rh) {
+  return (Rh + 31) / 32 * (d.W / 128) <= (fc_ready<8>(ctx, d) ? 640 : 256);
+}
+
 // Rows per group: the fewest that keep all groups of the chains side by side resident at once (a cluster of 8 SMs each,
 // about one cluster per GPC stays unused), where a step costs the least time; with more groups than that, the most rows
 // that fit, because every group reads all the weights.  0: none fits (W beyond about 4000).  The choice changes no bit.
@@ -457,7 +472,7 @@ int gchain_clusters_of(const csd_ctx* ctx, int W) {
 int gchain_clusters(const csd_ctx* ctx, int dtype, int W) {
   return dtype == CSD_F16 ? gchain_clusters_of<__half, 0>(ctx, W) : gchain_clusters_of<__nv_bfloat16, 1>(ctx, W);
 }
-constexpr size_t kGcChunkBytes = size_t(512) << 20;   // condition products of one chunk of steps
+constexpr size_t kGcChunkBytes = size_t(512) << 20;   // most bytes of condition products of one chunk of steps
 
 // One head's denoising chain for R token rows on stream `st` with workspace slot `slot`:
 // begin() enqueues the per-call work (timestep embedding, condition projection, first boundary
@@ -469,6 +484,7 @@ struct Chain {
   int Rh = 0, W = 0, L = 0, T = 0, tn = kTileN;
   bool gck = false, gfold = false;   // the whole chain runs in the group chain kernel (groupchain.cuh), in its folded form
   bool pck = false;       // the whole chain runs in the persistent chain kernel (pchain.cuh)
+  int gc_rows = 0, gc_most = 0;      // its rows (groups x 16) and the most steps of a chunk
   int fcg = 0;            // fp32 head: the whole chain runs in the fp32 chain kernel with groups of this many rows (f32chain.cuh)
   bool fold = false;      // blocks 1.. run as two kernels (fold.cuh) instead of three
   CUtensorMap tm_ap{};
@@ -591,9 +607,11 @@ struct Chain {
     gck = tc && (ctx->chain_mode == CSD_CHAIN_LAYERS || ctx->chain_mode == CSD_CHAIN_SMALL_BATCH) && hd->gc_ready &&
           slot != 2 && !batch_Rin && !lv_min && !ctx->prof_on &&
           (R + (cfg ? 7 : 15)) / (cfg ? 8 : 16) <= gchain_clusters(ctx, d.dtype, W);
-    if (gck) { fold = false; pair = false; }
     // Its folded form is a quarter faster a layer and less precise: only in the mode that says so, up to the rows that it names
-    gfold = gck && ctx->chain_mode == CSD_CHAIN_SMALL_BATCH && Rh <= 128 && hd->gf_ready;
+    gfold = gck && ctx->chain_mode == CSD_CHAIN_SMALL_BATCH && Rh <= 128;
+    int rc = CSD_OK;
+    if (gck && (rc = reserve_group_chain())) return rc;
+    if (gck) { fold = false; pair = false; }
     // One wave of 128 x 128 tiles per layer and W = 1024: one persistent kernel per chain (pchain.cuh).  Row blocks are
     // paired: an odd number is rounded up with a block of rows that belong to no token.
     {
@@ -605,9 +623,9 @@ struct Chain {
       if (pck) { fold = false; pair = false; }
     }
     // fp32 heads: one persistent kernel per chain, except where a row's bits have to be those of a batched pass
-    fcg = !tc && ctx->chain_mode != CSD_CHAIN_LAYERS_PLAIN && !batch_Rin && !ctx->prof_on ? fc_rows(ctx, d, R, cfg, chains) : 0;
+    fcg = !tc && ctx->chain_mode != CSD_CHAIN_LAYERS_PLAIN && !batch_Rin && !ctx->prof_on && fc_pays(ctx, d, Rh) ? fc_rows(ctx, d, R, cfg, chains) : 0;
     ChainWs& ws = ctx->ws[slot];
-    int rc = batch_Rin ? ensure_ws(ctx, ws, d, ws_steps * batch_Rin * (cfg ? 2 : 1), ws_steps * batch_Rin, Ts)
+    rc = batch_Rin ? ensure_ws(ctx, ws, d, ws_steps * batch_Rin * (cfg ? 2 : 1), ws_steps * batch_Rin, Ts)
                        : ensure_ws(ctx, ws, d, Rh, R, Ts);
     if (rc) return rc;
     if (fcg) return launch_f32_chain();
@@ -810,35 +828,44 @@ struct Chain {
     return CSD_OK;
   }
 
+  // Weight rows of the condition products, and the bytes of a chunk of steps of them.
+  size_t gc_wrows() const { return static_cast<size_t>(gfold ? 4 * L + 3 : 3 * L + 2) * W; }
+  size_t gc_chunk_bytes(int steps) const { return gc_wrows() * ((static_cast<size_t>(steps) * gc_rows + 255) / 256) * 256 * 4; }
+
+  // Buffers of the group chain kernel.  Shorter chunks cost a launch each and change no bit, so a chunk is halved until its two
+  // buffers can be had; where one step does not fit the chain falls back to the layer kernels (gck), which need none of it.
+  int reserve_group_chain() {
+    gc_rows = (R + (cfg ? 7 : 15)) / (cfg ? 8 : 16) * kGcRows;
+    auto have = [&](HostIo& io, size_t& refused, size_t need, const char* what) {
+      if (need <= io.cap) return static_cast<int>(CSD_OK);
+      const int rc = need < refused ? ensure_side(ctx, io, need, what) : static_cast<int>(CSD_ERR_WORKSPACE);
+      if (rc == CSD_ERR_WORKSPACE && need < refused) refused = need;
+      return rc;
+    };
+    int rc = have(ctx->gc[slot], ctx->gc_refused[slot], static_cast<size_t>(Ts) * gc_rows * W * 2, "the condition vectors of all steps");
+    gc_most = Ts < kGcMaxSteps ? Ts : kGcMaxSteps;
+    while (gc_most > 1 && gc_chunk_bytes(gc_most) > kGcChunkBytes) gc_most = (gc_most + 1) / 2;
+    if (!rc)
+      while ((rc = have(ctx->gm[slot], ctx->gm_refused[slot], 2 * gc_chunk_bytes(gc_most), "the condition products")) == CSD_ERR_WORKSPACE && gc_most > 1)
+        gc_most = (gc_most + 1) / 2;
+    if (rc == CSD_ERR_WORKSPACE) { gck = gfold = false; ctx->err[0] = 0; rc = CSD_OK; }
+    return rc;
+  }
+
   // The group chain kernel: s of every step in its row order, then chunk by chunk the condition products (on the slot's
   // own stream, ahead of the chain) and the chain.
   int launch_group_chain() {
     const csd_head_desc& d = hd->d;
     ChainWs& ws = ctx->ws[slot];
-    const int per = cfg ? 8 : 16, groups = (R + per - 1) / per, rows = groups * kGcRows, cl = W / 128;
-    size_t off = 0;
-    auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 1024); return o; };
-    const size_t o_s = take(static_cast<size_t>(Ts) * rows * W * 2), o_sched = take(static_cast<size_t>(3) * Ts * 4);
-    int rc = ensure_side(ctx, ctx->gc[slot], off, "the group chain buffers");
-    if (rc) return rc;
-    // Steps per chunk: a first chunk of a tile's width of rows, because nothing overlaps its products; then twice as many
-    // each time, as far as the buffers go.
-    const size_t wrows = static_cast<size_t>((gfold ? 4 : 3) * L + 2) * W;
-    auto chunk_bytes = [&](int steps) { return wrows * ((static_cast<size_t>(steps) * rows + 255) / 256) * 256 * 4; };
-    int most = Ts;
-    while (most > 1 && chunk_bytes(most) > kGcChunkBytes) most = (most + 1) / 2;
-    if ((rc = ensure_side(ctx, ctx->gm[slot], 2 * chunk_bytes(most), "the condition products"))) return rc;
-    char* b = static_cast<char*>(ctx->gc[slot].base);
+    const int rows = gc_rows, groups = rows / kGcRows, cl = W / 128, most = gc_most;
+    const size_t wrows = gc_wrows();
+    int rc;
+    void* const s_all = ctx->gc[slot].base;
     CUtensorMap tm_s{};
-    if ((rc = make_tmap(ctx, &tm_s, d.dtype, b + o_s, static_cast<uint64_t>(Ts) * rows, W, W, kTileM))) return rc;
-    float* d_sched = reinterpret_cast<float*>(b + o_sched);
-    // pageable source: staged by the runtime before the call returns
-    std::vector<float> hs(static_cast<size_t>(3) * Ts);
-    for (int t = 0; t < Ts; ++t) { hs[t] = sc->a[t]; hs[Ts + t] = sc->b[t]; hs[2 * Ts + t] = sc->sigma[t]; }
-    CSD_CUDA(ctx, cudaMemcpyAsync(d_sched, hs.data(), hs.size() * 4, cudaMemcpyHostToDevice, st));
+    if ((rc = make_tmap(ctx, &tm_s, d.dtype, s_all, static_cast<uint64_t>(Ts) * rows, W, W, kTileM))) return rc;
     const dim3 sgrid(static_cast<unsigned>(rows), static_cast<unsigned>((Ts + kCondSteps - 1) / kCondSteps));
-    if (d.dtype == CSD_F16) cond_all_kernel<__half, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__half*>(b + o_s), R, cfg, W, rows, Ts);
-    else cond_all_kernel<__nv_bfloat16, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__nv_bfloat16*>(b + o_s), R, cfg, W, rows, Ts);
+    if (d.dtype == CSD_F16) cond_all_kernel<__half, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, static_cast<__half*>(s_all), R, cfg, W, rows, Ts);
+    else cond_all_kernel<__nv_bfloat16, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, static_cast<__nv_bfloat16*>(s_all), R, cfg, W, rows, Ts);
     ctx->launches++;
     CSD_CUDA(ctx, cudaGetLastError());
     cudaStream_t gst = ctx->aux[slot];
@@ -848,22 +875,24 @@ struct Chain {
     p.R = R; p.cfg = cfg; p.W = W; p.L = L; p.C = d.C; p.T = Ts; p.rows = rows; p.sample_last = sample_last; p.cfg_scale = cfg_scale;
     p.maps = hd->d_gc_maps; p.c1 = hd->c1[0]; p.bsh = hd->bsh[0]; p.bsc = hd->bsc[0]; p.bg = hd->bg[0]; p.b1 = hd->b1[0]; p.b2 = hd->b2[0];
     p.bfsh = hd->bfsh; p.bfsc = hd->bfsc;
-    p.sched = d_sched; p.win = hd->win; p.bin = hd->bin; p.wout_t = hd->wout_t; p.bout = hd->bout; p.x_T = x_T; p.eps = eps;
+    p.win = hd->win; p.bin = hd->bin; p.wout_t = hd->wout_t; p.bout = hd->bout; p.x_T = x_T; p.eps = eps;
     p.x = ws.x; p.x0 = x0; p.mu1 = mu1; p.x1 = x1; p.traj_x = traj_x; p.traj_mu = traj_mu; p.err = ctx->d_err; p.status = ctx->d_err + 1;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t lc{};
     lc.attrs = at; lc.numAttrs = 1;
+    // Steps per chunk: a first chunk of a tile's width of rows, because nothing overlaps its products; then twice as many
+    // each time, as far as the buffers go.
     int n = (256 + rows - 1) / rows;
     for (int t_hi = Ts, c = 0; t_hi >= 1; ++c, n *= 2) {
       if (n > most) n = most;
       if (n > t_hi) n = t_hi;
       const int t_lo = t_hi - n + 1, buf = c & 1;
-      float4* mods = reinterpret_cast<float4*>(static_cast<char*>(ctx->gm[slot].base) + buf * chunk_bytes(most));
+      float4* mods = reinterpret_cast<float4*>(static_cast<char*>(ctx->gm[slot].base) + buf * gc_chunk_bytes(most));
       MgParams m{};
       m.nkb = W / kBlockK; m.tiles_n = (n * rows + 255) / 256; m.units = m.tiles_n * static_cast<int>(wrows / 256);
-      m.run = gfold ? static_cast<int>(wrows / 256) : 3 * W / 256; m.stride = 5 * W;   // plain: a block's layers lie between
+      m.wrow = hd->d_gc_rows + (gfold ? (3 * L + 2) * W / 256 : 0);
       m.s_row0 = (t_lo - 1) * rows; m.out = mods; m.err = ctx->d_err;
       if (c >= 2) CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_read[slot][buf], 0));
       // beside a running chain the products take the SMs it leaves
@@ -872,11 +901,12 @@ struct Chain {
       if (pairs > m.units) pairs = m.units;
       lc.gridDim = dim3(static_cast<unsigned>(2 * pairs)); lc.blockDim = dim3(kMgThreads); lc.dynamicSmemBytes = kMgSmemBytes; lc.stream = gst;
       at[0].val.clusterDim.x = 2;
-      if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<0>, gfold ? hd->Wm : hd->Wrows, tm_s, m));
-      else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<1>, gfold ? hd->Wm : hd->Wrows, tm_s, m));
+      if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<0>, hd->Wrows, hd->Wx, tm_s, m));
+      else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, mods_gemm_kernel<1>, hd->Wrows, hd->Wx, tm_s, m));
       CSD_CUDA(ctx, cudaEventRecord(ctx->ev_mods[slot][buf], gst));
       CSD_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_mods[slot][buf], 0));
       p.t_hi = t_hi; p.t_lo = t_lo; p.mods = mods; p.nq = m.tiles_n * 64;
+      for (int i = 0; i < n; ++i) { p.ca[i] = sc->a[t_lo - 1 + i]; p.cb[i] = sc->b[t_lo - 1 + i]; p.sigma[i] = sc->sigma[t_lo - 1 + i]; }
       lc.gridDim = dim3(static_cast<unsigned>(groups * cl)); lc.blockDim = dim3(kGcThreads); lc.dynamicSmemBytes = gc_layout(W).total + 1024; lc.stream = st;
       at[0].val.clusterDim.x = static_cast<unsigned>(cl);
       if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, gfold ? group_chain_kernel<__half, 0, true> : group_chain_kernel<__half, 0, false>, p));
@@ -1037,8 +1067,20 @@ int accept_scan_lv(csd_ctx* ctx, cudaStream_t st, int B, int gamma, int C, const
                       u, logratio, log_sigma_rows, n_accept, mask);
 }
 
+// The word through which the blocks of a resampling launch count the sequences that reached the cap, or null, with cap_hits
+// zeroed, where launches of this context may run side by side: a capturing stream (the graph's launches run whenever and
+// wherever the caller says), the per-thread stream handle (one stream for every thread).
+int cap_hits_tally(csd_ctx* ctx, cudaStream_t st, int32_t* cap_hits, unsigned long long** tally) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  CSD_CUDA(ctx, cudaStreamIsCapturing(st, &capture));
+  *tally = capture == cudaStreamCaptureStatusNone && st != cudaStreamPerThread ? ctx->tally() : nullptr;
+  if (!*tally) CSD_CUDA(ctx, cudaMemsetAsync(cap_hits, 0, sizeof(int32_t), st));
+  return CSD_OK;
+}
+
 template <bool LV>
-int launch_resample(csd_ctx* ctx, cudaStream_t st, const ResampleParams& p) {
+int launch_resample(csd_ctx* ctx, cudaStream_t st, ResampleParams& p) {
+  if (int rc = cap_hits_tally(ctx, st, p.cap_hits, &p.tally)) return rc;
   return launch_short(ctx, st, resample_kernel<LV>, (p.B + 3) / 4, 128, 0, p);
 }
 
@@ -1048,7 +1090,7 @@ int resample_lv(csd_ctx* ctx, cudaStream_t st, int B, int gamma, int C, int cap,
   ResampleParams p{};
   p.B = B; p.gamma = gamma; p.C = C; p.cap = cap; p.log_sigma_rows = log_sigma_rows; p.lv_p = lv_p; p.lv_q = lv_q;
   p.n_accept = n_accept; p.mu_p = mu_p; p.mu_q = mu_q; p.xi = xi; p.v = v; p.x_new = x_new; p.n_prop = n_prop; p.flags = flags;
-  p.cap_hits = cap_hits; p.tally = ctx->tally();
+  p.cap_hits = cap_hits;
   return launch_resample<true>(ctx, st, p);
 }
 
@@ -1075,7 +1117,7 @@ int resample(csd_ctx* ctx, cudaStream_t st, int B, int gamma, int C, int cap, do
   p.B = B; p.gamma = gamma; p.C = C; p.cap = cap; p.log_sigma = static_cast<float>(log_sigma); p.sp1 = sp1; p.sq1 = sq1;
   p.log_sp1 = static_cast<float>(std::log(static_cast<double>(sp1))); p.log_sq1 = static_cast<float>(std::log(static_cast<double>(sq1)));
   p.n_accept = n_accept; p.mu_p = mu_p; p.mu_q = mu_q; p.xi = xi; p.v = v; p.x_new = x_new; p.n_prop = n_prop; p.flags = flags;
-  p.cap_hits = cap_hits; p.tally = ctx->tally();
+  p.cap_hits = cap_hits;
   return launch_resample<false>(ctx, st, p);
 }
 
@@ -1484,7 +1526,6 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
       }
       if (!rc) rc = make_tmap(ctx, &tm.Wfss, d.dtype, h->Wfss, 2 * W, W, W, 2 * tn);
     }
-    std::vector<float> ms;    // the matrix multiplied by s for the group chain kernel
     if (!rc && (folded || gck)) {
       // xblob: Wgs_0 .. Wgs_{L-2} | Wf_1 .. Wf_{L-1} | Wf_0 (where block 0 is folded too), each [2 W, W] in operand format
       const size_t per = 2 * W * W, nx = (2 * (L - 1) + (gck ? 1 : 0)) * per;
@@ -1493,16 +1534,6 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
       try { xs.resize(nx); } catch (...) { return bail(CSD_ERR_WORKSPACE, "out of host memory"); }
       float *dA = nullptr, *dB = nullptr, *dC = nullptr;
       std::vector<float> f1(W * W), f2(W * W);
-      auto mput = [&](const float* src, size_t sec) { memcpy(&ms[sec * W * W], src, W * W * 4); };
-      if (gck) {
-        try { ms.resize((4 * L + 2) * W * W); } catch (...) { return bail(CSD_ERR_WORKSPACE, "out of host memory"); }
-        mput(w->Wada + W * W, 0);
-        for (size_t k = 0; k < L; ++k) {
-          mput(w->Wada + k * 3 * W * W + 2 * W * W, 3 + 4 * k);
-          if (k + 1 < L) mput(w->Wada + (k + 1) * 3 * W * W + W * W, 4 + 4 * k);
-        }
-        mput(w->Wfada, 4 * L); mput(w->Wfada + W * W, 4 * L + 1);
-      }
       bool okx = cudaMalloc(&dA, W * W * 4) == cudaSuccess && cudaMalloc(&dB, W * W * 4) == cudaSuccess && cudaMalloc(&dC, W * W * 4) == cudaSuccess;
       for (size_t k = 0; k + 1 < L && okx; ++k)     // gate of block k | scale of block k + 1
         interleave(w->Wada + k * 3 * W * W + 2 * W * W, w->Wada + (k + 1) * 3 * W * W + W * W, &xs[k * per]);
@@ -1517,7 +1548,6 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
         if (okx) square_matmul_kernel<<<grid, 256>>>(dA, dB, dC, static_cast<int>(W));
         okx = okx && cudaMemcpy(f2.data(), dC, W * W * 4, cudaMemcpyDeviceToHost) == cudaSuccess;
         if (okx) interleave(f1.data(), f2.data(), &xs[wf_slot(k) * per]);
-        if (okx && gck) { mput(f1.data(), 1 + 4 * k); mput(f2.data(), 2 + 4 * k); }
       }
       if (dA) cudaFree(dA);
       if (dB) cudaFree(dB);
@@ -1545,17 +1575,20 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
       // tables of the group chain kernel
       std::vector<CUtensorMap> maps;
       for (size_t k = 0; k < L; ++k) { maps.push_back(h->tm[1].W1[k]); maps.push_back(h->tm[1].W2[k]); }
-      std::vector<uint16_t> mb;
-      try { mb.resize(ms.size()); } catch (...) { return bail(CSD_ERR_WORKSPACE, "out of host memory"); }
-      if (d.dtype == CSD_BF16) { for (size_t i = 0; i < ms.size(); ++i) mb[i] = f32_to_bf16_bits(ms[i]); }
-      else { for (size_t i = 0; i < ms.size(); ++i) { const __half hv = __float2half_rn(ms[i]); memcpy(&mb[i], &hv, 2); } }
-      if (cudaMalloc(&h->mblob, mb.size() * 2) != cudaSuccess ||
+      std::vector<int> rows;
+      auto tiles = [&](size_t row, size_t n) { for (size_t r = 0; r < n; r += 256) rows.push_back(static_cast<int>(row + r)); };
+      for (size_t k = 0; k < L; ++k) tiles(5 * k * W, 3 * W);
+      tiles(5 * L * W, 2 * W);
+      const size_t nx = (4 * L - 2) * W;                     // rows of xblob
+      for (size_t r = 0; r < nx; r += 256) rows.push_back(~static_cast<int>(r));
+      tiles(0, 2 * W); tiles((5 * (L - 1) + 2) * W, W); tiles(5 * L * W, 2 * W);
+      if (cudaMalloc(&h->d_gc_rows, rows.size() * sizeof(int)) != cudaSuccess ||
           cudaMalloc(&h->d_gc_maps, maps.size() * sizeof(CUtensorMap)) != cudaSuccess) { cudaGetLastError(); return bail(CSD_ERR_WORKSPACE, "cannot allocate device memory for the group-chain tables"); }
-      if (cudaMemcpy(h->mblob, mb.data(), mb.size() * 2, cudaMemcpyHostToDevice) != cudaSuccess ||
+      if (cudaMemcpy(h->d_gc_rows, rows.data(), rows.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
           cudaMemcpy(h->d_gc_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess) return bail(CSD_ERR_CUDA, "group-chain table upload failed");
-      if ((rc = make_tmap(ctx, &h->Wm, d.dtype, h->mblob, (4 * L + 2) * W, W, W, kTileM)) ||
-          (rc = make_tmap(ctx, &h->Wrows, d.dtype, h->Wss[0], (5 * L + 2) * W, W, W, kTileM))) { csd_head_destroy(h); return rc; }
-      h->gc_ready = h->gf_ready = true;
+      if ((rc = make_tmap(ctx, &h->Wrows, d.dtype, h->Wss[0], (5 * L + 2) * W, W, W, kTileM)) ||
+          (rc = make_tmap(ctx, &h->Wx, d.dtype, h->xblob, nx, W, W, kTileM))) { csd_head_destroy(h); return rc; }
+      h->gc_ready = true;
     }
     if (gck && W / kTileN == static_cast<size_t>(kPcColTiles)) {
       // tables of the persistent chain kernel: phases B, (W1_k, GATE_k) for every block, F
@@ -1595,7 +1628,7 @@ int csd_head_destroy(csd_head* h) {
   if (h->d_pc_maps) cudaFree(h->d_pc_maps);
   if (h->d_pc_bias) cudaFree(h->d_pc_bias);
   if (h->d_gc_maps) cudaFree(h->d_gc_maps);
-  if (h->mblob) cudaFree(h->mblob);
+  if (h->d_gc_rows) cudaFree(h->d_gc_rows);
   cudaGetLastError();
   delete h;
   return CSD_OK;
@@ -2145,7 +2178,8 @@ int csd_gmm_resample(csd_ctx* ctx, int B, int gamma, int C, int cap, const csd_g
   if (cap < 1) return fail(ctx, CSD_ERR_INVALID_ARG, "cap = %d must be >= 1", cap);
   if (!n_accept || !w || !xi || !v || !x_new || !n_prop || !flags || !cap_hits) return fail(ctx, CSD_ERR_INVALID_ARG, "null array argument");
   CSD_DEVICE(ctx);
-  GmmResampleParams r{B, gamma, C, cap, gmm_view(q), gmm_view(p), n_accept, w, xi, v, x_new, n_prop, flags, cap_hits, ctx->tally()};
+  GmmResampleParams r{B, gamma, C, cap, gmm_view(q), gmm_view(p), n_accept, w, xi, v, x_new, n_prop, flags, cap_hits, nullptr};
+  if ((rc = cap_hits_tally(ctx, ctx->stream, cap_hits, &r.tally))) return rc;
   const size_t smem = gmm_resample_smem_floats(q->K, p->K, C) * 4;
   const bool fits = smem <= 48 * 1024;
   auto kern = C <= 16 ? (fits ? gmm_resample_kernel<16, true> : gmm_resample_kernel<16, false>)

@@ -394,7 +394,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
           tma_store_commit();
         }
       }
-      if (Cfg::kOutOverH && i + 1 < my_tiles) {  // the next tile's h once the piece has left
+      if (Cfg::kOutOverH && ok && i + 1 < my_tiles) {  // the next tile's h once the piece has left
         if (stores) tma_store_wait_read();
         __syncwarp();
         h_request(i + 1);
@@ -434,6 +434,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
       }
     }
     if (Cfg::kStagedOut && stores) tma_store_wait_all();
+    if (Cfg::kHChunks && !ok) settle();          // a block of h may be on its way
   }
   tc_fence_before_sync();
   __syncthreads();

@@ -35,15 +35,11 @@ constexpr int kMgEpiWarps = 8;
 constexpr int kMgThreads = (kMgEpiWarps + 3) * 32;
 constexpr int kMgSmemBytes = 1024 + kMgStages * kMgStageBytes + 256;
 
-// After a wait that ran out, copies may be in flight that nobody waits for: they land within microseconds.
-__device__ __forceinline__ void gc_settle(const int* err) {
-  if (*reinterpret_cast<const volatile int*>(err) != 0)
-    for (int i = 0; i < 64; ++i) __nanosleep(1000);
-}
+__device__ __forceinline__ void gc_settle(const int* err) { if (*reinterpret_cast<const volatile int*>(err) != 0) settle(); }
 
 struct MgParams {
   int nkb, tiles_n, units;     // k-blocks; tiles of 256 rows of s; tiles in all (s fastest: the weights stream past once)
-  int run, stride;             // tiles of 256 weight rows come in runs of this many, whose first rows lie this far apart
+  const int* wrow;             // first row of each tile of 256 weight rows in the first matrix, or ~row in the second
   int s_row0;                  // first row of s
   float4* out;                 // [weight row / 128][row of s / 4][128 weight rows][4 rows of s]
   int* err;
@@ -54,7 +50,8 @@ struct MgParams {
 // steps, 14 sections of 1024: 0.53 ms in all on the 84 SMs that the chain leaves, 715 TFLOP/s, hidden behind it.
 template <int AB_FMT>
 __global__ void __launch_bounds__(kMgThreads, 1)
-mods_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmS, const MgParams p) {
+mods_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmS,
+                 const MgParams p) {
   constexpr int S = kMgStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -69,7 +66,7 @@ mods_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   const int unit0 = static_cast<int>(blockIdx.x >> 1), nunits = static_cast<int>(gridDim.x >> 1);
   const int my_tiles = (p.units - unit0 + nunits - 1) / nunits;
   if (threadIdx.x == 0) {
-    tma_prefetch_desc(&tmW); tma_prefetch_desc(&tmS);
+    tma_prefetch_desc(&tmW); tma_prefetch_desc(&tmX); tma_prefetch_desc(&tmS);
     for (int s = 0; s < S; ++s) { mbar_init(&full_bar[s], 2); mbar_init(&empty_bar[s], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 2 * kMgEpiWarps); }
     tmem_base_s[1] = *reinterpret_cast<const volatile int*>(p.err) == 0;    // one reading for all warps
@@ -87,16 +84,17 @@ mods_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     const bool is_w = warp == 0;
     if (lane == 0) {
       bool ok = true;
-      int it = 0;
+      int it = 0, next = is_w ? __ldg(p.wrow + unit0 / p.tiles_n) : 0;
       for (int i = 0; i < my_tiles && ok; ++i) {
         const int u = unit0 + i * nunits;
-        const int wt = u / p.tiles_n;
-        const int row = (is_w ? wt / p.run * p.stride + wt % p.run * 256 : p.s_row0 + (u - wt * p.tiles_n) * 256) + rank * 128;
+        const CUtensorMap* const tm = !is_w ? &tmS : next < 0 ? &tmX : &tmW;
+        const int row = (!is_w ? p.s_row0 + u % p.tiles_n * 256 : next < 0 ? ~next : next) + rank * 128;
+        if (is_w && i + 1 < my_tiles) next = __ldg(p.wrow + (u + nunits) / p.tiles_n);
         for (int kb = 0; kb < p.nkb; ++kb, ++it) {
           const int s = it % S;
           if (it >= S && !ch_wait<false>(&empty_bar[s], ((it / S) & 1) ^ 1, p.err)) { ch_fail(p.err, DEV_ERR_TMA_WAIT, 1, it); ok = false; break; }
           if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], 32768);     // both CTAs' bytes of this operand
-          tma_load_2d_pair(smem + s * kMgStageBytes + (is_w ? 0 : 16384), is_w ? &tmW : &tmS, mapa_shared(smem_u32(&full_bar[s]), 0), kb * kBlockK, row);
+          tma_load_2d_pair(smem + s * kMgStageBytes + (is_w ? 0 : 16384), tm, mapa_shared(smem_u32(&full_bar[s]), 0), kb * kBlockK, row);
         }
       }
     }
@@ -185,7 +183,7 @@ __host__ __device__ inline GcLayout gc_layout(int W) {
   l.stats = take(W / 32 * kGcRows * 8);   // [32-column group][row] (mean, M2)
   l.part = take(kGcRows * kCPad * 4);     // the outgoing output-projection partial
   l.misc = take(1024 + 512 + 512);        // x [16 tokens][16], (mean, rstd) per epilogue warp [8][8], barriers
-  l.stages = (226 * 1024 - o) / 16384;    // all that is left streams weights: 12, 9, 6 stages
+  l.stages = (226 * 1024 - o) / 16384;    // all that is left streams weights: 9, 9, 6 stages at W = 512, 1024, 1536
   l.stages = (l.stages > kGcMaxStages ? kGcMaxStages : l.stages) / kGcMma * kGcMma;
   l.ring = take(0);
   o = (o + 1023) / 1024 * 1024;
@@ -195,18 +193,20 @@ __host__ __device__ inline GcLayout gc_layout(int W) {
   return l;
 }
 
+constexpr int kGcMaxSteps = 128;          // steps per launch: their coefficients travel as kernel parameters
+
 struct GcParams {
   int R, cfg, W, L, C, T, t_hi, t_lo, rows, sample_last;   // rows: kernel rows (groups x 16)
   float cfg_scale;
   const CUtensorMap* maps;     // [2 L]: W1_k, W2_k in boxes of 128 rows
   const float4* mods; int nq;  // products of the chunk, nq row quads per weight row
   const float *c1, *bsh, *bsc, *bg, *b1, *b2, *bfsh, *bfsc;   // block 0; c1_k | c2_k (FOLD) are 2 W floats a block, the others 5 W apart
-  const float* sched;          // a[T], b[T], sigma[T]
   const float *win, *bin, *wout_t, *bout;
   const float *x_T, *eps;
   float *x, *x0, *mu1, *x1, *traj_x, *traj_mu;
   int* err;
   int* status;
+  float ca[kGcMaxSteps], cb[kGcMaxSteps], sigma[kGcMaxSteps];   // index t - t_lo
 };
 
 // Shared memory of this CTA -> the same or another CTA of the cluster, completion counted in bytes on a barrier there.
@@ -331,6 +331,7 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
           // 128 rows, 3 x 1024, 100 steps)
           ok = ok && ch_wait<false>(lane & 1 ? &w_full[st] : &tile[src], lane & 1 ? par : use & 1, p.err);
           ok = __all_sync(0xffffffffu, ok);
+          __syncwarp();        // (a vote orders no memory: the leader issues on what the other lanes have waited for)
           if (!ok) { if (leader) ch_fail(p.err, DEV_ERR_MMA_WAIT, 2, ph); break; }
           tc_fence_after_sync();
           if (leader) {
@@ -365,13 +366,16 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
       const float4 a = gc_ld(src), b = gc_ld(src + 128);
       m[0] = a.x; m[1] = a.y; m[2] = a.z; m[3] = a.w; m[4] = b.x; m[5] = b.y; m[6] = b.z; m[7] = b.w;
     };
-    // FOLD: product `sec` (scale_0 | per block P1, P2, gate, next scale | final shift, scale) in this thread's column
-    auto take = [&](float (&m)[kGcHalf], int t, int sec) { take_row(m, t, sec * CL + rank, c); };
-    // Plain: shift and scale of block k (L: the final pair), whose rows are interleaved in groups of 64, and gate
-    auto take_ss = [&](float (&sh)[kGcHalf], float (&sc)[kGcHalf], int t, int k) {
-      const int tile = 3 * CL * k + 2 * rank + (c >> 6);
-      take_row(sh, t, tile, c & 63); take_row(sc, t, tile, 64 + (c & 63));
+    // two matrices whose rows are interleaved in groups of 64, from tile `base`, in this thread's column
+    auto take_pair = [&](float (&u)[kGcHalf], float (&v)[kGcHalf], int t, int base) {
+      const int tile = base + 2 * rank + (c >> 6);
+      take_row(u, t, tile, c & 63); take_row(v, t, tile, 64 + (c & 63));
     };
+    // Plain: per block shift | scale, gate; the final pair.  FOLD: gate_k | scale_{k+1} (k < L - 1), P1_k | P2_k (k = 1.., then 0),
+    // shift_0 | scale_0, the last gate, the final pair.
+    const int tail = (2 * L - 1) * 2 * CL;
+    auto take_ss = [&](float (&sh)[kGcHalf], float (&sc)[kGcHalf], int t, int k) { take_pair(sh, sc, t, 3 * CL * k); };
+    auto take_p12 = [&](float (&p1)[kGcHalf], float (&p2)[kGcHalf], int t, int k) { take_pair(p1, p2, t, 2 * CL * (k == 0 ? 2 * (L - 1) : L - 2 + k)); };
     auto take_gate = [&](float (&m)[kGcHalf], int t, int k) { take_row(m, t, 3 * CL * k + 2 * CL + rank, c); };
     // 16-bit tile of this CTA's columns: into its own activation buffer `buf`, and from there into every peer's
     auto send_tile = [&](const float (&v)[kGcHalf], int buf) {
@@ -463,7 +467,7 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
     const float4* const win4 = reinterpret_cast<const float4*>(p.win + static_cast<size_t>(col) * kCPad);
     const float bi = __ldg(p.bin + col), bs = __ldg(p.bsc + col), bh = FOLD ? 0.0f : __ldg(p.bsh + col);
     auto take_win = [&]() { w0 = gc_ld(win4); w1 = gc_ld(win4 + 1); w2 = gc_ld(win4 + 2); w3 = gc_ld(win4 + 3); };
-    auto take_first = [&](int t) { if constexpr (FOLD) take(m0, t, 0); else take_ss(m0, m1, t, 0); };
+    auto take_first = [&](int t) { if constexpr (FOLD) take_row(m0, t, tail + 2 * rank + (c >> 6), 64 + (c & 63)); else take_ss(m0, m1, t, 0); };
     take_first(p.t_hi);
     take_win();
     epi_sync();
@@ -485,7 +489,7 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
 #pragma unroll
           for (int i = 0; i < kGcHalf; ++i) a[i] = __fmul_rn(h[i], __fadd_rn(1.0f, __fadd_rn(m0[i], bs)));
           send_tile(a, 0);
-          take(m0, t, 1); take(m1, t, 2);
+          take_p12(m0, m1, t, 0);
           send_stats(h);
         } else {
           send_stats(h);
@@ -516,8 +520,8 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
         // ---- h += gate (v W2^T + b2); the next block's a' = h (1 + scale_{k+1}), or u
         const bool last = k + 1 == L;
         if constexpr (FOLD) {
-          take(m0, t, 4 * k + 3);
-          if (!last) take(m1, t, 4 * k + 4);
+          if (last) take_row(m0, t, tail + 2 * CL + rank, c);
+          else take_pair(m0, m1, t, 2 * CL * k);
           const float kg = __ldg(p.bg + static_cast<size_t>(5 * k) * W + col), kb = __ldg(p.b2 + static_cast<size_t>(5 * k) * W + col),
                       ks = last ? 0.0f : __ldg(p.bsc + static_cast<size_t>(5 * (k + 1)) * W + col);
           acc_load(a);
@@ -528,8 +532,8 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
             for (int i = 0; i < kGcHalf; ++i) a[i] = __fmul_rn(h[i], __fadd_rn(1.0f, __fadd_rn(m1[i], ks)));
             send_tile(a, 0);
           }
-          const int sec = last ? 4 * L : 4 * k + 5;           // the final shift and scale, or the next block's P1, P2
-          take(m0, t, sec); take(m1, t, sec + 1);
+          if (last) take_pair(m0, m1, t, tail + 3 * CL);
+          else take_p12(m0, m1, t, k + 1);
           send_stats(h);
         } else {
           take_gate(m0, t, k);
@@ -544,7 +548,7 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
         }
       }
       // ---- output projection of (LN(h)(1 + scale_f) + shift_f): this CTA's columns' part, to every CTA
-      const float sa = p.sched[t - 1], sb = p.sched[T + t - 1], sg = p.sched[2 * T + t - 1];
+      const float sa = p.ca[t - p.t_lo], sb = p.cb[t - p.t_lo], sg = p.sigma[t - p.t_lo];
       float noise = 0.0f;
       const int q = et >> 4, e = et & 15, tok = tok0 + q;                 // this thread's entry of the state
       const bool mine = et < per * kCPad && tok < p.R && e < p.C;

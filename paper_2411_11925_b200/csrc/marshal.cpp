@@ -5,6 +5,7 @@
 // No arithmetic and no policy: pointers and sizes go to the C ABI as they are, the status code comes back.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
+#include <exception>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "../../include/csd.h"
@@ -19,9 +20,14 @@ struct Args {
   template <typename T> T* ptr(PyObject* o) {
     if (!ok || o == Py_None) return nullptr;
     if (THPVariable_Check(o)) {
-      const at::Tensor& t = THPVariable_Unpack(o);
-      if (t.is_contiguous()) return static_cast<T*>(t.data_ptr());
-      PyErr_SetString(PyExc_AssertionError, "tensor must be contiguous");
+      // a tensor without strides or storage (nested, sparse, vmapped) throws: that stays a Python error
+      try {
+        const at::Tensor& t = THPVariable_Unpack(o);
+        if (t.is_contiguous()) return static_cast<T*>(t.data_ptr());
+        PyErr_SetString(PyExc_AssertionError, "tensor must be contiguous");
+      } catch (const std::exception& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+      }
       ok = false;
       return nullptr;
     }
@@ -59,8 +65,7 @@ struct Args {
     } else {
       PyObject** it = PySequence_Fast_ITEMS(s);
       m.logw = ptr<const float>(it[0]); m.mu = ptr<const float>(it[1]); m.log_sigma = ptr<const float>(it[2]);
-      if (ok && THPVariable_Check(it[0]) && THPVariable_Unpack(it[0]).dim() >= 2) m.K = static_cast<int>(THPVariable_Unpack(it[0]).size(1));
-      else if (ok) {
+      if (ok) {
         PyObject* sh = PyObject_GetAttrString(it[0], "shape");
         PyObject* k = sh ? PySequence_GetItem(sh, 1) : nullptr;
         m.K = k ? static_cast<int>(PyLong_AsLong(k)) : 0;

@@ -51,7 +51,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Same with acquire semantics at cluster scope: pairs with mbar_arrive_cluster of another CTA.
+// Same with acquire semantics at cluster scope: pairs with arrivals and copies of other CTAs.
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -103,6 +103,11 @@ __device__ __forceinline__ bool ch_wait(uint64_t* bar, uint32_t parity, const in
 // site << 4 | (count & 0xffff) << 8 | (block & 0x7f) << 24.  Later failures do not overwrite it.
 __device__ __forceinline__ void ch_fail(int* err, int role, int site, int count) {
   atomicCAS(err, 0, role | (site << 4) | ((count & 0xffff) << 8) | ((static_cast<int>(blockIdx.x) & 0x7f) << 24));
+}
+
+// After a wait that ran out, copies may be in flight that nobody waits for: they land within microseconds.
+__device__ __forceinline__ void settle() {
+  for (int i = 0; i < 64; ++i) __nanosleep(1000);
 }
 
 // ------------------------------------------------ programmatic dependent launch
@@ -219,25 +224,11 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t smem_addr, uint32_t ran
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// arrive on a barrier of another CTA of the cluster (shared::cluster address)
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// The same to say that tensor memory has been read: the reads are complete (tcgen05.wait::ld) and ordered by
-// tcgen05.fence::before_thread_sync, no ordinary memory is handed over.  A releasing arrive would wait for the thread's
+// Arrives on a barrier of another CTA of the cluster (shared::cluster address) to say that tensor memory has been read: the reads
+// are complete (tcgen05.wait::ld) and ordered by tcgen05.fence::before_thread_sync, no ordinary memory is handed over.  A releasing arrive would wait for the thread's
 // outstanding stores first: 2 to 3 k cycles per tile in the gated kernel's epilogue.
 __device__ __forceinline__ void mbar_arrive_cluster_tmem(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// Counter in shared memory that CTAs of the cluster bump remotely: relaxed add (the caller fences once
-// before a batch of them), read with acquire.
-__device__ __forceinline__ void red_add_cluster(uint32_t cluster_addr, uint32_t v) {
-  asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ uint32_t ld_acquire_cluster(const uint32_t* smem_word) {
-  uint32_t v;
-  asm volatile("ld.acquire.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(smem_word)) : "memory");
-  return v;
 }
 // TMA load into this CTA's shared memory whose byte count is credited to a barrier of the pair's
 // leader CTA (shared::cluster address).  No multicast.

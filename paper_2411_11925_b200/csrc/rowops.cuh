@@ -681,9 +681,14 @@ __device__ __forceinline__ float coord_tree_sum(float* v) {
 
 // The number of sequences whose cap was reached, summed over the blocks without a memset before the launch: every block
 // adds (its hits, 1) to one 64-bit word, the last one to arrive has the sum and leaves the word at zero for the context's
-// next call.  hits: this block's count, valid in thread 0.
+// next call.  The word serves one launch at a time: launches that others of the context may overlap (captured ones, whose
+// graphs run on any stream) get none and add to a cap_hits zeroed before them.  hits: this block's count, valid in thread 0.
 __device__ __forceinline__ void tally_cap_hits(int hits, unsigned long long* tally, int32_t* cap_hits) {
   if (threadIdx.x != 0) return;
+  if (!tally) {
+    if (hits) atomicAdd(cap_hits, hits);
+    return;
+  }
   unsigned long long before = 0;
   if (gridDim.x > 1) {
     before = atomicAdd(tally, (static_cast<unsigned long long>(hits) << 32) | 1ull);

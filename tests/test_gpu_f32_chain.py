@@ -68,3 +68,22 @@ def test_f32_predicted_variances_match_the_layer_kernels(kw):
     for k in ("hld_q", "hld_p"):
         assert float(np.max(np.abs(got[0][k] - got[1][k]))) <= 1e-6 * max(1.0, float(np.abs(got[1][k]).max())) * kw["T"] ** 0.5 + 1e-4, k
     r.ctx.close()
+
+
+@pytest.mark.parametrize("W,R,cfg", [(896, 91 * 32, False), (1536, 53 * 16, True), (2048, 512, False)])
+def test_most_rows_of_the_chain_kernel_and_one_more(W, R, cfg):
+    # 637, 636 and 256 tiles (groups of 16, 8 and 4 head rows); one token more runs as layer kernels, the same fp32 function summed in another order
+    from paper_2411_11925_b200 import api
+    from paper_2411_11925_b200.runner import DeviceRound
+    for rows, chain in ((R, True), (R + 1, False)):
+        dr = DeviceRound(gen.make_round_inputs(_wl(B=rows, gamma=1, T=2, cfg=cfg, cfg_scale=2.0, draft=gen.HeadSpec(1, W, 32), target=gen.HeadSpec(1, 128, 32))))
+        l0 = dr.ctx.launch_count()
+        dr.draft()
+        assert (dr.ctx.launch_count() - l0 == 3) == chain, (rows, dr.ctx.launch_count() - l0)
+        dr.ctx.sync()
+        x0 = dr.x0.clone()
+        dr.ctx.set_chain_mode(api.Context.CHAIN_LAYERS_PLAIN)
+        dr.draft()
+        dr.ctx.sync()
+        assert float((x0 - dr.x0).abs().max()) <= 2e-5 * float(dr.x0.abs().max())
+        dr.ctx.close()

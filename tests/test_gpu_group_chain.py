@@ -36,6 +36,27 @@ def test_group_chain_matches_checker_and_fused_round_matches_the_calls(kw):
     dr.ctx.close()
 
 
+@pytest.mark.parametrize("W,groups,cfg", [(512, 33, False), (512, 33, True), (1024, 15, True), (1536, 7, True)])
+def test_most_groups_and_one_more(W, groups, cfg):
+    # the last group full, then one token beyond it: layer kernels
+    from paper_2411_11925_b200 import api
+    from paper_2411_11925_b200.runner import DeviceRound
+    most = groups * (8 if cfg else 16)
+    for R, chain in ((most, True), (most + 1, False)):
+        inp = gen.make_round_inputs(_wl(bf16=True, B=R, gamma=1, T=3, cfg=cfg, cfg_scale=2.0, draft=H(1, W, 64), target=H(1, 128, 64)))
+        dr = DeviceRound(inp)
+        got = []
+        for mode in (api.Context.CHAIN_LAYERS, api.Context.CHAIN_LAYERS_PLAIN):
+            dr.ctx.set_chain_mode(mode)
+            l0 = dr.ctx.launch_count()
+            dr.draft()
+            dr.ctx.sync()
+            got.append((dr.x0.clone(), dr.ctx.launch_count() - l0))
+        assert (got[0][1] < 12) == chain and got[1][1] == 20, (R, got[0][1], got[1][1])
+        assert float((got[0][0] - got[1][0]).abs().max()) <= TOL_X["f16"] / 4
+        dr.ctx.close()
+
+
 @pytest.mark.parametrize("B,T", [(1, 16), (1, 17), (1, 49), (40, 5), (40, 6), (40, 17)])      # chunks of 16, 32, .. and of 5, 10, .. steps
 def test_trajectory_across_chunks_of_steps(B, T):
     from paper_2411_11925_b200 import api

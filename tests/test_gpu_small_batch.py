@@ -1,6 +1,5 @@
-"""The persistent small-batch chain kernel (CSD_CHAIN_SMALL_BATCH): chains of at most 128 head rows, the calling
-pattern of Alg. 1's draft loop (x_i ~ q_i one position at a time), against the float64 checker and against the
-layer kernels."""
+"""CSD_CHAIN_SMALL_BATCH: chains of at most 128 head rows, the calling pattern of Alg. 1's draft loop (x_i ~ q_i one position
+at a time), in the group chain kernel's folded form, against the float64 checker and against the layer kernels."""
 import numpy as np
 import pytest
 import torch
@@ -56,7 +55,7 @@ def test_small_batch_round_matches_checker_and_the_layer_kernels(op, kw):
     ref, s1 = _ref(inp)
     st = compare_round(a, ref, inp.wl, s1, s1, inp.u, inp.v, f"small batch {op} {kw}", xi=inp.xi)
     print("small batch", op, kw, {k: st[k] for k in ("x0_err", "mu1p_err", "logr_err_over_tol")}, "launches", launches)
-    # the fused round runs the same two kernels one after the other: same bits; and so does a repeat
+    # the fused round runs the same two chains side by side: same bits; and so does a repeat
     dr.fused_round()
     b = dr.results()
     dr.three_calls()
@@ -65,9 +64,11 @@ def test_small_batch_round_matches_checker_and_the_layer_kernels(op, kw):
         np.testing.assert_array_equal(a[k], b[k], err_msg=f"fused {k}")
         np.testing.assert_array_equal(a[k], c[k], err_msg=f"repeat {k}")
     # the layer kernels compute the same function with other roundings
-    dr.ctx.set_chain_mode(api.Context.CHAIN_LAYERS)
+    dr.ctx.set_chain_mode(api.Context.CHAIN_LAYER_KERNELS)
+    l0 = dr.ctx.launch_count()
     dr.three_calls()
     d = dr.results()
+    assert dr.ctx.launch_count() - l0 >= 2 * inp.wl.T * 4                  # three or more kernels a step besides the boundary
     for k in ("x0", "mu1_q", "mu1_p"):
         assert float(np.max(np.abs(a[k] - d[k]))) <= TOL_X[op] / (2 if op == "bf16" else 4), k   # both carry their own rounding
     dr.ctx.set_wait_limit(0)
@@ -93,17 +94,38 @@ def test_sequential_draft_calls_at_benchmark_size():
     wl = gen.Workload(**{**gen.WORKLOADS["mar256"].__dict__, "gamma": 1})
     inp = gen.make_round_inputs(wl)
     dr = _round(inp, api.Context.CHAIN_SMALL_BATCH)
+    l0 = dr.ctx.launch_count()
     dr.draft()
+    assert dr.ctx.launch_count() - l0 < 30
     dr.ctx.sync()
     x0 = dr.x0.cpu().numpy()
     sub = gen.select_sequences(inp, [0, 63])
     s = orc.ddpm_schedule(inp.beta, wl.tau)
     ref = orc.denoise(orc.make_mlp_head(sub.w_q, sub.z_q, sub.tfeat, wl.cfg, wl.cfg_scale), s, sub.x_T, sub.eps)
     err = float(np.max(np.abs(x0[sub.extras["rows"]] - ref["x0"])))
-    print("sequential draft call, small-batch kernel: x0 err", err)
+    print("sequential draft call, small-batch mode: x0 err", err)
     assert err <= TOL_X["f16"]
     dr.draft()
     dr.ctx.sync()
     np.testing.assert_array_equal(x0, dr.x0.cpu().numpy())
     dr.ctx.set_wait_limit(0)
     dr.ctx.close()
+
+
+def test_beyond_128_head_rows_the_mode_takes_the_plain_kernels():
+    # 129 rows: the group chain kernel's plain form, the default mode's bits; above its groups: three kernels per block
+    from paper_2411_11925_b200 import api
+    for B, other, few in ((129, api.Context.CHAIN_LAYERS, True), (241, api.Context.CHAIN_LAYERS_PLAIN, False)):
+        inp = gen.make_round_inputs(_wl(B=B, gamma=1, T=3, cfg=False, cfg_scale=1.0, draft=gen.HeadSpec(2, 1024, 64)))
+        dr = _round(inp, api.Context.CHAIN_SMALL_BATCH)
+        l0 = dr.ctx.launch_count()
+        dr.draft()
+        assert (dr.ctx.launch_count() - l0 < 15) == few
+        dr.ctx.sync()
+        x0 = dr.x0.clone()
+        dr.ctx.set_chain_mode(other)
+        dr.draft()
+        dr.ctx.sync()
+        assert bool((x0 == dr.x0).all())
+        dr.ctx.set_wait_limit(0)
+        dr.ctx.close()
