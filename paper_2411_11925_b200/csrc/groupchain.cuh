@@ -360,9 +360,10 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
     auto wait = [&](uint64_t* bar, uint32_t parity, int site) {
       if (ok && !ch_wait<true>(bar, parity, p.err)) { ch_fail(p.err, DEV_ERR_EPI_WAIT, site, static_cast<int>(n_acc)); ok = false; }
     };
+    const float4* const mods0 = p.mods + (grp * (kGcRows / 4) + r0 / 4) * 128;
     // product of step t with row `row` of tile `tile` of 128 weight rows, for this thread's rows of the group
     auto take_row = [&](float (&m)[kGcHalf], int t, int tile, int row) {
-      const float4* src = p.mods + (static_cast<size_t>(tile) * p.nq + (static_cast<size_t>(t - p.t_lo) * p.rows + grp * kGcRows + r0) / 4) * 128 + row;
+      const float4* src = mods0 + ((tile * p.nq + (t - p.t_lo) * (p.rows / 4)) * 128 + row);
       const float4 a = gc_ld(src), b = gc_ld(src + 128);
       m[0] = a.x; m[1] = a.y; m[2] = a.z; m[3] = a.w; m[4] = b.x; m[5] = b.y; m[6] = b.z; m[7] = b.w;
     };
