@@ -163,7 +163,7 @@ constexpr int kGcRows = 16;               // rows of a group = MMA N
 constexpr int kGcHalf = kGcRows / 2;      // rows of an epilogue thread
 constexpr int kGcEpi = 256;               // warps 0..7: epilogue
 // Three pairs of a loading warp (11..13) and an MMA-issuing warp (8..10), each with its own part of the weight ring and its own
-// accumulator, take k-blocks in turn.  One pair spends 370 cycles on loading and 530 on issuing a k-block (waits, the
+// accumulator, take k-blocks in turn (the same ones in every phase: the sums, hence the bits, do not depend on where a launch starts).  One pair spends 370 cycles on loading and 530 on issuing a k-block (waits, the
 // instructions' own latency, the commit), which the tensor pipe finishes in 160.  The ring is divided because waits on a
 // barrier's parity are only sound for one warp that follows its phases in order.
 constexpr int kGcMma = 3;
@@ -293,12 +293,12 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
     // ---------------------------------------------------------------- weights, k-blocks in this CTA's turn order
     if (lane == 0) {
       const int m = warp - 8 - kGcMma;
-      int j = m, s = 0;
+      int s = 0;
       uint32_t par = 1;
       bool ok = true;
       for (int t = p.t_hi; t >= p.t_lo && ok; --t)
-        for (int ph = 0; ph < 2 * L && ok; ++ph, j -= 2 * CL)
-          for (; j < 2 * CL; j += kGcMma) {
+        for (int ph = 0; ph < 2 * L && ok; ++ph)
+          for (int j = m; j < 2 * CL; j += kGcMma) {
             const int kb = 2 * rank + j < 2 * CL ? 2 * rank + j : 2 * rank + j - 2 * CL, st = m * SR + s;
             if (!ch_wait<false>(&w_empty[st], par, p.err)) { ch_fail(p.err, DEV_ERR_TMA_WAIT, 1, ph); ok = false; break; }   // (fresh: passes)
             mbar_arrive_expect_tx(&w_full[st], 16384);
@@ -315,17 +315,17 @@ __global__ void __launch_bounds__(kGcThreads, 1) group_chain_kernel(const __grid
     const int m = warp - 8;
     const uint32_t acc = tmem_base + m * kGcRows;
     bool ok = true;
-    int j = m, s = 0;
+    int s = 0;
     uint32_t par = 0, use = 0;
     for (int t = p.t_hi; t >= p.t_lo && ok; --t)
-      for (int ph = 0; ph < 2 * L && ok; ++ph, j -= 2 * CL) {
+      for (int ph = 0; ph < 2 * L && ok; ++ph) {
         const int buf = ph & 1;
         uint64_t* const tile = act_full + buf * kGcMaxCl;
         if (m == 0 && lane < CL && lane != rank) mbar_arrive_expect_tx(&tile[lane], kGcTile);   // (its own: the epilogue arrives)
         __syncwarp();
         ok = ch_wait<false>(&tile[rank], use & 1, p.err);      // this CTA's tile is also the word that the accumulators are free
         uint32_t more = 0;
-        for (; j < 2 * CL; j += kGcMma) {
+        for (int j = m; j < 2 * CL; j += kGcMma) {
           const int src = rank + (j >> 1) < CL ? rank + (j >> 1) : rank + (j >> 1) - CL, st = m * SR + s;
           // half of the lanes wait for the weights, half for the tile (one after the other: 2.79 instead of 2.73 ms a call of
           // 128 rows, 3 x 1024, 100 steps)
