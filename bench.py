@@ -26,10 +26,7 @@ import numpy as np  # noqa: E402
 
 # dram__bytes_read + dram__bytes_write per launch of a kernel class, from the ncu capture summarised under
 # profiles/ for (workload, class); absent = no capture of the kernel as it stands (reported as null)
-NCU_DRAM_BYTES_PER_LAUNCH = {
-    # profiles/mar256_persistent_chain_kernel_ncu.md: 6.02 GB read + 43.6 MB written per launch of the target chain
-    ("mar256", "pchain_target"): 6.062e9,
-}
+NCU_DRAM_BYTES_PER_LAUNCH = {}
 
 # Sequences of each workload that the float64 checker evaluates when it is timed (the first n of the batch): the
 # CPU-baseline leg and the reference arm time the very same sample.
@@ -309,8 +306,8 @@ def measure(name, args, peaks, steps, warmup, rounds_per_step, full):
         out["e2e_secs"] = float("nan")
 
     few = max(3, min(steps, 5))
-    # The two chains of a round on their own (csd_draft_denoise, csd_verify): with the persistent chain kernel a call
-    # is one launch, so this is the kernel's duration; and the same round from the layer kernels only.
+    # The two chains of a round on their own (csd_draft_denoise, csd_verify): with the wide chain kernel its launches and the
+    # condition products beside them; and the same round from the layer kernels only.
     if full:
         l1 = ctx.launch_count()
         timed(lambda i: rounds[i % nsets].draft(), 2)
@@ -324,7 +321,7 @@ def measure(name, args, peaks, steps, warmup, rounds_per_step, full):
         ctx.set_chain_mode(api.Context.CHAIN_LAYERS)
         out["chains"] = {"draft_ms": 1e3 * d_secs / few, "verify_ms": 1e3 * v_secs / few,
                          "draft_launches_per_call": int(d_launches),
-                         "persistent_chain_kernel": bool(d_launches < 50),
+                         "wide_chain_kernel": bool(d_launches < 100),
                          "layer_kernels_ms_per_round": 1e3 * lk_secs / few}
 
     # Sequential-draft variant: how an autoregressive loop has to call the draft head, one position at a time
@@ -510,21 +507,18 @@ def run_ours(args):
         line["decisions"] = m["decisions"]
         prof = m.get("prof")
         ch = m.get("chains")
-        if ch and ch["persistent_chain_kernel"] and wl.operand_format != "f32":
-            # the dominant kernel of the timed region is the target chain's persistent kernel: one launch per csd_verify
-            # call, timed by events around the call on the library's stream (the other kernels of the call take microseconds)
-            nb0 = -(-wl.R // (64 if wl.cfg else 128))
-            ctas = 8 * (nb0 + (nb0 & 1))            # one CTA per 128 x 128 tile of a layer, row blocks paired
+        if ch and ch["wide_chain_kernel"] and wl.operand_format != "f32":
+            # the kernels that decide the timed region are the target chain's: the wide chain kernel, chunk by chunk of steps, and
+            # beside it the dense products of the conditions; timed by events around a csd_verify call on the library's stream
             fl = wl.Rh * wl.T * wl.target.flops_per_row_step()
             ach = fl / (ch["verify_ms"] * 1e-3) / 1e12
-            line["roofline"] = {"bound": "tensor", "kernel": "pchain_kernel (target chain, one launch per call)",
+            line["roofline"] = {"bound": "tensor", "kernel": "wide_chain_kernel with wide_mods_kernel beside it (target chain, one call)",
                                 "achieved": ach, "peak": peaks["tflops_sustained"], "unit": "TFLOP/s",
                                 "frac": ach / peaks["tflops_sustained"],
-                                "traffic": NCU_DRAM_BYTES_PER_LAUNCH.get((wl.name, "pchain_target")),
+                                "traffic": NCU_DRAM_BYTES_PER_LAUNCH.get((wl.name, "wide_target")),
                                 "peak_source": f"{peaks['source']} bf16 sustained (fp16 has the same nominal rate)",
-                                "avg_launch_us": 1e3 * ch["verify_ms"], "flops_per_launch": fl,
-                                "sms_used": f"{ctas} of 148 (the draft chain's kernel runs beside it on others)",
-                                "draft_chain": {"avg_launch_us": 1e3 * ch["draft_ms"],
+                                "avg_call_us": 1e3 * ch["verify_ms"], "flops_per_call": fl,
+                                "draft_chain": {"avg_call_us": 1e3 * ch["draft_ms"],
                                                 "achieved": wl.Rh * wl.T * wl.draft.flops_per_row_step() / (ch["draft_ms"] * 1e-3) / 1e12}}
             line["chains"] = ch
         elif prof:

@@ -129,16 +129,16 @@ int64_t csd_launch_count(const csd_ctx *ctx);
 
 /* How the blocks of a denoising chain (the T steps of Eq. 3 for one head) are split into kernels.
  *   CSD_CHAIN_LAYERS  (default): the library picks by size.
- *                     - Layers of one wave of 128 x 128 tiles on a 16-bit head with W = 1024, var_out = 0 and an
- *                       even number of row blocks (128 head rows each: 64 tokens with guidance, 128 without; a few
- *                       hundred to about a thousand head rows) run as ONE persistent kernel per chain: a pair of
- *                       CTAs owns its output tiles for every layer and step, the residual stream stays in tensor
- *                       memory, the CTAs that share rows meet at a counter once per layer.  Draft and target chain
- *                       of csd_round then run side by side without competing for SMs.  Its buffers grow with T
- *                       (the condition vectors of all steps: T x rows x W 16-bit values).  A chain that has the GPU
- *                       to itself (csd_draft_denoise or csd_verify called alone) is about a tenth faster with
- *                       CSD_CHAIN_LAYER_KERNELS, whose kernels spread over the idle SMs; the default is chosen
- *                       per chain, not per call, so that csd_round and the three separate calls give the same bits.
+ *                     - A chain of more than 256 and up to 4608 head rows (R (1 + cfg)) on a 16-bit head with W a multiple of
+ *                       256 from 768 to 2048 runs as the wide chain kernel: everything that depends on the condition
+ *                       vector only is formed ahead, some steps at a time, and groups of W / 128 CTA pairs carry 256 or
+ *                       512 rows each through the steps, the residual stream in tensor memory.  Blocks are not folded: its
+ *                       error is that of three kernels per block.  The two chains of a round run side by side where
+ *                       their CTAs leave SMs to the condition products, else one after the other.  Its buffers, kept by
+ *                       the context per chain of a round: two chunks of condition products, fp32, (3 L + 2) W x rows x
+ *                       steps, at most 1 GB each as long as one step is less (1024 rows of 6 x 1024: 12 steps, 1 GB), the
+ *                       condition vectors of a chunk, operands and partials of one step.  Where the device has less
+ *                       free, chunks are shorter (the same bits); where not even one step fits, the layer kernels run.
  *                     - A chain of few rows on a 16-bit head with W in {512, 1024, 1536} and var_out = 0 (groups of
  *                       16 tokens, or 8 with guidance: up to 33, 15 and 7 groups) runs as the group chain kernel:
  *                       everything that depends on the condition vector only is formed ahead, for many steps at a
@@ -225,8 +225,8 @@ int csd_draft_denoise(csd_ctx *ctx, const csd_head *head, const csd_schedule *sc
 /* csd_draft_denoise without any allocation (the paper has no counterpart: this is a deployment
  * variant of the call above with the same arguments; it runs the kernels of CSD_CHAIN_LAYER_KERNELS, so its results are
  * bit-identical to csd_draft_denoise in the modes CSD_CHAIN_LAYER_KERNELS and CSD_CHAIN_LAYERS_PLAIN, and
- * in the default mode whenever that call takes neither the persistent nor the group chain kernel,
- * whose buffers grow with T and cannot live in a fixed array; otherwise the two agree within the parity tolerance).
+ * in the default mode whenever that call takes neither the wide nor the group chain kernel,
+ * whose buffers are too large for a fixed array; otherwise the two agree within the parity tolerance).
  * Who needs it: code that must not, or cannot, reach the CUDA allocator when the call is made -
  * a serving process whose framework has handed all free device memory to its own pool so that
  * cudaMalloc fails, a latency-critical loop where cudaMalloc's implicit device synchronisation is

@@ -228,7 +228,7 @@ class Context:
     CHAIN_LAYERS, CHAIN_SMALL_BATCH, CHAIN_LAYERS_PLAIN, CHAIN_LAYER_KERNELS = 0, 1, 2, 3
 
     def set_chain_mode(self, mode: int):
-        """csd_set_chain_mode: CHAIN_LAYERS (default: the group or the persistent chain kernel where one applies, else one
+        """csd_set_chain_mode: CHAIN_LAYERS (default: the group or the wide chain kernel where one applies, else one
         kernel per layer with folded blocks where they apply), CHAIN_LAYER_KERNELS (neither chain kernel),
         CHAIN_LAYERS_PLAIN (three kernels per block everywhere) or CHAIN_SMALL_BATCH (as CHAIN_LAYERS_PLAIN, with the group chain
         kernel for few rows, folded up to 128 head rows: faster, rounded more often)."""

@@ -21,7 +21,7 @@
 #include "gmm.cuh"
 #include "rowops.cuh"
 #include "groupchain.cuh"
-#include "pchain.cuh"
+#include "widechain.cuh"
 #include "f32chain.cuh"
 
 using namespace csd;
@@ -72,10 +72,10 @@ struct csd_ctx {
   HostIo un;       // csd_verify_unaligned: per-row noise terms
   HostIo bn;       // csd_bonus_token: samples of every sequence before the selection
   HostIo sp;       // csd_verify_single_path: schedule constants, mu^p of one pass, running log-ratio
-  HostIo pc[3];    // persistent chain kernel (per chain slot): s of all steps, a', v, partials, counters, schedule
-  HostIo gc[2];    // group chain kernel (per chain slot): s of all steps
-  HostIo gm[2];    // its condition products: two chunks of steps
-  size_t gc_refused[2] = {SIZE_MAX, SIZE_MAX}, gm_refused[2] = {SIZE_MAX, SIZE_MAX};   // sizes that could not be had: not asked for again
+  HostIo gc[2];    // group and wide chain kernels (per chain slot): s of all steps, or of a chunk of steps
+  HostIo gm[2];    // their condition products: two chunks of steps
+  HostIo wx[2];    // wide chain kernel: what its column tiles exchange
+  size_t gc_refused[2] = {SIZE_MAX, SIZE_MAX}, gm_refused[2] = {SIZE_MAX, SIZE_MAX}, wx_refused[2] = {SIZE_MAX, SIZE_MAX};   // (wx: all of a wide chain's) sizes that could not be had: not asked for again
   cudaStream_t aux[2] = {nullptr, nullptr};        // (per chain slot) where they are formed
   cudaEvent_t ev_prep[2] = {}, ev_mods[2][2] = {}, ev_read[2][2] = {};   // preparation done; a chunk is written / has been read
   cudaEvent_t ev_on[2] = {};                       // every block of a chunk's chain kernel has its SM
@@ -118,10 +118,10 @@ struct csd_head {
   CUtensorMap* d_gc_maps = nullptr;
   CUtensorMap Wrows{}, Wx{};
   int* d_gc_rows = nullptr;     // plain form, then folded form: first rows (~row: of xblob)
-  // persistent chain kernel (pchain.cuh): per phase the early and the dependent weight maps; per phase three bias rows
-  bool pc_ready = false;
-  CUtensorMap* d_pc_maps = nullptr;
-  const float** d_pc_bias = nullptr;
+  // wide chain kernel (widechain.cuh): W1_k, W2_k in boxes of 64 rows; per tile of 256 weight rows its first row and its biases
+  CUtensorMap* d_wc_maps = nullptr;
+  int* d_wc_rows = nullptr;
+  float* d_wc_bias = nullptr;
 };
 
 namespace {
@@ -201,6 +201,18 @@ int make_tmap(csd_ctx* ctx, CUtensorMap* m, int dtype, const void* ptr, uint64_t
   const CUresult r = ctx->encode(m, dtype == CSD_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), gdim, gstride, box,
                                  estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(ctx, CSD_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
+  return CSD_OK;
+}
+
+// [lines, 256] elements as they lie, in boxes of 32 lines (16 KB).
+int make_plain_tmap(csd_ctx* ctx, CUtensorMap* m, int dtype, const void* ptr, uint64_t lines) {
+  const cuuint64_t gdim[2] = {256, lines};
+  const cuuint64_t gstride[1] = {512};
+  const cuuint32_t box[2] = {256, 32};
+  const cuuint32_t estr[2] = {1, 1};
+  const CUresult r = ctx->encode(m, dtype == CSD_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), gdim, gstride, box,
+                                 estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(ctx, CSD_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
   return CSD_OK;
 }
@@ -352,12 +364,6 @@ int check_sched(csd_ctx* ctx, const csd_schedule* s, bool full) {
   return CSD_OK;
 }
 
-// Chains whose layers are one wave of tiles run as one persistent kernel (pchain.cuh) where it applies.
-#ifndef CSD_PERSISTENT_CHAINS
-#define CSD_PERSISTENT_CHAINS 1
-#endif
-constexpr bool kPersistentChains = CSD_PERSISTENT_CHAINS != 0;
-
 // Folded blocks run as CTA pairs when a layer's row tiles pair up.
 #ifndef CSD_FOLD_PAIRS
 #define CSD_FOLD_PAIRS 1
@@ -429,20 +435,6 @@ bool fold_kernels_ready(const csd_ctx* ctx, const csd_head_desc& d) {
 
 int ensure_side(csd_ctx* ctx, HostIo& io, size_t need, const char* what);
 
-// Shared-memory opt-in of the persistent chain kernel, once per device and operand type.
-bool pchain_kernel_ready(const csd_ctx* ctx, int dtype) {
-  static int known[kMaxDevices][2] = {};
-  int& k = known[ctx->device][dtype == CSD_F16 ? 0 : 1];
-  if (k == 0) {
-    const bool ok = dtype == CSD_F16
-        ? cudaFuncSetAttribute(pchain_kernel<__half, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPcSmemBytes) == cudaSuccess
-        : cudaFuncSetAttribute(pchain_kernel<__nv_bfloat16, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPcSmemBytes) == cudaSuccess;
-    cudaGetLastError();
-    k = ok ? 1 : -1;
-  }
-  return k == 1;
-}
-
 // Clusters of the group chain kernel for width W that the device holds at a time (0: it cannot run), and its opt-ins, once
 // per device and operand type.
 template <typename ACT, int FMT>
@@ -475,6 +467,71 @@ int gchain_clusters(const csd_ctx* ctx, int dtype, int W) {
 }
 constexpr size_t kGcChunkBytes = size_t(512) << 20;   // most bytes of condition products of one chunk of steps
 
+// Wide chain kernel (widechain.cuh): the heads it takes.
+bool wide_width(const csd_head_desc& d) {
+  return d.dtype != CSD_F32 && d.W % 256 == 0 && d.W >= 768 && d.W <= 128 * kWcMaxCt &&
+         wc_layout(d.L, d.var_out ? kCPad2 : kCPad, 1).stages >= kWcMinStages;
+}
+typedef void (*WideKernel)(CUtensorMap, CUtensorMap, WcParams);
+template <typename ACT, int FMT>
+WideKernel wide_kernel_of(bool lv, int halves) {
+  if (halves == 2) return lv ? wide_chain_kernel<ACT, FMT, true, 2> : wide_chain_kernel<ACT, FMT, false, 2>;
+  return lv ? wide_chain_kernel<ACT, FMT, true, 1> : wide_chain_kernel<ACT, FMT, false, 1>;
+}
+WideKernel wide_kernel(int dtype, bool lv, int halves) { return dtype == CSD_F16 ? wide_kernel_of<__half, 0>(lv, halves) : wide_kernel_of<__nv_bfloat16, 1>(lv, halves); }
+bool wide_ready(const csd_ctx* ctx, int dtype) {
+  static int known[kMaxDevices][2] = {};
+  int& k = known[ctx->device][dtype == CSD_F16 ? 0 : 1];
+  if (k == 0) {
+    bool ok = (dtype == CSD_F16 ? cudaFuncSetAttribute(wide_mods_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMgSmemBytes)
+                                : cudaFuncSetAttribute(wide_mods_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMgSmemBytes)) == cudaSuccess;
+    for (int i = 0; i < 4; ++i) ok = ok && cudaFuncSetAttribute(wide_kernel(dtype, (i & 1) != 0, 1 + (i >> 1)), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
+    cudaGetLastError();
+    k = ok ? 1 : -1;
+  }
+  return k == 1;
+}
+// How a chain of R token rows is cut up: slots of 256 rows; the form of the kernel (halves 1: two slots a group, 2: one slot with
+// twice the epilogue warps); slots of a launch (a part of the rows where not all of a launch's CTAs would find an SM).
+struct WideCut { int nb, slots, part, ctas, halves; };
+WideCut wide_cut(const csd_ctx* ctx, const csd_head_desc& d, int R, int cfg, int halves) {
+  WideCut c{};
+  const int nb = cfg ? (R + 63) / 64 : (R + 127) / 128, group = 2 * (d.W / 128), most = ctx->num_sms / group, gs = 2 / halves;
+  c.nb = nb + (nb & 1); c.slots = c.nb / 2; c.halves = halves;
+  const int groups = (c.slots + gs - 1) / gs, parts = (groups + most - 1) / most;
+  c.part = ((c.slots + parts - 1) / parts + gs - 1) / gs * gs;
+  c.ctas = ((c.part < c.slots ? c.part : c.slots) + gs - 1) / gs * group;
+  return c;
+}
+bool wide_halves(const csd_head_desc& d) { return wc_layout(d.L, d.var_out ? kCPad2 : kCPad, 2).stages >= kWcMinStages; }
+// Which form, and whether two chains go side by side, by a model of one step in us, fitted to measured steps (W = 1024, 1024 rows: 3
+// blocks 68 in one-slot groups, 82 in two-slot groups; 6 blocks 106 and 158; 12 x 1536 259 and 420).  The choice changes no bit.
+double wide_step_us(const csd_head_desc& d, int halves) { return halves == 2 ? 30.0 + 12.7 * d.L * d.W / 1024 : 20.0 + 22.0 * d.L * d.W / 1024; }
+double wide_mods_sm_us(const csd_head_desc& d, int slots) { return 2.0 * (3 * d.L + 2) * d.W * d.W * kWcRows * slots / 8.8e6; }   // 8.8 TFLOP/s an SM
+// Beside chains that hold at most half of the SMs the products have the rest to themselves; else everything shares the GPU, at about
+// 120 of 148 SMs' worth.
+double wide_us(const csd_ctx* ctx, double chain_us, double chain_sm_us, double mods_sm_us, int held) {
+  const double other = held <= ctx->num_sms / 2 ? mods_sm_us / (ctx->num_sms - held) : (mods_sm_us + chain_sm_us) / (0.81 * ctx->num_sms);
+  return chain_us > other ? chain_us : other;
+}
+WideCut wide_cut_alone(const csd_ctx* ctx, const csd_head_desc& d, int R, int cfg) {
+  const WideCut one = wide_cut(ctx, d, R, cfg, 2), two = wide_cut(ctx, d, R, cfg, 1);
+  if (!wide_halves(d) || one.part < one.slots) return two;
+  auto us = [&](const WideCut& c) { const double t = wide_step_us(d, c.halves); return wide_us(ctx, t, t * c.ctas, wide_mods_sm_us(d, c.slots), c.ctas); };
+  return us(one) <= us(two) ? one : two;
+}
+constexpr size_t kWcChunkBytes = size_t(1) << 30;     // most bytes of condition products of one chunk of steps
+// More than one slot of rows, up to what two-slot groups of 1024-wide heads cover at a time.  Beyond that the layer kernels' waves of tiles
+// fill the GPU as well, and the chain's hand-overs cost more than the dense product of the conditions saves.  ms a round of 20 steps with
+// guidance, before (persistent chain or layer kernels) / this kernel, at 512, 1024, 2048, 4096 and 8192 head rows of each head:
+//   3 and 6 x 1024:   3.13 / 2.25   3.16 / 2.93   6.44 / 5.23   11.3 / 10.6   18.8 / 21.2
+//   6 x 1024, 12 x 1536:  5.89 / 5.32   10.8 / 8.05   18.6 / 17.1   34.0 / 32.9   61.7 / 66.9
+constexpr int kWcMostRows = 4608;
+bool wide_takes(const csd_ctx* ctx, const csd_head* hd, int R, int cfg, int slot, bool batch) {
+  const int rows = R * (cfg ? 2 : 1);
+  return wide_width(hd->d) && ctx->chain_mode == CSD_CHAIN_LAYERS && slot != 2 && !batch && !ctx->prof_on && rows > kWcRows && rows <= kWcMostRows &&
+         wide_ready(ctx, hd->d.dtype);
+}
 // One head's denoising chain for R token rows on stream `st` with workspace slot `slot`:
 // begin() enqueues the per-call work (timestep embedding, condition projection, first boundary
 // kernel), step(t) enqueues the kernels of step t.  Two chains can be interleaved launch by launch.
@@ -484,7 +541,10 @@ struct Chain {
   int chains = 1;   // chains that run concurrently with this one (itself included)
   int Rh = 0, W = 0, L = 0, T = 0, tn = kTileN;
   bool gck = false, gfold = false;   // the whole chain runs in the group chain kernel (groupchain.cuh), in its folded form
-  bool pck = false;       // the whole chain runs in the persistent chain kernel (pchain.cuh)
+  bool wck = false;       // the whole chain runs in the wide chain kernel (widechain.cuh)
+  int beside = 0;         // CTAs that the other chain's wide chain kernel holds meanwhile
+  WideCut wc{};
+  int wc_most = 0;        // the most steps of a chunk
   int gc_rows = 0, gc_most = 0;      // its rows (groups x 16) and the most steps of a chunk
   int fcg = 0;            // fp32 head: the whole chain runs in the fp32 chain kernel with groups of this many rows (f32chain.cuh)
   bool fold = false;      // blocks 1.. run as two kernels (fold.cuh) instead of three
@@ -613,16 +673,9 @@ struct Chain {
     int rc = CSD_OK;
     if (gck && (rc = reserve_group_chain())) return rc;
     if (gck) { fold = false; pair = false; }
-    // One wave of 128 x 128 tiles per layer and W = 1024: one persistent kernel per chain (pchain.cuh).  Row blocks are
-    // paired: an odd number is rounded up with a block of rows that belong to no token.
-    {
-      const int row_tiles = (Rh + kTileM - 1) / kTileM, nb = cfg ? (R + 63) / 64 : (R + 127) / 128;
-      const int t128 = (W / kTileN) * row_tiles;
-      pck = kPersistentChains && tc && ctx->chain_mode == CSD_CHAIN_LAYERS && !pair && !gck && slot != 2 && hd->pc_ready &&
-            8 * t128 > ctx->num_sms && 2 * t128 <= ctx->num_sms && W / kTileN == kPcColTiles && row_tiles == nb &&
-            !batch_Rin && !lv_min && !ctx->prof_on && d.C <= kCPad && pchain_kernel_ready(ctx, d.dtype);
-      if (pck) { fold = false; pair = false; }
-    }
+    wck = !gck && wide_takes(ctx, hd, R, cfg, slot, batch_Rin != 0);
+    if (wck && (rc = reserve_wide_chain())) return rc;
+    if (wck) { fold = false; pair = false; }
     // fp32 heads: one persistent kernel per chain, except where a row's bits have to be those of a batched pass
     fcg = !tc && ctx->chain_mode != CSD_CHAIN_LAYERS_PLAIN && !batch_Rin && !ctx->prof_on && fc_pays(ctx, d, Rh) ? fc_rows(ctx, d, R, cfg, chains) : 0;
     ChainWs& ws = ctx->ws[slot];
@@ -666,7 +719,7 @@ struct Chain {
     if (rc) return rc;
     sbuf[0] = ws.s2; sbuf[1] = ws.s;
     if (gck) return launch_group_chain();
-    if (pck) return launch_pchain();
+    if (wck) return launch_wide_chain();
     if (batch_Rin) return launch_batch(0);   // a pass has one step (t = 1): its s is sbuf[1]
     sp.traj_x = traj_x; sp.traj_mu = nullptr; sp.status = ctx->d_err + 1;
     sp.lv1 = lv1; sp.half_logdet = half_logdet; sp.lv_min = 0.0f; sp.lv_max = 0.0f;
@@ -718,55 +771,6 @@ struct Chain {
       else { if (fp) CSD_FOLD_LAUNCH(__nv_bfloat16, 1, FOLD_GATE, true); else CSD_FOLD_LAUNCH(__nv_bfloat16, 1, FOLD_GATE, false); }
     }
 #undef CSD_FOLD_LAUNCH
-    ctx->launches++;
-    return CSD_OK;
-  }
-
-  // The persistent chain kernel: s of every step in the kernel's row order, zeroed counters, the schedule on the
-  // device, one launch of CTA pairs.
-  int launch_pchain() {
-    const csd_head_desc& d = hd->d;
-    ChainWs& ws = ctx->ws[slot];
-    const size_t asz = 2;
-    const int nb0 = cfg ? (R + 63) / 64 : (R + 127) / 128, nb = nb0 + (nb0 & 1);   // row blocks, paired
-    const size_t rows = static_cast<size_t>(nb) * kTileM, G = W / kStatCols;
-    size_t off = 0;
-    auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 1024); return o; };
-    const size_t o_s = take(static_cast<size_t>(Ts) * rows * W * asz), o_ap = take(rows * W * asz), o_v = take(rows * W * asz),
-                 o_st = take(rows * G * 8), o_ep = take(rows * G * kCPad * 4), o_sync = take(static_cast<size_t>(nb / 2) * 4),
-                 o_sched = take(static_cast<size_t>(3) * Ts * 4);
-    int rc = ensure_side(ctx, ctx->pc[slot], off, "the persistent chain buffers");
-    if (rc) return rc;
-    char* b = static_cast<char*>(ctx->pc[slot].base);
-    CUtensorMap tm_s{}, tm_a{}, tm_vv{};
-    if ((rc = make_tmap(ctx, &tm_s, d.dtype, b + o_s, static_cast<uint64_t>(Ts) * rows, W, W, kTileM))) return rc;
-    if ((rc = make_tmap(ctx, &tm_a, d.dtype, b + o_ap, rows, W, W, kTileM))) return rc;
-    if ((rc = make_tmap(ctx, &tm_vv, d.dtype, b + o_v, rows, W, W, kTileM))) return rc;
-    CSD_CUDA(ctx, cudaMemsetAsync(b + o_sync, 0, static_cast<size_t>(nb / 2) * 4, st));
-    float* d_sched = reinterpret_cast<float*>(b + o_sched);
-    CSD_CUDA(ctx, cudaMemcpyAsync(d_sched, sc->a, Ts * sizeof(float), cudaMemcpyHostToDevice, st));
-    CSD_CUDA(ctx, cudaMemcpyAsync(d_sched + Ts, sc->b, Ts * sizeof(float), cudaMemcpyHostToDevice, st));
-    CSD_CUDA(ctx, cudaMemcpyAsync(d_sched + 2 * Ts, sc->sigma, Ts * sizeof(float), cudaMemcpyHostToDevice, st));
-    const dim3 sgrid(static_cast<unsigned>(rows), static_cast<unsigned>((Ts + kCondSteps - 1) / kCondSteps));
-    if (d.dtype == CSD_F16) cond_all_kernel<__half, 128><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__half*>(b + o_s), R, cfg, W, static_cast<int>(rows), Ts);
-    else cond_all_kernel<__nv_bfloat16, 128><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, reinterpret_cast<__nv_bfloat16*>(b + o_s), R, cfg, W, static_cast<int>(rows), Ts);
-    ctx->launches++;
-    CSD_CUDA(ctx, cudaGetLastError());
-    PcParams p{};
-    p.R = R; p.cfg = cfg; p.W = W; p.L = L; p.T = Ts; p.C = d.C; p.sample_last = sample_last; p.nblk = nb; p.cfg_scale = cfg_scale;
-    p.maps = hd->d_pc_maps; p.bias = hd->d_pc_bias; p.sched = d_sched;
-    p.win = hd->win; p.bin = hd->bin; p.wout_t = hd->wout_t; p.bout = hd->bout; p.x_T = x_T; p.eps = eps;
-    p.x0 = x0; p.mu1 = mu1; p.x1 = x1; p.x = ws.x; p.traj_x = traj_x; p.traj_mu = traj_mu;
-    p.stats = reinterpret_cast<float*>(b + o_st); p.epart = reinterpret_cast<float*>(b + o_ep);
-    p.sync = reinterpret_cast<unsigned*>(b + o_sync); p.err = ctx->d_err; p.status = ctx->d_err + 1;
-    cudaLaunchConfig_t lc{};
-    lc.gridDim = dim3(static_cast<unsigned>(nb) * kPcColTiles); lc.blockDim = dim3(kPcThreads); lc.dynamicSmemBytes = kPcSmemBytes; lc.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    lc.attrs = at; lc.numAttrs = 1;
-    if (d.dtype == CSD_F16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, pchain_kernel<__half, 0>, tm_s, tm_a, tm_vv, p));
-    else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, pchain_kernel<__nv_bfloat16, 1>, tm_s, tm_a, tm_vv, p));
     ctx->launches++;
     return CSD_OK;
   }
@@ -833,16 +837,18 @@ struct Chain {
   size_t gc_wrows() const { return static_cast<size_t>(gfold ? 4 * L + 3 : 3 * L + 2) * W; }
   size_t gc_chunk_bytes(int steps) const { return gc_wrows() * ((static_cast<size_t>(steps) * gc_rows + 255) / 256) * 256 * 4; }
 
+  // ensure_side for buffers that a call can do without: a size that could not be had is not asked for again.
+  int have(HostIo& io, size_t& refused, size_t need, const char* what) {
+    if (need <= io.cap) return CSD_OK;
+    const int rc = need < refused ? ensure_side(ctx, io, need, what) : static_cast<int>(CSD_ERR_WORKSPACE);
+    if (rc == CSD_ERR_WORKSPACE && need < refused) refused = need;
+    return rc;
+  }
+
   // Buffers of the group chain kernel.  Shorter chunks cost a launch each and change no bit, so a chunk is halved until its two
   // buffers can be had; where one step does not fit the chain falls back to the layer kernels (gck), which need none of it.
   int reserve_group_chain() {
     gc_rows = (R + (cfg ? 7 : 15)) / (cfg ? 8 : 16) * kGcRows;
-    auto have = [&](HostIo& io, size_t& refused, size_t need, const char* what) {
-      if (need <= io.cap) return static_cast<int>(CSD_OK);
-      const int rc = need < refused ? ensure_side(ctx, io, need, what) : static_cast<int>(CSD_ERR_WORKSPACE);
-      if (rc == CSD_ERR_WORKSPACE && need < refused) refused = need;
-      return rc;
-    };
     int rc = have(ctx->gc[slot], ctx->gc_refused[slot], static_cast<size_t>(Ts) * gc_rows * W * 2, "the condition vectors of all steps");
     gc_most = Ts < kGcMaxSteps ? Ts : kGcMaxSteps;
     while (gc_most > 1 && gc_chunk_bytes(gc_most) > kGcChunkBytes) gc_most = (gc_most + 1) / 2;
@@ -865,8 +871,8 @@ struct Chain {
     CUtensorMap tm_s{};
     if ((rc = make_tmap(ctx, &tm_s, d.dtype, s_all, static_cast<uint64_t>(Ts) * rows, W, W, kTileM))) return rc;
     const dim3 sgrid(static_cast<unsigned>(rows), static_cast<unsigned>((Ts + kCondSteps - 1) / kCondSteps));
-    if (d.dtype == CSD_F16) cond_all_kernel<__half, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, static_cast<__half*>(s_all), R, cfg, W, rows, Ts);
-    else cond_all_kernel<__nv_bfloat16, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, static_cast<__nv_bfloat16*>(s_all), R, cfg, W, rows, Ts);
+    if (d.dtype == CSD_F16) cond_all_kernel<__half, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, static_cast<__half*>(s_all), R, cfg, W, rows, 0, Ts);
+    else cond_all_kernel<__nv_bfloat16, 16><<<sgrid, 128, 0, st>>>(ws.cz, ws.te, static_cast<__nv_bfloat16*>(s_all), R, cfg, W, rows, 0, Ts);
     ctx->launches++;
     CSD_CUDA(ctx, cudaGetLastError());
     cudaStream_t gst = ctx->aux[slot];
@@ -924,8 +930,138 @@ struct Chain {
     return CSD_OK;
   }
 
+  size_t wc_chunk_rows(int steps) const { return static_cast<size_t>(steps) * (wc.part < wc.slots ? wc.part : wc.slots) * kWcRows; }
+  size_t wc_chunk_bytes(int steps) const { return wc_chunk_rows(steps) * (3 * L + 2) * W * 4; }
+
+  // Buffers of the wide chain kernel; where memory is short, shorter chunks (same bits), then the layer kernels (wck), which find
+  // their workspace taken first and everything else given back.
+  int reserve_wide_chain() {
+    if (!wc.slots) wc = wide_cut_alone(ctx, hd->d, R, cfg);
+    int rc = ensure_ws(ctx, ctx->ws[slot], hd->d, Rh, R, Ts);
+    if (rc) return rc;
+    const size_t exchange = wx_layout().total, least = exchange + wc_chunk_rows(1) * W * 2 + 2 * wc_chunk_bytes(1);
+    if (least >= ctx->wx_refused[slot]) { wck = false; return CSD_OK; }
+    const size_t s_refused = ctx->gc_refused[slot], m_refused = ctx->gm_refused[slot];
+    rc = exchange <= ctx->wx[slot].cap ? static_cast<int>(CSD_OK) : ensure_side(ctx, ctx->wx[slot], exchange, "the chain's exchange buffers");
+    wc_most = Ts < kWcMaxSteps ? Ts : kWcMaxSteps;
+    while (wc_most > 1 && wc_chunk_bytes(wc_most) > kWcChunkBytes) --wc_most;
+    for (; !rc; wc_most = (wc_most + 1) / 2) {
+      rc = have(ctx->gc[slot], ctx->gc_refused[slot], wc_chunk_rows(wc_most) * W * 2, "the condition vectors of a chunk of steps");
+      if (!rc) rc = have(ctx->gm[slot], ctx->gm_refused[slot], 2 * wc_chunk_bytes(wc_most) + 256, "the condition products");
+      if (rc != CSD_ERR_WORKSPACE || wc_most == 1) break;
+      rc = CSD_OK;
+    }
+    if (rc != CSD_ERR_WORKSPACE) return rc;
+    ctx->wx_refused[slot] = least; ctx->gc_refused[slot] = s_refused; ctx->gm_refused[slot] = m_refused;
+    ctx->err[0] = 0;
+    wck = false;
+    CSD_CUDA(ctx, cudaStreamSynchronize(st));
+    CSD_CUDA(ctx, cudaStreamSynchronize(ctx->aux[slot]));
+    for (HostIo* io : {&ctx->wx[slot], &ctx->gc[slot], &ctx->gm[slot]}) {
+      if (io->base) CSD_CUDA(ctx, cudaFree(io->base));
+      io->base = nullptr; io->cap = 0;
+    }
+    return CSD_OK;
+  }
+  struct WxLayout { size_t stats, epart, xll, cnt, zeroed, u, v, hsum, total; };
+  WxLayout wx_layout() const {
+    const size_t rows = static_cast<size_t>(wc.nb) * kTileM, G = W / 128;
+    size_t off = 0;
+    auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 1024); return o; };
+    WxLayout l{};
+    l.stats = take(rows * G * 16); l.epart = take(rows * G * (lv_min ? kCPad2 : kCPad) * 8); l.xll = take(rows * kCPad * 8);
+    l.cnt = take(static_cast<size_t>(wc.nb) * 512);
+    l.zeroed = off;              // what precedes starts at zero
+    l.u = take(rows * W * 2); l.v = take(rows * W * 2); l.hsum = take(lv_min ? rows * kCPad * 4 : 0);
+    l.total = off;
+    return l;
+  }
+
+  // The wide chain kernel, chunk by chunk of steps and part by part of the rows: s and the condition products on the slot's
+  // own stream, ahead of the chain.
+  int launch_wide_chain() {
+    const csd_head_desc& d = hd->d;
+    ChainWs& ws = ctx->ws[slot];
+    const WxLayout l = wx_layout();
+    char* const xb = static_cast<char*>(ctx->wx[slot].base);
+    char* const gm = static_cast<char*>(ctx->gm[slot].base);
+    const size_t chunk = wc_chunk_bytes(wc_most);
+    int* const tickets = reinterpret_cast<int*>(gm + 2 * chunk);
+    const bool f16 = d.dtype == CSD_F16, lv = lv_min != nullptr;
+    int rc;
+    CUtensorMap tm_s{}, tm_uu{}, tm_vv{};
+    if ((rc = make_tmap(ctx, &tm_s, d.dtype, ctx->gc[slot].base, wc_chunk_rows(wc_most), W, W, kTileM))) return rc;
+    const uint64_t lines = static_cast<uint64_t>(wc.nb) * kTileM * W / 256;      // u, v as lines of 256 elements: 32 of them a k-block
+    if ((rc = make_plain_tmap(ctx, &tm_uu, d.dtype, xb + l.u, lines)) || (rc = make_plain_tmap(ctx, &tm_vv, d.dtype, xb + l.v, lines))) return rc;
+    CSD_CUDA(ctx, cudaMemsetAsync(xb, 0, l.zeroed, st));
+    cudaStream_t gst = ctx->aux[slot];
+    CSD_CUDA(ctx, cudaEventRecord(ctx->ev_prep[slot], st));
+    CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_prep[slot], 0));
+    WcParams p{};
+    p.R = R; p.cfg = cfg; p.W = W; p.L = L; p.C = d.C; p.T = Ts; p.sample_last = sample_last; p.cfg_scale = cfg_scale;
+    p.maps = hd->d_wc_maps; p.b1 = hd->b1[0]; p.b2 = hd->b2[0]; p.win = hd->win; p.bin = hd->bin; p.wout_t = hd->wout_t; p.bout = hd->bout;
+    p.x_T = x_T; p.eps = eps; p.x = ws.x; p.x0 = x0; p.mu1 = mu1; p.x1 = x1; p.traj_x = traj_x; p.traj_mu = traj_mu;
+    p.u = xb + l.u; p.v = xb + l.v; p.stats = reinterpret_cast<ulonglong2*>(xb + l.stats); p.epart = reinterpret_cast<ulonglong2*>(xb + l.epart);
+    p.xll = reinterpret_cast<ulonglong2*>(xb + l.xll); p.cnt = reinterpret_cast<unsigned*>(xb + l.cnt); p.hsum = reinterpret_cast<float*>(xb + l.hsum);
+    p.lv1 = lv1; p.half_logdet = half_logdet; p.err = ctx->d_err; p.status = ctx->d_err + 1;
+    WmParams m{};
+    m.nkb = W / kBlockK; m.nwt = (3 * L + 2) * W / 256; m.sb = 32; m.wrow = hd->d_wc_rows; m.bias = hd->d_wc_bias; m.err = ctx->d_err;
+    cudaLaunchAttribute at[3];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeLaunchCompletionEvent;
+    at[1].val.launchCompletionEvent.event = ctx->ev_on[slot]; at[1].val.launchCompletionEvent.flags = 0;
+    at[2].id = cudaLaunchAttributeCooperative;      // its CTAs wait for one another
+    at[2].val.cooperative = 1;
+    cudaLaunchConfig_t lc{};
+    lc.attrs = at;
+    // Beside chains that leave most of the GPU free the products take only what is left, so that the next chunk's chain finds
+    // its SMs; a chain that holds most of it takes turns with them.
+    const int held = wc.ctas + beside, free_pairs = (held <= ctx->num_sms / 2 ? ctx->num_sms - held : ctx->num_sms) / 2;
+    // Steps per chunk: one first, because nothing overlaps its products; then twice as many each time, as far as the buffers go.
+    int n = 1, c = 0;
+    for (int t_hi = Ts; t_hi >= 1; n *= 2) {
+      if (t_hi <= 4) n = t_hi;      // (short schedules)
+      if (n > wc_most) n = wc_most;
+      if (n > t_hi) n = t_hi;
+      const int t_lo = t_hi - n + 1;
+      for (int i = 0; i < n; ++i) {
+        p.ca[i] = sc->a[t_lo - 1 + i]; p.cb[i] = sc->b[t_lo - 1 + i];
+        p.s0[i] = lv ? lv_min[t_lo - 1 + i] : sc->sigma[t_lo - 1 + i]; p.s1[i] = lv ? lv_max[t_lo - 1 + i] : 0.0f;
+      }
+      for (int s0 = 0; s0 < wc.slots; s0 += wc.part, ++c) {
+        const int slots = wc.slots - s0 < wc.part ? wc.slots - s0 : wc.part, rows = slots * kWcRows, buf = c & 1;
+        float* const mods = reinterpret_cast<float*>(gm + buf * chunk);
+        if (c >= 2) CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_read[slot][buf], 0));
+        if (c >= 1) CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_on[slot], 0));
+        CSD_CUDA(ctx, cudaMemsetAsync(tickets + buf, 0, sizeof(int), gst));
+        const dim3 sgrid(static_cast<unsigned>(rows), static_cast<unsigned>((n + kCondSteps - 1) / kCondSteps));
+        const float* te = ws.te + static_cast<size_t>(t_lo - 1) * W;
+        if (f16) cond_all_kernel<__half, 128><<<sgrid, 128, 0, gst>>>(ws.cz, te, static_cast<__half*>(ctx->gc[slot].base), R, cfg, W, rows, s0 * kWcRows, n);
+        else cond_all_kernel<__nv_bfloat16, 128><<<sgrid, 128, 0, gst>>>(ws.cz, te, static_cast<__nv_bfloat16*>(ctx->gc[slot].base), R, cfg, W, rows, s0 * kWcRows, n);
+        CSD_CUDA(ctx, cudaGetLastError());
+        m.nst = n * slots; m.ticket = tickets + buf; m.out = mods;
+        int pairs = c == 0 ? ctx->num_sms / 2 : free_pairs;
+        if (pairs > m.nst * m.nwt) pairs = m.nst * m.nwt;
+        lc.gridDim = dim3(static_cast<unsigned>(2 * pairs)); lc.blockDim = dim3(kMgThreads); lc.dynamicSmemBytes = kMgSmemBytes; lc.stream = gst; lc.numAttrs = 1;
+        if (f16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, wide_mods_kernel<0>, hd->Wrows, tm_s, m));
+        else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, wide_mods_kernel<1>, hd->Wrows, tm_s, m));
+        CSD_CUDA(ctx, cudaEventRecord(ctx->ev_mods[slot][buf], gst));
+        CSD_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_mods[slot][buf], 0));
+        p.t_hi = t_hi; p.t_lo = t_lo; p.slot0 = s0; p.slots = slots; p.mods = mods;
+        lc.gridDim = dim3(static_cast<unsigned>((wc.halves == 2 ? slots : (slots + 1) / 2) * 2 * (W / 128))); lc.blockDim = dim3(kWcThreads);
+        lc.dynamicSmemBytes = wc_layout(L, lv ? kCPad2 : kCPad, wc.halves).total + 1024; lc.stream = st; lc.numAttrs = 3;
+        CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, wide_kernel(d.dtype, lv, wc.halves), tm_uu, tm_vv, p));
+        CSD_CUDA(ctx, cudaEventRecord(ctx->ev_read[slot][buf], st));
+        ctx->launches += 3;
+      }
+      t_hi = t_lo - 1;
+    }
+    return CSD_OK;
+  }
+
   int step(int t) {
-    if (gck || pck || fcg) return CSD_OK;   // already enqueued by begin()
+    if (gck || wck || fcg) return CSD_OK;   // already enqueued by begin()
     const csd_head_desc& d = hd->d;
     ChainWs& ws = ctx->ws[slot];
     cur_t = t;
@@ -1017,6 +1153,28 @@ struct Chain {
     return launch_step(t > 1 ? STEP_MID : STEP_LAST);
   }
 };
+
+// The two chains of a round in the wide chain kernel: side by side in the forms that take the least time by the model, as long as they
+// leave some SMs to the condition products; else one after the other.
+void place_wide_chains(Chain& a, Chain& b) {
+  csd_ctx* ctx = a.ctx;
+  if (!wide_takes(ctx, a.hd, a.R, a.cfg, a.slot, false) || !wide_takes(ctx, b.hd, b.R, b.cfg, b.slot, false)) return;
+  const csd_head_desc &da = a.hd->d, &db = b.hd->d;
+  double best = 0.0;
+  for (int i = 0; i < 4; ++i) {
+    const int ha = 1 + (i & 1), hb = 1 + (i >> 1);
+    if ((ha == 2 && !wide_halves(da)) || (hb == 2 && !wide_halves(db))) continue;
+    const WideCut ca = wide_cut(ctx, da, a.R, a.cfg, ha), cb = wide_cut(ctx, db, b.R, b.cfg, hb);
+    const int held = ca.ctas + cb.ctas;
+    if (ca.part < ca.slots || cb.part < cb.slots || held > ctx->num_sms - 18) continue;
+    const double ta = wide_step_us(da, ha), tb = wide_step_us(db, hb);
+    const double us = wide_us(ctx, ta > tb ? ta : tb, ta * ca.ctas + tb * cb.ctas, wide_mods_sm_us(da, ca.slots) + wide_mods_sm_us(db, cb.slots), held);
+    if (best > 0.0 && us >= best) continue;
+    best = us;
+    a.wc = ca; b.wc = cb; a.beside = cb.ctas; b.beside = ca.ctas;
+  }
+  if (best <= 0.0) a.st = b.st;
+}
 
 int run_chain(csd_ctx* ctx, int slot, cudaStream_t st, const csd_head* hd, const csd_schedule* sc, int R, int cfg,
               float cfg_scale, const float* z, const float* x_T, const float* eps, int sample_last, float* x0,
@@ -1264,7 +1422,7 @@ int csd_destroy(csd_ctx* c) {
   if (c->bn.base) cudaFree(c->bn.base);
   for (HostIo& b : c->gc) if (b.base) cudaFree(b.base);
   for (HostIo& b : c->gm) if (b.base) cudaFree(b.base);
-  for (HostIo& b : c->pc) if (b.base) cudaFree(b.base);
+  for (HostIo& b : c->wx) if (b.base) cudaFree(b.base);
   if (c->d_err) cudaFree(c->d_err);
   cudaGetLastError();
   delete c;
@@ -1490,7 +1648,7 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
   const size_t f_bfsh = put(w->bfada, W), f_bfsc = put(w->bfada + W, W);
   // folded blocks: c1_k = W1_k (1 + bscale_k), c2_k = W1_k bshift_k + b1_k  (double accumulation, rounded once)
   const bool folded = d.dtype != CSD_F32 && L >= 2;
-  // the group chain kernel and the persistent chain kernel fold every block, the first included
+  // the group chain kernel folds every block, the first included
   const bool gck = d.dtype != CSD_F32 && W % 512 == 0 && W <= static_cast<size_t>(kGcMaxW) && !d.var_out;
   const size_t kfold0 = gck ? 0 : 1;      // first block that has folded weights
   std::vector<size_t> f_c1(L, 0), f_c2(L, 0);
@@ -1598,25 +1756,28 @@ int csd_head_create(csd_ctx* ctx, const csd_head_desc* desc, const csd_head_weig
           (rc = make_tmap(ctx, &h->Wx, d.dtype, h->xblob, nx, W, W, kTileM))) { csd_head_destroy(h); return rc; }
       h->gc_ready = true;
     }
-    if (gck && W / kTileN == static_cast<size_t>(kPcColTiles)) {
-      // tables of the persistent chain kernel: phases B, (W1_k, GATE_k) for every block, F
-      const size_t NP = 2 * L + 2;
-      std::vector<CUtensorMap> maps(2 * NP);
-      std::vector<const float*> bt(3 * NP, nullptr);
-      maps[0] = h->tm[0].Wss[0]; bt[0] = h->bsc[0];
+    if (wide_width(d)) {
+      std::vector<CUtensorMap> maps;
+      for (size_t k = 0; k < L; ++k) { maps.push_back(h->tm[0].W1[k]); maps.push_back(h->tm[0].W2[k]); }
+      std::vector<int> rows;
+      std::vector<float> bias;
+      auto pair_rows = [&](size_t row, const float* shift, const float* scale) {     // shift | scale rows, interleaved by 64
+        for (size_t r = 0; r < 2 * W; r += 256) rows.push_back(static_cast<int>(row + r));
+        for (size_t j = 0; j < W; j += kStatCols) { bias.insert(bias.end(), shift + j, shift + j + kStatCols); bias.insert(bias.end(), scale + j, scale + j + kStatCols); }
+      };
       for (size_t k = 0; k < L; ++k) {
-        const size_t w1 = 1 + 2 * k, gt = 2 + 2 * k;
-        maps[w1] = h->Wf_half[k]; maps[NP + w1] = h->tm[0].W1[k]; bt[3 * w1] = h->c1[k]; bt[3 * w1 + 1] = h->c2[k];
-        maps[gt] = k + 1 < L ? h->Wgs_half[k] : h->tm[0].Wg[k]; maps[NP + gt] = h->tm[0].W2[k];
-        bt[3 * gt] = h->bg[k]; bt[3 * gt + 1] = h->b2[k]; bt[3 * gt + 2] = k + 1 < L ? h->bsc[k + 1] : nullptr;
+        const float* ba = w->bada + k * 3 * W;
+        pair_rows(5 * k * W, ba, ba + W);
+        for (size_t r = 0; r < W; r += 256) rows.push_back(~static_cast<int>((5 * k + 2) * W + r));
+        bias.insert(bias.end(), ba + 2 * W, ba + 3 * W);
       }
-      maps[NP - 1] = h->tm[0].Wfss; bt[3 * (NP - 1)] = h->bfsh; bt[3 * (NP - 1) + 1] = h->bfsc;
-      maps[NP] = h->tm[0].W1[0]; maps[2 * NP - 1] = h->tm[0].W1[0];   // unused entries: any valid map
-      if (cudaMalloc(&h->d_pc_maps, maps.size() * sizeof(CUtensorMap)) != cudaSuccess ||
-          cudaMalloc(&h->d_pc_bias, bt.size() * sizeof(float*)) != cudaSuccess) { cudaGetLastError(); return bail(CSD_ERR_WORKSPACE, "cannot allocate device memory for the persistent-chain tables"); }
-      if (cudaMemcpy(h->d_pc_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess ||
-          cudaMemcpy(h->d_pc_bias, bt.data(), bt.size() * sizeof(float*), cudaMemcpyHostToDevice) != cudaSuccess) return bail(CSD_ERR_CUDA, "persistent-chain table upload failed");
-      h->pc_ready = true;
+      pair_rows(5 * L * W, w->bfada, w->bfada + W);
+      if (cudaMalloc(&h->d_wc_rows, rows.size() * sizeof(int)) != cudaSuccess || cudaMalloc(&h->d_wc_bias, bias.size() * sizeof(float)) != cudaSuccess ||
+          cudaMalloc(&h->d_wc_maps, maps.size() * sizeof(CUtensorMap)) != cudaSuccess) { cudaGetLastError(); return bail(CSD_ERR_WORKSPACE, "cannot allocate device memory for the wide-chain tables"); }
+      if (cudaMemcpy(h->d_wc_rows, rows.data(), rows.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
+          cudaMemcpy(h->d_wc_bias, bias.data(), bias.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
+          cudaMemcpy(h->d_wc_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess) return bail(CSD_ERR_CUDA, "wide-chain table upload failed");
+      if ((rc = make_tmap(ctx, &h->Wrows, d.dtype, h->Wss[0], (5 * L + 2) * W, W, W, kTileM))) { csd_head_destroy(h); return rc; }
     }
   }
   *out = h;
@@ -1633,10 +1794,11 @@ int csd_head_destroy(csd_head* h) {
   if (h->wblob) cudaFree(h->wblob);
   if (h->fblob) cudaFree(h->fblob);
   if (h->xblob) cudaFree(h->xblob);
-  if (h->d_pc_maps) cudaFree(h->d_pc_maps);
-  if (h->d_pc_bias) cudaFree(h->d_pc_bias);
   if (h->d_gc_maps) cudaFree(h->d_gc_maps);
   if (h->d_gc_rows) cudaFree(h->d_gc_rows);
+  if (h->d_wc_maps) cudaFree(h->d_wc_maps);
+  if (h->d_wc_rows) cudaFree(h->d_wc_rows);
+  if (h->d_wc_bias) cudaFree(h->d_wc_bias);
   cudaGetLastError();
   delete h;
   return CSD_OK;
@@ -1968,6 +2130,7 @@ static int round_impl(csd_ctx* ctx, const csd_head* head_q, const csd_head* head
   Chain cp = bonus ? Chain{ctx, 1, st_p, head_p, sched_p, Rp, cfg, cfg_scale, bb.z, bb.x_T, bb.eps, 1, bb.x0, bb.mu1, nullptr}
                    : Chain{ctx, 1, st_p, head_p, sched_p, R, cfg, cfg_scale, z_p, x_T, eps, 0, nullptr, mu1_p, nullptr};
   cq.chains = cp.chains = 2;
+  place_wide_chains(cq, cp);
   rc = cp.begin();
   int rc2 = cq.begin();
   for (int t = sched_p->T; t >= 1 && !rc && !rc2; --t) {
@@ -2121,6 +2284,7 @@ int csd_round_lv(csd_ctx* ctx, const csd_head* head_q, const csd_head* head_p, c
   Chain cp = make_lv_chain(ctx, 1, ctx->side[1 - sq], head_p, &vp, sched_p, R, cfg, cfg_scale, z_p, x_T, eps, 0, nullptr, mu1_p,
                            lv1_p, half_logdet_p, nullptr);
   cq.chains = cp.chains = 2;
+  place_wide_chains(cq, cp);
   rc = cp.begin();
   int rc2 = cq.begin();
   for (int t = sched_p->T; t >= 1 && !rc && !rc2; --t) {

@@ -104,15 +104,15 @@ __device__ __forceinline__ int group_row_token(int rho, int cfg, int* rep) {
 }
 
 // s_t = SiLU(cz + te_t) of every step, in that row order and operand format: s_all[(t - 1) rows + rho][col]; rows of tokens
-// beyond R are zero.  A block keeps its row of cz in registers over kCondSteps steps: one step per block was bound by the
+// beyond R are zero.  rows rows from rho0 on, T steps from te on.  A block keeps its row of cz in registers over kCondSteps steps: one step per block was bound by the
 // trip to memory (115 us for 1024 rows of 1024 and 100 steps, 210 MB written).
 constexpr int kCondSteps = 10;
 template <typename ACT, int G>
 __global__ void __launch_bounds__(128) cond_all_kernel(const float* __restrict__ cz, const float* __restrict__ te, ACT* __restrict__ s_all,
-                                                       int R, int cfg, int W, int rows, int T) {
+                                                       int R, int cfg, int W, int rows, int rho0, int T) {
   const int rho = blockIdx.x, t0 = blockIdx.y * kCondSteps, t1 = min(T, t0 + kCondSteps);
   int rep;
-  const int i = group_row_token<G>(rho, cfg, &rep);
+  const int i = group_row_token<G>(rho0 + rho, cfg, &rep);
   for (int j = threadIdx.x; j < W / 8; j += blockDim.x) {
     uint4* dst = reinterpret_cast<uint4*>(s_all + static_cast<size_t>(rho) * W) + j;     // 8 values per store
     const size_t step = static_cast<size_t>(rows) * W / 8;

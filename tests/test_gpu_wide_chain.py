@@ -1,0 +1,154 @@
+"""The wide chain kernel (more than 256 head rows, 16-bit heads, W a multiple of 256) at its edges: the fewest and the most rows it takes
+and one more on either side, ragged and odd slots, rows in several parts, every width class, chunk boundaries, predicted variances,
+little memory; its error against the layer kernels'."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import csd_oracle as orc
+from paper_2411_11925_b200 import inputs as gen
+from _parity import TOL_X
+from test_gpu_parity import _check, _wl
+
+pytestmark = pytest.mark.gpu
+
+H = gen.HeadSpec
+
+
+def _draft_both_modes(dr):
+    from paper_2411_11925_b200 import api
+    got = []
+    for mode in (api.Context.CHAIN_LAYERS, api.Context.CHAIN_LAYERS_PLAIN):
+        dr.ctx.set_chain_mode(mode)
+        l0 = dr.ctx.launch_count()
+        dr.draft()
+        dr.ctx.sync()
+        got.append((dr.x0.clone(), dr.ctx.launch_count() - l0))
+    dr.ctx.set_chain_mode(api.Context.CHAIN_LAYERS)
+    return got
+
+
+@pytest.mark.parametrize("kw", [
+    dict(B=257, gamma=1, T=3, draft=H(1, 768, 64), target=H(2, 1024, 64)),                                            # one row in the second slot
+    dict(B=43, gamma=3, T=4, cfg=True, cfg_scale=2.0, operand="bf16", draft=H(2, 1280, 64), target=H(1, 768, 128)),   # one token in the last row block
+    dict(B=33, gamma=8, T=6, cfg=True, cfg_scale=3.0, draft=H(3, 1024, 64), target=H(1, 1536, 64)),                   # three slots: a group of one
+    dict(B=130, gamma=5, T=2, draft=H(1, 2048, 64), target=H(2, 1792, 64)),                                           # widest; ragged
+])
+def test_wide_chain_round_matches_checker_and_fused_round_matches_the_calls(kw):
+    from paper_2411_11925_b200.runner import DeviceRound
+    inp = gen.make_round_inputs(_wl(**{"bf16": True, **kw}))
+    _, a, _ = _check(inp, f"wide chain {kw}")
+    dr = DeviceRound(inp)
+    dr.fused_round()          # other forms of the kernel (slots a group), another order of launches: the same bits
+    b = dr.results()
+    for k in ("x0", "mu1_q", "mu1_p", "logratio"):
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+    dr.ctx.close()
+
+
+@pytest.mark.parametrize("rows,W,wide", [(256, 1024, False), (258, 1024, True), (4608, 768, True), (4610, 768, False), (3074, 1536, True), (1000, 640, False)])
+def test_rows_and_widths_it_takes(rows, W, wide):
+    from paper_2411_11925_b200.runner import DeviceRound
+    dr = DeviceRound(gen.make_round_inputs(_wl(bf16=True, B=rows // 2, gamma=1, T=5, cfg=True, cfg_scale=2.0, draft=H(2, W, 64), target=H(1, 128, 64))))
+    (x, n), (y, m) = _draft_both_modes(dr)
+    assert m == 5 * 8 + 5 and (n <= 16) == wide, (n, m)          # three launches a chunk and part of the rows, five or eight a step
+    assert float((x - y).abs().max()) <= TOL_X["f16"] / 4
+    dr.ctx.close()
+
+
+@pytest.mark.parametrize("T", [4, 5, 17, 70])       # one chunk; 1 + 4; 1, 2, 4, ..; more than a launch's steps
+def test_trajectory_across_chunks_of_steps(T):
+    from paper_2411_11925_b200 import api
+    from paper_2411_11925_b200.runner import DeviceRound
+    dr = DeviceRound(gen.make_round_inputs(_wl(bf16=True, B=150, gamma=2, T=T, draft=H(1, 768, 64), target=H(1, 128, 64))))
+    dr.draft_traj()
+    dr.ctx.sync()
+    x, mu = dr.traj_x.clone(), dr.traj_mu.clone()
+    dr.draft()
+    dr.ctx.sync()
+    assert bool((x[-1] == dr.x0).all()) and bool((mu[-1] == dr.mu1_q).all())
+    dr.ctx.set_chain_mode(api.Context.CHAIN_LAYERS_PLAIN)
+    dr.draft_traj()
+    dr.ctx.sync()
+    # both carry their own rounding
+    assert float((x - dr.traj_x).abs().max()) <= TOL_X["f16"] / 4 and float((mu - dr.traj_mu).abs().max()) <= TOL_X["f16"] / 4
+    dr.ctx.close()
+
+
+def test_little_memory_left_shorter_chunks_and_the_same_bits():
+    from paper_2411_11925_b200.runner import DeviceRound
+    # 600 rows of 2 x 1024, 40 steps: 3 x 256 x 8 x 1024 x 4 = 25 MB of condition products a step
+    inp = gen.make_round_inputs(_wl(bf16=True, B=600, gamma=1, T=40, draft=H(2, 1024, 64), target=H(1, 128, 64)))
+    ref = DeviceRound(inp)
+    (want, n), (_, m) = _draft_both_modes(ref)
+    tight, none = DeviceRound(inp), DeviceRound(inp)
+    got = torch.empty_like(want)
+    torch.cuda.synchronize()
+    hog = []
+
+    def leave(mb):
+        while (free := torch.cuda.mem_get_info()[0]) > (mb + 4) << 20:
+            hog.append(torch.empty((free - (mb << 20)) >> 21 << 21, dtype=torch.uint8, device="cuda"))
+
+    try:
+        leave(240)
+        l0 = tight.ctx.launch_count()
+        tight.draft()
+        tight.ctx.sync()
+        assert n < tight.ctx.launch_count() - l0 < n + 60
+        got.copy_(tight.x0)
+        assert bool((got == want).all())
+        tight.ctx.close()
+        leave(40)                                                   # room for the workspace, not for the products
+        l0 = none.ctx.launch_count()
+        none.draft()
+        none.ctx.sync()
+        assert none.ctx.launch_count() - l0 > n + 60
+        assert float((none.x0 - want).abs().max()) <= TOL_X["f16"] / 4
+    finally:
+        hog.clear()
+        torch.cuda.empty_cache()
+    for d in (ref, none):
+        d.ctx.close()
+
+
+def test_captured_round_replays():
+    from paper_2411_11925_b200 import api
+    from paper_2411_11925_b200.runner import DeviceRound
+    side = torch.cuda.Stream()
+    dr = DeviceRound(gen.make_round_inputs(_wl(bf16=True, B=40, gamma=8, T=9, draft=H(1, 768, 64), target=H(2, 1024, 64))), ctx=api.Context(0, side))
+    torch.cuda.synchronize()
+    dr.fused_round()                                  # workspaces
+    want = dr.results()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=side):
+        dr.fused_round()
+    dr.x0.zero_()
+    dr.mu1_p.zero_()
+    torch.cuda.synchronize()
+    g.replay()
+    torch.cuda.synchronize()
+    got = dr.results()
+    for k in ("x0", "mu1_q", "mu1_p", "logratio", "n_accept"):
+        np.testing.assert_array_equal(got[k], want[k], err_msg=k)
+    dr.ctx.close()
+
+
+@pytest.mark.parametrize("op", ["f16", "bf16"])
+def test_default_mode_is_as_precise_as_three_kernels_per_block(op):
+    # relative error (2-norm) of 4 x 300 tokens against the checker, wide chain over plain layer kernels: the same roundings, sums in another
+    # order; 1.00 +- 0.02 over such draws
+    from paper_2411_11925_b200 import api
+    from paper_2411_11925_b200.runner import DeviceRound
+    inps = [gen.make_round_inputs(_wl(bf16=True, operand=op, B=300, gamma=1, T=12, draft=H(3, 768, 128), target=H(1, 128, 64)), seed_offset=i) for i in range(4)]
+    err = {}
+    for inp in inps:
+        inp.w_q = inps[0].w_q
+        ref = orc.denoise(orc.make_mlp_head(inp.w_q, inp.z_q, inp.tfeat, False, 1.0), orc.ddpm_schedule(inp.beta, 1.0), inp.x_T, inp.eps)["x0"]
+        dr = DeviceRound(inp)
+        for mode, (x, _) in zip((api.Context.CHAIN_LAYERS, api.Context.CHAIN_LAYERS_PLAIN), _draft_both_modes(dr)):
+            err.setdefault(mode, []).append(float(np.linalg.norm(x.cpu().numpy() - ref) / np.linalg.norm(ref)))
+        dr.ctx.close()
+    ratio = np.exp(np.mean(np.log(err[api.Context.CHAIN_LAYERS])) - np.mean(np.log(err[api.Context.CHAIN_LAYERS_PLAIN])))
+    print("wide chain error over layer kernels'", op, ratio, err)
+    assert ratio <= 1.07, (ratio, err)
