@@ -1006,13 +1006,13 @@ struct Chain {
     p.lv1 = lv1; p.half_logdet = half_logdet; p.err = ctx->d_err; p.status = ctx->d_err + 1;
     WmParams m{};
     m.nkb = W / kBlockK; m.nwt = (3 * L + 2) * W / 256; m.sb = 32; m.wrow = hd->d_wc_rows; m.bias = hd->d_wc_bias; m.err = ctx->d_err;
-    cudaLaunchAttribute at[3];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     at[1].id = cudaLaunchAttributeLaunchCompletionEvent;
     at[1].val.launchCompletionEvent.event = ctx->ev_on[slot]; at[1].val.launchCompletionEvent.flags = 0;
-    at[2].id = cudaLaunchAttributeCooperative;      // its CTAs wait for one another
-    at[2].val.cooperative = 1;
+    // (Not a cooperative launch: only the CTAs of a row block, neighbours in the grid, wait for each other, so a launch of which some groups
+    // have no SM yet gets on; and a cooperative one fails under the profiler.)
     cudaLaunchConfig_t lc{};
     lc.attrs = at;
     // Beside chains that leave most of the GPU free the products take only what is left, so that the next chunk's chain finds
@@ -1050,7 +1050,7 @@ struct Chain {
         CSD_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_mods[slot][buf], 0));
         p.t_hi = t_hi; p.t_lo = t_lo; p.slot0 = s0; p.slots = slots; p.mods = mods;
         lc.gridDim = dim3(static_cast<unsigned>((wc.halves == 2 ? slots : (slots + 1) / 2) * 2 * (W / 128))); lc.blockDim = dim3(kWcThreads);
-        lc.dynamicSmemBytes = wc_layout(L, lv ? kCPad2 : kCPad, wc.halves).total + 1024; lc.stream = st; lc.numAttrs = 3;
+        lc.dynamicSmemBytes = wc_layout(L, lv ? kCPad2 : kCPad, wc.halves).total + 1024; lc.stream = st; lc.numAttrs = 2;
         CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, wide_kernel(d.dtype, lv, wc.halves), tm_uu, tm_vv, p));
         CSD_CUDA(ctx, cudaEventRecord(ctx->ev_read[slot][buf], st));
         ctx->launches += 3;
