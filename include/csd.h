@@ -104,7 +104,10 @@ typedef struct {
 /* Context: owns a growable device workspace and the stream association.  `cuda_stream` is a
  * cudaStream_t (NULL = legacy default stream).  csd_destroy synchronises the stream and frees.
  * Several contexts, also on different devices (ordinals below 64), may live in one process.  Every call
- * makes the context's device current while it runs and puts the caller's current device back on return. */
+ * makes the context's device current while it runs and puts the caller's current device back on return.
+ * Calls may be captured into CUDA graphs once a call of the same sizes has been made (a captured call cannot grow the
+ * workspace).  What a captured call used stays allocated until csd_destroy, also where a later call needs more and gets
+ * memory of its own: a graph may be launched as long as its context and heads live. */
 int csd_create(csd_ctx **out, int device, void *cuda_stream);
 int csd_destroy(csd_ctx *ctx);
 const char *csd_last_error(const csd_ctx *ctx);
@@ -136,8 +139,8 @@ int64_t csd_launch_count(const csd_ctx *ctx);
  *                       error is that of three kernels per block.  The two chains of a round run side by side where
  *                       their CTAs leave SMs to the condition products, else one after the other.  Its buffers, kept by
  *                       the context per chain of a round: two chunks of condition products, fp32, (3 L + 2) W x rows x
- *                       steps, at most 1 GB each as long as one step is less (1024 rows of 6 x 1024: 12 steps, 1 GB), the
- *                       condition vectors of a chunk, operands and partials of one step.  Where the device has less
+ *                       steps, and the condition vectors of a chunk, at most 2 GB together as long as one step is less
+ *                       (1024 rows of 6 x 1024: 12 steps); operands and partials of one step.  Where the device has less
  *                       free, chunks are shorter (the same bits); where not even one step fits, the layer kernels run.
  *                     - A chain of few rows on a 16-bit head with W in {512, 1024, 1536} and var_out = 0 (groups of
  *                       16 tokens, or 8 with guidance: up to 33, 15 and 7 groups) runs as the group chain kernel:

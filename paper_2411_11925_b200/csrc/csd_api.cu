@@ -43,15 +43,17 @@ struct ChainWs {
   void* ap = nullptr;   // a' = h (1 + scale) of the folded blocks
   float* hid = nullptr; // hidden layer of the timestep embedding [T, W]
   bool owned = true;    // false: base is memory the library did not allocate and must never free or grow
+  bool in_graph = false;
 };
 
 constexpr int kMaxDevices = 64;   // device ordinals the per-device tables below cover
 
 struct ProfRec { cudaEvent_t a, b; int cls; double flops; };
 
-struct HostIo {  // device mirrors for csd_round_host
+struct HostIo {  // a device buffer that grows on demand
   void* base = nullptr;
   size_t cap = 0;
+  bool in_graph = false;   // a captured call used it: its graph holds the address
 };
 
 }  // namespace
@@ -68,12 +70,13 @@ struct csd_ctx {
   int chain_mode = CSD_CHAIN_LAYERS;   // csd_set_chain_mode
   EncodeTiledFn encode = nullptr;
   ChainWs ws[3];   // draft chain, target chain, static-scratch calls
-  HostIo io;
+  std::vector<void*> in_graphs;   // replaced buffers whose addresses graphs hold: freed with the context
+  HostIo io;       // device mirrors for csd_round_host
   HostIo un;       // csd_verify_unaligned: per-row noise terms
   HostIo bn;       // csd_bonus_token: samples of every sequence before the selection
   HostIo sp;       // csd_verify_single_path: schedule constants, mu^p of one pass, running log-ratio
-  HostIo gc[2];    // group and wide chain kernels (per chain slot): s of all steps, or of a chunk of steps
-  HostIo gm[2];    // their condition products: two chunks of steps
+  HostIo gc[2];    // group chain kernel (per chain slot): s of all steps
+  HostIo gm[2];    // group and wide chain kernels: condition products of two chunks of steps (wide: s of a chunk before them)
   HostIo wx[2];    // wide chain kernel: what its column tiles exchange
   size_t gc_refused[2] = {SIZE_MAX, SIZE_MAX}, gm_refused[2] = {SIZE_MAX, SIZE_MAX}, wx_refused[2] = {SIZE_MAX, SIZE_MAX};   // (wx: all of a wide chain's) sizes that could not be had: not asked for again
   cudaStream_t aux[2] = {nullptr, nullptr};        // (per chain slot) where they are formed
@@ -242,21 +245,45 @@ WsLayout ws_layout(const csd_head_desc& d, int Rh, int R, int T) {
   return l;
 }
 
+bool capturing(const csd_ctx* ctx) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &s) != cudaSuccess) { cudaGetLastError(); return false; }
+  return s != cudaStreamCaptureStatusNone;
+}
+
+// Gives a buffer up, once nothing in flight uses it; what a graph may still use on its next launch stays until csd_destroy.
+template <typename Buf>
+int give_up(csd_ctx* ctx, Buf& b) {
+  void* const base = b.base;
+  const bool keep = b.in_graph;
+  b.base = nullptr; b.cap = 0; b.in_graph = false;
+  if (base && keep) ctx->in_graphs.push_back(base);
+  else if (base) CSD_CUDA(ctx, cudaFree(base));
+  return CSD_OK;
+}
+
+// At least need bytes in b for the call that is being made.
+template <typename Buf>
+int ensure_buffer(csd_ctx* ctx, Buf& b, size_t need, const char* what) {
+  if (need > b.cap) {
+    CSD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    for (int i = 0; i < 2; ++i) { CSD_CUDA(ctx, cudaStreamSynchronize(ctx->side[i])); CSD_CUDA(ctx, cudaStreamSynchronize(ctx->aux[i])); }
+    if (int rc = give_up(ctx, b)) return rc;
+    if (cudaMalloc(&b.base, need) != cudaSuccess) {
+      cudaGetLastError();
+      b.base = nullptr;
+      return fail(ctx, CSD_ERR_WORKSPACE, "cannot allocate %zu bytes for %s", need, what);
+    }
+    b.cap = need;
+  }
+  b.in_graph = b.in_graph || capturing(ctx);
+  return CSD_OK;
+}
+
 int ensure_ws(csd_ctx* ctx, ChainWs& ws, const csd_head_desc& d, int Rh, int R, int T) {
   const WsLayout l = ws_layout(d, Rh, R, T);
-  if (l.total > ws.cap) {
-    if (!ws.owned) return fail(ctx, CSD_ERR_WORKSPACE, "the fixed scratch holds %zu bytes, this call needs %zu", ws.cap, l.total);
-    CSD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    for (int i = 0; i < 2; ++i) CSD_CUDA(ctx, cudaStreamSynchronize(ctx->side[i]));
-    if (ws.base) CSD_CUDA(ctx, cudaFree(ws.base));
-    ws.base = nullptr;
-    ws.cap = 0;
-    if (cudaMalloc(&ws.base, l.total) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(ctx, CSD_ERR_WORKSPACE, "cannot allocate %zu bytes of workspace", l.total);
-    }
-    ws.cap = l.total;
-  }
+  if (l.total > ws.cap && !ws.owned) return fail(ctx, CSD_ERR_WORKSPACE, "the fixed scratch holds %zu bytes, this call needs %zu", ws.cap, l.total);
+  if (int rc = ensure_buffer(ctx, ws, l.total, "the workspace")) return rc;
   char* b = static_cast<char*>(ws.base);
   ws.zc = b + l.zc; ws.s = b + l.s; ws.u = b + l.u; ws.v = b + l.v;
   ws.cz = reinterpret_cast<float*>(b + l.cz); ws.te = reinterpret_cast<float*>(b + l.te);
@@ -433,8 +460,6 @@ bool fold_kernels_ready(const csd_ctx* ctx, const csd_head_desc& d) {
   return k == 1;
 }
 
-int ensure_side(csd_ctx* ctx, HostIo& io, size_t need, const char* what);
-
 // Clusters of the group chain kernel for width W that the device holds at a time (0: it cannot run), and its opt-ins, once
 // per device and operand type.
 template <typename ACT, int FMT>
@@ -520,7 +545,7 @@ WideCut wide_cut_alone(const csd_ctx* ctx, const csd_head_desc& d, int R, int cf
   auto us = [&](const WideCut& c) { const double t = wide_step_us(d, c.halves); return wide_us(ctx, t, t * c.ctas, wide_mods_sm_us(d, c.slots), c.ctas); };
   return us(one) <= us(two) ? one : two;
 }
-constexpr size_t kWcChunkBytes = size_t(1) << 30;     // most bytes of condition products of one chunk of steps
+constexpr size_t kWcBufferBytes = size_t(2) << 30;    // most bytes of a chunk of steps: s and two buffers of condition products
 // More than one slot of rows, up to what two-slot groups of 1024-wide heads cover at a time.  Beyond that the layer kernels' waves of tiles
 // fill the GPU as well, and the chain's hand-overs cost more than the dense product of the conditions saves.  ms a round of 20 steps with
 // guidance, before (persistent chain or layer kernels) / this kernel, at 512, 1024, 2048, 4096 and 8192 head rows of each head:
@@ -837,24 +862,28 @@ struct Chain {
   size_t gc_wrows() const { return static_cast<size_t>(gfold ? 4 * L + 3 : 3 * L + 2) * W; }
   size_t gc_chunk_bytes(int steps) const { return gc_wrows() * ((static_cast<size_t>(steps) * gc_rows + 255) / 256) * 256 * 4; }
 
-  // ensure_side for buffers that a call can do without: a size that could not be had is not asked for again.
+  // ensure_buffer for buffers that a call can do without: a size that could not be had is not asked for again.
   int have(HostIo& io, size_t& refused, size_t need, const char* what) {
-    if (need <= io.cap) return CSD_OK;
-    const int rc = need < refused ? ensure_side(ctx, io, need, what) : static_cast<int>(CSD_ERR_WORKSPACE);
+    const int rc = need <= io.cap || need < refused ? ensure_buffer(ctx, io, need, what) : static_cast<int>(CSD_ERR_WORKSPACE);
     if (rc == CSD_ERR_WORKSPACE && need < refused) refused = need;
     return rc;
   }
 
-  // Buffers of the group chain kernel.  Shorter chunks cost a launch each and change no bit, so a chunk is halved until its two
-  // buffers can be had; where one step does not fit the chain falls back to the layer kernels (gck), which need none of it.
+  // Buffers of the group chain kernel: bytes by the steps that a call has and the limit, so that no call of fewer steps or rows has to replace
+  // them.  Shorter chunks cost a launch each and change no bit, so the buffers are halved until they can be had; where one step does
+  // not fit the chain falls back to the layer kernels (gck), which need none of it.
   int reserve_group_chain() {
     gc_rows = (R + (cfg ? 7 : 15)) / (cfg ? 8 : 16) * kGcRows;
     int rc = have(ctx->gc[slot], ctx->gc_refused[slot], static_cast<size_t>(Ts) * gc_rows * W * 2, "the condition vectors of all steps");
     gc_most = Ts < kGcMaxSteps ? Ts : kGcMaxSteps;
-    while (gc_most > 1 && gc_chunk_bytes(gc_most) > kGcChunkBytes) gc_most = (gc_most + 1) / 2;
-    if (!rc)
-      while ((rc = have(ctx->gm[slot], ctx->gm_refused[slot], 2 * gc_chunk_bytes(gc_most), "the condition products")) == CSD_ERR_WORKSPACE && gc_most > 1)
-        gc_most = (gc_most + 1) / 2;
+    const size_t step = gc_chunk_bytes(1), all = gc_chunk_bytes(gc_most);
+    size_t chunk = all < kGcChunkBytes ? all : kGcChunkBytes;
+    if (chunk < step) chunk = step;
+    while (!rc && (rc = have(ctx->gm[slot], ctx->gm_refused[slot], 2 * chunk, "the condition products")) == CSD_ERR_WORKSPACE && chunk > step) {
+      rc = CSD_OK;
+      chunk = chunk / 2 < step ? step : chunk / 2;
+    }
+    while (gc_most > 1 && gc_chunk_bytes(gc_most) > chunk) gc_most = (gc_most + 1) / 2;
     if (rc == CSD_ERR_WORKSPACE) { gck = gfold = false; ctx->err[0] = 0; rc = CSD_OK; }
     return rc;
   }
@@ -932,45 +961,44 @@ struct Chain {
 
   size_t wc_chunk_rows(int steps) const { return static_cast<size_t>(steps) * (wc.part < wc.slots ? wc.part : wc.slots) * kWcRows; }
   size_t wc_chunk_bytes(int steps) const { return wc_chunk_rows(steps) * (3 * L + 2) * W * 4; }
+  size_t wc_step_bytes() const { return wc_chunk_rows(1) * W * 2 + 2 * wc_chunk_bytes(1); }
 
-  // Buffers of the wide chain kernel; where memory is short, shorter chunks (same bits), then the layer kernels (wck), which find
-  // their workspace taken first and everything else given back.
+  // Buffers of the wide chain kernel.  Bytes by the steps that a call has and the limit, and not a whole number of its steps: of two calls the
+  // one of fewer rows or blocks may have room for more steps, and must not have to replace what the other uses.  Where memory is
+  // short, shorter chunks (same bits), then the layer kernels (wck), which find their workspace taken first and everything else given back.
   int reserve_wide_chain() {
     if (!wc.slots) wc = wide_cut_alone(ctx, hd->d, R, cfg);
     int rc = ensure_ws(ctx, ctx->ws[slot], hd->d, Rh, R, Ts);
     if (rc) return rc;
-    const size_t exchange = wx_layout().total, least = exchange + wc_chunk_rows(1) * W * 2 + 2 * wc_chunk_bytes(1);
+    const size_t exchange = wx_layout().total, step = wc_step_bytes(), least = exchange + step;
     if (least >= ctx->wx_refused[slot]) { wck = false; return CSD_OK; }
-    const size_t s_refused = ctx->gc_refused[slot], m_refused = ctx->gm_refused[slot];
-    rc = exchange <= ctx->wx[slot].cap ? static_cast<int>(CSD_OK) : ensure_side(ctx, ctx->wx[slot], exchange, "the chain's exchange buffers");
+    const size_t m_refused = ctx->gm_refused[slot];
     wc_most = Ts < kWcMaxSteps ? Ts : kWcMaxSteps;
-    while (wc_most > 1 && wc_chunk_bytes(wc_most) > kWcChunkBytes) --wc_most;
-    for (; !rc; wc_most = (wc_most + 1) / 2) {
-      rc = have(ctx->gc[slot], ctx->gc_refused[slot], wc_chunk_rows(wc_most) * W * 2, "the condition vectors of a chunk of steps");
-      if (!rc) rc = have(ctx->gm[slot], ctx->gm_refused[slot], 2 * wc_chunk_bytes(wc_most) + 256, "the condition products");
-      if (rc != CSD_ERR_WORKSPACE || wc_most == 1) break;
+    size_t want = wc_most * step < kWcBufferBytes ? wc_most * step : kWcBufferBytes;
+    if (want < step) want = step;
+    rc = ensure_buffer(ctx, ctx->wx[slot], exchange, "the chain's exchange buffers");
+    while (!rc && (rc = have(ctx->gm[slot], ctx->gm_refused[slot], want, "the condition products")) == CSD_ERR_WORKSPACE && want > step) {
       rc = CSD_OK;
+      want = want / 2 < step ? step : want / 2;
     }
+    if (!rc && static_cast<size_t>(wc_most) > want / step) wc_most = static_cast<int>(want / step);
     if (rc != CSD_ERR_WORKSPACE) return rc;
-    ctx->wx_refused[slot] = least; ctx->gc_refused[slot] = s_refused; ctx->gm_refused[slot] = m_refused;
+    ctx->wx_refused[slot] = least; ctx->gm_refused[slot] = m_refused;
     ctx->err[0] = 0;
     wck = false;
     CSD_CUDA(ctx, cudaStreamSynchronize(st));
     CSD_CUDA(ctx, cudaStreamSynchronize(ctx->aux[slot]));
-    for (HostIo* io : {&ctx->wx[slot], &ctx->gc[slot], &ctx->gm[slot]}) {
-      if (io->base) CSD_CUDA(ctx, cudaFree(io->base));
-      io->base = nullptr; io->cap = 0;
-    }
-    return CSD_OK;
+    if ((rc = give_up(ctx, ctx->wx[slot]))) return rc;
+    return give_up(ctx, ctx->gm[slot]);
   }
-  struct WxLayout { size_t stats, epart, xll, cnt, zeroed, u, v, hsum, total; };
+  struct WxLayout { size_t stats, epart, xll, cnt, ticket, zeroed, u, v, hsum, total; };
   WxLayout wx_layout() const {
     const size_t rows = static_cast<size_t>(wc.nb) * kTileM, G = W / 128;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 1024); return o; };
     WxLayout l{};
     l.stats = take(rows * G * 16); l.epart = take(rows * G * (lv_min ? kCPad2 : kCPad) * 8); l.xll = take(rows * kCPad * 8);
-    l.cnt = take(static_cast<size_t>(wc.nb) * 512);
+    l.cnt = take(static_cast<size_t>(wc.nb) * 512); l.ticket = take(2 * sizeof(int));
     l.zeroed = off;              // what precedes starts at zero
     l.u = take(rows * W * 2); l.v = take(rows * W * 2); l.hsum = take(lv_min ? rows * kCPad * 4 : 0);
     l.total = off;
@@ -984,13 +1012,14 @@ struct Chain {
     ChainWs& ws = ctx->ws[slot];
     const WxLayout l = wx_layout();
     char* const xb = static_cast<char*>(ctx->wx[slot].base);
-    char* const gm = static_cast<char*>(ctx->gm[slot].base);
     const size_t chunk = wc_chunk_bytes(wc_most);
-    int* const tickets = reinterpret_cast<int*>(gm + 2 * chunk);
+    void* const s_chunk = ctx->gm[slot].base;
+    char* const gm = static_cast<char*>(s_chunk) + wc_chunk_rows(wc_most) * W * 2;
+    int* const tickets = reinterpret_cast<int*>(xb + l.ticket);
     const bool f16 = d.dtype == CSD_F16, lv = lv_min != nullptr;
     int rc;
     CUtensorMap tm_s{}, tm_uu{}, tm_vv{};
-    if ((rc = make_tmap(ctx, &tm_s, d.dtype, ctx->gc[slot].base, wc_chunk_rows(wc_most), W, W, kTileM))) return rc;
+    if ((rc = make_tmap(ctx, &tm_s, d.dtype, s_chunk, wc_chunk_rows(wc_most), W, W, kTileM))) return rc;
     const uint64_t lines = static_cast<uint64_t>(wc.nb) * kTileM * W / 256;      // u, v as lines of 256 elements: 32 of them a k-block
     if ((rc = make_plain_tmap(ctx, &tm_uu, d.dtype, xb + l.u, lines)) || (rc = make_plain_tmap(ctx, &tm_vv, d.dtype, xb + l.v, lines))) return rc;
     CSD_CUDA(ctx, cudaMemsetAsync(xb, 0, l.zeroed, st));
@@ -1037,8 +1066,8 @@ struct Chain {
         CSD_CUDA(ctx, cudaMemsetAsync(tickets + buf, 0, sizeof(int), gst));
         const dim3 sgrid(static_cast<unsigned>(rows), static_cast<unsigned>((n + kCondSteps - 1) / kCondSteps));
         const float* te = ws.te + static_cast<size_t>(t_lo - 1) * W;
-        if (f16) cond_all_kernel<__half, 128><<<sgrid, 128, 0, gst>>>(ws.cz, te, static_cast<__half*>(ctx->gc[slot].base), R, cfg, W, rows, s0 * kWcRows, n);
-        else cond_all_kernel<__nv_bfloat16, 128><<<sgrid, 128, 0, gst>>>(ws.cz, te, static_cast<__nv_bfloat16*>(ctx->gc[slot].base), R, cfg, W, rows, s0 * kWcRows, n);
+        if (f16) cond_all_kernel<__half, 128><<<sgrid, 128, 0, gst>>>(ws.cz, te, static_cast<__half*>(s_chunk), R, cfg, W, rows, s0 * kWcRows, n);
+        else cond_all_kernel<__nv_bfloat16, 128><<<sgrid, 128, 0, gst>>>(ws.cz, te, static_cast<__nv_bfloat16*>(s_chunk), R, cfg, W, rows, s0 * kWcRows, n);
         CSD_CUDA(ctx, cudaGetLastError());
         m.nst = n * slots; m.ticket = tickets + buf; m.out = mods;
         int pairs = c == 0 ? ctx->num_sms / 2 : free_pairs;
@@ -1298,20 +1327,6 @@ size_t bonus_buf_bytes(const csd_head_desc& d, int Rt, int cfg, int T) {
   return align_up(rt * m * d.Dz * 4, 256) + align_up(rt * d.C * 4, 256) * 3 + align_up(static_cast<size_t>(T) * rt * d.C * 4, 256);
 }
 
-int ensure_side(csd_ctx* ctx, HostIo& io, size_t need, const char* what) {
-  if (need <= io.cap) return CSD_OK;
-  CSD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  for (int i = 0; i < 2; ++i) { CSD_CUDA(ctx, cudaStreamSynchronize(ctx->side[i])); CSD_CUDA(ctx, cudaStreamSynchronize(ctx->aux[i])); }
-  if (io.base) CSD_CUDA(ctx, cudaFree(io.base));
-  io.base = nullptr; io.cap = 0;
-  if (cudaMalloc(&io.base, need) != cudaSuccess) {
-    cudaGetLastError();
-    return fail(ctx, CSD_ERR_WORKSPACE, "cannot allocate %zu bytes for %s", need, what);
-  }
-  io.cap = need;
-  return CSD_OK;
-}
-
 // Carves the (already large enough) side buffer and enqueues the gathering copies on `st`.
 int gather_bonus_inputs(csd_ctx* ctx, cudaStream_t st, const csd_head_desc& d, int R, int B, int cfg, int T,
                         const float* z, const float* x_T, const float* eps, const float* z_next,
@@ -1416,6 +1431,7 @@ int csd_destroy(csd_ctx* c) {
     if (w.base && w.owned) cudaFree(w.base);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
+  for (void* b : c->in_graphs) cudaFree(b);
   if (c->io.base) cudaFree(c->io.base);
   if (c->sp.base) cudaFree(c->sp.base);
   if (c->un.base) cudaFree(c->un.base);
@@ -1888,7 +1904,7 @@ static int verify_impl(csd_ctx* ctx, const csd_head* head_p, const csd_schedule*
   const int R = B * gamma, C = head_p->d.C, T = sched_p->T;
   BonusBuf bb{};
   if (bonus) {
-    if ((rc = ensure_side(ctx, ctx->bn, bonus_buf_bytes(head_p->d, R + B, cfg, T), "the bonus rows"))) return rc;
+    if ((rc = ensure_buffer(ctx, ctx->bn, bonus_buf_bytes(head_p->d, R + B, cfg, T), "the bonus rows"))) return rc;
     if ((rc = gather_bonus_inputs(ctx, ctx->stream, head_p->d, R, B, cfg, T, z_p, x_T, eps, z_next, x_T_next, eps_next, bb))) return rc;
     // every row samples at the last step; only the bonus rows' samples are used
     rc = run_chain(ctx, 1, ctx->stream, head_p, sched_p, R + B, cfg, cfg_scale, bb.z, bb.x_T, bb.eps, 1, bb.x0, bb.mu1, nullptr);
@@ -1939,16 +1955,7 @@ int csd_verify_unaligned(csd_ctx* ctx, const csd_head* head_p, const csd_schedul
   CSD_DEVICE(ctx);
   const int R = B * gamma, C = head_p->d.C, T = sched_p->T;
   const size_t need = static_cast<size_t>(R) * 4;
-  if (need > ctx->un.cap) {
-    CSD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    if (ctx->un.base) CSD_CUDA(ctx, cudaFree(ctx->un.base));
-    ctx->un.base = nullptr; ctx->un.cap = 0;
-    if (cudaMalloc(&ctx->un.base, need) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(ctx, CSD_ERR_WORKSPACE, "cannot allocate %zu bytes for the noise terms", need);
-    }
-    ctx->un.cap = need;
-  }
+  if ((rc = ensure_buffer(ctx, ctx->un, need, "the noise terms"))) return rc;
   float* d_off = static_cast<float*>(ctx->un.base);
   rc = run_chain(ctx, 1, ctx->stream, head_p, sched_p, R, cfg, cfg_scale, z_p, x_T, eps_p, 0, nullptr, mu1_p, nullptr);
   if (rc) return rc;
@@ -1969,7 +1976,7 @@ int csd_bonus_token(csd_ctx* ctx, const csd_head* head_p, const csd_schedule* sc
   if (!n_accept || !x_bonus) return fail(ctx, CSD_ERR_INVALID_ARG, "n_accept / x_bonus is null");
   CSD_DEVICE(ctx);
   const int C = head_p->d.C;
-  if ((rc = ensure_side(ctx, ctx->bn, static_cast<size_t>(2) * B * C * 4, "the bonus samples"))) return rc;
+  if ((rc = ensure_buffer(ctx, ctx->bn, static_cast<size_t>(2) * B * C * 4, "the bonus samples"))) return rc;
   float* d_x0 = static_cast<float*>(ctx->bn.base);
   float* d_mu = d_x0 + static_cast<size_t>(B) * C;
   // the masks live on the device, so every sequence is sampled and the selection is a kernel: no host round trip
@@ -2029,16 +2036,7 @@ int csd_verify_single_path(csd_ctx* ctx, const csd_head* head_p, const csd_sched
   const size_t o_acc = align_up(o_mu + static_cast<size_t>(tb) * R * C * 4, 256);
   const size_t need = o_acc + static_cast<size_t>(T) * R * 4;
   cudaStream_t st = ctx->stream;
-  if (need > ctx->sp.cap) {
-    CSD_CUDA(ctx, cudaStreamSynchronize(st));
-    if (ctx->sp.base) CSD_CUDA(ctx, cudaFree(ctx->sp.base));
-    ctx->sp.base = nullptr; ctx->sp.cap = 0;
-    if (cudaMalloc(&ctx->sp.base, need) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(ctx, CSD_ERR_WORKSPACE, "cannot allocate %zu bytes for the single-path buffers", need);
-    }
-    ctx->sp.cap = need;
-  }
+  if ((rc = ensure_buffer(ctx, ctx->sp, need, "the single-path buffers"))) return rc;
   char* base = static_cast<char*>(ctx->sp.base);
   float* d_sched = reinterpret_cast<float*>(base);
   float* d_mu = reinterpret_cast<float*>(base + o_mu);
@@ -2116,7 +2114,7 @@ static int round_impl(csd_ctx* ctx, const csd_head* head_q, const csd_head* head
   // workspaces first (growing one synchronises), then fork the two chains
   if ((rc = ensure_ws(ctx, ctx->ws[0], head_q->d, R * (cfg ? 2 : 1), R, sched_q->T))) return rc;
   if ((rc = ensure_ws(ctx, ctx->ws[1], head_p->d, Rp * (cfg ? 2 : 1), Rp, sched_p->T))) return rc;
-  if (bonus && (rc = ensure_side(ctx, ctx->bn, bonus_buf_bytes(head_p->d, Rp, cfg, T), "the bonus rows"))) return rc;
+  if (bonus && (rc = ensure_buffer(ctx, ctx->bn, bonus_buf_bytes(head_p->d, Rp, cfg, T), "the bonus rows"))) return rc;
   CSD_CUDA(ctx, cudaEventRecord(ctx->ev_fork, ctx->stream));
   for (int i = 0; i < 2; ++i) CSD_CUDA(ctx, cudaStreamWaitEvent(ctx->side[i], ctx->ev_fork, 0));
   // the two chains' launches are interleaved step by step so that neither stream starves
@@ -2388,13 +2386,7 @@ int csd_round_host(csd_ctx* ctx, const csd_head* head_q, const csd_head* head_p,
       {nullptr, cap_hits, 4, 0, false}};
   size_t total = 0;
   for (Item& it : items) { it.off = total; total = align_up(total + it.bytes, 256); }
-  if (total > ctx->io.cap) {
-    CSD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    if (ctx->io.base) CSD_CUDA(ctx, cudaFree(ctx->io.base));
-    ctx->io.base = nullptr; ctx->io.cap = 0;
-    if (cudaMalloc(&ctx->io.base, total) != cudaSuccess) { cudaGetLastError(); return fail(ctx, CSD_ERR_WORKSPACE, "cannot allocate %zu bytes for the host-call mirrors", total); }
-    ctx->io.cap = total;
-  }
+  if (int rc = ensure_buffer(ctx, ctx->io, total, "the host-call mirrors")) return rc;
   char* base = static_cast<char*>(ctx->io.base);
   auto dp = [&](int i) { return base + items[i].off; };
   for (int i = 0; i < 7; ++i) CSD_CUDA(ctx, cudaMemcpyAsync(dp(i), items[i].src, items[i].bytes, cudaMemcpyHostToDevice, ctx->stream));

@@ -134,6 +134,43 @@ def test_captured_round_replays():
     dr.ctx.close()
 
 
+def test_captured_round_outlives_the_buffers_of_other_calls():
+    # by the steps that fit, 592 rows of the target would take more bytes (31 steps) than 1024 (23): the smaller call replaces nothing.  A larger
+    # call and one of few rows, which grow buffers, leave the graph what it holds.
+    from paper_2411_11925_b200 import api
+    from paper_2411_11925_b200.runner import DeviceRound
+    side = torch.cuda.Stream()
+    inps = [gen.make_round_inputs(_wl(bf16=True, B=B, gamma=8, T=40, cfg=True, cfg_scale=2.0, draft=H(1, 1024, 64), target=H(3, 1024, 64)), seed_offset=B)
+            for B in (64, 37, 80, 1)]
+    dr = DeviceRound(inps[0], ctx=api.Context(0, side))
+    others = [DeviceRound(i, ctx=dr.ctx, heads=(dr.head_q, dr.head_p)) for i in inps[1:]]
+    torch.cuda.synchronize()
+    dr.fused_round()
+    want = dr.results()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=side):
+        dr.fused_round()
+    free = torch.cuda.mem_get_info()[0]
+    others[0].fused_round()
+    dr.ctx.sync()
+    assert torch.cuda.mem_get_info()[0] == free
+    for o in others[1:]:
+        o.fused_round()
+    dr.ctx.sync()
+    others_memory = torch.full((6 << 30,), 255, dtype=torch.uint8, device="cuda")     # where freed buffers would have been
+    dr.x0.zero_()
+    dr.mu1_p.zero_()
+    torch.cuda.synchronize()
+    g.replay()
+    torch.cuda.synchronize()
+    got = dr.results()
+    for k in ("x0", "mu1_q", "mu1_p", "logratio", "n_accept"):
+        np.testing.assert_array_equal(got[k], want[k], err_msg=k)
+    assert bool((others_memory == 255).all())
+    del g
+    dr.ctx.close()
+
+
 @pytest.mark.parametrize("op", ["f16", "bf16"])
 def test_default_mode_is_as_precise_as_three_kernels_per_block(op):
     # relative error (2-norm) of 4 x 300 tokens against the checker, wide chain over plain layer kernels: the same roundings, sums in another
