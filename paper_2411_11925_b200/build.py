@@ -12,7 +12,7 @@ LIB_PATH = os.path.join(PKG_DIR, "libcsd.so")
 MARSHAL_PATH = os.path.join(PKG_DIR, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
 ABI_HEADER = os.path.join(os.path.dirname(PKG_DIR), "include", "csd.h")
 SOURCES = ["csd_api.cu"]
-HEADERS = ["ptx.cuh", "epilogue.cuh", "gemm.cuh", "rowops.cuh", "fold.cuh", "groupchain.cuh", "widechain.cuh", "gmm.cuh", "f32chain.cuh"]
+HEADERS = ["ptx.cuh", "epilogue.cuh", "gemm.cuh", "rowops.cuh", "fold.cuh", "groupchain.cuh", "wideplan.h", "widechain.cuh", "gmm.cuh", "f32chain.cuh"]
 
 
 def _nvcc() -> str:

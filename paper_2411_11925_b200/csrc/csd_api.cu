@@ -504,29 +504,29 @@ WideKernel wide_kernel_of(bool lv, int halves) {
   return lv ? wide_chain_kernel<ACT, FMT, true, 1> : wide_chain_kernel<ACT, FMT, false, 1>;
 }
 WideKernel wide_kernel(int dtype, bool lv, int halves) { return dtype == CSD_F16 ? wide_kernel_of<__half, 0>(lv, halves) : wide_kernel_of<__nv_bfloat16, 1>(lv, halves); }
-bool wide_ready(const csd_ctx* ctx, int dtype) {
+// CTA pairs of the wide chain kernel that the device holds at a time (0: it cannot run), and the opt-ins, once per device and operand type.
+int wide_pairs(const csd_ctx* ctx, int dtype) {
   static int known[kMaxDevices][2] = {};
   int& k = known[ctx->device][dtype == CSD_F16 ? 0 : 1];
   if (k == 0) {
     bool ok = (dtype == CSD_F16 ? cudaFuncSetAttribute(wide_mods_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMgSmemBytes)
                                 : cudaFuncSetAttribute(wide_mods_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMgSmemBytes)) == cudaSuccess;
     for (int i = 0; i < 4; ++i) ok = ok && cudaFuncSetAttribute(wide_kernel(dtype, (i & 1) != 0, 1 + (i >> 1)), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3(2); lc.blockDim = dim3(kWcThreads); lc.dynamicSmemBytes = 227 * 1024;
+    lc.attrs = at; lc.numAttrs = 1;
+    int n = 0;
+    ok = ok && cudaOccupancyMaxActiveClusters(&n, wide_kernel(dtype, false, 2), &lc) == cudaSuccess;
     cudaGetLastError();
-    k = ok ? 1 : -1;
+    k = ok && n > 0 ? n : -1;
   }
-  return k == 1;
+  return k < 0 ? 0 : k;
 }
-// How a chain of R token rows is cut up: slots of 256 rows; the form of the kernel (halves 1: two slots a group, 2: one slot with
-// twice the epilogue warps); slots of a launch (a part of the rows where not all of a launch's CTAs would find an SM).
-struct WideCut { int nb, slots, part, ctas, halves; };
 WideCut wide_cut(const csd_ctx* ctx, const csd_head_desc& d, int R, int cfg, int halves) {
-  WideCut c{};
-  const int nb = cfg ? (R + 63) / 64 : (R + 127) / 128, group = 2 * (d.W / 128), most = ctx->num_sms / group, gs = 2 / halves;
-  c.nb = nb + (nb & 1); c.slots = c.nb / 2; c.halves = halves;
-  const int groups = (c.slots + gs - 1) / gs, parts = (groups + most - 1) / most;
-  c.part = ((c.slots + parts - 1) / parts + gs - 1) / gs * gs;
-  c.ctas = ((c.part < c.slots ? c.part : c.slots) + gs - 1) / gs * group;
-  return c;
+  return csd::wide_cut(wide_groups(wide_pairs(ctx, d.dtype), d.W), d.W, R, cfg, halves);
 }
 bool wide_halves(const csd_head_desc& d) { return wc_layout(d.L, d.var_out ? kCPad2 : kCPad, 2).stages >= kWcMinStages; }
 // Which form, and whether two chains go side by side, by a model of one step in us, fitted to measured steps (W = 1024, 1024 rows: 3
@@ -555,7 +555,7 @@ constexpr int kWcMostRows = 4608;
 bool wide_takes(const csd_ctx* ctx, const csd_head* hd, int R, int cfg, int slot, bool batch) {
   const int rows = R * (cfg ? 2 : 1);
   return wide_width(hd->d) && ctx->chain_mode == CSD_CHAIN_LAYERS && slot != 2 && !batch && !ctx->prof_on && rows > kWcRows && rows <= kWcMostRows &&
-         wide_ready(ctx, hd->d.dtype);
+         wide_groups(wide_pairs(ctx, hd->d.dtype), hd->d.W) >= 1;      // (a device, or a part of one, with fewer SMs than a group has CTAs)
 }
 // One head's denoising chain for R token rows on stream `st` with workspace slot `slot`:
 // begin() enqueues the per-call work (timestep embedding, condition projection, first boundary

@@ -30,6 +30,7 @@
 // own step number (value | tag, value | tag): the reader polls the data itself and no fence stands in between.
 #pragma once
 #include "groupchain.cuh"
+#include "wideplan.h"
 
 namespace csd {
 
@@ -201,7 +202,6 @@ wide_mods_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 }
 
 // ------------------------------------------------------------------------------------------ the chain
-constexpr int kWcRows = 256;              // rows of a slot
 constexpr int kWcMmaWarp = 8, kWcActWarp = 9, kWcWeightWarp = 10;
 constexpr int kWcThreads = 11 * 32;
 constexpr int kWcAhead = 4;               // pieces of the products that an epilogue thread has in flight
