@@ -767,7 +767,7 @@ wide_chain_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant
           tmem_ld16(t_acc + i * 16, a);
           tmem_ld16(t_h + i * 16, hv);
           tmem_ld_wait();
-          if (i == CW / 16 - 1) release_acc();
+          if (i == CW / 16 - 1 && k + 1 < L) release_acc();      // (the last block's columns serve the output projection first)
           const float4* b4 = reinterpret_cast<const float4*>(bias_s + (2 * k + 1) * 128 + hf * CW + i * 16);
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
@@ -793,7 +793,7 @@ wide_chain_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant
           if (c0 + j < p.C) nz[j] = __ldg(p.eps + (static_cast<size_t>(t - 1) * p.R + tok) * p.C + c0 + j);
       {
         if (t > p.t_lo) ahead(ss_at(t - 1, 0), 32768 / HV);
-        // into the (free) accumulator columns, and back in fragment order: four rows a thread, as above
+        // into the accumulator columns, which the MMAs get back only after it, and back in fragment order: four rows a thread, as above
         modulate(ss_at(t, L), [&](int i, const float (&o)[8]) { tmem_st8(t_acc + i * 8, o); });
         tmem_st_wait();
 #pragma unroll 1
@@ -859,6 +859,7 @@ wide_chain_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant
             for (int c = 0; c < kCPad; c += 2) wc_put(dst + (c / 2) * 128, o[c], o[c + 1], step + 1);
           }
         }
+        release_acc();
       }
       // ---- guidance and Eq. 3 for this CTA's tokens; the new state to every column tile
       if (upd) {
