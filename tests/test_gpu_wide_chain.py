@@ -7,6 +7,7 @@ import torch
 
 from oracle import csd_oracle as orc
 from paper_2411_11925_b200 import inputs as gen
+import test_gpu_learned_variance as lv
 from _parity import TOL_X
 from test_gpu_parity import _check, _wl
 
@@ -169,6 +170,28 @@ def test_captured_round_outlives_the_buffers_of_other_calls():
     assert bool((others_memory == 255).all())
     del g
     dr.ctx.close()
+
+
+@pytest.mark.parametrize("kw", [
+    dict(B=43, gamma=3, T=4, cfg=True, cfg_scale=2.0, operand="bf16", draft=H(2, 1280, 64), target=H(1, 1024, 128)),      # one token in the last row block
+    dict(B=393, gamma=1, T=1, cfg=False, draft=H(2, 768, 64, C=5), target=H(2, 1536, 64, C=5)),                           # a single step; a partial slot
+    dict(B=165, gamma=3, T=5, cfg=False, operand="bf16", draft=H(3, 1024, 64, C=3), target=H(2, 1792, 64, C=3)),          # a partial slot
+    dict(B=100, gamma=3, T=9, cfg=True, cfg_scale=3.0, draft=H(2, 2048, 64), target=H(2, 768, 64)),                       # three slots; chunks 1, 1 or 2, ..
+    dict(B=130, gamma=2, T=70, cfg=False, draft=H(2, 768, 64), target=H(2, 1024, 64)),                                    # more than a launch's steps
+])
+def test_predicted_variances_match_checker_and_fused_round_matches_the_calls(kw):
+    r = lv.LvRound(lv._inputs(lv._wl(bf16=True, **{"operand": "f16", **kw})), 1.0, 0.95)
+    l0 = r.ctx.launch_count()
+    r.three_calls()
+    a = r.results()
+    assert r.ctx.launch_count() - l0 < 40 + 6 * kw["T"] // 5      # neither chain ran the layer kernels
+    lv._compare(a, lv._ref(r.inp, 1.0, 0.95), r.wl, r.inp.u, label=f"wide chain lv {kw}")
+    for _ in range(2):            # other forms of the kernel (slots a group), another order of launches, whatever overlaps: the same bits
+        r.fused()
+        b = r.results()
+        for k in lv.LvRound.NAMES:
+            np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+    r.ctx.close()
 
 
 @pytest.mark.parametrize("op", ["f16", "bf16"])
