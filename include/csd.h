@@ -117,15 +117,16 @@ const char *csd_last_error(const csd_ctx *ctx);
  * word, else CSD_OK.  Clears the status.  After a failed wait every later launch of the context returns
  * at once until csd_sync has been called. */
 int csd_sync(csd_ctx *ctx);
-/* Every device-side wait of the library (on an mbarrier of a TMA / MMA / epilogue pipeline) is bounded:
+/* Every device-side wait of the library (on an mbarrier of a TMA / MMA / epilogue pipeline, on a word that another block writes) is bounded:
  * after `cycles` SM clock cycles (default 4e9, about two seconds; cycles <= 0 restores the default) it
  * gives up and raises the status csd_sync reports.  The limit is one value per GPU and process (all
  * contexts on that device share it).  Synchronises the context's streams. */
 int csd_set_wait_limit(csd_ctx *ctx, int64_t cycles);
-/* Diagnostic: enqueues one tiny kernel whose only thread waits on a barrier nobody arrives at, i.e. a wait
- * that is certain to run into the limit above.  Used to check the reporting path (csd_sync returns
- * CSD_ERR_TIMEOUT, "wait self-test") without disturbing the GPU: nothing faults or traps, and the wait
- * ends at the limit.  Set a short limit first (1e5 cycles) or the call takes the default two seconds. */
+/* Diagnostic: enqueues one tiny kernel whose only thread polls words nobody writes, then waits on a barrier nobody
+ * arrives at, i.e. two waits that are certain to run into the limit above.  Used to check the reporting path (csd_sync
+ * returns CSD_ERR_TIMEOUT, "wait self-test"; iteration = cycles of the first wait, per cent of the limit) without
+ * disturbing the GPU: nothing faults or traps, and the waits end at the limit.  Set a short limit first (1e5 cycles)
+ * or the call takes twice the default two seconds. */
 int csd_selftest_wait_timeout(csd_ctx *ctx);
 /* Number of kernels this context has launched so far (bookkeeping for benchmarks). */
 int64_t csd_launch_count(const csd_ctx *ctx);

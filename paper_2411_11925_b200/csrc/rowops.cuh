@@ -784,14 +784,4 @@ __global__ void __launch_bounds__(128) resample_kernel(const ResampleParams p) {
   tally_cap_hits(hit_s[0] + hit_s[1] + hit_s[2] + hit_s[3], p.tally, p.cap_hits);
 }
 
-// Self-test of the bounded waits: one thread waits on a barrier on which nobody ever arrives, so the wait runs
-// into the limit (csd_set_wait_limit), gives up and records role 4, site 1 in the context's error word.  Nothing
-// else happens: no fault, no trap, no wait beyond the limit.
-__global__ void wait_timeout_selftest_kernel(int* err) {
-  __shared__ uint64_t bar;
-  if (threadIdx.x == 0) { mbar_init(&bar, 1); fence_mbar_init(); }
-  __syncthreads();
-  if (threadIdx.x == 0 && !ch_wait<false>(&bar, 0, err)) ch_fail(err, 4, 1, 0);
-}
-
 }  // namespace csd

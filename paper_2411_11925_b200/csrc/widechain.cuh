@@ -296,13 +296,13 @@ __device__ __forceinline__ void wc_put(ulonglong2* p, float a, float b, uint32_t
   asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(t | __float_as_uint(a)), "l"(t | __float_as_uint(b)) : "memory");
 }
 // Eight words, two (2 KB apart) from each of four places, polled until all carry the tag.  False: the context's error word is up, or
-// limit polls were not enough.  (One block of assembly: as a C++ loop the words are held twice.)
-__device__ __forceinline__ bool wc_poll8(ulonglong2 (&w)[8], const ulonglong2* a, const ulonglong2* b, const ulonglong2* c, const ulonglong2* d,
-                                         uint32_t tag, const int* err, uint32_t limit) {
+// the wait took longer than the bound of every other one, in cycles of the SM clock.  (One block of assembly: as a C++ loop the words are held twice.)
+__device__ __forceinline__ bool wc_poll(ulonglong2 (&w)[8], const ulonglong2* a, const ulonglong2* b, const ulonglong2* c, const ulonglong2* d,
+                                        uint32_t tag, const int* err) {
   uint32_t bad;
   asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b32 n, x, lo, hi;\n\t"
-      "mov.u32 n, 0;\n"
+      "{\n\t.reg .pred p;\n\t.reg .b32 x, lo, hi, t0;\n\t.reg .b64 now, most;\n\t"
+      "mov.u64 now, %%clock64;\n\tshr.u64 now, now, 10;\n\tcvt.u32.u64 t0, now;\n"      // units of 1024 cycles
       "AGAIN:\n\t"
       "ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%17];\n\t"
       "ld.relaxed.gpu.global.v2.b64 {%2, %3}, [%17 + 2048];\n\t"
@@ -320,13 +320,16 @@ __device__ __forceinline__ bool wc_poll8(ulonglong2 (&w)[8], const ulonglong2* a
 #undef WC_CHECK
       "setp.ne.u32 p, %16, 0;\n\t@p bra DONE;\n\t"
       "setp.eq.u32 p, x, 0;\n\t@p bra DONE;\n\t"
-      "add.u32 n, n, 1;\n\t"
-      "setp.lt.u32 p, n, %23;\n\t@p bra AGAIN;\n\t"
+      "mov.u64 now, %%clock64;\n\tshr.u64 now, now, 10;\n\tcvt.u32.u64 x, now;\n\tsub.u32 x, x, t0;\n\t"
+      "setp.lt.u32 p, x, 64;\n\t@p bra AGAIN;\n\t"                                           // (the limit is read only then)
+      "cvt.u64.u32 now, x;\n\t"
+      "ld.volatile.global.u64 most, [%23];\n\tshr.u64 most, most, 10;\n\t"
+      "setp.le.u64 p, now, most;\n\t@p bra AGAIN;\n\t"
       "mov.u32 %16, 1;\n"
       "DONE:\n\t}"
       : "=&l"(w[0].x), "=&l"(w[0].y), "=&l"(w[1].x), "=&l"(w[1].y), "=&l"(w[2].x), "=&l"(w[2].y), "=&l"(w[3].x), "=&l"(w[3].y),
         "=&l"(w[4].x), "=&l"(w[4].y), "=&l"(w[5].x), "=&l"(w[5].y), "=&l"(w[6].x), "=&l"(w[6].y), "=&l"(w[7].x), "=&l"(w[7].y), "=&r"(bad)
-      : "l"(a), "l"(b), "l"(c), "l"(d), "r"(tag), "l"(err), "r"(limit)
+      : "l"(a), "l"(b), "l"(c), "l"(d), "r"(tag), "l"(err), "l"(&g_wait_limit_cycles)
       : "memory");
   return bad == 0;
 }
@@ -504,11 +507,8 @@ wide_chain_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant
     // HV == 2: the second half's warp has left something for the first half's in shared memory
     auto hand_over = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(3 + q) : "memory"); };
     // eight words of this lane, or the word that it gives up
-    const long long wait_cycles = *reinterpret_cast<volatile long long*>(&g_wait_limit_cycles);
-    const uint32_t polls = wait_cycles < (1ll << 40) ? static_cast<uint32_t>(wait_cycles / 512) + 64u : 0x7fffffffu;      // a poll takes more than 512 cycles
     auto poll = [&](ulonglong2 (&w)[8], const ulonglong2* a, const ulonglong2* b, const ulonglong2* c, const ulonglong2* d, uint32_t tag, int site) {
-      // (once given up, one poll and no wait; a branch around the loads would have the words held twice)
-      const bool got = wc_poll8(w, a, b, c, d, tag, p.err, ok ? polls : 0u);
+      const bool got = wc_poll(w, a, b, c, d, tag, p.err);      // (once given up, the error word ends it at once; a branch around it would have the words held twice)
       if (ok && !got) ch_fail(p.err, DEV_ERR_EPI_WAIT, site, static_cast<int>(tag));
       ok = __all_sync(0xffffffffu, ok && got);
     };
@@ -943,6 +943,24 @@ wide_chain_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant
   gc_settle(p.err);
   cluster_arrive(); cluster_wait();   // neither CTA leaves while the pair's MMAs or signals may touch it
   if (warp == kWcMmaWarp) tmem_dealloc_pair(tmem_base, 512);
+}
+
+// Self-test of the bounded waits: one thread polls words that nobody writes, then waits on a barrier on which nobody arrives, so both waits
+// run into the limit (csd_set_wait_limit) and give up.  Recorded in the context's error word: role 4, site 1 (2: the poll
+// succeeded), and as the iteration the cycles that the poll took, in per cent of the limit.  Nothing else happens: no
+// fault, no trap, no wait beyond the limit.
+__device__ ulonglong2 g_selftest_words[256];
+__global__ void wait_timeout_selftest_kernel(int* err) {
+  __shared__ uint64_t bar;
+  if (threadIdx.x == 0) { mbar_init(&bar, 1); fence_mbar_init(); }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  ulonglong2 w[8];
+  const ulonglong2* const a = g_selftest_words;
+  const long long t0 = clock64();
+  const bool got = wc_poll(w, a, a, a, a, 1, err);
+  const long long percent = (clock64() - t0) * 100 / *reinterpret_cast<volatile long long*>(&g_wait_limit_cycles);
+  if (!ch_wait<false>(&bar, 0, err)) ch_fail(err, 4, got ? 2 : 1, static_cast<int>(percent < 0xffff ? percent : 0xffff));
 }
 
 }  // namespace csd

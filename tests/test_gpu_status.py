@@ -1,7 +1,7 @@
 """Device-side status words: a bounded wait that runs out, and a non-finite value at a step update.
 
-Neither case faults, traps or hangs anything.  The wait that runs out is a one-thread kernel waiting, with a limit
-of 1e5 cycles, on a barrier nobody arrives at; the non-finite value is an fp16 activation beyond 65504 produced by a
+Neither case faults, traps or hangs anything.  The waits that run out are a one-thread kernel's, with a limit
+of 1e5 cycles (1e7 where the limit is measured), on words nobody writes and on a barrier nobody arrives at; the non-finite value is an fp16 activation beyond 65504 produced by a
 head whose first MLP layer is scaled up."""
 import time
 
@@ -49,6 +49,21 @@ def test_wait_that_runs_out_returns_timeout_and_the_context_recovers():
     for k in KEYS:
         np.testing.assert_array_equal(before[k], after[k], err_msg=k)
     dr.ctx.close()
+
+
+def test_polled_words_are_given_up_at_the_limit():
+    from paper_2411_11925_b200 import api
+    ctx = api.Context(0)
+    try:
+        ctx.set_wait_limit(10_000_000)
+        ctx.selftest_wait_timeout()
+        with pytest.raises(api.CsdError) as e:
+            ctx.sync()
+        percent = int(str(e.value).split("iteration ")[1].split(",")[0])
+        assert 100 <= percent <= 110, str(e.value)        # the clock is read at every poll, some 1000 cycles
+    finally:
+        ctx.set_wait_limit(0)
+        ctx.close()
 
 
 def test_fp16_activation_overflow_is_reported_as_nonfinite_and_bf16_operands_take_the_same_head():
