@@ -143,6 +143,9 @@ int64_t csd_launch_count(const csd_ctx *ctx);
  *                       steps, and the condition vectors of a chunk, at most 2 GB together as long as one step is less
  *                       (1024 rows of 6 x 1024: 12 steps); operands and partials of one step.  Where the device has less
  *                       free, chunks are shorter (the same bits); where not even one step fits, the layer kernels run.
+ *                       The two chains of a round share what there is: one does not take long chunks while the other
+ *                       finds no room for one step, and if one falls back both do.  Later calls ask again once there
+ *                       is room.
  *                     - A chain of few rows on a 16-bit head with W in {512, 1024, 1536} and var_out = 0 (groups of
  *                       16 tokens, or 8 with guidance: up to 33, 15 and 7 groups) runs as the group chain kernel:
  *                       everything that depends on the condition vector only is formed ahead, for many steps at a

@@ -78,7 +78,7 @@ struct csd_ctx {
   HostIo gc[2];    // group chain kernel (per chain slot): s of all steps
   HostIo gm[2];    // group and wide chain kernels: condition products of two chunks of steps (wide: s of a chunk before them)
   HostIo wx[2];    // wide chain kernel: what its column tiles exchange
-  size_t gc_refused[2] = {SIZE_MAX, SIZE_MAX}, gm_refused[2] = {SIZE_MAX, SIZE_MAX}, wx_refused[2] = {SIZE_MAX, SIZE_MAX};   // (wx: all of a wide chain's) sizes that could not be had: not asked for again
+  size_t gc_refused[2] = {SIZE_MAX, SIZE_MAX}, gm_refused[2] = {SIZE_MAX, SIZE_MAX}, wc_refused[2] = {SIZE_MAX, SIZE_MAX};   // sizes that could not be had (wc: gm and wx of a wide chain): asked for again where the device has as much free
   cudaStream_t aux[2] = {nullptr, nullptr};        // (per chain slot) where they are formed
   cudaEvent_t ev_prep[2] = {}, ev_mods[2][2] = {}, ev_read[2][2] = {};   // preparation done; a chunk is written / has been read
   cudaEvent_t ev_on[2] = {};                       // every block of a chunk's chain kernel has its SM
@@ -262,12 +262,17 @@ int give_up(csd_ctx* ctx, Buf& b) {
   return CSD_OK;
 }
 
+int sync_streams(csd_ctx* ctx) {
+  CSD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  for (int i = 0; i < 2; ++i) { CSD_CUDA(ctx, cudaStreamSynchronize(ctx->side[i])); CSD_CUDA(ctx, cudaStreamSynchronize(ctx->aux[i])); }
+  return CSD_OK;
+}
+
 // At least need bytes in b for the call that is being made.
 template <typename Buf>
 int ensure_buffer(csd_ctx* ctx, Buf& b, size_t need, const char* what) {
   if (need > b.cap) {
-    CSD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    for (int i = 0; i < 2; ++i) { CSD_CUDA(ctx, cudaStreamSynchronize(ctx->side[i])); CSD_CUDA(ctx, cudaStreamSynchronize(ctx->aux[i])); }
+    if (int rc = sync_streams(ctx)) return rc;
     if (int rc = give_up(ctx, b)) return rc;
     if (cudaMalloc(&b.base, need) != cudaSuccess) {
       cudaGetLastError();
@@ -278,6 +283,13 @@ int ensure_buffer(csd_ctx* ctx, Buf& b, size_t need, const char* what) {
   }
   b.in_graph = b.in_graph || capturing(ctx);
   return CSD_OK;
+}
+
+// Whether the device has need bytes free, counting `back` that would be given up first, and a little more.
+bool room_for(size_t need, size_t back) {
+  size_t free = 0, total = 0;
+  if (cudaMemGetInfo(&free, &total) != cudaSuccess) { cudaGetLastError(); return false; }
+  return free + back >= need + (size_t(32) << 20);
 }
 
 int ensure_ws(csd_ctx* ctx, ChainWs& ws, const csd_head_desc& d, int Rh, int R, int T) {
@@ -567,6 +579,7 @@ struct Chain {
   int Rh = 0, W = 0, L = 0, T = 0, tn = kTileN;
   bool gck = false, gfold = false;   // the whole chain runs in the group chain kernel (groupchain.cuh), in its folded form
   bool wck = false;       // the whole chain runs in the wide chain kernel (widechain.cuh)
+  bool wc_asked = false;  // its buffers have been asked for; wc_most 0: refused
   int beside = 0;         // CTAs that the other chain's wide chain kernel holds meanwhile
   WideCut wc{};
   int wc_most = 0;        // the most steps of a chunk
@@ -651,9 +664,11 @@ struct Chain {
     return CSD_OK;
   }
 
+  void sizes() { Rh = R * (cfg ? 2 : 1); W = hd->d.W; L = hd->d.L; Ts = sc->T; }
+
   int begin() {
     const csd_head_desc& d = hd->d;
-    Rh = R * (cfg ? 2 : 1); W = d.W; L = d.L; Ts = sc->T;
+    sizes();
     T = batch_Rin ? 1 : Ts;   // a batched pass runs the layers once
     tc = d.dtype != CSD_F32;
     // 64-wide output tiles when 128-wide ones (of all chains running side by side) would occupy at most a
@@ -699,7 +714,9 @@ struct Chain {
     if (gck && (rc = reserve_group_chain())) return rc;
     if (gck) { fold = false; pair = false; }
     wck = !gck && wide_takes(ctx, hd, R, cfg, slot, batch_Rin != 0);
-    if (wck && (rc = reserve_wide_chain())) return rc;
+    Chain* const self = this;
+    if (wck && !wc_asked && (rc = reserve_wide_chains(ctx, &self, 1))) return rc;
+    wck = wck && wc_most > 0;
     if (wck) { fold = false; pair = false; }
     // fp32 heads: one persistent kernel per chain, except where a row's bits have to be those of a batched pass
     fcg = !tc && ctx->chain_mode != CSD_CHAIN_LAYERS_PLAIN && !batch_Rin && !ctx->prof_on && fc_pays(ctx, d, Rh) ? fc_rows(ctx, d, R, cfg, chains) : 0;
@@ -862,9 +879,10 @@ struct Chain {
   size_t gc_wrows() const { return static_cast<size_t>(gfold ? 4 * L + 3 : 3 * L + 2) * W; }
   size_t gc_chunk_bytes(int steps) const { return gc_wrows() * ((static_cast<size_t>(steps) * gc_rows + 255) / 256) * 256 * 4; }
 
-  // ensure_buffer for buffers that a call can do without: a size that could not be had is not asked for again.
+  // ensure_buffer for buffers that a call can do without: a size that could not be had is asked for again only where there is room.
   int have(HostIo& io, size_t& refused, size_t need, const char* what) {
-    const int rc = need <= io.cap || need < refused ? ensure_buffer(ctx, io, need, what) : static_cast<int>(CSD_ERR_WORKSPACE);
+    if (need > io.cap && need >= refused && (capturing(ctx) || !room_for(need, io.in_graph ? 0 : io.cap))) return CSD_ERR_WORKSPACE;
+    const int rc = ensure_buffer(ctx, io, need, what);
     if (rc == CSD_ERR_WORKSPACE && need < refused) refused = need;
     return rc;
   }
@@ -872,6 +890,7 @@ struct Chain {
   // Buffers of the group chain kernel: bytes by the steps that a call has and the limit, so that no call of fewer steps or rows has to replace
   // them.  Shorter chunks cost a launch each and change no bit, so the buffers are halved until they can be had; where one step does
   // not fit the chain falls back to the layer kernels (gck), which need none of it.
+  static int reserve_wide_chains(csd_ctx* ctx, Chain* const* c, int n);
   int reserve_group_chain() {
     gc_rows = (R + (cfg ? 7 : 15)) / (cfg ? 8 : 16) * kGcRows;
     int rc = have(ctx->gc[slot], ctx->gc_refused[slot], static_cast<size_t>(Ts) * gc_rows * W * 2, "the condition vectors of all steps");
@@ -963,33 +982,12 @@ struct Chain {
   size_t wc_chunk_bytes(int steps) const { return wc_chunk_rows(steps) * (3 * L + 2) * W * 4; }
   size_t wc_step_bytes() const { return wc_chunk_rows(1) * W * 2 + 2 * wc_chunk_bytes(1); }
 
-  // Buffers of the wide chain kernel.  Bytes by the steps that a call has and the limit, and not a whole number of its steps: of two calls the
-  // one of fewer rows or blocks may have room for more steps, and must not have to replace what the other uses.  Where memory is
-  // short, shorter chunks (same bits), then the layer kernels (wck), which find their workspace taken first and everything else given back.
-  int reserve_wide_chain() {
-    if (!wc.slots) wc = wide_cut_alone(ctx, hd->d, R, cfg);
-    int rc = ensure_ws(ctx, ctx->ws[slot], hd->d, Rh, R, Ts);
-    if (rc) return rc;
-    const size_t exchange = wx_layout().total, step = wc_step_bytes(), least = exchange + step;
-    if (least >= ctx->wx_refused[slot]) { wck = false; return CSD_OK; }
-    const size_t m_refused = ctx->gm_refused[slot];
-    wc_most = Ts < kWcMaxSteps ? Ts : kWcMaxSteps;
-    size_t want = wc_most * step < kWcBufferBytes ? wc_most * step : kWcBufferBytes;
-    if (want < step) want = step;
-    rc = ensure_buffer(ctx, ctx->wx[slot], exchange, "the chain's exchange buffers");
-    while (!rc && (rc = have(ctx->gm[slot], ctx->gm_refused[slot], want, "the condition products")) == CSD_ERR_WORKSPACE && want > step) {
-      rc = CSD_OK;
-      want = want / 2 < step ? step : want / 2;
-    }
-    if (!rc && static_cast<size_t>(wc_most) > want / step) wc_most = static_cast<int>(want / step);
-    if (rc != CSD_ERR_WORKSPACE) return rc;
-    ctx->wx_refused[slot] = least; ctx->gm_refused[slot] = m_refused;
-    ctx->err[0] = 0;
-    wck = false;
-    CSD_CUDA(ctx, cudaStreamSynchronize(st));
-    CSD_CUDA(ctx, cudaStreamSynchronize(ctx->aux[slot]));
-    if ((rc = give_up(ctx, ctx->wx[slot]))) return rc;
-    return give_up(ctx, ctx->gm[slot]);
+  // Bytes of the wide chain kernel's chunk buffer: by the steps that a call has and the limit, and not a whole number of its steps - of two calls
+  // the one of fewer rows or blocks may have room for more steps, and must not have to replace what the other uses.  halvings: where
+  // memory is short, shorter chunks (same bits), down to one step.
+  size_t wc_need(int halvings) const {
+    const size_t step = wc_step_bytes(), all = step * (Ts < kWcMaxSteps ? Ts : kWcMaxSteps), want = all < kWcBufferBytes ? all : kWcBufferBytes;
+    return (want >> halvings) > step ? want >> halvings : step;
   }
   struct WxLayout { size_t stats, epart, xll, cnt, ticket, zeroed, u, v, hsum, total; };
   WxLayout wx_layout() const {
@@ -1183,11 +1181,84 @@ struct Chain {
   }
 };
 
+// Buffers of one wide chain, or of the two of a round, which find their workspaces taken first.  Where memory is short the chunks of both
+// get shorter; where not one step of each can be had both run the layer kernels (wc_most 0), so that equal heads of a round
+// run equal kernels, and everything is given back.
+int Chain::reserve_wide_chains(csd_ctx* ctx, Chain* const* c, int n) {
+  int rc = CSD_OK;
+  for (int i = 0; i < n; ++i) {
+    Chain& a = *c[i];
+    a.sizes();
+    a.wc_asked = true; a.wc_most = 0;
+    if (!a.wc.slots) a.wc = wide_cut_alone(ctx, a.hd->d, a.R, a.cfg);
+    if ((rc = ensure_ws(ctx, ctx->ws[a.slot], a.hd->d, a.Rh, a.R, a.Ts))) return rc;
+  }
+  auto drop = [&](bool exchange) {       // (what a graph holds would not come back)
+    rc = sync_streams(ctx);
+    for (int i = 0; i < n && !rc; ++i) {
+      if (!ctx->gm[c[i]->slot].in_graph) rc = give_up(ctx, ctx->gm[c[i]->slot]);
+      if (!rc && exchange && !ctx->wx[c[i]->slot].in_graph) rc = give_up(ctx, ctx->wx[c[i]->slot]);
+    }
+  };
+  bool tried = false;
+  for (int h = 0;; ++h) {
+    size_t need[2], grow = 0, back = 0, whole = 0, whole_back = 0;
+    bool refused = false, least = h > 0;
+    for (int i = 0; i < n; ++i) {
+      const int slot = c[i]->slot;
+      const HostIo* io[2] = {&ctx->gm[slot], &ctx->wx[slot]};
+      need[i] = c[i]->wc_need(h);
+      least = least && c[i]->wc_need(h - 1) == c[i]->wc_step_bytes();
+      const size_t want[2] = {need[i], c[i]->wx_layout().total};
+      for (int j = 0; j < 2; ++j) {
+        const size_t own = io[j]->in_graph ? 0 : io[j]->cap;
+        if (want[j] > io[j]->cap) { grow += want[j]; back += own; }
+        if (want[j] > io[j]->cap || own) { whole += want[j]; whole_back += own; }
+      }
+      refused = refused || want[0] + want[1] >= ctx->wc_refused[slot];
+    }
+    if (least) {                                  // one step of each was not to be had
+      if (tried) drop(true);
+      return rc;
+    }
+    if (grow && refused) {
+      if (capturing(ctx)) continue;
+      if (!room_for(grow, back)) {                // perhaps what one chain has and does not need serves both
+        if (!room_for(whole, whole_back)) continue;
+        drop(true);
+        if (rc) return rc;
+      }
+    }
+    for (int i = 0; i < n && !rc; ++i) {
+      tried = tried || grow;
+      rc = ensure_buffer(ctx, ctx->wx[c[i]->slot], c[i]->wx_layout().total, "the chain's exchange buffers");
+      if (!rc) rc = ensure_buffer(ctx, ctx->gm[c[i]->slot], need[i], "the condition products");
+    }
+    if (!rc) {
+      for (int i = 0; i < n; ++i) {
+        const int most = c[i]->Ts < kWcMaxSteps ? c[i]->Ts : kWcMaxSteps, fit = static_cast<int>(need[i] / c[i]->wc_step_bytes());
+        c[i]->wc_most = fit < most ? fit : most;
+      }
+      return CSD_OK;
+    }
+    if (rc != CSD_ERR_WORKSPACE) return rc;
+    rc = CSD_OK;
+    ctx->err[0] = 0;
+    for (int i = 0; i < n; ++i) {
+      size_t& r = ctx->wc_refused[c[i]->slot];
+      const size_t all = need[i] + c[i]->wx_layout().total;
+      if (all < r) r = all;
+    }
+    drop(false);
+    if (rc) return rc;
+  }
+}
+
 // The two chains of a round in the wide chain kernel: side by side in the forms that take the least time by the model, as long as they
 // leave some SMs to the condition products; else one after the other.
-void place_wide_chains(Chain& a, Chain& b) {
+int place_wide_chains(Chain& a, Chain& b) {
   csd_ctx* ctx = a.ctx;
-  if (!wide_takes(ctx, a.hd, a.R, a.cfg, a.slot, false) || !wide_takes(ctx, b.hd, b.R, b.cfg, b.slot, false)) return;
+  if (!wide_takes(ctx, a.hd, a.R, a.cfg, a.slot, false) || !wide_takes(ctx, b.hd, b.R, b.cfg, b.slot, false)) return CSD_OK;
   const csd_head_desc &da = a.hd->d, &db = b.hd->d;
   double best = 0.0;
   for (int i = 0; i < 4; ++i) {
@@ -1202,7 +1273,10 @@ void place_wide_chains(Chain& a, Chain& b) {
     best = us;
     a.wc = ca; b.wc = cb; a.beside = cb.ctas; b.beside = ca.ctas;
   }
-  if (best <= 0.0) a.st = b.st;
+  Chain* const both[2] = {&b, &a};
+  if (int rc = Chain::reserve_wide_chains(ctx, both, 2)) return rc;
+  if (best <= 0.0 && b.wc_most > 0) a.st = b.st;
+  return CSD_OK;
 }
 
 int run_chain(csd_ctx* ctx, int slot, cudaStream_t st, const csd_head* hd, const csd_schedule* sc, int R, int cfg,
@@ -2128,7 +2202,7 @@ static int round_impl(csd_ctx* ctx, const csd_head* head_q, const csd_head* head
   Chain cp = bonus ? Chain{ctx, 1, st_p, head_p, sched_p, Rp, cfg, cfg_scale, bb.z, bb.x_T, bb.eps, 1, bb.x0, bb.mu1, nullptr}
                    : Chain{ctx, 1, st_p, head_p, sched_p, R, cfg, cfg_scale, z_p, x_T, eps, 0, nullptr, mu1_p, nullptr};
   cq.chains = cp.chains = 2;
-  place_wide_chains(cq, cp);
+  if ((rc = place_wide_chains(cq, cp))) return rc;
   rc = cp.begin();
   int rc2 = cq.begin();
   for (int t = sched_p->T; t >= 1 && !rc && !rc2; --t) {
@@ -2282,7 +2356,7 @@ int csd_round_lv(csd_ctx* ctx, const csd_head* head_q, const csd_head* head_p, c
   Chain cp = make_lv_chain(ctx, 1, ctx->side[1 - sq], head_p, &vp, sched_p, R, cfg, cfg_scale, z_p, x_T, eps, 0, nullptr, mu1_p,
                            lv1_p, half_logdet_p, nullptr);
   cq.chains = cp.chains = 2;
-  place_wide_chains(cq, cp);
+  if ((rc = place_wide_chains(cq, cp))) return rc;
   rc = cp.begin();
   int rc2 = cq.begin();
   for (int t = sched_p->T; t >= 1 && !rc && !rc2; --t) {

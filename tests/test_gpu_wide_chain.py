@@ -113,6 +113,41 @@ def test_little_memory_left_shorter_chunks_and_the_same_bits():
         d.ctx.close()
 
 
+def test_round_of_equal_heads_with_little_memory_left_runs_equal_kernels():
+    # room for one step's products of both chains, or for several of the first to ask: both get one; and all they want once there is room again
+    from paper_2411_11925_b200 import api
+    from paper_2411_11925_b200.runner import DeviceRound
+    inp = gen.make_round_inputs(_wl(bf16=True, B=600, gamma=1, T=40, draft=H(2, 1024, 64), target=H(2, 1024, 64)))
+    inp.w_q, inp.z_q = inp.w_p, inp.z_p
+    ref, tight = DeviceRound(inp), DeviceRound(inp)
+
+    def launches(dr):
+        l0 = dr.ctx.launch_count()
+        dr.fused_round()
+        dr.ctx.sync()
+        return dr.ctx.launch_count() - l0
+
+    n = launches(ref)
+    tight.ctx.set_chain_mode(api.Context.CHAIN_LAYER_KERNELS)       # (workspaces, and kernels loaded)
+    launches(tight)
+    tight.ctx.set_chain_mode(api.Context.CHAIN_LAYERS)
+    same = torch.zeros((), dtype=torch.bool, device="cuda")
+    torch.cuda.synchronize()
+    hog = []
+    try:
+        while (free := torch.cuda.mem_get_info()[0]) > 154 << 20:
+            hog.append(torch.empty((free - (150 << 20)) >> 21 << 21, dtype=torch.uint8, device="cuda"))
+        m = launches(tight)
+        same.copy_((tight.x0 == ref.x0).all() & (tight.logratio == 0).all())
+    finally:
+        hog.clear()
+        torch.cuda.empty_cache()
+    assert bool(same) and n + 100 < m < 300, (n, m)                # three launches a step and chain; the layer kernels are eight and one
+    assert launches(tight) == n and bool((tight.x0 == ref.x0).all())
+    for d in (ref, tight):
+        d.ctx.close()
+
+
 def test_captured_round_replays():
     from paper_2411_11925_b200 import api
     from paper_2411_11925_b200.runner import DeviceRound
