@@ -583,6 +583,7 @@ struct Chain {
   int beside = 0;         // CTAs that the other chain's wide chain kernel holds meanwhile
   WideCut wc{};
   int wc_most = 0;        // the most steps of a chunk
+  struct { WcParams p; CUtensorMap tm_s, tm_u, tm_v; int t_hi, n, launched; } wq{};   // first step and number of steps of the next and the last chunk, launches so far
   int gc_rows = 0, gc_most = 0;      // its rows (groups x 16) and the most steps of a chunk
   int fcg = 0;            // fp32 head: the whole chain runs in the fp32 chain kernel with groups of this many rows (f32chain.cuh)
   bool fold = false;      // blocks 1.. run as two kernels (fold.cuh) instead of three
@@ -761,7 +762,7 @@ struct Chain {
     if (rc) return rc;
     sbuf[0] = ws.s2; sbuf[1] = ws.s;
     if (gck) return launch_group_chain();
-    if (wck) return launch_wide_chain();
+    if (wck) return begin_wide_chain();
     if (batch_Rin) return launch_batch(0);   // a pass has one step (t = 1): its s is sbuf[1]
     sp.traj_x = traj_x; sp.traj_mu = nullptr; sp.status = ctx->d_err + 1;
     sp.lv1 = lv1; sp.half_logdet = half_logdet; sp.lv_min = 0.0f; sp.lv_max = 0.0f;
@@ -1003,34 +1004,40 @@ struct Chain {
     return l;
   }
 
-  // The wide chain kernel, chunk by chunk of steps and part by part of the rows: s and the condition products on the slot's
-  // own stream, ahead of the chain.
-  int launch_wide_chain() {
+  // The wide chain kernel, chunk by chunk of steps (launched with a chunk's first step) and part by part of the rows: s and the
+  // condition products on the slot's own stream, ahead of the chain.
+  int begin_wide_chain() {
     const csd_head_desc& d = hd->d;
     ChainWs& ws = ctx->ws[slot];
     const WxLayout l = wx_layout();
     char* const xb = static_cast<char*>(ctx->wx[slot].base);
-    const size_t chunk = wc_chunk_bytes(wc_most);
-    void* const s_chunk = ctx->gm[slot].base;
-    char* const gm = static_cast<char*>(s_chunk) + wc_chunk_rows(wc_most) * W * 2;
-    int* const tickets = reinterpret_cast<int*>(xb + l.ticket);
-    const bool f16 = d.dtype == CSD_F16, lv = lv_min != nullptr;
     int rc;
-    CUtensorMap tm_s{}, tm_uu{}, tm_vv{};
-    if ((rc = make_tmap(ctx, &tm_s, d.dtype, s_chunk, wc_chunk_rows(wc_most), W, W, kTileM))) return rc;
+    if ((rc = make_tmap(ctx, &wq.tm_s, d.dtype, ctx->gm[slot].base, wc_chunk_rows(wc_most), W, W, kTileM))) return rc;
     const uint64_t lines = static_cast<uint64_t>(wc.nb) * kTileM * W / 256;      // u, v as lines of 256 elements: 32 of them a k-block
-    if ((rc = make_plain_tmap(ctx, &tm_uu, d.dtype, xb + l.u, lines)) || (rc = make_plain_tmap(ctx, &tm_vv, d.dtype, xb + l.v, lines))) return rc;
+    if ((rc = make_plain_tmap(ctx, &wq.tm_u, d.dtype, xb + l.u, lines)) || (rc = make_plain_tmap(ctx, &wq.tm_v, d.dtype, xb + l.v, lines))) return rc;
     CSD_CUDA(ctx, cudaMemsetAsync(xb, 0, l.zeroed, st));
-    cudaStream_t gst = ctx->aux[slot];
     CSD_CUDA(ctx, cudaEventRecord(ctx->ev_prep[slot], st));
-    CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_prep[slot], 0));
-    WcParams p{};
+    CSD_CUDA(ctx, cudaStreamWaitEvent(ctx->aux[slot], ctx->ev_prep[slot], 0));
+    WcParams& p = wq.p;
     p.R = R; p.cfg = cfg; p.W = W; p.L = L; p.C = d.C; p.T = Ts; p.sample_last = sample_last; p.cfg_scale = cfg_scale;
     p.maps = hd->d_wc_maps; p.b1 = hd->b1[0]; p.b2 = hd->b2[0]; p.win = hd->win; p.bin = hd->bin; p.wout_t = hd->wout_t; p.bout = hd->bout;
     p.x_T = x_T; p.eps = eps; p.x = ws.x; p.x0 = x0; p.mu1 = mu1; p.x1 = x1; p.traj_x = traj_x; p.traj_mu = traj_mu;
     p.u = xb + l.u; p.v = xb + l.v; p.stats = reinterpret_cast<ulonglong2*>(xb + l.stats); p.epart = reinterpret_cast<ulonglong2*>(xb + l.epart);
     p.xll = reinterpret_cast<ulonglong2*>(xb + l.xll); p.cnt = reinterpret_cast<unsigned*>(xb + l.cnt); p.hsum = reinterpret_cast<float*>(xb + l.hsum);
     p.lv1 = lv1; p.half_logdet = half_logdet; p.err = ctx->d_err; p.status = ctx->d_err + 1;
+    wq.t_hi = Ts;
+    return CSD_OK;
+  }
+  int launch_wide_chunk() {
+    const csd_head_desc& d = hd->d;
+    ChainWs& ws = ctx->ws[slot];
+    const size_t chunk = wc_chunk_bytes(wc_most);
+    void* const s_chunk = ctx->gm[slot].base;
+    char* const gm = static_cast<char*>(s_chunk) + wc_chunk_rows(wc_most) * W * 2;
+    int* const tickets = reinterpret_cast<int*>(static_cast<char*>(ctx->wx[slot].base) + wx_layout().ticket);
+    const bool f16 = d.dtype == CSD_F16, lv = lv_min != nullptr;
+    cudaStream_t gst = ctx->aux[slot];
+    WcParams& p = wq.p;
     WmParams m{};
     m.nkb = W / kBlockK; m.nwt = (3 * L + 2) * W / 256; m.sb = 32; m.wrow = hd->d_wc_rows; m.bias = hd->d_wc_bias; m.err = ctx->d_err;
     cudaLaunchAttribute at[2];
@@ -1046,49 +1053,50 @@ struct Chain {
     // its SMs; a chain that holds most of it takes turns with them.
     const int held = wc.ctas + beside, free_pairs = (held <= ctx->num_sms / 2 ? ctx->num_sms - held : ctx->num_sms) / 2;
     // Steps per chunk: one first, because nothing overlaps its products; then twice as many each time, as far as the buffers go.
-    int n = 1, c = 0;
-    for (int t_hi = Ts; t_hi >= 1; n *= 2) {
-      if (t_hi <= 4) n = t_hi;      // (short schedules)
-      if (n > wc_most) n = wc_most;
-      if (n > t_hi) n = t_hi;
-      const int t_lo = t_hi - n + 1;
-      for (int i = 0; i < n; ++i) {
-        p.ca[i] = sc->a[t_lo - 1 + i]; p.cb[i] = sc->b[t_lo - 1 + i];
-        p.s0[i] = lv ? lv_min[t_lo - 1 + i] : sc->sigma[t_lo - 1 + i]; p.s1[i] = lv ? lv_max[t_lo - 1 + i] : 0.0f;
-      }
-      for (int s0 = 0; s0 < wc.slots; s0 += wc.part, ++c) {
-        const int slots = wc.slots - s0 < wc.part ? wc.slots - s0 : wc.part, rows = slots * kWcRows, buf = c & 1;
-        float* const mods = reinterpret_cast<float*>(gm + buf * chunk);
-        if (c >= 2) CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_read[slot][buf], 0));
-        if (c >= 1) CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_on[slot], 0));
-        CSD_CUDA(ctx, cudaMemsetAsync(tickets + buf, 0, sizeof(int), gst));
-        const dim3 sgrid(static_cast<unsigned>(rows), static_cast<unsigned>((n + kCondSteps - 1) / kCondSteps));
-        const float* te = ws.te + static_cast<size_t>(t_lo - 1) * W;
-        if (f16) cond_all_kernel<__half, 128><<<sgrid, 128, 0, gst>>>(ws.cz, te, static_cast<__half*>(s_chunk), R, cfg, W, rows, s0 * kWcRows, n);
-        else cond_all_kernel<__nv_bfloat16, 128><<<sgrid, 128, 0, gst>>>(ws.cz, te, static_cast<__nv_bfloat16*>(s_chunk), R, cfg, W, rows, s0 * kWcRows, n);
-        CSD_CUDA(ctx, cudaGetLastError());
-        m.nst = n * slots; m.ticket = tickets + buf; m.out = mods;
-        int pairs = c == 0 ? ctx->num_sms / 2 : free_pairs;
-        if (pairs > m.nst * m.nwt) pairs = m.nst * m.nwt;
-        lc.gridDim = dim3(static_cast<unsigned>(2 * pairs)); lc.blockDim = dim3(kMgThreads); lc.dynamicSmemBytes = kMgSmemBytes; lc.stream = gst; lc.numAttrs = 1;
-        if (f16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, wide_mods_kernel<0>, hd->Wrows, tm_s, m));
-        else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, wide_mods_kernel<1>, hd->Wrows, tm_s, m));
-        CSD_CUDA(ctx, cudaEventRecord(ctx->ev_mods[slot][buf], gst));
-        CSD_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_mods[slot][buf], 0));
-        p.t_hi = t_hi; p.t_lo = t_lo; p.slot0 = s0; p.slots = slots; p.mods = mods;
-        lc.gridDim = dim3(static_cast<unsigned>((wc.halves == 2 ? slots : (slots + 1) / 2) * 2 * (W / 128))); lc.blockDim = dim3(kWcThreads);
-        lc.dynamicSmemBytes = wc_layout(L, lv ? kCPad2 : kCPad, wc.halves).total + 1024; lc.stream = st; lc.numAttrs = 2;
-        CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, wide_kernel(d.dtype, lv, wc.halves), tm_uu, tm_vv, p));
-        CSD_CUDA(ctx, cudaEventRecord(ctx->ev_read[slot][buf], st));
-        ctx->launches += 3;
-      }
-      t_hi = t_lo - 1;
+    int& n = wq.n;
+    const int t_hi = wq.t_hi;
+    n = n ? 2 * n : 1;
+    if (t_hi <= 4) n = t_hi;      // (short schedules)
+    if (n > wc_most) n = wc_most;
+    if (n > t_hi) n = t_hi;
+    const int t_lo = t_hi - n + 1;
+    for (int i = 0; i < n; ++i) {
+      p.ca[i] = sc->a[t_lo - 1 + i]; p.cb[i] = sc->b[t_lo - 1 + i];
+      p.s0[i] = lv ? lv_min[t_lo - 1 + i] : sc->sigma[t_lo - 1 + i]; p.s1[i] = lv ? lv_max[t_lo - 1 + i] : 0.0f;
     }
+    for (int s0 = 0; s0 < wc.slots; s0 += wc.part, ++wq.launched) {
+      const int slots = wc.slots - s0 < wc.part ? wc.slots - s0 : wc.part, rows = slots * kWcRows, c = wq.launched, buf = c & 1;
+      float* const mods = reinterpret_cast<float*>(gm + buf * chunk);
+      if (c >= 2) CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_read[slot][buf], 0));
+      if (c >= 1) CSD_CUDA(ctx, cudaStreamWaitEvent(gst, ctx->ev_on[slot], 0));
+      CSD_CUDA(ctx, cudaMemsetAsync(tickets + buf, 0, sizeof(int), gst));
+      const dim3 sgrid(static_cast<unsigned>(rows), static_cast<unsigned>((n + kCondSteps - 1) / kCondSteps));
+      const float* te = ws.te + static_cast<size_t>(t_lo - 1) * W;
+      if (f16) cond_all_kernel<__half, 128><<<sgrid, 128, 0, gst>>>(ws.cz, te, static_cast<__half*>(s_chunk), R, cfg, W, rows, s0 * kWcRows, n);
+      else cond_all_kernel<__nv_bfloat16, 128><<<sgrid, 128, 0, gst>>>(ws.cz, te, static_cast<__nv_bfloat16*>(s_chunk), R, cfg, W, rows, s0 * kWcRows, n);
+      CSD_CUDA(ctx, cudaGetLastError());
+      m.nst = n * slots; m.ticket = tickets + buf; m.out = mods;
+      int pairs = c == 0 ? ctx->num_sms / 2 : free_pairs;
+      if (pairs > m.nst * m.nwt) pairs = m.nst * m.nwt;
+      lc.gridDim = dim3(static_cast<unsigned>(2 * pairs)); lc.blockDim = dim3(kMgThreads); lc.dynamicSmemBytes = kMgSmemBytes; lc.stream = gst; lc.numAttrs = 1;
+      if (f16) CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, wide_mods_kernel<0>, hd->Wrows, wq.tm_s, m));
+      else CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, wide_mods_kernel<1>, hd->Wrows, wq.tm_s, m));
+      CSD_CUDA(ctx, cudaEventRecord(ctx->ev_mods[slot][buf], gst));
+      CSD_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_mods[slot][buf], 0));
+      p.t_hi = t_hi; p.t_lo = t_lo; p.slot0 = s0; p.slots = slots; p.mods = mods;
+      lc.gridDim = dim3(static_cast<unsigned>((wc.halves == 2 ? slots : (slots + 1) / 2) * 2 * (W / 128))); lc.blockDim = dim3(kWcThreads);
+      lc.dynamicSmemBytes = wc_layout(L, lv ? kCPad2 : kCPad, wc.halves).total + 1024; lc.stream = st; lc.numAttrs = 2;
+      CSD_CUDA(ctx, cudaLaunchKernelEx(&lc, wide_kernel(d.dtype, lv, wc.halves), wq.tm_u, wq.tm_v, p));
+      CSD_CUDA(ctx, cudaEventRecord(ctx->ev_read[slot][buf], st));
+      ctx->launches += 3;
+    }
+    wq.t_hi = t_lo - 1;
     return CSD_OK;
   }
 
   int step(int t) {
-    if (gck || wck || fcg) return CSD_OK;   // already enqueued by begin()
+    if (gck || fcg) return CSD_OK;   // already enqueued by begin()
+    if (wck) return t == wq.t_hi ? launch_wide_chunk() : static_cast<int>(CSD_OK);
     const csd_head_desc& d = hd->d;
     ChainWs& ws = ctx->ws[slot];
     cur_t = t;
