@@ -546,9 +546,9 @@ bool wide_halves(const csd_head_desc& d) { return wc_layout(d.L, d.var_out ? kCP
 double wide_step_us(const csd_head_desc& d, int halves) { return halves == 2 ? 30.0 + 12.7 * d.L * d.W / 1024 : 20.0 + 22.0 * d.L * d.W / 1024; }
 double wide_mods_sm_us(const csd_head_desc& d, int slots) { return 2.0 * (3 * d.L + 2) * d.W * d.W * kWcRows * slots / 8.8e6; }   // 8.8 TFLOP/s an SM
 // Beside chains that hold at most half of the SMs the products have the rest to themselves; else everything shares the GPU, at about
-// 120 of 148 SMs' worth.
-double wide_us(const csd_ctx* ctx, double chain_us, double chain_sm_us, double mods_sm_us, int held) {
-  const double other = held <= ctx->num_sms / 2 ? mods_sm_us / (ctx->num_sms - held) : (mods_sm_us + chain_sm_us) / (0.81 * ctx->num_sms);
+// 120 of 148 SMs' worth (two chains, which fill each other's gaps: 133).
+double wide_us(const csd_ctx* ctx, double chain_us, double chain_sm_us, double mods_sm_us, int held, double share = 0.81) {
+  const double other = held <= ctx->num_sms / 2 ? mods_sm_us / (ctx->num_sms - held) : (mods_sm_us + chain_sm_us) / (share * ctx->num_sms);
   return chain_us > other ? chain_us : other;
 }
 WideCut wide_cut_alone(const csd_ctx* ctx, const csd_head_desc& d, int R, int cfg) {
@@ -1276,7 +1276,10 @@ int place_wide_chains(Chain& a, Chain& b) {
     const int held = ca.ctas + cb.ctas;
     if (ca.part < ca.slots || cb.part < cb.slots || held > ctx->num_sms - 18) continue;
     const double ta = wide_step_us(da, ha), tb = wide_step_us(db, hb);
-    const double us = wide_us(ctx, ta > tb ? ta : tb, ta * ca.ctas + tb * cb.ctas, wide_mods_sm_us(da, ca.slots) + wide_mods_sm_us(db, cb.slots), held);
+    // Beside another chain and its products a step of two-slot groups takes a quarter longer: 1, 2, 4, 8 x 1024, 1024 rows of each chain, 49, 79,
+    // 133, 241 us where the formula has 42, 64, 108, 196.
+    const double la = ta * (ha == 1 ? 1.25 : 1.0), lb = tb * (hb == 1 ? 1.25 : 1.0);
+    const double us = wide_us(ctx, la > lb ? la : lb, ta * ca.ctas + tb * cb.ctas, wide_mods_sm_us(da, ca.slots) + wide_mods_sm_us(db, cb.slots), held, 0.9);
     if (best > 0.0 && us >= best) continue;
     best = us;
     a.wc = ca; b.wc = cb; a.beside = cb.ctas; b.beside = ca.ctas;
