@@ -558,15 +558,9 @@ WideCut wide_cut_alone(const csd_ctx* ctx, const csd_head_desc& d, int R, int cf
   return us(one) <= us(two) ? one : two;
 }
 constexpr size_t kWcBufferBytes = size_t(2) << 30;    // most bytes of a chunk of steps: s and two buffers of condition products
-// More than one slot of rows, up to what two-slot groups of 1024-wide heads cover at a time.  Beyond that the layer kernels' waves of tiles
-// fill the GPU as well, and the chain's hand-overs cost more than the dense product of the conditions saves.  ms a round of 20 steps with
-// guidance, before (persistent chain or layer kernels) / this kernel, at 512, 1024, 2048, 4096 and 8192 head rows of each head:
-//   3 and 6 x 1024:   3.13 / 2.25   3.16 / 2.93   6.44 / 5.23   11.3 / 10.6   18.8 / 21.2
-//   6 x 1024, 12 x 1536:  5.89 / 5.32   10.8 / 8.05   18.6 / 17.1   34.0 / 32.9   61.7 / 66.9
-constexpr int kWcMostRows = 4608;
 bool wide_takes(const csd_ctx* ctx, const csd_head* hd, int R, int cfg, int slot, bool batch) {
   const int rows = R * (cfg ? 2 : 1);
-  return wide_width(hd->d) && ctx->chain_mode == CSD_CHAIN_LAYERS && slot != 2 && !batch && !ctx->prof_on && rows > kWcRows && rows <= kWcMostRows &&
+  return wide_width(hd->d) && ctx->chain_mode == CSD_CHAIN_LAYERS && slot != 2 && !batch && !ctx->prof_on && wide_pays(hd->d.L, hd->d.W, rows) &&
          wide_groups(wide_pairs(ctx, hd->d.dtype), hd->d.W) >= 1;      // (a device, or a part of one, with fewer SMs than a group has CTAs)
 }
 // One head's denoising chain for R token rows on stream `st` with workspace slot `slot`:

@@ -14,6 +14,7 @@ def plan(tmp_path_factory):
     src = d / "plan.cpp"
     src.write_text('#include "wideplan.h"\n'
                    'extern "C" int groups(int pairs, int W) { return csd::wide_groups(pairs, W); }\n'
+                   'extern "C" int pays(int L, int W, int rows) { return csd::wide_pays(L, W, rows); }\n'
                    'extern "C" void cut(int most, int W, int R, int cfg, int halves, int* o) {\n'
                    '  const csd::WideCut c = csd::wide_cut(most, W, R, cfg, halves);\n'
                    '  o[0] = c.nb; o[1] = c.slots; o[2] = c.part; o[3] = c.ctas;\n}\n')
@@ -52,3 +53,9 @@ def test_cuts_of_a_whole_device(plan):
     assert _cut(plan, plan.groups(74, 1024), 1024, 512, 1, 2) == [8, 4, 4, 64]
     assert _cut(plan, plan.groups(74, 1536), 1536, 2048, 1, 1) == [32, 16, 8, 96]
     assert _cut(plan, plan.groups(74, 2048), 2048, 1536, 1, 2) == [24, 12, 4, 128]
+
+
+def test_rows_that_take_the_kernel(plan):
+    for L, W, least, most in ((1, 768, 683, 4608), (1, 1024, 512, 4608), (1, 1280, 410, 3710), (1, 1536, 385, 3092), (1, 2048, 385, 2319),
+                              (2, 768, 257, 4608), (2, 1024, 257, 4608), (12, 1280, 257, 3710), (12, 1536, 385, 3092), (8, 2048, 385, 2319)):
+        assert [plan.pays(L, W, r) for r in (1, least - 1, least, most, most + 1, 1 << 30)] == [0, 0, 1, 1, 0, 0], (L, W)
