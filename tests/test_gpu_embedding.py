@@ -22,7 +22,8 @@ def _cancelling(rng, rows, K):
 
 @pytest.mark.parametrize("op,mode,L,W,R,T,F", [
     ("f16", 0, 2, 512, 5, 3, 256),         # group chain kernel
-    ("f16", 0, 1, 1024, 300, 2, 10),       # persistent chain kernel; feature rows of 40 bytes
+    ("f16", 0, 1, 1024, 300, 2, 10),       # layer kernels; feature rows of 40 bytes
+    ("f16", 0, 2, 1024, 300, 2, 10),       # wide chain kernel
     ("bf16", 2, 1, 256, 3, 65, 30),        # layer kernels; more steps than two tiles of rows
     ("f16", 2, 1, 128, 3, 64, 256),
     ("f32", 2, 1, 384, 3, 9, 33),

@@ -233,19 +233,22 @@ def test_constant_variance_output_reproduces_the_fixed_variance_calls():
 def test_mar256_shaped_round_sampled_sequences():
     # B=64, gamma=8, T=100, guidance, 3x1024 and 6x1024 heads with 32 output columns; the checker evaluates the
     # first and last sequence and both sides of a 128-row tile boundary
+    from paper_2411_11925_b200 import api
     inp = _inputs(gen.WORKLOADS["mar256"])
-    wl = inp.wl
     r = LvRound(inp)
-    r.fused()
-    g = r.results()
-    assert np.all(np.isfinite(g["x0"])) and np.all(np.isfinite(g["logratio"]))
     seqs = [0, 15, 16, 63]
     sub = gen.select_sequences(inp, seqs)
-    _compare(g, _ref(sub), sub.wl, sub.u, rows=sub.extras["rows"], seqs=seqs, label="lv mar256-shaped")
-    r.fused()
-    again = r.results()
-    for k in LvRound.NAMES:
-        np.testing.assert_array_equal(g[k], again[k], err_msg=k)
+    ref = _ref(sub)
+    for mode in (api.Context.CHAIN_LAYERS, api.Context.CHAIN_LAYER_KERNELS):        # wide chain kernel; layer kernels, folded blocks
+        r.ctx.set_chain_mode(mode)
+        r.fused()
+        g = r.results()
+        assert np.all(np.isfinite(g["x0"])) and np.all(np.isfinite(g["logratio"]))
+        _compare(g, ref, sub.wl, sub.u, rows=sub.extras["rows"], seqs=seqs, label=f"lv mar256-shaped, chain mode {mode}")
+        r.fused()
+        again = r.results()
+        for k in LvRound.NAMES:
+            np.testing.assert_array_equal(g[k], again[k], err_msg=k)
     r.ctx.close()
 
 

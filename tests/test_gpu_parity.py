@@ -207,11 +207,22 @@ def test_argument_errors_are_reported_not_raised_by_the_device():
 
 
 def _sampled(name, seqs, label):
-    wl = gen.WORKLOADS[name]
-    inp = gen.make_round_inputs(wl)
-    dr, out = _run(inp, fused=True)
+    # in the default mode and with the layer kernels only, which run these sizes where the wide chain kernel does not
+    from paper_2411_11925_b200 import api
+    from paper_2411_11925_b200.runner import DeviceRound
+    inp = gen.make_round_inputs(gen.WORKLOADS[name])
+    dr = DeviceRound(inp)
     sub = gen.select_sequences(inp, seqs)
-    ref, s1q, s1p = _ref(sub)
+    ref = _ref(sub)
+    for mode in (api.Context.CHAIN_LAYERS, api.Context.CHAIN_LAYER_KERNELS):
+        dr.ctx.set_chain_mode(mode)
+        dr.fused_round()
+        _check_sampled(inp.wl, dr.results(), sub, ref, seqs, f"{label}, chain mode {mode}")
+    dr.ctx.close()
+
+
+def _check_sampled(wl, out, sub, ref, seqs, label):
+    ref, s1q, s1p = ref
     rows = sub.extras["rows"]
     gsub = {k: (out[k][rows] if out[k].shape[0] == wl.R else out[k][seqs]) for k in out if k != "cap_hits"}
     gsub["cap_hits"] = out["cap_hits"]
@@ -222,8 +233,6 @@ def _sampled(name, seqs, label):
     np.testing.assert_array_equal(out["flags"] & 1, (out["n_accept"] < wl.gamma).astype(out["flags"].dtype))
     assert np.all(np.isfinite(out["x0"])) and np.all(np.isfinite(out["logratio"]))
     assert int(out["cap_hits"][0]) == int(((out["flags"] & 2) != 0).sum())
-    dr.ctx.close()
-    return st
 
 
 # Sampled sequences at full size: the first and the last sequence, both sides of the first 128-row tile boundary
@@ -261,8 +270,8 @@ def test_mar512_full_size_sampled_sequences():
 
 
 def test_large_target_full_size_sampled_sequences():
-    # B=128, gamma=16, T=100, guidance: 4096 head rows = 32 row tiles in CTA pairs, W=1536 = 12 column tiles; eight
-    # sequences per tile: 7 | 8 straddle a tile, 15 | 16 a pair
+    # B=128, gamma=16, T=100, guidance: 4096 head rows = 32 row tiles, W=1536 = 12 column tiles, in CTA pairs (the target in
+    # either mode); eight sequences per tile: 7 | 8 straddle a tile, 15 | 16 a pair
     _sampled("large_target", [0, 7, 8, 15, 16, 64, 126, 127], "large_target sampled")
 
 
@@ -293,10 +302,27 @@ def test_degenerate_sizes_single_row_single_step_widest_scan(op):
 
 
 @pytest.mark.parametrize("op", ["bf16", "f16"])
+@pytest.mark.parametrize("B", [100, 130])       # three row tiles: single CTAs; four: CTA pairs
+def test_folded_blocks_match_checker(op, B):
+    from paper_2411_11925_b200 import api
+    from paper_2411_11925_b200.runner import DeviceRound
+    inp = gen.make_round_inputs(_wl(B=B, gamma=3, T=4, bf16=True, operand=op, draft=gen.HeadSpec(2, 1024, 64), target=gen.HeadSpec(3, 1280, 64)))
+    dr = DeviceRound(inp)
+    dr.ctx.set_chain_mode(api.Context.CHAIN_LAYER_KERNELS)
+    l0 = dr.ctx.launch_count()
+    dr.three_calls()
+    out = dr.results()
+    assert dr.ctx.launch_count() - l0 == 4 * (7 + 9) + 2 * 5 + 2        # 2 L + 3 kernels a step: blocks folded
+    ref, s1q, s1p = _ref(inp)
+    compare_round(out, ref, inp.wl, s1q, s1p, inp.u, inp.v, f"folded {op} {B}", xi=inp.xi)
+    dr.ctx.close()
+
+
+@pytest.mark.parametrize("op", ["bf16", "f16"])
 def test_chain_layouts_agree(op):
-    # csd_set_chain_mode.  CHAIN_LAYERS_PLAIN runs three kernels per block everywhere.  The default layout folds
-    # LayerNorm into the first layer's epilogue from the second block on where its grid rule applies: the same
-    # function rounded differently, so it is held to a quarter of a trajectory's tolerance (short chains here: far
+    # csd_set_chain_mode.  CHAIN_LAYERS_PLAIN runs three kernels per block everywhere.  The default layout runs the wide chain kernel
+    # where its rule applies, else it folds LayerNorm into the first layer's epilogue from the second block on where that rule
+    # applies: the same function rounded differently, so it is held to a quarter of a trajectory's tolerance (short chains here: far
     # inside it).  In either layout csd_round returns the bits of the three calls, and a repeat returns the same bits.
     from paper_2411_11925_b200.runner import DeviceRound
     from paper_2411_11925_b200 import api

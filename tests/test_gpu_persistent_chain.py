@@ -1,6 +1,7 @@
-"""The persistent chain kernel (one launch per chain when a layer is one wave of 128 x 128 tiles and W = 1024): whole
-rounds against the float64 checker, against the three-kernel layer layout, fused against separate calls, with guidance
-and without, ragged token counts, both operand formats, one-block and several-block heads."""
+"""Chains whose kernels run through all steps of a chunk, at the sizes of a round of 1024-wide heads (the wide chain kernel; a
+one-block draft of few rows runs the layer kernels): whole rounds against the float64 checker, against the three-kernel layer
+layout, fused against separate calls, with guidance and without, ragged token counts, both operand formats, one-block and
+several-block heads."""
 import numpy as np
 import pytest
 
@@ -47,11 +48,11 @@ def test_persistent_chain_round_matches_checker_and_the_plain_layers(op, kw):
     dr.three_calls()
     a = dr.results()
     launches = dr.ctx.launch_count() - l0
-    assert launches < 30, launches           # two chains of one kernel each (plus their set-up), not 2 T (2L + 3)
+    assert launches < 30, launches           # two chains of three kernels a chunk of steps (plus their set-up), not T (2L + 3) each
     ref, s1 = _ref(inp)
     st = compare_round(a, ref, inp.wl, s1, s1, inp.u, inp.v, f"persistent chain {op} {kw}", xi=inp.xi)
     print("persistent chain", op, kw, {k: st[k] for k in ("x0_err", "mu1p_err", "logr_err_over_tol")}, "launches", launches)
-    # the fused round launches the same two kernels side by side: same bits; and so does a repeat
+    # the fused round runs the two chains side by side: same bits; and so does a repeat
     dr.fused_round()
     b = dr.results()
     dr.three_calls()
@@ -87,7 +88,7 @@ def test_identical_heads_give_exactly_zero_in_the_persistent_chain():
 
 
 def test_recorded_trajectory_is_the_chain_itself():
-    # csd_draft_denoise_traj through the persistent kernel: the records' last slots are the call's outputs, every
+    # csd_draft_denoise_traj through the wide chain kernel: the records' last slots are the call's outputs, every
     # recorded state is the recorded mean plus the step's noise, and the plain call returns the same bits
     import torch
     from paper_2411_11925_b200 import api

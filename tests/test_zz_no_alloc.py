@@ -103,7 +103,7 @@ def test_static_scratch_near_the_limit_runs_the_folded_blocks():
                                     got[0], got[1], None)
     dr.ctx.sync()
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
-    # ... and in the default mode, where this shape (4 row blocks, W = 1024) takes the persistent chain kernel, the same
+    # ... and in the default mode, where this shape (4 row blocks, W = 1024) takes the wide chain kernel, the same
     # function within the rounding of the two layouts
     dr.ctx.set_chain_mode(api.Context.CHAIN_LAYERS)
     l0 = dr.ctx.launch_count()
