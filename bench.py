@@ -24,9 +24,12 @@ if ROOT not in sys.path:
 
 import numpy as np  # noqa: E402
 
-# dram__bytes_read + dram__bytes_write per launch of a kernel class, from the ncu capture summarised under
-# profiles/ for (workload, class); absent = no capture of the kernel as it stands (reported as null)
-NCU_DRAM_BYTES_PER_LAUNCH = {}
+# dram__bytes_read + dram__bytes_write per launch of a kernel class (wide_target: per csd_verify call), from the ncu capture summarised
+# under profiles/ for (workload, class); absent = no capture of the kernel as it stands (reported as null)
+NCU_DRAM_BYTES_PER_LAUNCH = {
+    # profiles/wide_chain_kernels_ncu.md: 880 MB for five of the hundred steps, both kernels
+    ("mar256", "wide_target"): 17.6e9,
+}
 
 # Sequences of each workload that the float64 checker evaluates when it is timed (the first n of the batch): the
 # CPU-baseline leg and the reference arm time the very same sample.

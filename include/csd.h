@@ -133,9 +133,8 @@ int64_t csd_launch_count(const csd_ctx *ctx);
 
 /* How the blocks of a denoising chain (the T steps of Eq. 3 for one head) are split into kernels.
  *   CSD_CHAIN_LAYERS  (default): the library picks by size.
- *                     - A chain of more than 256 head rows (R (1 + cfg); more than 384 beyond W = 1280; on one block rows x W of
- *                       2^19 at least) and up to 4608, or rows x W of 4.75 million, on a 16-bit head with W a multiple of
- *                       256 from 768 to 2048 runs as the wide chain kernel: everything that depends on the condition
+ *                     - A chain of more than 256 head rows (R (1 + cfg); on one block rows x W of 2^19 at least) and up
+ *                       to 4608, or rows x W of 4.75 million, on a 16-bit head with W a multiple of 256 from 768 to 2048 runs as the wide chain kernel: everything that depends on the condition
  *                       vector only is formed ahead, some steps at a time, and groups of W / 128 CTA pairs carry 256 or
  *                       512 rows each through the steps, the residual stream in tensor memory.  Blocks are not folded: its
  *                       error is that of three kernels per block.  The two chains of a round run side by side where

@@ -8,13 +8,15 @@ constexpr int kWcRows = 256;              // rows of a slot
 // Whether the wide chain kernel is the faster one for a head of L blocks and so many head rows.  Time over that of the layer kernels, chain
 // alone | round of two equal heads, with guidance, 20 steps (100 steps: 0.05 to 0.1 less):
 //   few rows, where a second slot is nearly empty      258: 2 x 768 1.02 | 0.84, 4 x 1024 0.97 | 0.85, 4 x 1280 0.91 | 1.00, 8 x 1536 0.99 | 1.21,
-//                                                      8 x 2048 1.00 | 1.25; 384: 8 x 1536 0.89 | 1.09, 8 x 2048 0.87 | 1.10; 514: 0.90 | 0.95, 0.78 | 0.95
+//                                                      8 x 2048 1.00 | 1.25 (100 steps 1.00 and 1.02); 514: 0.90 | 0.95, 0.78 | 0.95.  Taken all the
+//                                                      same: beside a narrower head in this kernel it is the better one (272 rows of 6 x 1024 and
+//                                                      12 x 1536, 100 steps, ms a round: 26.8; the target in layer kernels 31.4, both 29.4)
 //   one block, where a step is mostly its projections  512: 1 x 768 1.30 | 0.81, 1 x 1024 1.23 | 0.91; 1024: 1.12 | 0.72, 1.00 | 0.78; 384 of 1 x 1280 1.04 | 0.89
 //   many rows, whose tiles fill the GPU in waves       2560: 4 x 1280 0.79 | 0.81, 4 x 1536 0.86 | 0.86, 4 x 1792 0.90 | 0.83, 4 x 2048 0.92 | 0.98;
 //                                                      3400: 1.01 | 0.94, 1.03 | 1.02, 1.03 | 1.03, 1.02 | 1.04; 4608: 4 x 768 0.86 | 0.89, 4 x 1024 0.98 | 0.97
 // Beyond the last line a step's products alone are up to 1 GB, for no gain.
 inline bool wide_pays(int L, int W, int rows) {
-  if (rows <= (W > 1280 ? 384 : kWcRows) || rows > 4608) return false;
+  if (rows <= kWcRows || rows > 4608) return false;
   return (L > 1 || rows * W >= 1 << 19) && rows * W <= 4750000;
 }
 

@@ -50,7 +50,7 @@ def test_wide_chain_round_matches_checker_and_fused_round_matches_the_calls(kw):
 
 
 @pytest.mark.parametrize("rows,W,wide", [(256, 1024, False), (258, 1024, True), (4608, 768, True), (4610, 768, False), (3074, 1536, True), (1000, 640, False),
-                                         (384, 1280, True), (384, 1536, False), (386, 1536, True), (3092, 1536, True), (3094, 1536, False), (2318, 2048, True), (2320, 2048, False)])
+                                         (258, 1536, True), (3092, 1536, True), (3094, 1536, False), (2318, 2048, True), (2320, 2048, False)])
 def test_rows_and_widths_it_takes(rows, W, wide):
     from paper_2411_11925_b200.runner import DeviceRound
     dr = DeviceRound(gen.make_round_inputs(_wl(bf16=True, B=rows // 2, gamma=1, T=5, cfg=True, cfg_scale=2.0, draft=H(2, W, 64), target=H(1, 128, 64))))
