@@ -134,8 +134,9 @@ int64_t csd_launch_count(const csd_ctx *ctx);
 /* How the blocks of a denoising chain (the T steps of Eq. 3 for one head) are split into kernels.
  *   CSD_CHAIN_LAYERS  (default): the library picks by size.
  *                     - A chain of more than 256 head rows (R (1 + cfg); on one block rows x W of 2^19 at least) and up
- *                       to 4608, or rows x W of 4.75 million, on a 16-bit head with W a multiple of 256 from 768 to 2048 runs as the wide chain kernel: everything that depends on the condition
- *                       vector only is formed ahead, some steps at a time, and groups of W / 128 CTA pairs carry 256 or
+ *                       to 4608, or rows x W of 4.75 million, on a 16-bit head with W a multiple of 256 from 768 to 2048
+ *                       runs as the wide chain kernel: everything that depends on the condition vector only is
+ *                       formed ahead, some steps at a time, and groups of W / 128 CTA pairs carry 256 or
  *                       512 rows each through the steps, the residual stream in tensor memory.  Blocks are not folded: its
  *                       error is that of three kernels per block.  The two chains of a round run side by side where
  *                       their CTAs leave SMs to the condition products, else one after the other.  Its buffers, kept by
@@ -145,7 +146,8 @@ int64_t csd_launch_count(const csd_ctx *ctx);
  *                       free, chunks are shorter (the same bits); where not even one step fits, the layer kernels run.
  *                       The two chains of a round share what there is: one does not take long chunks while the other
  *                       finds no room for one step, and if one falls back both do.  Later calls ask again once there
- *                       is room.
+ *                       is room.  The blocks of a group (12 to 32, a block per SM) wait for each other: other work that keeps
+ *                       some of them from their SMs for longer than the wait limit ends the call with CSD_ERR_TIMEOUT.
  *                     - A chain of few rows on a 16-bit head with W in {512, 1024, 1536} and var_out = 0 (groups of
  *                       16 tokens, or 8 with guidance: up to 33, 15 and 7 groups) runs as the group chain kernel:
  *                       everything that depends on the condition vector only is formed ahead, for many steps at a

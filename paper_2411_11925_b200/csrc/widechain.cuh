@@ -16,11 +16,11 @@
 // What made the epilogues: words that are polled in one block of assembly (as a C++ loop ptxas held them twice and spilled: 27 k cycles more a
 // step), few and wide tensor-memory reads (a read and its wait take some 300 cycles beside running MMAs), rolled loops, projections with
 // four rows a thread so that a weight read from shared memory serves four (18 k -> 9 k cycles).  Taken back: sixteen epilogue warps
-// (96 registers: spills), a register hand-over between warpgroups by setmaxnreg (illegal instruction, cause not found), half
+// (96 registers: spills), a register hand-over between warpgroups by setmaxnreg (illegal instruction: the last warpgroup has three warps), half
 // tiles published by a warp of their own (its fence and release wait for all of the SM's stores: 15.7 -> 16.4 ms a round).
 //
-// 1024 rows each of 3 and 6 x 1024 heads, T = 100: chains alone 8.4 -> 6.8 and 15.1 -> 11.2 ms, a round 16.8 -> 14.0 ms (15.9 when repeated for
-// seconds: the GPU is at its power cap then, at 1.67 GHz instead of 1.76).  Before: one persistent kernel per chain that formed the condition
+// 1024 rows each of 3 and 6 x 1024 heads, T = 100: chains alone 8.4 -> 6.8 and 15.1 -> 11.2 ms, a single round 16.6 -> 14.0 ms (repeated for
+// seconds 16.7 -> 16.1: the GPU is at its power cap then, at 1.67 GHz instead of 1.76).  Before: one persistent kernel per chain that formed the condition
 // products itself, folded blocks.
 //
 // Accumulators and the residual stream h stay in tensor memory (128 columns each per slot).  The 16-bit operands u and v cross
